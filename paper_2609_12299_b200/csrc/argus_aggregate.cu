@@ -51,19 +51,11 @@ struct AggArgs {
   u64* iter_copies;   // global path: private copies of the iteration table, one per group of blocks (null: none)
   u32 num_copies;
   int iter_inline;    // global path taken inside k_agg_streams_compact (one read of the intervals serves both)
-  // overlap span selection in the same pass over the intervals (argus_synthesize); ov.ov_spans null = off
+  // overlap selection in the pass over the digests (argus_synthesize)
   ArgusFuseArgs ov;
-  const u64* digest;  // digests of the intervals (k_agg_streams_digest), null = read the records
+  const u64* digest;  // digests of the intervals (k_agg_streams_digest; overwritten with entries where overlap is selected), null = read the records
   u64 interval_limit; // records the interval array holds: a stream whose offsets reach beyond it is reported, not read
 };
-
-
-// The slots of a reserved chunk that the warp leaves unused are tagged, so that the list needs no clearing
-// (a warp that holds no chunk has used == the chunk size: nothing to tag).
-__device__ __forceinline__ void agg_ov_retire(const ArgusFuseArgs& ov, u64 base, u32 used, u32 lane) {
-  for (u32 i = used + lane; i < ov.ov_chunk; i += 32)
-    if (base + i < ov.ov_capacity) ov.ov_seg[base + i] = 0xffffffffu;
-}
 
 __device__ __forceinline__ bool mask_bit(const u32* mask, u32 i) { return !mask || ((mask[i >> 5] >> (i & 31)) & 1u); }
 
@@ -160,26 +152,9 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
   ArgusAggCell* const ctab = reinterpret_cast<ArgusAggCell*>(sh_raw);
   const u32 R = a.num_regions;
   const u32 cells = R * kCell;
-  const u32 lane = threadIdx.x & 31;
-  // overlap selection: bitmap of the regions that appear in a pair, and the pair list, after the table
-  u32* const pairbits = reinterpret_cast<u32*>(ctab + R);
-  u32* const pairs_sm = pairbits + (R + 31) / 32;
-  const bool has_ov = a.ov.ov_spans != nullptr && a.ov.num_pairs != 0;
   // iteration table too large for shared memory: this block's private copy in global memory (or the table itself)
   u64* const iter_base = !a.iter_inline ? nullptr
                          : a.iter_copies ? a.iter_copies + (u64)(blockIdx.x % a.num_copies) * a.num_iters * cells : a.iter_tab;
-  u64 ovc_base = 0;             // warp-uniform: current chunk of the global span list
-  u32 ovc_used = a.ov.ov_chunk;  // none held yet
-  if (has_ov) {
-    for (u32 i = threadIdx.x; i < (R + 31) / 32; i += blockDim.x) pairbits[i] = 0;
-    __syncthreads();
-    for (u32 i = threadIdx.x; i < 2 * a.ov.num_pairs; i += blockDim.x) {
-      const u32 r = a.ov.pairs[i];
-      pairs_sm[i] = r;
-      if (r < R) atomicOr(&pairbits[r >> 5], 1u << (r & 31));
-    }
-    __syncthreads();
-  }
   for (u32 s = blockIdx.x; s < a.num_streams; s += gridDim.x) {
     u64* row = a.warp_tab + (size_t)s * cells;
     // the global row takes flag counts' overflow path, bins outside the window and the ambiguity counters directly
@@ -188,63 +163,22 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
     __threadfence();
     __syncthreads();
     ArgusFuseCtx fx;
-    fx.tab = ctab; fx.pairbits = nullptr; fx.row = row; fx.sm_index = 0;
+    fx.tab = ctab; fx.row = row;
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
     const int sel = stream_in_scope(a, s);
     if (sel == 2 && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, a.cta_sm[s / a.warps_per_cta]);
-    u32 sm_index = 0;
-    if (has_ov) {
-      const u32 m = a.cta_sm[s / a.warps_per_cta];
-      if (m >= a.num_sms && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, m);
-      sm_index = m < a.num_sms ? m : 0;
-    }
     if (hi < lo || hi > a.interval_limit) {
       if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
     } else if (sel == 1) {
-      // every lane of a warp runs the same number of rounds, so that spans can be appended a warp at a time
-      for (u64 base = lo + (threadIdx.x & ~31u); base < hi; base += blockDim.x) {
-        const u64 i = base + lane;
-        bool cand = false;
-        u32 region = 0;
-        u64 t0 = 0, incl = 0;
-        if (i < hi) {
-          const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
-          const uint4 q0 = __ldg(p), q1 = __ldg(p + 1), q2 = __ldg(p + 2);
-          region = q1.z;
-          if (region >= R) {
-            argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i);
-          } else if (record_in_scope(a, q1.w, region)) {
-            t0 = (u64)q0.x | ((u64)q0.y << 32);
-            incl = (u64)q0.z | ((u64)q0.w << 32);
-            const u64 excl = (u64)q1.x | ((u64)q1.y << 32);
-            argus_fuse_aggregate(fx, region, incl, excl, q2.w >> 16);
-            if (a.iter_inline) agg_add_interval_lean(iter_base + (u64)(q1.w - a.ctx_lo) * cells, region, incl, excl, q2.w >> 16);
-            cand = has_ov && incl && ((pairbits[region >> 5] >> (region & 31)) & 1u);
-          }
-        }
-        if (has_ov && __ballot_sync(0xffffffffu, cand)) {
-          for (u32 k = 0; k < 2 * a.ov.num_pairs; ++k) {
-            const bool pick = cand && pairs_sm[k] == region;
-            const u32 bal = __ballot_sync(0xffffffffu, pick);
-            if (!bal) continue;
-            const u32 c = __popc(bal);
-            if (ovc_used + c > a.ov.ov_chunk) {
-              agg_ov_retire(a.ov, ovc_base, ovc_used, lane);
-              u64 nb64 = 0;
-              if (lane == 0) nb64 = atomicAdd(a.ov.ov_count, (u64)a.ov.ov_chunk);
-              ovc_base = __shfl_sync(0xffffffffu, nb64, 0);
-              ovc_used = 0;
-            }
-            if (pick) {
-              const u64 slot = ovc_base + ovc_used + __popc(bal & ((1u << lane) - 1u));
-              if (slot < a.ov.ov_capacity) {
-                a.ov.ov_spans[slot] = make_ulonglong2(t0, t0 + incl);
-                a.ov.ov_seg[slot] = ((k >> 1) * a.num_sms + sm_index) * 2 + (k & 1u);
-              }
-            }
-            ovc_used += c;
-          }
-        }
+      for (u64 i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
+        const uint4 q0 = __ldg(p), q1 = __ldg(p + 1), q2 = __ldg(p + 2);
+        const u32 region = q1.z;
+        if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
+        if (!record_in_scope(a, q1.w, region)) continue;
+        const u64 incl = (u64)q0.z | ((u64)q0.w << 32), excl = (u64)q1.x | ((u64)q1.y << 32);
+        argus_fuse_aggregate(fx, region, incl, excl, q2.w >> 16);
+        if (a.iter_inline) agg_add_interval_lean(iter_base + (u64)(q1.w - a.ctx_lo) * cells, region, incl, excl, q2.w >> 16);
       }
     }
     if (a.ambig && a.ambig_offsets && sel == 1) {
@@ -262,7 +196,6 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
     argus_fuse_flush(ctab, row, R, threadIdx.x, blockDim.x);
     __syncthreads();
   }
-  if (has_ov) agg_ov_retire(a.ov, ovc_base, ovc_used, lane);
 }
 
 // ---- the pass over the intervals' 8-byte digests (what argus_synthesize's pairing wrote beside the records) ----
@@ -273,8 +206,8 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
 // cells: never a bank conflict), which are folded into the region's cell when the stream ends. The last word of
 // a region's cell (meta) holds what a lane needs to know about its region: histogram window base, copy slot,
 // whether the region appears in an overlap pair. A digest marked wide (a duration of 2^23 ticks or more) sends
-// its lane to the record and to 64-bit atomics on the global row. Overlap candidates take their start time from
-// the record. The table is addressed with 32-bit shared-memory addresses and the fields by constant offsets.
+// its lane to the record and to 64-bit atomics on the global row. Every warp walks a slice of the stream, so that overlap
+// candidates stay in order; their entries replace digests that the warp has consumed: no list, no atomics. The table is addressed with 32-bit shared-memory addresses and the fields by constant offsets.
 constexpr u32 kDigestHot = 4;
 constexpr u32 kDgSumInclLo = 0, kDgSumInclHi = 1, kDgSumExclLo = 2, kDgSumExclHi = 3, kDgMin = 4, kDgMax = 5, kDgFlag = 6,
               kDgCountOut = 7, kDgBins = 8, kDgMeta = kDgBins + kAggWindow, kDgWords = kDgMeta + 1;
@@ -321,26 +254,24 @@ __device__ __noinline__ u32 digest_bin_rare(u32* meta_word, u32 bin, u32 cell, u
 // (512 threads, three blocks per SM: the same 48 warps as six blocks of 256, but a stream's set-up, the choice of its hot
 // regions and the write-back of its row are shared by twice the threads; measured 2.33 ms against 2.45 ms on trace 3)
 constexpr int kDgThreads = 512;
+constexpr u32 kDgSlices = kDgThreads / 32;     // slices of a stream, one per warp (also the slices of the overlap entries)
 __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a) {
   extern __shared__ __align__(16) unsigned char sh_raw[];
   u32* const tab = reinterpret_cast<u32*>(sh_raw);
   const u32 R = a.num_regions;
   const u32 num_cells = R + kDigestHot * 32;
   u32* const pairbits = tab + (size_t)kDgWords * num_cells;
-  u32* const pairs_sm = pairbits + (R + 31) / 32;
   __shared__ u32 hot_region[kDigestHot];
   const u32 tab_addr = (u32)__cvta_generic_to_shared(tab);
   const u32 cells = R * kCell;
   const u32 lane = threadIdx.x & 31;
-  const bool has_ov = a.ov.ov_spans != nullptr && a.ov.num_pairs != 0;
-  u64 ovc_base = 0;
-  u32 ovc_used = a.ov.ov_chunk;  // none held yet
+  const u32 warp = threadIdx.x >> 5;
+  const bool has_ov = a.ov.num_pairs != 0;
   for (u32 i = threadIdx.x; i < (R + 31) / 32; i += blockDim.x) pairbits[i] = 0;
   __syncthreads();
   if (has_ov) {
     for (u32 i = threadIdx.x; i < 2 * a.ov.num_pairs; i += blockDim.x) {
       const u32 r = a.ov.pairs[i];
-      pairs_sm[i] = r;
       if (r < R) atomicOr(&pairbits[r >> 5], 1u << (r & 31));
     }
     __syncthreads();
@@ -358,23 +289,27 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
     __threadfence();
     __syncthreads();
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
-    u32 sm_index = 0;
-    if (has_ov) {
+    if (has_ov && threadIdx.x == 0) {
       const u32 m = a.cta_sm[s / a.warps_per_cta];
-      if (m >= a.num_sms && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, m);
-      sm_index = m < a.num_sms ? m : 0;
+      if (m >= a.num_sms) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, m);
     }
+    u32 out_count = 0, out_first = 0;  // warp-uniform: entries of the warp's slice, where they start in the stream
     if (hi < lo || hi > a.interval_limit || ((hi - lo) >> 32)) {
       if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
     } else {
       const u32 n = (u32)(hi - lo);
       const u64* const dgs = a.digest + lo;
       const argus_interval_t* const ivs = a.intervals + lo;
-      // two legs: the probe (every interval into its region's cell), then, hot regions chosen, the rest of the stream
-      const u32 probe_end = n >= kDigestMinStream ? kDigestProbe : n;
+      u32 i0, i1;
+      argus_ov_slice(n, kDgSlices, warp, &i0, &i1);
+      out_first = i0;
+      u64* const ents = a.ov.entries + lo + i0;
+      u64* const starts = a.ov.starts + lo + i0;
+      // two legs: the probe (the first intervals of every slice, each into its region's cell), then, hot regions chosen, the rest
+      const u32 probe_end = n >= kDigestMinStream ? (i0 + 32 < i1 ? i0 + 32 : i1) : i1;
       for (int leg = 0; leg < 2; ++leg) {
-        const u32 leg_lo = leg ? probe_end : 0u, leg_hi = leg ? n : probe_end;
-        if (leg && leg_lo < leg_hi) {
+        const u32 leg_lo = leg ? probe_end : i0, leg_hi = leg ? i1 : probe_end;
+        if (leg && n >= kDigestMinStream) {
           // warp 0 ranks the regions by their counts so far; kDigestHot rounds of a warp-wide maximum
           if (threadIdx.x < 32) {
             for (u32 h = 0; h < kDigestHot; ++h) {
@@ -396,16 +331,19 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
           }
           __syncthreads();
         }
-        // every lane of a warp runs the same number of rounds, so that spans can be appended a warp at a time
-        u32 b = leg_lo + (threadIdx.x & ~31u);
+        // every lane of a warp runs the same number of rounds, so that entries can be appended a warp at a time
+        u32 b = leg_lo;
+        bool late = false;  // the lane's candidate of the round before: its begin time may still be on its way
+        u64 late_t0 = 0;
+        u64* late_start = nullptr;
         // digests are asked for two rounds ahead (one round is shorter than a loaded DRAM access)
-        u64 dg_next = b + lane < leg_hi ? __ldg(dgs + b + lane) : 0ull;
-        u64 dg_next2 = b + lane + kDgThreads < leg_hi ? __ldg(dgs + b + lane + kDgThreads) : 0ull;
-        for (; b < leg_hi; b += kDgThreads) {
+        u64 dg_next = b + lane < leg_hi ? dgs[b + lane] : 0ull;
+        u64 dg_next2 = b + lane + 32 < leg_hi ? dgs[b + lane + 32] : 0ull;
+        for (; b < leg_hi; b += 32) {
           const u32 i = b + lane;
           const u64 dg = dg_next;
           dg_next = dg_next2;
-          dg_next2 = i + 2 * kDgThreads < leg_hi ? __ldg(dgs + i + 2 * kDgThreads) : 0ull;
+          dg_next2 = i + 64 < leg_hi ? dgs[i + 64] : 0ull;
           const u32 dlo = (u32)dg, dhi = (u32)(dg >> 32);
           const bool in = i < leg_hi;
           const u32 region = dlo & 0xffffu;
@@ -455,34 +393,27 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
             }
           }
           const bool cand = ok && ((meta >> 16) & 1u) && span;
-          if (has_ov && __ballot_sync(0xffffffffu, cand)) {
-            u64 t0 = 0;
-            if (cand) t0 = __ldg(reinterpret_cast<const u64*>(ivs + i));
-            for (u32 k = 0; k < 2 * a.ov.num_pairs; ++k) {
-              const bool pick = cand && pairs_sm[k] == region;
-              const u32 bal = __ballot_sync(0xffffffffu, pick);
-              if (!bal) continue;
-              const u32 c = __popc(bal);
-              if (ovc_used + c > a.ov.ov_chunk) {
-                agg_ov_retire(a.ov, ovc_base, ovc_used, lane);
-                u64 nb64 = 0;
-                if (lane == 0) nb64 = atomicAdd(a.ov.ov_count, (u64)a.ov.ov_chunk);
-                ovc_base = __shfl_sync(0xffffffffu, nb64, 0);
-                ovc_used = 0;
-              }
-              if (pick) {
-                const u64 slot_o = ovc_base + ovc_used + __popc(bal & ((1u << lane) - 1u));
-                if (slot_o < a.ov.ov_capacity) {
-                  a.ov.ov_spans[slot_o] = make_ulonglong2(t0, t0 + span);
-                  a.ov.ov_seg[slot_o] = ((k >> 1) * a.num_sms + sm_index) * 2 + (k & 1u);
-                }
-              }
-              ovc_used += c;
+          const u32 bal = __ballot_sync(0xffffffffu, cand);
+          if (late) late_start[0] = late_t0;  // asked for a round ago
+          late = cand;
+          if (bal) {  // (the entries of a slice never reach the digests that are still to be read)
+            const u32 at = out_count + __popc(bal & ((1u << lane) - 1u));
+            if (cand) {
+              ents[at] = argus_entry_pack(dg, i - i0);
+              late_start = starts + at;
+              late_t0 = __ldg(reinterpret_cast<const u64*>(ivs + i));
             }
+            out_count += __popc(bal);
           }
         }
+        if (late) late_start[0] = late_t0;
         __syncthreads();
       }
+    }
+    if (has_ov && lane == 0) {
+      ArgusOvPiece e;
+      e.pos = lo + out_first; e.count = out_count; e.next = kOvNone;
+      a.ov.pieces[s * kDgSlices + warp] = e;
     }
     if (a.ambig && a.ambig_offsets) {
       const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
@@ -545,7 +476,6 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
     }
     __syncthreads();
   }
-  if (has_ov) agg_ov_retire(a.ov, ovc_base, ovc_used, lane);
 }
 
 __device__ __forceinline__ u64 combine(u32 field, u64 x, u64 y) {
@@ -708,7 +638,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
                                     size_t workspace_bytes, void* cuda_stream, bool reset_status,
                                     const ArgusFuseArgs* ov_select, const uint64_t* digest, uint64_t interval_limit) {
   if (!interval_offsets || !status || !workspace) return ARGUS_ERR_INVALID_ARG;
-  if (ov_select && (num_regions > kAggCompactRegions || ov_select->num_pairs > kFuseMaxPairs)) return ARGUS_ERR_INVALID_ARG;
+  if (ov_select && !digest) return ARGUS_ERR_INVALID_ARG;
   if (warps_per_cta == 0 || num_streams % warps_per_cta != 0) return ARGUS_ERR_INVALID_ARG;
   if (num_regions == 0 || num_regions > ARGUS_MAX_REGIONS) return ARGUS_ERR_INVALID_ARG;
   if ((sm_tab || (scope && scope->sm_mask)) && ((!cta_sm && num_streams) || num_sms == 0)) return ARGUS_ERR_INVALID_ARG;
@@ -741,7 +671,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   a.warp_mask = scope ? scope->warp_mask : ~0ull;
   a.sm_mask = scope ? scope->sm_mask : nullptr; a.region_mask = scope ? scope->region_mask : nullptr;
   a.role_tab = (u64*)role_tab; a.iter_tab = (u64*)iter_tab; a.num_iters = num_iters;
-  if (ov_select) { a.ov = *ov_select; } else { a.ov.ov_spans = nullptr; a.ov.num_pairs = 0; a.ov.ov_chunk = 256; }
+  if (ov_select) { a.ov = *ov_select; } else { a.ov = ArgusFuseArgs(); }
   a.digest = !scope && !role_tab && !iter_tab && num_regions <= kAggCompactRegions ? (const u64*)digest : nullptr;
   a.interval_limit = interval_limit;
   const size_t smem = (size_t)num_regions * sizeof(argus_agg_t);
@@ -770,11 +700,11 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   }
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 0);
   if (num_regions <= kAggCompactRegions) {
-    const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell) + ((num_regions + 31) / 32) * 4 + (size_t)a.ov.num_pairs * 8;
+    const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell);
     if (compact > 48 * 1024)
       ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_compact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)compact));
     if (a.digest) {
-      const size_t dg = digest_table_words(num_regions) * 4 + ((num_regions + 31) / 32) * 4 + (size_t)a.ov.num_pairs * 8;
+      const size_t dg = digest_table_words(num_regions) * 4 + ((num_regions + 31) / 32) * 4;
       if (dg > 48 * 1024)
         ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_digest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
       k_agg_streams_digest<<<num_streams, kDgThreads, dg, stream>>>(a);
@@ -824,9 +754,8 @@ int argus_internal_aggregate(const argus_interval_t* intervals, const uint64_t* 
                                          nullptr, interval_limit);
 }
 
-bool argus_aggregate_can_select_overlap(uint32_t num_regions, uint32_t num_pairs) {
-  return num_regions <= kAggCompactRegions && num_pairs <= kFuseMaxPairs;
-}
+bool argus_aggregate_can_read_digests(uint32_t num_regions) { return num_regions <= kAggCompactRegions; }
+uint32_t argus_aggregate_digest_slices() { return kDgSlices; }
 
 extern "C" int argus_aggregate(const argus_interval_t* intervals, const uint64_t* interval_offsets,
                                const argus_ambiguity_t* ambig, const uint64_t* ambig_offsets, uint32_t num_streams,

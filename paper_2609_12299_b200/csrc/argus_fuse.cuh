@@ -1,13 +1,11 @@
 // argus_fuse.cuh — what the pairing kernels and the aggregation passes share: the compact shared-memory
-// form of a stream's row of the warp-scope table, the 8-byte digest of an interval, and the arguments of
-// overlap span selection.
+// form of a stream's row of the warp-scope table, the 8-byte digest of an interval, and the form in which
+// intervals are handed to the overlap kernel.
 //
 // Compact row: per region the sums, min, max, counts and a 16-bin window of the 64-bin log2 histogram
 // (bins outside the window go straight to the global row); the CTA that aggregates a stream keeps the row
 // in shared memory and writes it to the global row when the stream ends. All updates are integer atomics,
 // so thread order is irrelevant.
-// Overlap selection: spans of intervals whose region appears in a (producer, consumer) pair are appended to
-// a global list tagged with their (pair, SM, role) segment; the overlap kernels take it from there.
 #ifndef ARGUS_FUSE_CUH_
 #define ARGUS_FUSE_CUH_
 
@@ -15,7 +13,6 @@
 
 constexpr u32 kAggWindow = 16;          // histogram bins kept in shared memory per region
 constexpr u32 kAggUnset = 0xffffffffu;  // window base not chosen yet
-constexpr u32 kFuseMaxPairs = 128;      // span selection keeps the pair list (8 bytes a pair) in shared memory
 constexpr u32 kAggCellWords = 72;       // u64 words of one argus_agg_t
 
 struct ArgusAggCell {  // 112 bytes
@@ -24,24 +21,42 @@ struct ArgusAggCell {  // 112 bytes
   u32 h[kAggWindow];                 // the interval count of the region is count_out + the sum of these
 };
 
-struct ArgusFuseArgs {
-  u64* warp_tab;          // unused by span selection (kept for layout)
-  const u32* cta_sm;      // [C]
-  u32 warps_per_cta, num_sms;
+// Overlap selection. The intervals whose region appears in a pair are handed to the overlap kernel as 8-byte entries, slice
+// by slice of a stream and in order. A slice is a run of consecutive intervals that one warp looks at; its entries lie in
+// one piece or in a chain of pieces. Entries from digests: the digest with the interval's place in its slice instead of the
+// exclusive duration, or, when it is wide or the place does not fit, region, wide bit and place; the piece lies where the
+// slice's digests did, so position + place is the record's index. Entries from records: index within the stream (low word),
+// region (high word).
+constexpr u32 kOvNone = 0xffffffffu;
+struct ArgusOvPiece {  // 16 bytes; piece [stream * slices + slice] is the slice's first
+  u64 pos;             // first entry
+  u32 count, next;     // entries; the slice's next piece or kOvNone
+};
+struct ArgusOvCtl {    // zeroed before the selection
+  u64 num_entries;     // entries appended (selection that appends; may exceed the room)
+  u64 num_spans;       // room asked for by the blocks of the overlap kernel (may exceed the capacity)
+  u32 num_pieces;      // later pieces taken from the pool
+  u32 asked;           // blocks that have asked for room
+};
+// Intervals [*i0, *i1) of a stream of n are slice `slice` of `slices`: whole warps' worth, equal but for the last ones.
+__device__ __forceinline__ void argus_ov_slice(u32 n, u32 slices, u32 slice, u32* i0, u32* i1) {
+  const u64 per = (((u64)n + slices - 1) / slices + 31) & ~31ull;
+  const u64 a = per * slice, b = a + per;
+  *i0 = a < n ? (u32)a : n;
+  *i1 = b < n ? (u32)b : n;
+}
+
+struct ArgusFuseArgs {    // selection inside the pass over the digests
   const u32* pairs;       // [K][2]
-  u32 num_pairs;
-  ulonglong2* ov_spans;   // appended (start, end); null = no fused overlap selection
-  u32* ov_seg;            // segment of each appended span: (pair * num_sms + sm) * 2 + role
-  u64 ov_capacity;
-  u32 ov_chunk;           // list slots a warp reserves at a time: a power of two from 32 to 256
-  u64* ov_count;          // spans appended so far (may exceed the capacity)
+  u32 num_pairs;          // 0 = no selection
+  u64* entries;           // the digest array: a warp writes the entries of its slice over the digests it has consumed
+  u64* starts;            // begin times of the entries' intervals, same positions
+  ArgusOvPiece* pieces;   // [S][slices]
 };
 
 struct ArgusFuseCtx {     // per CTA, for the stream it is aggregating
   ArgusAggCell* tab;      // shared memory [R]; null = aggregation off
-  const u32* pairbits;    // shared memory bitmap over regions: region appears in some pair; null = overlap off
   u64* row;               // global row of this stream in the warp-scope table
-  u32 sm_index;           // SM of this stream's CTA
 };
 
 // Digest of an interval (8 bytes): all that aggregation needs of it. argus_synthesize lets the pairing kernels
@@ -49,12 +64,19 @@ struct ArgusFuseCtx {     // per CTA, for the stream it is aggregating
 // instead of 48. Bits 0-15 region, 16 any flag set, 17 wide (a duration does not fit: take both from the
 // record; the duration bits then mean nothing), 18-40 inclusive, 41-63 exclusive duration.
 constexpr u32 kDigestBits = 23;
+constexpr u32 kDigestFlag = 1u << 16, kDigestWide = 1u << 17;
+constexpr u32 kEntryIndexShift = 18 + kDigestBits;        // an entry's place in its slice
 __device__ __forceinline__ u64 argus_digest_pack(u32 region, u64 incl, u64 excl, u32 flags) {
   const u32 il = (u32)incl, el = (u32)excl;
   const bool wide = (((il | el) >> kDigestBits) | (u32)(incl >> 32) | (u32)(excl >> 32)) != 0;
   const u32 lo = region | (flags ? 1u << 16 : 0u) | (wide ? 1u << 17 : 0u) | (il << 18);
   const u32 hi = ((il >> 14) & 0x1ffu) | (el << 9);
   return (u64)lo | ((u64)hi << 32);
+}
+
+__device__ __forceinline__ u64 argus_entry_pack(u64 digest, u32 place) {
+  if (((u32)digest & kDigestWide) || place >> (64 - kEntryIndexShift)) return ((u64)place << 18) | kDigestWide | ((u32)digest & 0xffffu);
+  return (digest & ((1ull << kEntryIndexShift) - 1ull)) | ((u64)place << kEntryIndexShift);
 }
 
 __device__ __forceinline__ u32 argus_log2_bin(u64 d) { return d ? 63u - (u32)__clzll((long long)d) : 0u; }

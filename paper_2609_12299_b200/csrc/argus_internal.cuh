@@ -23,8 +23,9 @@ int argus_internal_aggregate(const argus_interval_t* intervals, const uint64_t* 
                              argus_agg_t* warp_tab, argus_agg_t* cta_tab, argus_agg_t* sm_tab, argus_agg_t* kernel_tab,
                              argus_status_t* status, void* workspace, size_t workspace_bytes, void* cuda_stream,
                              bool reset_status, uint64_t interval_limit = ~0ull);
-// scope, role_tab, iter_tab nullable; ov_select (nullable): also append the overlap spans of the selected intervals;
+// scope, role_tab, iter_tab nullable;
 // digest (nullable; needs no scope, no role or iteration table, at most 400 regions): the intervals' digests, read instead of the records;
+// ov_select (nullable, needs digest): also select the overlap candidates, whose entries replace digests;
 // interval_limit: records the interval array holds (a stream whose offsets reach beyond it is reported as ARGUS_ERR_BAD_OFFSETS, not read)
 int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uint64_t* interval_offsets,
                                     const argus_ambiguity_t* ambig, const uint64_t* ambig_offsets, uint32_t num_streams,
@@ -35,7 +36,8 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
                                     size_t workspace_bytes, void* cuda_stream, bool reset_status,
                                     const ArgusFuseArgs* ov_select, const uint64_t* digest = nullptr,
                                     uint64_t interval_limit = ~0ull);
-bool argus_aggregate_can_select_overlap(uint32_t num_regions, uint32_t num_pairs);
+bool argus_aggregate_can_read_digests(uint32_t num_regions);
+uint32_t argus_aggregate_digest_slices();  // slices per stream in which that pass selects overlap candidates
 
 // argus_ring.cu — stream_offsets (and dropped) of the records that survive in the slots of a ring container;
 // status->code = ARGUS_ERR_CAPACITY if they exceed event_capacity. The status block is not cleared.
@@ -47,9 +49,12 @@ int argus_internal_overlap(const argus_interval_t* intervals, uint64_t max_inter
                            uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm, uint32_t num_sms,
                            const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out, argus_status_t* status,
                            void* workspace, size_t workspace_bytes, void* cuda_stream, bool reset_status);
-// overlap from a list of selected spans (spans + segment of each; *list_count slots reserved, unused ones tagged 0xffffffff)
-int argus_internal_overlap_from_list(const void* list_spans, const uint32_t* list_seg, const uint64_t* list_count,
-                                     uint64_t list_capacity, uint32_t num_sms, uint32_t num_pairs, argus_overlap_t* out,
-                                     argus_status_t* status, void* workspace, size_t workspace_bytes, void* cuda_stream);
+size_t argus_internal_overlap_bytes(uint64_t max_spans, uint32_t num_streams);  // workspace for at most max_spans selected spans
+// overlap from what the pass over the digests selected; `starts`: begin times, at the entries' positions; `spans`: 32 bytes for
+// each of max_spans
+int argus_internal_overlap_from_digests(const argus_interval_t* intervals, const uint64_t* starts, const uint64_t* entries, const ArgusOvPiece* pieces,
+                                        uint32_t slices, uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm,
+                                        uint32_t num_sms, const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out,
+                                        argus_status_t* status, ArgusOvCtl* ctl, void* spans, uint64_t max_spans, void* cuda_stream);
 
 #endif  // ARGUS_INTERNAL_CUH_

@@ -1,42 +1,43 @@
 // argus_overlap.cu — argus_overlap: per-SM overlap time of producer/consumer region pairs.
 //
-// Segment = (pair k, SM m, role) with role 0 = producer, 1 = consumer.
-//   k_ov_select  : one pass over the intervals: selected spans appended to an unordered list with their segment
-//                  (argus_synthesize gets the same list from the aggregation pass or the pairing kernel instead)
-//   k_ov_list_count_or_scatter : spans counted per segment, then copied into their segment (order irrelevant)
-//   k_ov_scan    : segment bases; capacity check
-//   k_ov_sort    : one CTA per segment: sort by (start, end) — by buckets of start time with one warp per bucket,
-//                  or by a bitonic network on shared-memory tiles when the starts crowd; then turn the sorted spans into the
-//                  disjoint pieces of their union, piece i = [max(start_i, E_{i-1}), E_i) with
-//                  E_i = max end of spans 0..i, and the running length before each piece
-//   k_ov_measure : one CTA per (k, m): |U_P|, |U_C|, and |U_P ∩ U_C| = sum over producer pieces of
-//                  F_C(b) - F_C(a), F_C(t) = covered length of U_C before t (threads walk runs of producer pieces
-//                  and find each boundary among the C pieces from the one before)
+//   k_ov_select : one pass over the intervals: those whose region appears in a pair are appended, slice by slice of a
+//                 stream and in order, as entries {index within the stream, region} (argus_synthesize gets the same
+//                 entries from the aggregation pass, which writes them over the digests that it has consumed)
+//   k_ov_pair   : one block per (pair k, SM m): gathers the spans of the producer and of the consumer region from the
+//                 entries of the SM's streams, in stream and slice order; sorts a role by start time if it is not in order
+//                 already and cuts it into the disjoint pieces of its union if its spans overlap one another; then walks
+//                 the merged sequence of both roles, where every piece meets the last piece of the other role:
+//                 |U_P ∩ U_C| in one pass, |U_P| and |U_C| being sums of lengths.
+//
+// A region that is not nested in itself leaves its spans of one stream disjoint and in time order. The entries are kept in
+// order, so a role that sits in one warp of a CTA needs no sort, and spans of several warps are runs that need few merges.
 #include "argus_internal.cuh"
+
+#include <atomic>
 
 namespace {
 
-constexpr int kOvThreads = 1024;
-constexpr u32 kMaxPairs = ARGUS_MAX_PAIRS;
+constexpr int kSelThreads = 256;
+constexpr u32 kSelWarps = kSelThreads / 32;
+constexpr u32 kSelStage = 128;    // entries a warp collects before it appends them
+constexpr u32 kSelFilter = 4096;  // bits of the region filter
+constexpr unsigned kSelGrid = 148 * 8;
 
-struct OvArgs {
+struct OvSelectArgs {
   const argus_interval_t* intervals;
   const u64* interval_offsets;
   u64 max_intervals;  // records the interval array holds
   u32 num_streams, warps_per_cta, num_sms, num_pairs;
   const u32* cta_sm;
   const u32* pairs;
-  argus_overlap_t* out;
   argus_status_t* status;
-  u64* seg_count;   // [nseg]     (zeroed)
-  u64* seg_cursor;  // [nseg]     (zeroed)
-  u64* seg_base;    // [nseg + 1]
-  ulonglong2* spans;  // [capacity] (start, end) -> after k_ov_sort (piece begin, piece end)
-  ulonglong2* scratch;  // room k_ov_sort may use (the span list, which is dead by then); null = none
-  u64 scratch_capacity;
-  u64* cum;           // [capacity] covered length before piece i within its segment
-  u64 capacity;
-  u32 nseg;
+  u64* entries;
+  u64 entry_capacity;
+  ArgusOvPiece* pieces;  // [num_streams * slices] first pieces, then the pool of later ones
+  u32 slices;            // per stream, a multiple of kSelWarps
+  u32 piece_capacity;
+  int direct;            // the entry array has a place for every interval: a slice's entries start at its first interval's
+  ArgusOvCtl* ctl;
   // scope selection (argus_overlap_scoped): iteration window, warp mask, SM mask, region mask
   int scoped;
   u32 ctx_lo, ctx_hi;
@@ -47,590 +48,738 @@ struct OvArgs {
 
 __device__ __forceinline__ bool ov_mask_bit(const u32* mask, u32 i) { return !mask || ((mask[i >> 5] >> (i & 31)) & 1u); }
 
-// One pass over the intervals: spans of intervals whose region appears in a pair are appended to an unordered
-// list with their segment. A warp reserves `chunk` list slots at a time (one global atomic per chunk) and
-// marks the slots it leaves unused, so the list needs no clearing.
-struct OvSelectOut {
-  ulonglong2* spans;
-  u32* seg;
-  u64* count;      // slots reserved so far (zeroed before the kernel)
-  u64 capacity;
-  u32 chunk;       // power of two, at most 256
-};
-
-__device__ __forceinline__ void ov_retire_chunk(const OvSelectOut& o, u64 base, u32 used, u32 lane) {
-  for (u32 i = used + lane; i < o.chunk; i += 32)
-    if (base + i < o.capacity) o.seg[base + i] = 0xffffffffu;
-}
-
-__global__ void __launch_bounds__(256) k_ov_select(OvArgs a, OvSelectOut o) {
-  __shared__ u32 sh_pairs[2 * kMaxPairs];
-  for (u32 i = threadIdx.x; i < 2 * a.num_pairs; i += blockDim.x) sh_pairs[i] = a.pairs[i];
+// Bound by HBM: the 32-byte sectors of a record that hold its duration, region and ctx. A warp walks one slice of a stream.
+// Where the workspace has a place for every interval the entries go straight to their slice's; else the warp collects them
+// and appends about 100 at a time, exactly as many places as it needs, as pieces of a chain.
+__global__ void __launch_bounds__(kSelThreads) k_ov_select(OvSelectArgs a) {
+  __shared__ u32 filter[kSelFilter / 32];
+  __shared__ u32 sh_pairs[2 * ARGUS_MAX_PAIRS];
+  __shared__ u64 stage[kSelWarps][kSelStage];
+  for (u32 i = threadIdx.x; i < kSelFilter / 32; i += blockDim.x) filter[i] = 0;
   __syncthreads();
-  const u32 lane = threadIdx.x & 31;
-  u64 ovc_base = 0;          // warp-uniform: the chunk this warp is filling
-  u32 ovc_used = o.chunk;    // chunk size = none held yet
-  bool held = false;
-  for (u32 s = blockIdx.x; s < a.num_streams; s += gridDim.x) {
+  for (u32 i = threadIdx.x; i < 2 * a.num_pairs; i += blockDim.x) {
+    const u32 r = a.pairs[i];
+    sh_pairs[i] = r;
+    atomicOr(&filter[(r & (kSelFilter - 1)) >> 5], 1u << (r & 31));
+  }
+  __syncthreads();
+  const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 parts = a.slices / kSelWarps, heads = a.num_streams * a.slices;
+  u64* const mine = stage[warp];
+  for (u64 item = blockIdx.x; item < (u64)a.num_streams * parts; item += gridDim.x) {
+    const u32 s = (u32)(item / parts), slice = (u32)(item % parts) * kSelWarps + warp;
+    const u32 head = s * a.slices + slice;
     const u32 m = a.cta_sm[s / a.warps_per_cta];
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
-    if (m >= a.num_sms || hi < lo || hi > a.max_intervals) {  // offsets beyond the interval array are reported, not read
+    bool take = true;
+    if (m >= a.num_sms || hi < lo || hi > a.max_intervals || ((hi - lo) >> 32)) {  // offsets beyond the interval array are reported, not read
       if (threadIdx.x == 0) argus_set_error(a.status, m >= a.num_sms ? ARGUS_ERR_INVALID_ARG : ARGUS_ERR_BAD_OFFSETS, s, m);
-      continue;
-    }
-    if (a.scoped) {  // warp-role and SM tests: one answer per stream
+      take = false;
+    } else if (a.scoped) {  // warp-role and SM tests: one answer per stream
       const u32 w = s % a.warps_per_cta;
-      if (a.warp_mask != ~0ull && (w >= 64 || !((a.warp_mask >> w) & 1ull))) continue;
-      if (!ov_mask_bit(a.sm_mask, m)) continue;
+      if (a.warp_mask != ~0ull && (w >= 64 || !((a.warp_mask >> w) & 1ull))) take = false;
+      if (!ov_mask_bit(a.sm_mask, m)) take = false;
     }
-    // every lane of a warp runs the same number of rounds, so that spans can be appended a warp at a time
-    for (u64 base = lo + (threadIdx.x & ~31u); base < hi; base += blockDim.x) {
-      const u64 i = base + lane;
+    const u32 n = take ? (u32)(hi - lo) : 0u;
+    u32 i0, i1;
+    argus_ov_slice(n, a.slices, slice, &i0, &i1);
+    const argus_interval_t* const ivs = a.intervals + lo;
+    u64* const to = a.direct ? a.entries + lo + i0 : mine;
+    u32 held = 0, last = head, total_pieces = 0;
+    if (lane == 0) { ArgusOvPiece e; e.pos = 0; e.count = 0; e.next = kOvNone; a.pieces[head] = e; }
+    for (u32 base = i0; base < i1 || (held && !a.direct); base += 32) {
+      const bool end = base >= i1;
+      u32 bal = 0, region = 0;
       bool cand = false;
-      u32 region = 0;
-      u64 t0 = 0, incl = 0;
-      if (i < hi) {
-        const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
-        const uint4 q0 = __ldg(p);
-        incl = (u64)q0.z | ((u64)q0.w << 32);
-        t0 = (u64)q0.x | ((u64)q0.y << 32);
-        region = __ldg(reinterpret_cast<const u32*>(p + 1) + 2);
-        cand = incl != 0;
-        if (cand && a.scoped) {  // iteration-window and region tests: one answer per interval
-          const u32 ctx = __ldg(reinterpret_cast<const u32*>(p + 1) + 3);
-          cand = ctx >= a.ctx_lo && ctx <= a.ctx_hi && ov_mask_bit(a.region_mask, region);
+      if (!end) {
+        const u32 i = base + lane;
+        if (i < i1) {
+          const uint4* p = reinterpret_cast<const uint4*>(ivs + i);
+          const u64 incl = __ldg(reinterpret_cast<const u64*>(p) + 1);
+          const uint2 rc = __ldg(reinterpret_cast<const uint2*>(p + 1) + 1);
+          region = rc.x;
+          cand = incl != 0 && ((filter[(region & (kSelFilter - 1)) >> 5] >> (region & 31)) & 1u);
+          // iteration-window and region tests: one answer per interval
+          if (cand && a.scoped) cand = rc.y >= a.ctx_lo && rc.y <= a.ctx_hi && ov_mask_bit(a.region_mask, region);
         }
-      }
-      for (u32 k = 0; k < 2 * a.num_pairs; ++k) {
-        const bool pick = cand && sh_pairs[k] == region;
-        const u32 bal = __ballot_sync(0xffffffffu, pick);
-        if (!bal) continue;
-        u32 todo = __popc(bal), done = 0;
-        while (todo) {  // a ballot may straddle chunks when the chunks are small
-          if (ovc_used == o.chunk) {
-            u64 nb64 = 0;
-            if (lane == 0) nb64 = atomicAdd(reinterpret_cast<unsigned long long*>(o.count), (unsigned long long)o.chunk);
-            ovc_base = __shfl_sync(0xffffffffu, nb64, 0);
-            ovc_used = 0;
-            held = true;
+        bal = __ballot_sync(0xffffffffu, cand);
+        if (bal) {  // the filter lets a few other regions through
+          if (cand) {
+            bool hit = false;
+            for (u32 k = 0; k < 2 * a.num_pairs && !hit; ++k) hit = sh_pairs[k] == region;
+            cand = hit;
           }
-          const u32 room = o.chunk - ovc_used, take = todo < room ? todo : room;
-          if (pick) {
-            const u32 rank = __popc(bal & ((1u << lane) - 1u));
-            if (rank >= done && rank < done + take) {
-              const u64 slot = ovc_base + ovc_used + (rank - done);
-              if (slot < o.capacity) {
-                o.spans[slot] = make_ulonglong2(t0, t0 + incl);
-                o.seg[slot] = ((k >> 1) * a.num_sms + m) * 2 + (k & 1u);
-              }
-            }
-          }
-          ovc_used += take; done += take; todo -= take;
+          bal = __ballot_sync(0xffffffffu, cand);
         }
-      }
-    }
-  }
-  if (held) ov_retire_chunk(o, ovc_base, ovc_used, lane);
-}
-
-// Same two roles for spans that the pairing kernel already selected: list entries carry their segment;
-// entries of reserved but unused slots have segment 0xffffffff.
-struct OvList {
-  const ulonglong2* spans;
-  const u32* seg;
-  const u64* count;  // slots reserved (may exceed capacity)
-  u64 capacity;
-};
-
-constexpr u32 kOvListSegs = 2048;   // segments a block can count in shared memory
-constexpr u32 kOvListChunk = 8192;  // list entries a block handles per iteration
-
-__global__ void __launch_bounds__(256) k_ov_list_count_or_scatter(OvArgs a, OvList l, int scatter) {
-  __shared__ u32 sh_cnt[kOvListSegs];
-  __shared__ u64 sh_base[kOvListSegs];
-  if (scatter && a.status->code != 0) return;
-  const u64 reserved = *l.count;
-  if (reserved > l.capacity && blockIdx.x == 0 && threadIdx.x == 0) {
-    argus_set_error(a.status, ARGUS_ERR_CAPACITY, 0, reserved);
-    a.status->intervals_required = reserved;
-  }
-  const u64 n = reserved < l.capacity ? reserved : l.capacity;
-  const bool local = a.nseg <= kOvListSegs;
-  for (u64 c0 = (u64)blockIdx.x * kOvListChunk; c0 < n; c0 += (u64)gridDim.x * kOvListChunk) {
-    const u64 c1 = c0 + kOvListChunk < n ? c0 + kOvListChunk : n;
-    if (!local) {  // too many segments for shared counters: global atomics per entry
-      for (u64 i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-        const u32 seg = l.seg[i];
-        if (seg >= a.nseg) continue;
-        if (!scatter) atomicAdd(&a.seg_count[seg], 1ull);
-        else {
-          const u64 slot = a.seg_base[seg] + atomicAdd(&a.seg_cursor[seg], 1ull);
-          if (slot < a.capacity) a.spans[slot] = l.spans[i];
-        }
-      }
-      continue;
-    }
-    for (u32 g = threadIdx.x; g < a.nseg; g += blockDim.x) sh_cnt[g] = 0;
-    __syncthreads();
-    for (int pass = 0; pass < (scatter ? 2 : 1); ++pass) {
-      for (u64 i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-        const u32 seg = l.seg[i];
-        if (seg >= a.nseg) continue;
-        const u32 pos = atomicAdd(&sh_cnt[seg], 1u);
-        if (pass == 1) {
-          const u64 slot = sh_base[seg] + pos;
-          if (slot < a.capacity) a.spans[slot] = l.spans[i];
-        }
-      }
-      __syncthreads();
-      for (u32 g = threadIdx.x; g < a.nseg; g += blockDim.x) {
-        if (pass == 0 && sh_cnt[g]) {
-          if (!scatter) atomicAdd(&a.seg_count[g], (u64)sh_cnt[g]);
-          else sh_base[g] = a.seg_base[g] + atomicAdd(&a.seg_cursor[g], (u64)sh_cnt[g]);
-        }
-        sh_cnt[g] = 0;
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kOvThreads) k_ov_scan(OvArgs a) {
-  __shared__ u64 sh[33];
-  u64 carry = 0;
-  for (u32 g0 = 0; g0 < a.nseg; g0 += kOvThreads) {
-    const u32 g = g0 + threadIdx.x;
-    const u64 c = g < a.nseg ? a.seg_count[g] : 0;
-    u64 total;
-    const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
-    if (g < a.nseg) a.seg_base[g] = carry + ex;
-    carry += total;
-  }
-  if (threadIdx.x == 0) {
-    a.seg_base[a.nseg] = carry;
-    if (carry > a.capacity) {
-      argus_set_error(a.status, ARGUS_ERR_CAPACITY, 0, carry);
-      a.status->intervals_required = carry;
-    }
-  }
-}
-
-__device__ __forceinline__ bool span_less(const ulonglong2& x, const ulonglong2& y) {
-  return x.x < y.x || (x.x == y.x && x.y < y.y);
-}
-
-__device__ __forceinline__ void cmp_swap(ulonglong2* d, u64 i, u64 l) {
-  const ulonglong2 x = d[i], y = d[l];
-  if (span_less(y, x)) { d[i] = y; d[l] = x; }
-}
-
-constexpr u32 kOvSortTile = 4096;  // spans of a segment sorted in shared memory at a time (64 KB)
-
-// Stages of the network whose partners lie inside one tile, on the tile in shared memory: the flip of block size k
-// (if `flip`) and then the distances j_top, j_top / 2, ..., 1. `tbase` is the tile's first index in the segment.
-// (every thread takes whole comparators: comparator c of a stage with distance bit h joins i = c with a zero
-// inserted at bit h, and its partner)
-__device__ __forceinline__ void ov_sort_tile_stages(ulonglong2* t, u64 tbase, u64 n, u32 k, bool flip, u32 j_top) {
-  if (flip) {
-    const u32 h = k >> 1;
-    for (u32 c = threadIdx.x; c < kOvSortTile / 2; c += blockDim.x) {
-      const u32 i = ((c & ~(h - 1)) << 1) | (c & (h - 1)), l = i ^ (k - 1);
-      if (tbase + l < n) cmp_swap(t, i, l);
-    }
-    __syncthreads();
-  }
-  for (u32 j = j_top; j > 0; j >>= 1) {
-    for (u32 c = threadIdx.x; c < kOvSortTile / 2; c += blockDim.x) {
-      const u32 i = ((c & ~(j - 1)) << 1) | (c & (j - 1)), l = i | j;
-      if (tbase + l < n) cmp_swap(t, i, l);
-    }
-    __syncthreads();
-  }
-}
-
-// Sort of a large segment in expected linear time: spans are spread over buckets of equal width in start time (about 32
-// a bucket for starts spread evenly), copied to `scratch` bucket by bucket, and every bucket is sorted by one warp with a
-// small bitonic network in shared memory and written back in place. Returns false, with `d` untouched, when some bucket
-// would hold more than kOvBucketMax spans (starts crowded in time): the caller then runs the full network.
-// Shared memory (kOvSortSmem bytes at `raw`): bucket offsets, bucket cursors, one slice of kOvBucketMax spans per warp.
-constexpr u32 kOvBucketMax = 128;
-constexpr u32 kOvBuckets = 4096;
-constexpr size_t kOvSortSmem = 2 * (kOvBuckets + 1) * 4 + 32 + (size_t)(kOvThreads / 32) * kOvBucketMax * sizeof(ulonglong2);
-
-__device__ bool ov_bucket_sort(ulonglong2* d, ulonglong2* scratch, u64 n, unsigned char* raw) {
-  u32* const off = reinterpret_cast<u32*>(raw);                 // [kOvBuckets + 1]
-  u32* const cur = off + kOvBuckets + 1;                        // [kOvBuckets + 1]
-  ulonglong2* const slices = reinterpret_cast<ulonglong2*>(raw + ((2 * (kOvBuckets + 1) * 4 + 15) & ~(size_t)15));
-  __shared__ u64 red[2][32];
-  __shared__ u32 sh_scan[33];
-  __shared__ u32 crowded;
-  const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (n >> 31) return false;
-  // range of the start times
-  u64 mn = ~0ull, mx = 0;
-  for (u64 i = threadIdx.x; i < n; i += blockDim.x) {
-    const u64 s = d[i].x;
-    mn = s < mn ? s : mn;
-    mx = s > mx ? s : mx;
-  }
-#pragma unroll
-  for (int dd = 16; dd > 0; dd >>= 1) {
-    const u64 a = __shfl_xor_sync(0xffffffffu, mn, dd), b = __shfl_xor_sync(0xffffffffu, mx, dd);
-    mn = a < mn ? a : mn;
-    mx = b > mx ? b : mx;
-  }
-  if (lane == 0) { red[0][warp] = mn; red[1][warp] = mx; }
-  if (threadIdx.x == 0) crowded = 0;
-  __syncthreads();
-  mn = red[0][0]; mx = red[1][0];
-  for (u32 w = 1; w < blockDim.x / 32; ++w) {
-    mn = red[0][w] < mn ? red[0][w] : mn;
-    mx = red[1][w] > mx ? red[1][w] : mx;
-  }
-  // buckets: a power of two of them, about 32 spans each; equal width, a power of two of ticks
-  u32 nb = 1;
-  while (nb < kOvBuckets && (u64)nb * 32 < n) nb <<= 1;
-  u32 shift = 0;
-  while (((mx - mn) >> shift) >= nb) ++shift;
-  for (u32 b = threadIdx.x; b <= nb; b += blockDim.x) { off[b] = 0; cur[b] = 0; }
-  __syncthreads();
-  for (u64 i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&off[(u32)((d[i].x - mn) >> shift)], 1u);
-  __syncthreads();
-  for (u32 b = threadIdx.x; b < nb; b += blockDim.x)
-    if (off[b] > kOvBucketMax) crowded = 1;
-  __syncthreads();
-  if (crowded) return false;  // uniform: every thread read the same word after the barrier
-  // exclusive prefix of the counts (nb <= 4 x 1024)
-  u32 carry = 0;
-  for (u32 b0 = 0; b0 < nb; b0 += blockDim.x) {
-    const u32 b = b0 + threadIdx.x;
-    const u32 c = b < nb ? off[b] : 0u;
-    u32 total;
-    const u32 ex = argus_block_exclusive_scan<u32>(c, sh_scan, &total);
-    if (b < nb) off[b] = carry + ex;
-    carry += total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) off[nb] = (u32)n;
-  __syncthreads();
-  for (u64 i = threadIdx.x; i < n; i += blockDim.x) {
-    const ulonglong2 sp = d[i];
-    const u32 b = (u32)((sp.x - mn) >> shift);
-    scratch[off[b] + atomicAdd(&cur[b], 1u)] = sp;
-  }
-  __syncthreads();
-  // one warp per bucket: small network in the warp's slice, then back in place (buckets are in time order)
-  ulonglong2* const sl = slices + (size_t)warp * kOvBucketMax;
-  for (u32 b = warp; b < nb; b += blockDim.x / 32) {
-    const u32 lo = off[b], c = off[b + 1] - lo;
-    if (c == 0) continue;
-    u32 m = 1;
-    while (m < c) m <<= 1;
-    for (u32 t = lane; t < m; t += 32) sl[t] = t < c ? scratch[lo + t] : make_ulonglong2(~0ull, ~0ull);
-    __syncwarp();
-    for (u32 k = 2; k <= m; k <<= 1) {
-      const u32 h = k >> 1;
-      for (u32 q = lane; q < m / 2; q += 32) {
-        const u32 i = ((q & ~(h - 1)) << 1) | (q & (h - 1));
-        cmp_swap(sl, i, i ^ (k - 1));
-      }
-      __syncwarp();
-      for (u32 j = k >> 2; j > 0; j >>= 1) {
-        for (u32 q = lane; q < m / 2; q += 32) {
-          const u32 i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
-          cmp_swap(sl, i, i | j);
-        }
+        if (cand) to[held + __popc(bal & ((1u << lane) - 1u))] = (u64)i | ((u64)region << 32);
+        held += __popc(bal);
         __syncwarp();
       }
+      if (!a.direct && (held > kSelStage - 32 || end)) {
+        u64 pos = 0;
+        u32 piece = head;
+        if (lane == 0) {
+          pos = atomicAdd(&a.ctl->num_entries, (u64)held);
+          if (total_pieces) piece = heads + atomicAdd(&a.ctl->num_pieces, 1u);
+        }
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        piece = __shfl_sync(0xffffffffu, piece, 0);
+        if (pos + held <= a.entry_capacity && piece < a.piece_capacity) {  // else the counter tells that they did not fit
+          for (u32 t = lane; t < held; t += 32) a.entries[pos + t] = mine[t];
+          if (lane == 0) {
+            ArgusOvPiece e; e.pos = pos; e.count = held; e.next = kOvNone;
+            a.pieces[piece] = e;
+            if (total_pieces) a.pieces[last].next = piece;
+          }
+          last = piece;
+          ++total_pieces;
+        }
+        held = 0;
+        __syncwarp();
+        if (end) break;
+      }
     }
-    for (u32 t = lane; t < c; t += 32) d[lo + t] = sl[t];
+    if (a.direct && lane == 0) { ArgusOvPiece e; e.pos = lo + i0; e.count = held; e.next = kOvNone; a.pieces[head] = e; }
     __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------------------------------------------------------------
+constexpr int kPairThreads = 1024;
+constexpr u32 kPairWarps = kPairThreads / 32;
+constexpr u32 kVT = 9;                                 // spans a thread merges at a time (odd: lanes that far apart hit different banks)
+constexpr u32 kTile = kPairThreads * kVT;              // spans in shared memory at a time (144 KB)
+constexpr u32 kBatch = kPairThreads;                   // slices whose spans are placed at a time
+constexpr u32 kGather = 4;                             // entries a thread asks for at a time
+constexpr size_t kPairSmem = (size_t)kTile * sizeof(ulonglong2);
+
+struct OvPairArgs {
+  const argus_interval_t* intervals;
+  const u64* interval_offsets;
+  const u64* starts;    // begin times, at the entries' positions (entries from digests)
+  const u64* entries;
+  const ArgusOvPiece* pieces;
+  u32 slices, num_streams, warps_per_cta, num_sms, num_pairs, blocks;
+  const u32* cta_sm;
+  const u32* pairs;
+  argus_overlap_t* out;
+  argus_status_t* status;
+  ulonglong2* spans;    // [capacity] (start, end) of the producer role, from the block's base on; what it leaves, the other side of a merge
+  ulonglong2* scratch;  // [capacity] the same for the consumer role
+  u64 capacity, entry_capacity;
+  ArgusOvCtl* ctl;
+};
+
+__device__ __forceinline__ bool before_or_at(const ulonglong2& x, const ulonglong2& y) { return x.x <= y.x; }
+
+// Number of the first `diag` elements of the merge of A and B that come from A (elements of A first on ties).
+__device__ __forceinline__ u32 merge_split(const ulonglong2* A, u32 na, const ulonglong2* B, u32 nb, u32 diag) {
+  u32 lo = diag > nb ? diag - nb : 0u, hi = diag < na ? diag : na;
+  while (lo < hi) {
+    const u32 mid = (lo + hi) >> 1;
+    if (before_or_at(A[mid], B[diag - 1 - mid])) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// The same by one warp, 32 probes a round (for arrays in global memory, where a probe is a round trip to the L2).
+__device__ __forceinline__ u64 merge_split_warp(const ulonglong2* A, u64 na, const ulonglong2* B, u64 nb, u64 diag, u32 lane) {
+  u64 lo = diag > nb ? diag - nb : 0ull, hi = diag < na ? diag : na;
+  while (lo < hi) {
+    const u64 step = (hi - lo + 31) >> 5, mid = lo + lane * step;
+    const bool yes = mid < hi && __ldcg(&A[mid].x) <= __ldcg(&B[diag - 1 - mid].x);
+    const u32 c = __popc(__ballot_sync(0xffffffffu, yes));  // the probes that say yes come first
+    if (c == 0) break;
+    const u64 nlo = lo + (c - 1) * step + 1, nhi = lo + c * step;
+    lo = nlo;
+    if (nhi < hi) hi = nhi;
+  }
+  return lo;
+}
+
+// One thread's share of a merge in shared memory: kVT elements from A[a..na) and B[b..nb) into registers; elements past the
+// end of both are left alone.
+__device__ __forceinline__ void merge_serial(const ulonglong2* A, u32 a, u32 na, const ulonglong2* B, u32 b, u32 nb, ulonglong2 (&v)[kVT]) {
+#pragma unroll
+  for (u32 j = 0; j < kVT; ++j) {
+    if (a < na || b < nb) {
+      const ulonglong2 x = A[a < na ? a : 0], y = B[b < nb ? b : 0];
+      const bool take_a = b >= nb || (a < na && before_or_at(x, y));
+      v[j] = take_a ? x : y;
+      if (take_a) ++a; else ++b;
+    }
+  }
+}
+
+// Sorts t[0..cnt) in shared memory by start time: kVT elements a thread in registers, then merges of doubling width.
+__device__ __noinline__ void sort_tile(ulonglong2* t, u32 cnt) {
+  const u32 at = threadIdx.x * kVT;
+  ulonglong2 v[kVT];
+  if (at < cnt) {
+#pragma unroll
+    for (u32 j = 0; j < kVT; ++j) v[j] = at + j < cnt ? t[at + j] : make_ulonglong2(~0ull, ~0ull);
+#pragma unroll
+    for (u32 r = 0; r < kVT; ++r)  // odd-even transposition
+#pragma unroll
+      for (u32 j = r & 1u; j + 1 < kVT; j += 2)
+        if (v[j + 1].x < v[j].x) { const ulonglong2 x = v[j]; v[j] = v[j + 1]; v[j + 1] = x; }
+    // (padding has the largest key; equal keys keep their order, so padding stays last)
+#pragma unroll
+    for (u32 j = 0; j < kVT; ++j) if (at + j < cnt) t[at + j] = v[j];
+  }
+  __syncthreads();
+  for (u32 width = kVT; width < cnt; width <<= 1) {
+    const u32 a0 = at / (2 * width) * (2 * width), b0 = a0 + width < cnt ? a0 + width : cnt, e0 = a0 + 2 * width < cnt ? a0 + 2 * width : cnt;
+    const bool work = at < cnt && b0 < e0 && t[b0].x < t[b0 - 1].x;  // runs that follow one another need no merge
+    if (work) {
+      const u32 na = b0 - a0, nb = e0 - b0, diag = at - a0;
+      const u32 a = merge_split(t + a0, na, t + b0, nb, diag);
+      merge_serial(t + a0, a, na, t + b0, diag - a, nb, v);
+    }
+    __syncthreads();
+    if (work) {
+#pragma unroll
+      for (u32 j = 0; j < kVT; ++j) if (at + j < cnt) t[at + j] = v[j];
+    }
+    __syncthreads();
+  }
+}
+
+// Sorts d[0..n) in global memory by start time; `scratch` has as much room. Returns where the sorted spans lie.
+__device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratch, u64 n, ulonglong2* t, u64* sh) {
+  for (u64 t0 = 0; t0 < n; t0 += kTile) {
+    const u32 cnt = (u32)(n - t0 < kTile ? n - t0 : kTile);
+    for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) t[i] = d[t0 + i];
+    __syncthreads();
+    sort_tile(t, cnt);
+    for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) d[t0 + i] = t[i];
+    __syncthreads();
+  }
+  const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (u64 width = kTile; width < n; width <<= 1) {
+    for (u64 t0 = 0; t0 < n; t0 += kTile) {  // every tile of the output lies inside one merge (widths are multiples of a tile)
+      const u64 a0 = t0 / (2 * width) * (2 * width), b0 = a0 + width < n ? a0 + width : n, e0 = a0 + 2 * width < n ? a0 + 2 * width : n;
+      const u64 d0 = t0 - a0, d1 = (t0 + kTile < e0 ? t0 + kTile : e0) - a0;
+      if (warp < 2) {
+        const u64 sp = merge_split_warp(d + a0, b0 - a0, d + b0, e0 - b0, warp ? d1 : d0, lane);
+        if (lane == 0) sh[warp] = sp;
+      }
+      __syncthreads();
+      const u64 aA = sh[0], aB = sh[1];
+      const u32 na = (u32)(aB - aA), cnt = (u32)(d1 - d0), nb = cnt - na;
+      for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) t[i] = i < na ? d[a0 + aA + i] : d[b0 + (d0 - aA) + (i - na)];
+      __syncthreads();
+      const u32 at = threadIdx.x * kVT;
+      ulonglong2 v[kVT];
+      if (at < cnt) {
+        const u32 a = merge_split(t, na, t + na, nb, at);
+        merge_serial(t, a, na, t + na, at - a, nb, v);
+      }
+      __syncthreads();
+#pragma unroll
+      for (u32 j = 0; j < kVT; ++j) if (at + j < cnt) t[at + j] = v[j];
+      __syncthreads();
+      for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) scratch[t0 + i] = t[i];
+      __syncthreads();
+    }
+    ulonglong2* const x = d; d = scratch; scratch = x;
+  }
+  return d;
+}
+
+// Sort of both roles together, up to kTile spans (in0[0..n0), in1[0..n1); a role that is in order already comes with n = 0),
+// into out0 and out1: spans are spread over buckets of equal width in start time, about one for a span, and a span's place is
+// the number of earlier ones in its bucket. Elements are 8 bytes, start time relative to the role's earliest (50 bits) and place (14
+// bits); the spans follow once (4,096 spans a role: 20 us; merging runs pairwise took 50 us). Returns false, the same for all threads and with nothing written, when a bucket would hold
+// more than kBucketMost (starts that crowd) or a role's starts spread over 2^50 ticks: the caller then merges.
+constexpr u32 kBuckets = 8192, kBucketMost = 32;  // buckets of a role at most
+__host__ __device__ constexpr u32 bucket_word(u32 b) { return b + (b >> 5); }  // padded: threads sum up runs of counters without bank conflicts
+constexpr size_t kBucketSmem = (size_t)kTile * 8 + bucket_word(2 * kBuckets) * 4;
+static_assert(kTile <= 1u << 14 && kBucketSmem <= (size_t)kTile * sizeof(ulonglong2), "places fit 14 bits, buckets the tile's room");
+__device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong2* in1, u32 n0, u32 n1, ulonglong2* out0, ulonglong2* out1,
+                                          ulonglong2* room, u64 (*red)[kPairWarps + 1], u32* scan) {
+  u64* const t = reinterpret_cast<u64*>(room);
+  u32* const cnt = reinterpret_cast<u32*>(t + kTile);  // a role's counters after the other's; then where a bucket ends
+  const u32 n = n0 + n1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  u32 bits = 5;  // 2^bits buckets a role
+  while (bits < 13 && (2u << bits) < n) ++bits;
+  const u32 nb = 2u << bits;
+  for (u32 b = threadIdx.x; b < nb; b += kPairThreads) cnt[bucket_word(b)] = 0;
+  u64 low0 = ~0ull, low1 = ~0ull, high0 = 0, high1 = 0;
+#pragma unroll 3
+  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
+    const u64 x = i < n0 ? in0[i].x : in1[i - n0].x;
+    if (i < n0) { low0 = x < low0 ? x : low0; high0 = x > high0 ? x : high0; }
+    else { low1 = x < low1 ? x : low1; high1 = x > high1 ? x : high1; }
+  }
+  u32 shift0 = 0, shift1 = 0;
+#pragma unroll 1
+  for (int role = 0; role < 2; ++role) {
+    u64 mn = role ? low1 : low0, mx = role ? high1 : high0;
+#pragma unroll 1
+    for (int step = 0; step < 2; ++step) {
+#pragma unroll
+      for (int dd = 16; dd > 0; dd >>= 1) {
+        const u64 a = __shfl_xor_sync(0xffffffffu, mn, dd), b = __shfl_xor_sync(0xffffffffu, mx, dd);
+        mn = a < mn ? a : mn; mx = b > mx ? b : mx;
+      }
+      if (step) break;
+      if (lane == 0) { red[0][warp] = mn; red[1][warp] = mx; }
+      __syncthreads();
+      mn = red[0][lane]; mx = red[1][lane];
+      __syncthreads();
+    }
+    const u64 range = mx > mn ? mx - mn : 0ull;
+    if (range >> 50) return false;
+    const u32 have = 64u - (u32)__clzll((long long)range), sh = have > bits ? have - bits : 0u;  // range < 2^have
+    if (role) { low1 = mn; shift1 = sh; } else { low0 = mn; shift0 = sh; }
+  }
+#pragma unroll 3
+  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
+    const bool role = i >= n0;
+    const u64 x = role ? in1[i - n0].x - low1 : in0[i].x - low0;
+    atomicAdd(&cnt[bucket_word((role ? 1u << bits : 0u) + (u32)(x >> (role ? shift1 : shift0)))], 1u);
+  }
+  __syncthreads();
+  const u32 per = (nb + kPairThreads - 1) / kPairThreads, c0 = threadIdx.x * per;  // counters a thread sums up: consecutive ones
+  u32 mine = 0, most = 0;
+  for (u32 b = c0; b < c0 + per && b < nb; ++b) { const u32 c = cnt[bucket_word(b)]; mine += c; most = c > most ? c : most; }
+  if (__syncthreads_or(most > kBucketMost)) return false;
+  u32 total;
+  u32 at = argus_block_exclusive_scan<u32>(mine, scan, &total);
+  for (u32 b = c0; b < c0 + per && b < nb; ++b) { const u32 c = cnt[bucket_word(b)]; cnt[bucket_word(b)] = at; at += c; }
+  __syncthreads();
+#pragma unroll 3
+  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
+    const bool role = i >= n0;
+    const u64 x = role ? in1[i - n0].x - low1 : in0[i].x - low0;
+    t[atomicAdd(&cnt[bucket_word((role ? 1u << bits : 0u) + (u32)(x >> (role ? shift1 : shift0)))], 1u)] = (x << 14) | i;
+  }
+  __syncthreads();
+#pragma unroll 3
+  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {  // the counter of a bucket is now where it ends
+    const bool role = i >= n0;  // (the first n0 elements are role 0's)
+    const u64 v = t[i];
+    const u32 b = (role ? 1u << bits : 0u) + (u32)((v >> 14) >> (role ? shift1 : shift0)), from = (u32)v & 0x3fffu;
+    const u32 b0 = b ? cnt[bucket_word(b - 1)] : 0u, b1 = cnt[bucket_word(b)];
+    u32 to = b0;
+    for (u32 k = b0; k < b1; ++k) to += t[k] < v;
+    if (role) out1[to - n0] = in1[from - n0]; else out0[to] = in0[from];
   }
   __syncthreads();
   return true;
 }
 
-__global__ void __launch_bounds__(kOvThreads) k_ov_sort(OvArgs a) {
-  extern __shared__ __align__(16) unsigned char sort_raw[];
-  ulonglong2* const tile = reinterpret_cast<ulonglong2*>(sort_raw);
-  __shared__ u64 sh[33];
-  __shared__ u64 sh_carry_e, sh_carry_len;
-  if (a.status->code != 0) return;
-  const u32 seg = blockIdx.x;
-  const u64 base = a.seg_base[seg];
-  const u64 n = a.seg_base[seg + 1] - base;
-  if (n == 0) return;
-  ulonglong2* d = a.spans + base;
-  if (a.scratch && base + n <= a.scratch_capacity && n > kOvBucketMax && ov_bucket_sort(d, a.scratch + base, n, sort_raw)) {
-    // sorted by buckets of start time
-  } else {
-  u64 p = 1;
-  while (p < n) p <<= 1;
-  // Bitonic network whose comparators all sort ascending; slots >= n act as +infinity and never move. A stage is a
-  // barrier apart from the next, and a segment larger than the L1 pays an L2 round trip per stage in global memory:
-  // so every run of stages whose partners lie within kOvSortTile spans is done on tiles in shared memory (one load
-  // and one store of the segment per run), and only the stages that reach across tiles work on global memory.
-  const u64 ntiles = (n + kOvSortTile - 1) / kOvSortTile;
-  for (u64 tI = 0; tI < ntiles; ++tI) {  // all block sizes up to a tile
-    const u64 tbase = tI * kOvSortTile;
-    const u32 cnt = (u32)(n - tbase < kOvSortTile ? n - tbase : kOvSortTile);
-    for (u32 i = threadIdx.x; i < cnt; i += blockDim.x) tile[i] = d[tbase + i];
-    __syncthreads();
-    for (u32 k = 2; k <= kOvSortTile && k <= p; k <<= 1) ov_sort_tile_stages(tile, tbase, n, k, true, k >> 2);
-    for (u32 i = threadIdx.x; i < cnt; i += blockDim.x) d[tbase + i] = tile[i];
-    __syncthreads();
-  }
-  for (u64 k = 2ull * kOvSortTile; k <= p; k <<= 1) {
-    const u64 h = k >> 1;
-    for (u64 c = threadIdx.x; c < p / 2; c += blockDim.x) {  // the flip and the long distances: across tiles
-      const u64 i = ((c & ~(h - 1)) << 1) | (c & (h - 1)), l = i ^ (k - 1);
-      if (l < n) cmp_swap(d, i, l);
-    }
-    __syncthreads();
-    u64 j = k >> 2;
-    for (; j >= kOvSortTile; j >>= 1) {
-      for (u64 c = threadIdx.x; c < p / 2; c += blockDim.x) {
-        const u64 i = ((c & ~(j - 1)) << 1) | (c & (j - 1)), l = i | j;
-        if (l < n) cmp_swap(d, i, l);
-      }
-      __syncthreads();
-    }
-    for (u64 tI = 0; tI < ntiles; ++tI) {  // the distances below a tile
-      const u64 tbase = tI * kOvSortTile;
-      const u32 cnt = (u32)(n - tbase < kOvSortTile ? n - tbase : kOvSortTile);
-      for (u32 i = threadIdx.x; i < cnt; i += blockDim.x) tile[i] = d[tbase + i];
-      __syncthreads();
-      ov_sort_tile_stages(tile, tbase, n, 0, false, (u32)j);
-      for (u32 i = threadIdx.x; i < cnt; i += blockDim.x) d[tbase + i] = tile[i];
-      __syncthreads();
-    }
-  }
-  }
-  // pieces of the union and running covered length
-  if (threadIdx.x == 0) { sh_carry_e = 0; sh_carry_len = 0; }
-  __syncthreads();
+// d[0..n) in start order -> the disjoint pieces of their union: piece i = [max(start_i, E), max(end_i, that)) with E the largest
+// end of the spans before i (pieces may be empty). Returns this thread's share of the sum of their lengths.
+__device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
+  constexpr u32 kPer = 4;  // consecutive spans a thread takes at a time
   const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (u64 i0 = 0; i0 < n; i0 += blockDim.x) {
-    const u64 i = i0 + threadIdx.x;
-    const bool live = i < n;
-    const ulonglong2 sp = live ? d[i] : make_ulonglong2(0, 0);
-    // inclusive prefix max of span ends (0 is the identity: ends are > starts >= 0)
-    u64 e = live ? sp.y : 0;
+  u64 carry = 0, len = 0;
+  for (u64 i0 = 0; i0 < n; i0 += kPer * kPairThreads) {
+    const u64 at = i0 + (u64)threadIdx.x * kPer;
+    ulonglong2 s[kPer];
+    u64 e = 0;
+#pragma unroll
+    for (u32 j = 0; j < kPer; ++j) s[j] = at + j < n ? d[at + j] : make_ulonglong2(0, 0);
+#pragma unroll
+    for (u32 j = 0; j < kPer; ++j) e = s[j].y > e ? s[j].y : e;
 #pragma unroll
     for (int dd = 1; dd < 32; dd <<= 1) {
       const u64 o = __shfl_up_sync(0xffffffffu, e, dd);
       if (lane >= (u32)dd && o > e) e = o;
     }
-    if (lane == 31) sh[warp] = e;
+    if (lane == 31) red[warp] = e;
     __syncthreads();
-    if (warp == 0) {
-      u64 w = sh[lane];
+    u64 w = red[lane];
 #pragma unroll
-      for (int dd = 1; dd < 32; dd <<= 1) {
-        const u64 o = __shfl_up_sync(0xffffffffu, w, dd);
-        if (lane >= (u32)dd && o > w) w = o;
-      }
-      sh[lane] = w;
+    for (int dd = 1; dd < 32; dd <<= 1) {
+      const u64 o = __shfl_up_sync(0xffffffffu, w, dd);
+      if (lane >= (u32)dd && o > w) w = o;
     }
-    __syncthreads();
-    const u64 carry_e = sh_carry_e;
-    u64 before = carry_e;  // max end of all earlier spans
-    if (warp > 0 && sh[warp - 1] > before) before = sh[warp - 1];
-    {
-      const u64 own_excl = __shfl_up_sync(0xffffffffu, e, 1);
-      if (lane > 0 && own_excl > before) before = own_excl;
-    }
-    u64 e_incl = e > before ? e : before;
-    const u64 pa = sp.x > before ? sp.x : before;
-    const u64 pb = e_incl > pa ? e_incl : pa;
-    const u64 len = live ? pb - pa : 0;
-    __syncthreads();
-    u64 total;
-    const u64 ex = argus_block_exclusive_scan<u64>(len, sh, &total);
-    const u64 carry_len = sh_carry_len;
-    if (live) {
-      d[i] = make_ulonglong2(pa, pb);
-      a.cum[base + i] = carry_len + ex;
-    }
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) {
-      sh_carry_e = e_incl > carry_e ? e_incl : carry_e;
-      sh_carry_len = carry_len + total;
-    }
-    __syncthreads();
-  }
-}
-
-constexpr int kOvMeasureThreads = 1024;
-
-// covered length of the consumer pieces before time t, given pos = number of pieces whose begin is < t
-__device__ __forceinline__ u64 covered_at(const ulonglong2* pc, const u64* cum, u64 pos, u64 t) {
-  if (pos == 0) return 0;
-  const ulonglong2 last = pc[pos - 1];
-  return cum[pos - 1] + ((t < last.y ? t : last.y) - last.x);
-}
-
-// pos = number of consumer pieces whose begin is < t, reached from an earlier boundary's pos (never past it): steps
-// of doubling length, then a binary search inside the last step, so a far boundary costs a logarithm of its distance
-__device__ __forceinline__ u64 advance_to(const ulonglong2* pc, u64 nc, u64 pos, u64 t) {
-  if (pos >= nc || !(pc[pos].x < t)) return pos;
-  u64 lo = pos, step = 1;  // pc[lo].x < t
-  while (lo + step < nc && pc[lo + step].x < t) { lo += step; step <<= 1; }
-  u64 hi = lo + step < nc ? lo + step : nc;  // the first piece with begin >= t lies in (lo, hi]
-  ++lo;
-  while (lo < hi) {
-    const u64 mid = lo + ((hi - lo) >> 1);
-    if (pc[mid].x < t) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-__global__ void __launch_bounds__(kOvMeasureThreads) k_ov_measure(OvArgs a) {
-  __shared__ u64 sh[kOvMeasureThreads / 32];
-  if (a.status->code != 0) return;
-  const u32 km = blockIdx.x;  // k * M + m
-  const u64 bp = a.seg_base[2 * km], bc = a.seg_base[2 * km + 1], be = a.seg_base[2 * km + 2];
-  const u64 np = bc - bp, nc = be - bc;
-  const ulonglong2* pp = a.spans + bp;
-  const ulonglong2* pc = a.spans + bc;
-  const u64* cum_c = a.cum + bc;
-  u64 acc = 0;
-  if (nc) {
-    // Every thread takes a run of consecutive producer pieces. Pieces are disjoint and in time order, so the
-    // boundaries a thread asks about never decrease: one binary search places the first, the rest are reached from
-    // the one before (usually the next consumer piece or two).
-    const u64 per = (np + blockDim.x - 1) / blockDim.x;
-    const u64 i0 = (u64)threadIdx.x * per, i1 = i0 + per < np ? i0 + per : np;
-    if (i0 < i1) {
-      u64 pos;  // number of consumer pieces whose begin is < the boundary at hand
-      {
-        const u64 t = pp[i0].x;
-        u64 lo = 0, hi = nc;
-        while (lo < hi) {
-          const u64 mid = lo + ((hi - lo) >> 1);
-          if (pc[mid].x < t) lo = mid + 1; else hi = mid;
-        }
-        pos = lo;
-      }
-      for (u64 i = i0; i < i1; ++i) {
-        const ulonglong2 piece = pp[i];
-        pos = advance_to(pc, nc, pos, piece.x);
-        const u64 before = covered_at(pc, cum_c, pos, piece.x);
-        pos = advance_to(pc, nc, pos, piece.y);
-        if (piece.y > piece.x) acc += covered_at(pc, cum_c, pos, piece.y) - before;
-      }
-    }
-  }
+    u64 before = __shfl_up_sync(0xffffffffu, e, 1);
+    if (lane == 0) before = 0;
+    const u64 warps_before = warp ? __shfl_sync(0xffffffffu, w, warp - 1) : 0ull, all = __shfl_sync(0xffffffffu, w, 31);
+    before = before > warps_before ? before : warps_before;
+    before = before > carry ? before : carry;
 #pragma unroll
-  for (int dd = 16; dd > 0; dd >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, dd);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+    for (u32 j = 0; j < kPer; ++j) {
+      if (at + j < n) {
+        const u64 a = s[j].x > before ? s[j].x : before, b = s[j].y > a ? s[j].y : a;
+        d[at + j] = make_ulonglong2(a, b);
+        len += b - a;
+        before = b > before ? b : before;
+      }
+    }
+    carry = all > carry ? all : carry;
+    __syncthreads();
+  }
+  return len;
+}
+
+// Latency decides (one block per SM and pair). The entries of up to kBatch slices are taken as one flat sequence, so that
+// every thread has kGather entries and then as many begin times (or pieces of records) in flight, whatever the slices hold.
+// 148 SMs, two roles of 16,000 spans each: 109 us (five kernels before it: 393 us); 2,048 spans a role from 16 interleaved
+// streams: 43 us (178 us); a few hundred spans: 28 us, most of it fixed steps one after the other (45 us).
+// DIGEST: entries as the pass over the digests leaves them (argus_fuse.cuh); else {index in the stream, region}.
+template <bool DIGEST>
+__global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
+  extern __shared__ __align__(16) unsigned char pair_raw[];
+  ulonglong2* const tile = reinterpret_cast<ulonglong2*>(pair_raw);
+  __shared__ u32 sh_hit[kPairThreads];             // CTAs of this SM among the ones just looked at
+  __shared__ u32 sh_ex[kBatch + 1];                // entries of the batch before slice i
+  __shared__ u64 sh_pos[kBatch], sh_iv[kBatch];    // where a slice's entries and its stream's intervals start
+  __shared__ u32 sh_scan[33];
+  __shared__ u64 sh64[4];
+  __shared__ u64 red[2][kPairWarps + 1];
+  __shared__ u32 sh_cnt[kGather * kPairWarps];
+  __shared__ u32 sh_u;
+  const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 k = blockIdx.x / a.num_sms, m = blockIdx.x % a.num_sms;
+  const u32 P = a.pairs[2 * k], C = a.pairs[2 * k + 1];
+  const u32 num_ctas = a.num_streams / a.warps_per_cta, per_cta = a.warps_per_cta * a.slices;
+  if (tid == 0) {
+    sh_u = a.status->code;
+    if (a.ctl->num_entries > a.entry_capacity) {  // the selection ran out of room
+      sh_u = ARGUS_ERR_CAPACITY;
+      if (blockIdx.x == 0) {
+        argus_set_error(a.status, ARGUS_ERR_CAPACITY, 0, a.ctl->num_entries);
+        a.status->intervals_required = a.ctl->num_entries;
+      }
+    }
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    u64 both = 0;
-    for (u32 w = 0; w < (blockDim.x >> 5); ++w) both += sh[w];
-    const u64 p_ns = np ? a.cum[bp + np - 1] + (pp[np - 1].y - pp[np - 1].x) : 0;
-    const u64 c_ns = nc ? a.cum[bc + nc - 1] + (pc[nc - 1].y - pc[nc - 1].x) : 0;
+  // (a capacity error that another block of this launch reports is not waited for: such a block has no room itself or is done)
+  if (sh_u != 0) return;
+
+  // ---- gather: round 0 counts, round 1 places, in stream and slice order ----
+  // With one pair every entry is in a role of it, and round 0 only adds up the pieces.
+  u64 nP = 0, nC = 0, base = 0;
+  bool suspect[2] = {false, false};  // this thread has seen a span of the role that starts before the end of the one before it
+  u64 len[2] = {0, 0};               // this thread's share of |U_P| and |U_C|
+  u64 carry_p = 0, carry_c = 0;      // end of the last span of a role
+  ArgusOvPiece held; held.pos = 0; held.count = 0; held.next = kOvNone;
+  bool hold = false;                 // one batch holds everything: its CTAs and first pieces are kept from round 0
+  u32 hits = 0;
+  for (int round = 0; round < 2; ++round) {
+    u64 my_all = 0, my_p = 0, my_c = 0;  // round 0, per thread
+    for (u32 c0 = 0; c0 < num_ctas; c0 += kPairThreads) {
+      if (!hold) {
+        const bool hit = c0 + tid < num_ctas && a.cta_sm[c0 + tid] == m;
+        const u32 ex = argus_block_exclusive_scan<u32>(hit ? 1u : 0u, sh_scan, &hits);
+        if (hit) sh_hit[ex] = c0 + tid;
+        __syncthreads();
+      }
+      const u64 heads = (u64)hits * per_cta;
+      hold = num_ctas <= kPairThreads && heads <= kBatch;
+      for (u64 h0 = 0; h0 < heads; h0 += kBatch) {
+        u32 piece = kOvNone;
+        u64 iv0 = 0;
+        if (h0 + tid < heads) {
+          const u32 cta = sh_hit[(h0 + tid) / per_cta], rest = (u32)((h0 + tid) % per_cta);
+          piece = cta * per_cta + rest;
+          if (!DIGEST) iv0 = a.interval_offsets[cta * a.warps_per_cta + rest / a.slices];
+        }
+        // (chains of pieces are taken one link at a time: the spans are then no longer in slice order, and get sorted)
+        do {
+          ArgusOvPiece pc; pc.pos = 0; pc.count = 0; pc.next = kOvNone;
+          if (piece != kOvNone) {
+            const bool first = piece < num_ctas * per_cta;
+            pc = round == 1 && hold && first ? held : a.pieces[piece];
+            if (hold && first) held = pc;
+          }
+          piece = pc.next;
+          if (round == 0 && a.num_pairs == 1) { my_all += pc.count; continue; }
+          // slices that hold something, one after the other: where each starts in the flat sequence
+          u64 all;
+          const u64 ex = argus_block_exclusive_scan<u64>((u64)pc.count | (pc.count ? 1ull << 32 : 0ull), red[0], &all);
+          const u32 total = (u32)all, slices = (u32)(all >> 32);
+          if (pc.count) {
+            const u32 at = (u32)(ex >> 32);
+            sh_ex[at] = (u32)ex;
+            sh_pos[at] = pc.pos;
+            if (!DIGEST) sh_iv[at] = iv0;
+          }
+          for (u32 i = slices + tid; i <= kBatch; i += kPairThreads) sh_ex[i] = total;
+          __syncthreads();
+          for (u32 e0 = 0; e0 < total; e0 += kPairThreads * kGather) {
+            u64 ent[kGather];
+            u32 at[kGather];
+            u32 is_p = 0, is_c = 0;
+#pragma unroll
+            for (u32 j = 0; j < kGather; ++j) {
+              at[j] = 0; ent[j] = 0;
+              if (e0 + j * kPairThreads >= total) continue;
+              const u32 f = e0 + j * kPairThreads + tid, f0 = f - lane;
+              // the slice of the warp's first entry: the last one that starts at or before it, 32 probes at a time
+              u32 lo = 32u * ((u32)__popc(__ballot_sync(0xffffffffu, sh_ex[32 * lane] <= f0)) - 1u);
+              lo += (u32)__popc(__ballot_sync(0xffffffffu, sh_ex[lo + lane] <= f0)) - 1u;
+              if (f < total) while (f >= sh_ex[lo + 1]) ++lo;
+              at[j] = lo;
+              if (f < total) ent[j] = __ldcg(a.entries + sh_pos[lo] + (f - sh_ex[lo]));
+            }
+#pragma unroll
+            for (u32 j = 0; j < kGather; ++j) {
+              const bool in = e0 + j * kPairThreads + tid < total;
+              const u32 region = DIGEST ? (u32)ent[j] & 0xffffu : (u32)(ent[j] >> 32);
+              if (in && region == P) is_p |= 1u << j;
+              if (in && region == C) is_c |= 1u << j;
+            }
+            if (round == 0) { my_p += __popc(is_p); my_c += __popc(is_c); continue; }
+            ulonglong2 q[kGather];  // begin time and duration
+#pragma unroll
+            for (u32 j = 0; j < kGather; ++j) {
+              if (!(((is_p | is_c) >> j) & 1u)) continue;
+              if (DIGEST) {
+                if ((u32)ent[j] & kDigestWide) {
+                  q[j] = __ldg(reinterpret_cast<const ulonglong2*>(a.intervals + sh_pos[at[j]] + (ent[j] >> 18)));
+                } else {
+                  q[j].x = __ldcg(a.starts + sh_pos[at[j]] + (e0 + j * kPairThreads + tid - sh_ex[at[j]]));
+                  q[j].y = (ent[j] >> 18) & ((1u << kDigestBits) - 1u);
+                }
+              } else {
+                q[j] = __ldg(reinterpret_cast<const ulonglong2*>(a.intervals + sh_iv[at[j]] + (u32)ent[j]));
+              }
+            }
+            // places: entries of a role before (j, warp, lane)
+            u32 bp[kGather], bc[kGather];
+#pragma unroll
+            for (u32 j = 0; j < kGather; ++j) {
+              bp[j] = __ballot_sync(0xffffffffu, (is_p >> j) & 1u);
+              bc[j] = __ballot_sync(0xffffffffu, (is_c >> j) & 1u);
+              if (lane == 0) sh_cnt[j * kPairWarps + warp] = (u32)__popc(bp[j]) | ((u32)__popc(bc[j]) << 16);
+            }
+            __syncthreads();
+            if (warp == 0) {
+              u32 c[kGather], sum = 0;
+#pragma unroll
+              for (u32 j = 0; j < kGather; ++j) { c[j] = sh_cnt[lane * kGather + j]; sum += c[j]; }
+              u32 incl = sum;
+#pragma unroll
+              for (int dd = 1; dd < 32; dd <<= 1) { const u32 o = __shfl_up_sync(0xffffffffu, incl, dd); if (lane >= (u32)dd) incl += o; }
+              u32 ex = incl - sum;
+#pragma unroll
+              for (u32 j = 0; j < kGather; ++j) { sh_cnt[lane * kGather + j] = ex; ex += c[j]; }
+              if (lane == 31) sh_u = incl;
+            }
+            __syncthreads();
+            const u32 tot = sh_u, tot_p = tot & 0xffffu, tot_c = tot >> 16, lt = (1u << lane) - 1u;
+            u64* const ends_p = reinterpret_cast<u64*>(tile);      // ends_p[i]: end of the role's span before place i of the group
+            u64* const ends_c = ends_p + kPairThreads * kGather + 1;
+            if (tid == 0) { ends_p[0] = carry_p; ends_c[0] = carry_c; }
+#pragma unroll
+            for (u32 j = 0; j < kGather; ++j) {
+              const ulonglong2 span = make_ulonglong2(q[j].x, q[j].x + q[j].y);
+              const u32 before = sh_cnt[j * kPairWarps + warp];
+              if ((is_p >> j) & 1u) {
+                const u32 r = (before & 0xffffu) + (u32)__popc(bp[j] & lt);
+                a.spans[base + nP + r] = span;
+                ends_p[r + 1] = span.y;
+                len[0] += span.y - span.x;
+              }
+              if ((is_c >> j) & 1u) {
+                const u32 r = (before >> 16) + (u32)__popc(bc[j] & lt);
+                a.scratch[base + nC + r] = span;
+                ends_c[r + 1] = span.y;
+                len[1] += span.y - span.x;
+              }
+            }
+            __syncthreads();
+#pragma unroll
+            for (u32 j = 0; j < kGather; ++j) {  // in order and disjoint so far?
+              const u64 e = q[j].x + q[j].y;
+              const u32 before = sh_cnt[j * kPairWarps + warp];
+              if ((is_p >> j) & 1u) suspect[0] |= q[j].x < ends_p[(before & 0xffffu) + (u32)__popc(bp[j] & lt)] || e < q[j].x;
+              if ((is_c >> j) & 1u) suspect[1] |= q[j].x < ends_c[(before >> 16) + (u32)__popc(bc[j] & lt)] || e < q[j].x;
+            }
+            carry_p = ends_p[tot_p];
+            carry_c = ends_c[tot_c];
+            nP += tot_p;
+            nC += tot_c;
+            __syncthreads();
+          }
+          __syncthreads();  // sh_ex and sh_pos are overwritten next
+        } while (__syncthreads_or(piece != kOvNone));
+      }
+      __syncthreads();  // sh_hit is overwritten next
+    }
+    if (round == 0) {
+      u64 mine = a.num_pairs == 1 ? (P == C ? 2 * my_all : my_all) : my_p + my_c;
+#pragma unroll
+      for (int dd = 16; dd > 0; dd >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, dd);
+      if (lane == 0) red[0][warp] = mine;
+      __syncthreads();
+      if (tid == 0) {  // room for this block's spans; the last block to ask knows whether everybody's fitted
+        u64 all = 0;
+        for (u32 w = 0; w < kPairWarps; ++w) all += red[0][w];
+        sh64[0] = all ? atomicAdd(&a.ctl->num_spans, all) : 0ull;
+        sh64[1] = all;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(&a.ctl->asked, 1u) == a.blocks - 1) {
+          const u64 total = *reinterpret_cast<volatile u64*>(&a.ctl->num_spans);
+          if (total > a.capacity) {
+            argus_set_error(a.status, ARGUS_ERR_CAPACITY, 0, total);
+            a.status->intervals_required = total;
+          }
+        }
+      }
+      base = sh64[0];
+      if (base + sh64[1] > a.capacity) return;
+      if (sh64[1] == 0) break;
+    }
+  }
+
+  // ---- sorted, disjoint pieces of both roles ----
+  const u64 total = nP + nC;
+  ulonglong2 *A = a.spans + base, *B = a.scratch + base;
+  {
+    const bool cut_a = __syncthreads_or(suspect[0]), cut_b = __syncthreads_or(suspect[1]);
+    ulonglong2 *const free_a = a.scratch + base + nC, *const free_b = a.spans + base + nP;  // as much room again for either role
+    if (cut_a || cut_b) {
+      if ((cut_a ? nP : 0ull) + (cut_b ? nC : 0ull) <= kTile &&
+          sort_buckets(A, B, cut_a ? (u32)nP : 0u, cut_b ? (u32)nC : 0u, free_a, free_b, tile, red, sh_scan)) {
+        if (cut_a) A = free_a;
+        if (cut_b) B = free_b;
+      } else {
+        if (cut_a) A = sort_spans(A, free_a, nP, tile, sh64);
+        if (cut_b) B = sort_spans(B, free_b, nC, tile, sh64);
+      }
+      if (cut_a) len[0] = cut_pieces(A, nP, red[0]);
+      if (cut_b) len[1] = cut_pieces(B, nC, red[1]);
+    }
+  }
+  __syncthreads();
+
+  // ---- walk of the merged sequence ----
+  // a piece that starts inside the last piece of the other role overlaps it, and no other
+  u64 both = 0;
+  u64 a0 = 0;  // producer pieces taken so far
+  for (u64 t0 = 0; nP && nC && t0 < total; t0 += kTile) {
+    const u32 cnt = (u32)(total - t0 < kTile ? total - t0 : kTile), step = (u32)((t0 / kTile) % kPairWarps);
+    if (step == 0) {  // where the next 32 tiles end, one warp each
+      const u64 to = t0 + (u64)(warp + 1) * kTile;
+      const u64 s1 = to >= total ? nP : merge_split_warp(A, nP, B, nC, to, lane);
+      if (lane == 0) red[0][warp] = s1;
+      __syncthreads();
+    }
+    const u64 a1 = red[0][step], b0 = t0 - a0;
+    const u32 na = (u32)(a1 - a0), nb = cnt - na;
+    const u64 last_a = a0 ? A[a0 - 1].y : 0ull, last_b = b0 ? B[b0 - 1].y : 0ull;
+#pragma unroll
+    for (u32 j = 0; j < kVT; ++j) {
+      const u32 i = j * kPairThreads + tid;
+      if (i < cnt) tile[i] = i < na ? A[a0 + i] : B[b0 + (i - na)];
+    }
+    __syncthreads();
+    const u32 at = tid * kVT;
+    if (at < cnt) {
+      u32 x = merge_split(tile, na, tile + na, nb, at), y = at - x;
+      u64 end_a = x ? tile[x - 1].y : last_a, end_b = y ? tile[na + y - 1].y : last_b;
+      ulonglong2 va = x < na ? tile[x] : make_ulonglong2(~0ull, ~0ull), vb = y < nb ? tile[na + y] : make_ulonglong2(~0ull, ~0ull);
+#pragma unroll
+      for (u32 j = 0; j < kVT; ++j) {
+        if (at + j < cnt) {
+          const bool take_a = y >= nb || (x < na && va.x <= vb.x);
+          const u64 s = take_a ? va.x : vb.x, e = take_a ? va.y : vb.y, other = take_a ? end_b : end_a;
+          const u64 upto = e < other ? e : other;
+          if (upto > s) both += upto - s;
+          if (take_a) { end_a = e; ++x; if (x < na) va = tile[x]; }
+          else { end_b = e; ++y; if (y < nb) vb = tile[na + y]; }
+        }
+      }
+    }
+    a0 = a1;
+    __syncthreads();
+  }
+#pragma unroll
+  for (int dd = 16; dd > 0; dd >>= 1) {
+    len[0] += __shfl_down_sync(0xffffffffu, len[0], dd);
+    len[1] += __shfl_down_sync(0xffffffffu, len[1], dd);
+    both += __shfl_down_sync(0xffffffffu, both, dd);
+  }
+  __syncthreads();
+  if (tid < 3) sh64[tid] = 0;
+  __syncthreads();
+  if (lane == 0) {
+    if (len[0]) atomicAdd(&sh64[0], len[0]);
+    if (len[1]) atomicAdd(&sh64[1], len[1]);
+    if (both) atomicAdd(&sh64[2], both);
+  }
+  __syncthreads();
+  if (tid == 0) {
     argus_overlap_t o;
-    o.overlap_ns = both; o.producer_ns = p_ns; o.consumer_ns = c_ns; o.either_ns = p_ns + c_ns - both;
-    a.out[km] = o;
+    o.producer_ns = sh64[0]; o.consumer_ns = sh64[1]; o.overlap_ns = sh64[2];
+    o.either_ns = o.producer_ns + o.consumer_ns - o.overlap_ns;
+    a.out[blockIdx.x] = o;
   }
 }
 
-struct OvLayout { size_t seg_count, seg_cursor, seg_base, spans, total_fixed; };
+// What the list path needs per span besides its fixed part: two places for the span, an entry, its share of a piece.
+constexpr size_t kBytesPerSpan = 16 + 16 + 8 + 1;
 
-OvLayout ov_layout(uint32_t nseg) {
-  OvLayout L;
-  size_t o = 0;
-  L.seg_count = o; o += argus_align_up((size_t)nseg * 8, 256);
-  L.seg_cursor = o; o += argus_align_up((size_t)nseg * 8, 256);
-  L.seg_base = o; o += argus_align_up(((size_t)nseg + 1) * 8, 256);
-  L.spans = o;
-  L.total_fixed = o;
-  return L;
+u32 select_slices(u32 num_streams) {
+  u32 parts = num_streams ? kSelGrid / num_streams : 1u;  // few streams: several blocks walk one
+  parts = parts < 1 ? 1 : parts > 8 ? 8 : parts;
+  return parts * kSelWarps;
+}
+
+size_t ov_fixed_bytes(u32 num_streams) {
+  return argus_align_up(sizeof(ArgusOvCtl), 256) + argus_align_up((size_t)num_streams * select_slices(num_streams) * sizeof(ArgusOvPiece), 256) + 1024;
+}
+
+template <bool DIGEST>
+int launch_pair(const OvPairArgs& a, cudaStream_t stream) {
+  static std::atomic<bool> opted_in[64];  // the shared-memory opt-in belongs to a device
+  int dev = 0;
+  ARGUS_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return ARGUS_ERR_INVALID_ARG;
+  if (!opted_in[dev].load(std::memory_order_acquire)) {
+    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_ov_pair<DIGEST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
+    opted_in[dev].store(true, std::memory_order_release);
+  }
+  argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);
+  k_ov_pair<DIGEST><<<a.blocks, kPairThreads, kPairSmem, stream>>>(a);
+  ARGUS_CHECK_LAUNCH();
+  argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 1);
+  return ARGUS_OK;
 }
 
 }  // namespace
 
-constexpr size_t kBytesPerSortedSpan = 24;  // (begin, end) + covered length before it
-constexpr size_t kBytesPerListedSpan = 20;  // (begin, end) + segment
-constexpr unsigned kSelectGrid = 148 * 8;
-constexpr unsigned kSelectWarps = kSelectGrid * 8;
-
-extern "C" size_t argus_overlap_workspace_bytes(uint64_t max_intervals, uint32_t /*num_streams*/, uint32_t num_pairs,
-                                                uint32_t num_sms) {
-  const OvLayout L = ov_layout(num_pairs * num_sms * 2);
-  // worst case: every interval selected in both roles of every pair, listed and then sorted; a third more
-  // list slots than spans cover the slots that warps reserve and leave unused
-  const size_t spans = (size_t)max_intervals * 2 * num_pairs;
-  return L.total_fixed + argus_align_up((spans + spans / 3 + 64) * (kBytesPerSortedSpan + kBytesPerListedSpan) + 1024, 256);
+extern "C" size_t argus_overlap_workspace_bytes(uint64_t max_intervals, uint32_t num_streams, uint32_t num_pairs,
+                                                uint32_t /*num_sms*/) {
+  // worst case: every interval selected in both roles of every pair
+  return ov_fixed_bytes(num_streams) + argus_align_up(((size_t)max_intervals * 2 * num_pairs + 64) * kBytesPerSpan, 256);
 }
 
-// Shared tail of both entry paths: from the list of selected spans to the overlap measures.
-static int ov_run(OvArgs& a, const OvList* list, cudaStream_t stream) {
-  for (int pass = 0; pass < 2; ++pass) {
-    k_ov_list_count_or_scatter<<<592, 256, 0, stream>>>(a, *list, pass);
-    ARGUS_CHECK_LAUNCH();
-    if (pass == 0) {
-      k_ov_scan<<<1, kOvThreads, 0, stream>>>(a);
-      ARGUS_CHECK_LAUNCH();
-    }
-  }
-  argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);
-  {
-    static bool opted_in[64];  // the shared-memory opt-in belongs to a device
-    int dev = 0;
-    ARGUS_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return ARGUS_ERR_INVALID_ARG;
-    if (!opted_in[dev]) {
-      ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_ov_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOvSortSmem));
-      opted_in[dev] = true;
-    }
-  }
-  a.scratch = const_cast<ulonglong2*>(list->spans);  // every listed span has been copied into its segment
-  a.scratch_capacity = list->capacity;
-  k_ov_sort<<<a.nseg, kOvThreads, kOvSortSmem, stream>>>(a);
-  ARGUS_CHECK_LAUNCH();
-  argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 1);
-  k_ov_measure<<<a.nseg / 2, kOvMeasureThreads, 0, stream>>>(a);
-  ARGUS_CHECK_LAUNCH();
-  return ARGUS_OK;
+size_t argus_internal_overlap_bytes(uint64_t max_spans, uint32_t num_streams) {
+  return ov_fixed_bytes(num_streams) + argus_align_up(((size_t)max_spans + 64) * kBytesPerSpan, 256);
 }
 
-static int ov_setup(OvArgs& a, uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm, uint32_t num_sms,
-                    const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out, argus_status_t* status, void* workspace,
-                    size_t workspace_bytes, cudaStream_t stream, size_t own_list_bytes = 0) {
-  const u32 nseg = num_pairs * num_sms * 2;
-  const OvLayout L = ov_layout(nseg);
-  if (workspace_bytes < L.total_fixed + 256 + own_list_bytes) return ARGUS_ERR_WORKSPACE;
-  workspace_bytes -= own_list_bytes;  // the caller keeps its list behind the part laid out here
-  char* ws = (char*)workspace;
-  a.intervals = nullptr; a.interval_offsets = nullptr; a.max_intervals = 0; a.num_streams = num_streams;
-  a.warps_per_cta = warps_per_cta; a.num_sms = num_sms; a.num_pairs = num_pairs; a.cta_sm = cta_sm; a.pairs = pairs;
-  a.out = out; a.status = status;
-  a.seg_count = (u64*)(ws + L.seg_count); a.seg_cursor = (u64*)(ws + L.seg_cursor); a.seg_base = (u64*)(ws + L.seg_base);
-  a.capacity = (workspace_bytes - L.total_fixed) / 24;
-  a.spans = (ulonglong2*)(ws + L.spans);
-  a.scratch = nullptr; a.scratch_capacity = 0;
-  a.cum = (u64*)(ws + L.spans + argus_align_up((size_t)a.capacity * 16, 16));
-  a.nseg = nseg;
-  a.scoped = 0; a.ctx_lo = 0; a.ctx_hi = 0xffffffffu; a.warp_mask = ~0ull; a.sm_mask = nullptr; a.region_mask = nullptr;
-  ARGUS_CUDA_TRY(cudaMemsetAsync(ws, 0, L.seg_base, stream));
-  ARGUS_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)num_pairs * num_sms * sizeof(argus_overlap_t), stream));
-  return ARGUS_OK;
+static OvPairArgs pair_args(const argus_interval_t* intervals, const uint64_t* interval_offsets, const uint64_t* entries, uint64_t entry_capacity,
+                            const ArgusOvPiece* pieces, uint32_t slices, uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm,
+                            uint32_t num_sms, const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out, argus_status_t* status,
+                            ArgusOvCtl* ctl, void* spans, uint64_t max_spans) {
+  OvPairArgs a;
+  a.intervals = intervals; a.interval_offsets = (const u64*)interval_offsets; a.starts = nullptr; a.entries = (const u64*)entries; a.pieces = pieces;
+  a.slices = slices; a.num_streams = num_streams; a.warps_per_cta = warps_per_cta; a.num_sms = num_sms; a.num_pairs = num_pairs;
+  a.blocks = num_pairs * num_sms; a.cta_sm = cta_sm; a.pairs = pairs; a.out = out; a.status = status;
+  a.spans = (ulonglong2*)spans; a.scratch = a.spans + max_spans; a.capacity = max_spans; a.entry_capacity = entry_capacity; a.ctl = ctl;
+  return a;
 }
 
-// Overlap from a span list appended by the pairing kernel (see argus_fuse.cuh).
-int argus_internal_overlap_from_list(const void* list_spans, const uint32_t* list_seg, const uint64_t* list_count,
-                                     uint64_t list_capacity, uint32_t num_sms, uint32_t num_pairs, argus_overlap_t* out,
-                                     argus_status_t* status, void* workspace, size_t workspace_bytes, void* cuda_stream) {
-  if (num_pairs == 0) return ARGUS_OK;
-  cudaStream_t stream = (cudaStream_t)cuda_stream;
-  OvArgs a;
-  const int rc = ov_setup(a, 0, 1, nullptr, num_sms, nullptr, num_pairs, out, status, workspace, workspace_bytes, stream);
-  if (rc != ARGUS_OK) return rc;
-  OvList l;
-  l.spans = (const ulonglong2*)list_spans; l.seg = list_seg; l.count = (const u64*)list_count; l.capacity = list_capacity;
-  return ov_run(a, &l, stream);
+// Overlap from what the pass over the digests selected: span area and scratch in `spans`.
+int argus_internal_overlap_from_digests(const argus_interval_t* intervals, const uint64_t* starts, const uint64_t* entries, const ArgusOvPiece* pieces,
+                                        uint32_t slices, uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm,
+                                        uint32_t num_sms, const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out,
+                                        argus_status_t* status, ArgusOvCtl* ctl, void* spans, uint64_t max_spans, void* cuda_stream) {
+  OvPairArgs a = pair_args(intervals, nullptr, entries, ~0ull, pieces, slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs, num_pairs,
+                           out, status, ctl, spans, max_spans);
+  a.starts = (const u64*)starts;
+  return launch_pair<true>(a, (cudaStream_t)cuda_stream);
 }
 
 static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_intervals, const uint64_t* interval_offsets,
@@ -641,46 +790,45 @@ static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_interv
   if (!interval_offsets || (!cta_sm && num_streams) || !status || !workspace) return ARGUS_ERR_INVALID_ARG;
   if (scope && scope->ctx_hi < scope->ctx_lo) return ARGUS_ERR_INVALID_ARG;
   if (warps_per_cta == 0 || num_streams % warps_per_cta != 0 || num_sms == 0) return ARGUS_ERR_INVALID_ARG;
-  if (num_pairs > kMaxPairs || (num_pairs && (!pairs || !out))) return ARGUS_ERR_INVALID_ARG;
+  if (num_pairs > ARGUS_MAX_PAIRS || (num_pairs && (!pairs || !out))) return ARGUS_ERR_INVALID_ARG;
   if ((max_intervals && !intervals) || ((uintptr_t)intervals & 15) || ((uintptr_t)workspace & 255) || ((uintptr_t)out & 7))
     return ARGUS_ERR_INVALID_ARG;
   if ((uint64_t)num_pairs * num_sms * 2 > 0x7fffffffull) return ARGUS_ERR_INVALID_ARG;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   if (reset_status) ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
   if (num_pairs == 0) return ARGUS_OK;
-  OvArgs a;
-  // split what the workspace offers beyond the fixed part between the list (20 B a slot) and the sorted spans
-  // (24 B each), with a third more list slots than sorted spans
-  const OvLayout L0 = ov_layout(num_pairs * num_sms * 2);
-  if (workspace_bytes < L0.total_fixed + 2048) return ARGUS_ERR_WORKSPACE;
-  const u64 span_cap = (workspace_bytes - L0.total_fixed - 1536) * 3 / (3 * kBytesPerSortedSpan + 4 * kBytesPerListedSpan);
-  const u64 list_cap = span_cap + span_cap / 3;
-  const size_t list_bytes = argus_align_up(256 + argus_align_up((size_t)list_cap * 4, 256) + (size_t)list_cap * 16, 256);
-  const int rc = ov_setup(a, num_streams, warps_per_cta, cta_sm, num_sms, pairs, num_pairs, out, status, workspace,
-                          workspace_bytes, stream, list_bytes);
-  if (rc != ARGUS_OK) return rc;
-  a.intervals = intervals; a.interval_offsets = (const u64*)interval_offsets; a.max_intervals = max_intervals;
-  if (scope) {
-    a.scoped = 1; a.ctx_lo = scope->ctx_lo; a.ctx_hi = scope->ctx_hi; a.warp_mask = scope->warp_mask;
-    a.sm_mask = scope->sm_mask; a.region_mask = scope->region_mask;
-  }
-  // the list of selected spans sits at the end of the workspace: counter, segments, spans
-  char* lbase = (char*)workspace + (workspace_bytes - list_bytes);
-  OvSelectOut o;
-  o.count = (u64*)lbase;
-  o.seg = (u32*)(lbase + 256);
-  o.spans = (ulonglong2*)(lbase + 256 + argus_align_up((size_t)list_cap * 4, 256));
-  o.capacity = list_cap;
-  o.chunk = 256;  // slots left unused are bounded by a quarter of the list: smaller chunks for small lists
-  while (o.chunk > 1 && (u64)kSelectWarps * o.chunk * 4 > list_cap) o.chunk >>= 1;
-  ARGUS_CUDA_TRY(cudaMemsetAsync(o.count, 0, 256, stream));
+  const size_t fixed = ov_fixed_bytes(num_streams);
+  if (workspace_bytes < fixed) return ARGUS_ERR_WORKSPACE;
+  const u64 cap = (workspace_bytes - fixed) / kBytesPerSpan;
+  const u32 slices = select_slices(num_streams), heads = num_streams * slices;
+  // control block, spans, scratch, entries, pieces
+  char* w = (char*)workspace;
+  ArgusOvCtl* const ctl = (ArgusOvCtl*)w;
+  w += argus_align_up(sizeof(ArgusOvCtl), 256);
+  void* const spans = w;
+  w += (size_t)cap * 32;
+  uint64_t* const entries = (uint64_t*)w;
+  w += argus_align_up((size_t)cap * 8, 16);
+  ArgusOvPiece* const pieces = (ArgusOvPiece*)w;
+  ARGUS_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(ArgusOvCtl), stream));
   if (num_streams) {
-    k_ov_select<<<num_streams < kSelectGrid ? num_streams : kSelectGrid, 256, 0, stream>>>(a, o);
+    OvSelectArgs o;
+    o.intervals = intervals; o.interval_offsets = (const u64*)interval_offsets; o.max_intervals = max_intervals;
+    o.num_streams = num_streams; o.warps_per_cta = warps_per_cta; o.num_sms = num_sms; o.num_pairs = num_pairs;
+    o.cta_sm = cta_sm; o.pairs = pairs; o.status = status; o.entries = (u64*)entries; o.entry_capacity = cap; o.pieces = pieces;
+    // a piece beyond a slice's first one holds more than kSelStage - 32 entries or is the slice's last, so one for every 96
+    // entries and one for every slice would do; the first ones are counted in the fixed part
+    o.slices = slices; o.piece_capacity = heads + (u32)(cap / 16 < 0x7fffffffu ? cap / 16 : 0x7fffffffu); o.ctl = ctl;
+    o.direct = max_intervals <= cap;
+    o.scoped = scope != nullptr;
+    o.ctx_lo = scope ? scope->ctx_lo : 0; o.ctx_hi = scope ? scope->ctx_hi : 0xffffffffu; o.warp_mask = scope ? scope->warp_mask : ~0ull;
+    o.sm_mask = scope ? scope->sm_mask : nullptr; o.region_mask = scope ? scope->region_mask : nullptr;
+    const u64 items = (u64)num_streams * (slices / kSelWarps);
+    k_ov_select<<<(unsigned)(items < kSelGrid ? items : kSelGrid), kSelThreads, 0, stream>>>(o);
     ARGUS_CHECK_LAUNCH();
   }
-  OvList l;
-  l.spans = o.spans; l.seg = o.seg; l.count = o.count; l.capacity = list_cap;
-  return ov_run(a, &l, stream);
+  return launch_pair<false>(pair_args(intervals, interval_offsets, entries, cap, pieces, slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs,
+                                      num_pairs, out, status, ctl, spans, cap), stream);
 }
 
 int argus_internal_overlap(const argus_interval_t* intervals, uint64_t max_intervals, const uint64_t* interval_offsets,

@@ -1,8 +1,8 @@
 // argus_synthesize.cu — the whole hot path in one call: pair -> aggregate -> overlap.
 //
 // Pairing writes, beside every 48-byte interval record, an 8-byte digest (region, both durations, a flag
-// bit); then ONE pass over the digests both aggregates the intervals and selects the overlap spans (a pass
-// over the records themselves reads six times the bytes). More than 400 regions or 128 pairs, or a call that
+// bit); then ONE pass over the digests both aggregates the intervals and selects the overlap candidates (a pass
+// over the records themselves reads six times the bytes). More than 400 regions, or a call that
 // asks for no table: the three plain calls. Results are identical in every mode. argus_synthesize_ring is the
 // same pipeline on a ring container.
 #include "argus_internal.cuh"
@@ -14,9 +14,8 @@ namespace {
 std::atomic<int> g_synth_mode_knob{-1};  // -1 = automatic
 
 struct SynLayout {
-  size_t pair, pair_bytes, agg, agg_bytes, list_count, list_seg, list_spans, ov, ov_bytes, digest, total;
-  uint64_t digest_capacity, list_capacity, list_slack;
-  uint32_t list_chunk;
+  size_t pair, pair_bytes, agg, agg_bytes, ov, ov_bytes, pieces, spans, digest, starts, total;
+  uint64_t digest_capacity;
 };
 
 SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_regions, uint64_t ambig_capacity,
@@ -25,25 +24,20 @@ SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_reg
   size_t o = 0;
   L.pair = o; L.pair_bytes = argus_pair_workspace_bytes(num_events, num_streams, ambig_capacity); o += argus_align_up(L.pair_bytes, 256);
   L.agg = o; L.agg_bytes = argus_aggregate_workspace_bytes(num_events / 2, num_streams, num_regions); o += argus_align_up(L.agg_bytes, 256);
-  // The span list: warps reserve slots in chunks and leave some unused, so the list is longer than the spans it
-  // may hold, by a quarter or by one smallest chunk for every warp that can append, whichever is more
-  // (the aggregation passes run at most one block of 8 warps per stream).
-  const uint64_t warps = (uint64_t)num_streams * 8 > 1024 ? (uint64_t)num_streams * 8 : 1024;
-  L.list_slack = num_pairs ? (max_overlap_spans / 4 > warps * 32 ? max_overlap_spans / 4 : warps * 32) : 0;
-  L.list_chunk = 256;
-  while (L.list_chunk > 32 && warps * L.list_chunk > L.list_slack) L.list_chunk >>= 1;
-  L.list_capacity = max_overlap_spans + L.list_slack;
-  L.list_count = o; o += 256;
-  L.list_seg = o; o += argus_align_up((size_t)L.list_capacity * 4 + 4, 256);
-  L.list_spans = o; o += argus_align_up((size_t)L.list_capacity * 16 + 16, 256);
+  // Overlap: the plain call's workspace, or control block, first pieces of the slices and 32 bytes a span (the entries
+  // lie in the digest array).
+  const bool digests = argus_aggregate_can_read_digests(num_regions);
+  const size_t pieces = (size_t)num_streams * argus_aggregate_digest_slices() * sizeof(ArgusOvPiece);
   L.ov = o;
-  // segment counters and the sorted spans (24 B each); a little more, so that the plain overlap call, which gets the
-  // list's room and this as one workspace and splits it itself (50.7 B a span), also holds max_overlap_spans
-  L.ov_bytes = argus_align_up((size_t)num_pairs * num_sms * 2 * 8 * 3 + 1024 + (size_t)max_overlap_spans * 27 + 4096, 256);
+  L.pieces = o + argus_align_up(sizeof(ArgusOvCtl), 256);
+  L.spans = L.pieces + argus_align_up(pieces, 256);
+  const size_t from_entries = L.spans - o + (size_t)max_overlap_spans * 32, plain = argus_internal_overlap_bytes(max_overlap_spans, num_streams);
+  L.ov_bytes = num_pairs ? argus_align_up(from_entries > plain ? from_entries : plain, 256) : 0;
   o += L.ov_bytes;
   // one digest per interval (a stream's intervals start at half its first event's position at the latest)
-  L.digest_capacity = argus_aggregate_can_select_overlap(num_regions, num_pairs) ? num_events / 2 + 1 : 0;
+  L.digest_capacity = digests ? num_events / 2 + 1 : 0;
   L.digest = o; o += argus_align_up((size_t)L.digest_capacity * 8, 256);
+  L.starts = o; o += num_pairs ? argus_align_up((size_t)L.digest_capacity * 8, 256) : 0;  // begin times of overlap candidates
   L.total = o;
   return L;
 }
@@ -51,7 +45,7 @@ SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_reg
 }  // namespace
 
 // Where argus_synthesize aggregates and selects overlap spans: -1 automatic, 1 in one pass over the intervals'
-// digests, 2 the plain calls, 3 in one pass over the interval records (test aid; results are identical).
+// digests, 2 the plain calls, 3 the same with the aggregation pass over the records (test aid; results are identical).
 extern "C" void argus_set_synthesize_mode(int mode) { g_synth_mode_knob.store(mode); }
 
 extern "C" size_t argus_synthesize_workspace_bytes(uint64_t num_events, uint32_t num_streams, uint32_t num_regions,
@@ -83,23 +77,16 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
   char* ws = (char*)workspace;
   const bool want_agg = warp_tab || cta_tab || sm_tab || kernel_tab;
 
-  ArgusFuseArgs f;
-  f.warp_tab = nullptr; f.cta_sm = cta_sm; f.warps_per_cta = warps_per_cta; f.num_sms = num_sms;
-  f.pairs = pairs; f.num_pairs = num_pairs; f.ov_spans = nullptr; f.ov_seg = nullptr; f.ov_capacity = 0; f.ov_count = nullptr; f.ov_chunk = L.list_chunk;
-  // where aggregation and overlap selection happen: 1 = in one pass over the intervals (their digests, or the
-  // records themselves) after pairing, 2 = the plain calls
-  const bool can_one_pass = num_streams > 0 && want_agg && argus_aggregate_can_select_overlap(num_regions, num_pairs);
-  int mode = can_one_pass ? 1 : 2;
-  if (g_synth_mode == 2) mode = 2;  // test aid: a forced mode applies when the inputs allow it
-  const bool list = mode != 2 && num_pairs;
-  if (list) {
-    f.ov_spans = (ulonglong2*)(ws + L.list_spans);
-    f.ov_seg = (u32*)(ws + L.list_seg);
-    f.ov_capacity = L.list_capacity;
-    f.ov_count = (u64*)(ws + L.list_count);
-    ARGUS_CUDA_TRY(cudaMemsetAsync(ws + L.list_count, 0, 256, stream));
+  // where aggregation and overlap selection happen: 1 = in one pass over the intervals' digests after pairing (or over the
+  // records, and then the plain overlap call), 2 = the plain calls
+  const bool can_one_pass = num_streams > 0 && want_agg && argus_aggregate_can_read_digests(num_regions) && num_pairs <= ARGUS_MAX_PAIRS;
+  const bool use_digest = can_one_pass && L.digest_capacity != 0 && g_synth_mode != 2 && g_synth_mode != 3;  // (test aid: modes 2 and 3)
+  ArgusOvCtl* const ov_ctl = (ArgusOvCtl*)(ws + L.ov);
+  ArgusFuseArgs f = ArgusFuseArgs();
+  if (use_digest && num_pairs) {
+    f.pairs = pairs; f.num_pairs = num_pairs; f.entries = (u64*)(ws + L.digest); f.starts = (u64*)(ws + L.starts); f.pieces = (ArgusOvPiece*)(ws + L.pieces);
+    ARGUS_CUDA_TRY(cudaMemsetAsync(ov_ctl, 0, sizeof(ArgusOvCtl), stream));
   }
-  const bool use_digest = mode == 1 && L.digest_capacity != 0 && g_synth_mode != 3;
   int rc = argus_internal_pair(events, num_events, stream_offsets, num_streams, num_regions, intervals, interval_capacity,
                                interval_offsets, ambig, ambig_capacity, ambig_offsets, status, ws + L.pair, L.pair_bytes,
                                cuda_stream, ring_written ? 2 : 0, ring_written == nullptr,
@@ -110,18 +97,18 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
     rc = argus_internal_aggregate_scoped(intervals, interval_offsets, ambig, ambig_offsets, num_streams, warps_per_cta,
                                          cta_sm, num_sms, num_regions, nullptr, warp_tab, cta_tab, sm_tab, kernel_tab,
                                          nullptr, nullptr, status, ws + L.agg, L.agg_bytes, cuda_stream, false,
-                                         mode == 1 && list ? &f : nullptr,
+                                         f.num_pairs ? &f : nullptr,
                                          use_digest ? (const uint64_t*)(ws + L.digest) : nullptr, interval_capacity);
     if (rc != ARGUS_OK) return rc;
   }
   if (num_pairs) {
-    if (mode != 2) {
-      rc = argus_internal_overlap_from_list(f.ov_spans, f.ov_seg, (const uint64_t*)f.ov_count, f.ov_capacity, num_sms, num_pairs, overlap_out,
-                                            status, ws + L.ov, L.ov_bytes, cuda_stream);
+    if (f.num_pairs) {
+      rc = argus_internal_overlap_from_digests(intervals, (const uint64_t*)f.starts, (const uint64_t*)f.entries, f.pieces,
+                                               argus_aggregate_digest_slices(), num_streams, warps_per_cta, cta_sm, num_sms, pairs,
+                                               num_pairs, overlap_out, status, ov_ctl, ws + L.spans, max_overlap_spans, cuda_stream);
     } else {
       rc = argus_internal_overlap(intervals, interval_capacity, interval_offsets, num_streams, warps_per_cta, cta_sm, num_sms,
-                                  pairs, num_pairs, overlap_out, status, ws + L.list_count, L.ov + L.ov_bytes - L.list_count,
-                                  cuda_stream, false);
+                                  pairs, num_pairs, overlap_out, status, ws + L.ov, L.ov_bytes, cuda_stream, false);
     }
     if (rc != ARGUS_OK) return rc;
   }

@@ -1,0 +1,57 @@
+"""argus_overlap's kernel at the sizes where its branches change: spans in order or not, one role or both, around the number of
+spans it holds in shared memory, starts that crowd, and a workspace too small for the plain layout of the entries."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_12299_b200 as argus
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+TILE = 9216  # spans of both roles that fit shared memory at a time
+
+
+def _intervals(rng, per_stream, S, order, other):
+    """S streams of per_stream intervals of regions 0 and 1 (every `other`-th of region 2), as pairing orders them: by end."""
+    iv = np.zeros(S * per_stream, argus.INTERVAL_DTYPE)
+    for s in range(S):
+        t = (1 << 40) + np.cumsum(rng.integers(1, 400, per_stream)).astype(np.uint64)
+        d = np.minimum(rng.integers(0, 300, per_stream), np.append(np.diff(t.astype(np.int64)), 100)).astype(np.uint64)
+        if order == "overlapping":
+            d += np.uint64(900)
+        elif order == "shuffled":
+            p = rng.permutation(per_stream)
+            t, d = t[p], d[p]
+        elif order == "crowded":
+            t = (1 << 40) + rng.integers(0, 50, per_stream).astype(np.uint64)
+            t[:2] += np.uint64(1 << 35)
+        sl = slice(s * per_stream, (s + 1) * per_stream)
+        iv["stream"][sl], iv["t_begin"][sl], iv["inclusive"][sl] = s, t, d
+        r = rng.integers(0, 2, per_stream)
+        r[::other] = 2
+        iv["region"][sl] = r
+    return iv
+
+
+@pytest.mark.parametrize("order", ["disjoint", "overlapping", "shuffled", "crowded"])
+@pytest.mark.parametrize("per_stream", [1, 33, TILE // 4, TILE // 2, TILE // 2 + 1, 23_000])
+def test_overlap_sizes_and_orders(order, per_stream):
+    rng = np.random.default_rng(per_stream)
+    S, W, M, other = 4, 2, 2, 3
+    iv = _intervals(rng, per_stream, S, order, other)
+    offs = (np.arange(S + 1) * per_stream).astype(np.uint64)
+    cta_sm = np.array([1, 0], np.uint32)
+    d_iv = torch.from_numpy(iv.view(np.uint8).reshape(-1).copy()).to(DEV)
+    d_off = torch.from_numpy(offs.view(np.int64).copy()).to(DEV)
+    d_sm = torch.from_numpy(cta_sm.view(np.int32)).to(DEV)
+    for pairs in ([(0, 1)], [(1, 0), (2, 2), (0, 9)]):
+        pairs_np = np.array(pairs, np.uint32)
+        d_pairs = torch.from_numpy(pairs_np.view(np.int32)).to(DEV)
+        _, want, _ = oracle.overlap(iv, offs, W, cta_sm, M, pairs_np)
+        spans = sum(int(((iv["region"] == r) & (iv["inclusive"] > 0)).sum()) for p in pairs for r in p)
+        # the whole workspace, and one with room for just the spans selected (fewer than the intervals)
+        for ws in (None, argus.argus_overlap_workspace_bytes((spans + 1) // 2, S, 1, M)):
+            out, st = argus.argus_overlap(d_iv, len(iv), d_off, W, d_sm, M, d_pairs, workspace_bytes=ws)
+            assert int(argus.argus_status_fetch(st)["code"]) == 0
+            assert out.cpu().numpy().view(argus.OVERLAP_DTYPE).reshape(want.shape).tobytes() == want.tobytes()

@@ -8,8 +8,8 @@
 //                   several CTAs fit an SM), for up to kAggCompactRegions regions;
 //   k_agg_streams : the same with a full 576 B-per-region copy in shared memory when that fits, else on
 //                   the global row itself. Integer atomics only: the result does not depend on thread order.
-//   k_agg_cta     : CTA-scope cells = reduction over the warps of each CTA (plain loads, no atomics).
-//   k_agg_init / k_agg_scatter : SM-scope and kernel-scope cells by atomic add/min/max of CTA cells.
+//   k_agg_rollup  : CTA-scope cells = reduction over the warps of each CTA; SM-scope and kernel-scope cells by atomic
+//                   add/min/max of CTA cells.
 //   k_agg_role    : warp-role cells = reduction over the CTAs of each warp index (plain loads).
 //   k_agg_iter    : per-iteration cells (key = ctx - ctx_lo) of the intervals of a scope.
 // A scope (iteration window, warp mask, SM mask, region mask) filters what k_agg_streams and
@@ -33,7 +33,6 @@ struct AggArgs {
   u32 num_streams, warps_per_cta, num_ctas, num_sms, num_regions;
   const u32* cta_sm;
   u64* warp_tab;  // [S][R][72] (caller's table or workspace)
-  u64* cta_tab;   // [C][R][72] (caller's table or workspace)
   u64* sm_tab;    // nullable
   u64* kernel_tab;  // nullable
   argus_status_t* status;
@@ -56,6 +55,13 @@ struct AggArgs {
   const u64* digest;  // digests of the intervals (k_agg_streams_digest; overwritten with entries where overlap is selected), null = read the records
   u64 interval_limit; // records the interval array holds: a stream whose offsets reach beyond it is reported, not read
 };
+
+// SM-scope and kernel-scope tables start empty; the kernel after the one that calls this adds to them.
+__device__ __forceinline__ void agg_empty_tables(const AggArgs& a) {
+  const u64 first = (u64)blockIdx.x * blockDim.x + threadIdx.x, stride = (u64)gridDim.x * blockDim.x, row = (u64)a.num_regions * kCell;
+  if (a.sm_tab) for (u64 i = first; i < a.num_sms * row; i += stride) a.sm_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
+  if (a.kernel_tab) for (u64 i = first; i < row; i += stride) a.kernel_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
+}
 
 __device__ __forceinline__ bool mask_bit(const u32* mask, u32 i) { return !mask || ((mask[i >> 5] >> (i & 31)) & 1u); }
 
@@ -104,6 +110,8 @@ __device__ __forceinline__ void agg_add_interval_lean(u64* tab, u32 region, u64 
 }
 
 __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
+  argus_kernel_begin_long();
+  agg_empty_tables(a);
   extern __shared__ __align__(16) u64 sh_tab[];
   const u32 R = a.num_regions;
   const u32 cells = R * kCell;
@@ -148,6 +156,8 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
 }
 
 __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) {
+  argus_kernel_begin_long();
+  agg_empty_tables(a);
   extern __shared__ __align__(16) unsigned char sh_raw[];
   ArgusAggCell* const ctab = reinterpret_cast<ArgusAggCell*>(sh_raw);
   const u32 R = a.num_regions;
@@ -207,7 +217,8 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
 // a region's cell (meta) holds what a lane needs to know about its region: histogram window base, copy slot,
 // whether the region appears in an overlap pair. A digest marked wide (a duration of 2^23 ticks or more) sends
 // its lane to the record and to 64-bit atomics on the global row. Every warp walks a slice of the stream, so that overlap
-// candidates stay in order; their entries replace digests that the warp has consumed: no list, no atomics. The table is addressed with 32-bit shared-memory addresses and the fields by constant offsets.
+// candidates stay in order; their entries replace digests that the warp has consumed: no list, no atomics. The table is
+// addressed with 32-bit shared-memory addresses and the fields by constant offsets.
 constexpr u32 kDigestHot = 4;
 constexpr u32 kDgSumInclLo = 0, kDgSumInclHi = 1, kDgSumExclLo = 2, kDgSumExclHi = 3, kDgMin = 4, kDgMax = 5, kDgFlag = 6,
               kDgCountOut = 7, kDgBins = 8, kDgMeta = kDgBins + kAggWindow, kDgWords = kDgMeta + 1;
@@ -256,6 +267,9 @@ __device__ __noinline__ u32 digest_bin_rare(u32* meta_word, u32 bin, u32 cell, u
 constexpr int kDgThreads = 512;
 constexpr u32 kDgSlices = kDgThreads / 32;     // slices of a stream, one per warp (also the slices of the overlap entries)
 __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a) {
+  argus_kernel_begin_long();
+  agg_empty_tables(a);
+  if (a.ov.num_pairs && blockIdx.x == 0 && threadIdx.x == 0) *a.ov.ctl = ArgusOvCtl{};
   extern __shared__ __align__(16) unsigned char sh_raw[];
   u32* const tab = reinterpret_cast<u32*>(sh_raw);
   const u32 R = a.num_regions;
@@ -482,33 +496,25 @@ __device__ __forceinline__ u64 combine(u32 field, u64 x, u64 y) {
   return field == 2 ? (x < y ? x : y) : field == 3 ? (x > y ? x : y) : x + y;
 }
 
-// cta_tab[c][r][j] = reduce over w of warp_tab[c*W + w][r][j]
-__global__ void __launch_bounds__(256) k_agg_cta(AggArgs a) {
-  const u64 per_cta = (u64)a.num_regions * kCell;
-  const u64 n = (u64)a.num_ctas * per_cta;
-  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-    const u64 c = i / per_cta, rem = i % per_cta;
-    const u32 field = (u32)(rem % kCell);
-    const u64* src = a.warp_tab + c * a.warps_per_cta * per_cta + rem;
-    u64 acc = src[0];
-    for (u32 w = 1; w < a.warps_per_cta; ++w) acc = combine(field, acc, src[(u64)w * per_cta]);
-    a.cta_tab[i] = acc;
-  }
-}
-
 __global__ void __launch_bounds__(256) k_agg_init(u64* tab, u64 n) {
+  argus_kernel_begin();
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x)
     tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
 }
 
-// SM-scope and kernel-scope cells from CTA cells (atomic add / min / max on integers).
-__global__ void __launch_bounds__(256) k_agg_scatter(AggArgs a) {
-  const u64 per_cta = (u64)a.num_regions * kCell;
-  const u64 n = (u64)a.num_ctas * per_cta;
+// CTA cells = reduction over the warps of each CTA (written if asked for), added to the SM-scope and kernel-scope cells (atomic
+// add / min / max on integers). Bound by the read of the warp-scope table; eight warps' words are asked for at a time.
+__global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
+  argus_kernel_begin_long();
+  const u64 per_cta = (u64)a.num_regions * kCell, n = (u64)a.num_ctas * per_cta;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
     const u64 c = i / per_cta, rem = i % per_cta;
     const u32 field = (u32)(rem % kCell);
-    const u64 v = a.cta_tab[i];
+    const u64* src = a.warp_tab + c * a.warps_per_cta * per_cta + rem;
+    u64 v = src[0];
+#pragma unroll 8
+    for (u32 w = 1; w < a.warps_per_cta; ++w) v = combine(field, v, src[(u64)w * per_cta]);
+    if (cta_out) cta_out[i] = v;
     if (field == 2 ? v == ~0ull : v == 0ull) continue;  // identity element: nothing to add
     if (a.sm_tab) {
       const u32 m = a.cta_sm[c];
@@ -525,6 +531,7 @@ __global__ void __launch_bounds__(256) k_agg_scatter(AggArgs a) {
 
 // role_tab[w][r][j] = reduce over c of warp_tab[c*W + w][r][j]
 __global__ void __launch_bounds__(256) k_agg_role(AggArgs a) {
+  argus_kernel_begin_long();
   const u64 per_row = (u64)a.num_regions * kCell;
   const u64 n = (u64)a.warps_per_cta * per_row;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
@@ -541,6 +548,7 @@ __global__ void __launch_bounds__(256) k_agg_role(AggArgs a) {
 // streams in a shared-memory copy of the table when that fits and adds the non-empty cells to the global
 // table (initialised by k_agg_init) at the end; otherwise it updates the global table record by record.
 __global__ void __launch_bounds__(kAggThreads) k_agg_iter(AggArgs a) {
+  argus_kernel_begin_long();
   extern __shared__ __align__(16) u64 sh_tab[];
   const u32 R = a.num_regions;
   const u64 cells = (u64)a.num_iters * R * kCell;
@@ -589,6 +597,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_iter(AggArgs a) {
 // iter_tab[i] = combination of cell word i over the private copies (none: iter_tab holds the sums already);
 // the interval count of a cell, which the global path leaves out, is the sum of its histogram bins.
 __global__ void __launch_bounds__(256) k_agg_iter_reduce(AggArgs a) {
+  argus_kernel_begin();
   const u64 cells = (u64)a.num_iters * a.num_regions * kCell;
   if (a.iter_copies) {
     for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < cells; i += (u64)gridDim.x * blockDim.x) {
@@ -611,14 +620,13 @@ __global__ void __launch_bounds__(256) k_agg_iter_reduce(AggArgs a) {
   }
 }
 
-struct AggLayout { size_t warp, cta, iter, total; };
+struct AggLayout { size_t warp, iter, total; };
 
 AggLayout agg_layout(uint32_t num_streams, uint32_t num_regions) {
   AggLayout L;
   const size_t row = (size_t)num_regions * sizeof(argus_agg_t);
   L.warp = 0;
-  L.cta = argus_align_up((size_t)num_streams * row, 256);
-  L.iter = L.cta + argus_align_up((size_t)num_streams * row, 256);  // C <= S
+  L.iter = argus_align_up((size_t)num_streams * row, 256);
   L.total = L.iter + kIterScratchBytes;
   return L;
 }
@@ -650,13 +658,13 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   const AggLayout L = agg_layout(num_streams, num_regions);
   if (workspace_bytes < L.total) return ARGUS_ERR_WORKSPACE;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  if (reset_status) ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
+  if (reset_status) { const int rc = argus_internal_clear(status, nullptr, 0, cuda_stream); if (rc != ARGUS_OK) return rc; }
   const u32 num_iters = iter_tab ? scope->ctx_hi - scope->ctx_lo + 1 : 0;
-  if (kernel_tab) { k_agg_init<<<16, 256, 0, stream>>>((u64*)kernel_tab, (u64)num_regions * kCell); ARGUS_CHECK_LAUNCH(); }
-  if (sm_tab) { k_agg_init<<<296, 256, 0, stream>>>((u64*)sm_tab, (u64)num_sms * num_regions * kCell); ARGUS_CHECK_LAUNCH(); }
   if (num_streams == 0) {
-    if (role_tab) { k_agg_init<<<64, 256, 0, stream>>>((u64*)role_tab, (u64)warps_per_cta * num_regions * kCell); ARGUS_CHECK_LAUNCH(); }
-    if (iter_tab) { k_agg_init<<<64, 256, 0, stream>>>((u64*)iter_tab, (u64)num_iters * num_regions * kCell); ARGUS_CHECK_LAUNCH(); }
+    if (kernel_tab) ARGUS_LAUNCH(k_agg_init, 16, 256, 0, stream, (u64*)kernel_tab, (u64)num_regions * kCell);
+    if (sm_tab) ARGUS_LAUNCH(k_agg_init, 296, 256, 0, stream, (u64*)sm_tab, (u64)num_sms * num_regions * kCell);
+    if (role_tab) { ARGUS_LAUNCH(k_agg_init, 64, 256, 0, stream, (u64*)role_tab, (u64)warps_per_cta * num_regions * kCell); }
+    if (iter_tab) { ARGUS_LAUNCH(k_agg_init, 64, 256, 0, stream, (u64*)iter_tab, (u64)num_iters * num_regions * kCell); }
     return ARGUS_OK;
   }
   AggArgs a;
@@ -664,7 +672,6 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   a.num_streams = num_streams; a.warps_per_cta = warps_per_cta; a.num_ctas = num_streams / warps_per_cta;
   a.num_sms = num_sms; a.num_regions = num_regions; a.cta_sm = cta_sm;
   a.warp_tab = warp_tab ? (u64*)warp_tab : (u64*)((char*)workspace + L.warp);
-  a.cta_tab = cta_tab ? (u64*)cta_tab : (u64*)((char*)workspace + L.cta);
   a.sm_tab = (u64*)sm_tab; a.kernel_tab = (u64*)kernel_tab; a.status = status;
   a.scoped = scope != nullptr;
   a.ctx_lo = scope ? scope->ctx_lo : 0; a.ctx_hi = scope ? scope->ctx_hi : 0xffffffffu;
@@ -691,12 +698,8 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   const u64 iter_cells = (u64)num_iters * num_regions * kCell;
   a.iter_inline = iter_tab && !a.iter_smem && num_regions <= kAggCompactRegions;
   if (iter_tab) {
-    if (a.iter_copies) {
-      k_agg_init<<<592, 256, 0, stream>>>(a.iter_copies, iter_cells * a.num_copies);
-    } else {
-      k_agg_init<<<296, 256, 0, stream>>>((u64*)iter_tab, iter_cells);
-    }
-    ARGUS_CHECK_LAUNCH();
+    if (a.iter_copies) ARGUS_LAUNCH(k_agg_init, 592, 256, 0, stream, a.iter_copies, iter_cells * a.num_copies);
+    else ARGUS_LAUNCH(k_agg_init, 296, 256, 0, stream, (u64*)iter_tab, iter_cells);
   }
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 0);
   if (num_regions <= kAggCompactRegions) {
@@ -707,37 +710,29 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       const size_t dg = digest_table_words(num_regions) * 4 + ((num_regions + 31) / 32) * 4;
       if (dg > 48 * 1024)
         ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_digest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
-      k_agg_streams_digest<<<num_streams, kDgThreads, dg, stream>>>(a);
+      ARGUS_LAUNCH(k_agg_streams_digest, num_streams, kDgThreads, dg, stream, a);
     } else {
-      k_agg_streams_compact<<<num_streams, kAggThreads, compact, stream>>>(a);
+      ARGUS_LAUNCH(k_agg_streams_compact, num_streams, kAggThreads, compact, stream, a);
     }
   } else {
-    k_agg_streams<<<num_streams, kAggThreads, need, stream>>>(a);
+    ARGUS_LAUNCH(k_agg_streams, num_streams, kAggThreads, need, stream, a);
   }
-  ARGUS_CHECK_LAUNCH();
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 1);
   if (iter_tab) {
     if (!a.iter_inline) {
       const unsigned iter_grid = a.iter_smem ? 296u : 148u * 8u;
-      k_agg_iter<<<num_streams < iter_grid ? num_streams : iter_grid, kAggThreads, need_iter, stream>>>(a);
-      ARGUS_CHECK_LAUNCH();
+      ARGUS_LAUNCH(k_agg_iter, num_streams < iter_grid ? num_streams : iter_grid, kAggThreads, need_iter, stream, a);
     }
     if (!a.iter_smem) {
-      k_agg_iter_reduce<<<296, 256, 0, stream>>>(a);
-      ARGUS_CHECK_LAUNCH();
+      ARGUS_LAUNCH(k_agg_iter_reduce, 296, 256, 0, stream, a);
     }
   }
   if (role_tab) {
-    k_agg_role<<<296, 256, 0, stream>>>(a);
-    ARGUS_CHECK_LAUNCH();
+    ARGUS_LAUNCH(k_agg_role, 296, 256, 0, stream, a);
   }
   if (cta_tab || sm_tab || kernel_tab) {
-    k_agg_cta<<<1184, 256, 0, stream>>>(a);
-    ARGUS_CHECK_LAUNCH();
-  }
-  if (sm_tab || kernel_tab) {
-    k_agg_scatter<<<1184, 256, 0, stream>>>(a);
-    ARGUS_CHECK_LAUNCH();
+    const u64 want = ((u64)a.num_ctas * num_regions * kCell + 255) / 256;
+    ARGUS_LAUNCH(k_agg_rollup, (unsigned)(want < 2368 ? want : 2368), 256, 0, stream, a, (u64*)cta_tab);
   }
   return ARGUS_OK;
 }

@@ -1,5 +1,5 @@
 // argus_api.cu — status fetch, error strings, version.
-#include "argus_common.cuh"
+#include "argus_internal.cuh"
 
 #include <atomic>
 #include <mutex>
@@ -12,7 +12,18 @@ thread_local int g_prof_suppress = 0;  // per host thread: a call that must not 
 std::mutex g_prof_mu;
 struct ProfPair { cudaEvent_t a, b; };
 std::vector<ProfPair> g_prof[ARGUS_PROF_SLOTS];
+
+__global__ void __launch_bounds__(256) k_clear(argus_status_t* status, u64* extra, u32 words) {
+  argus_kernel_begin();
+  if (status && threadIdx.x < sizeof(argus_status_t) / 8) reinterpret_cast<u64*>(status)[threadIdx.x] = 0;
+  for (u32 i = threadIdx.x; i < words; i += blockDim.x) extra[i] = 0;
+}
 }  // namespace
+
+int argus_internal_clear(argus_status_t* status, void* extra, size_t bytes, void* cuda_stream) {
+  ARGUS_LAUNCH(k_clear, 1, 256, 0, (cudaStream_t)cuda_stream, status, (u64*)extra, extra ? (u32)(bytes / 8) : 0u);
+  return ARGUS_OK;
+}
 
 void argus_count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 

@@ -32,6 +32,7 @@ __device__ __forceinline__ void shared_add64(u64* p64, u64 v) {
 __global__ void __launch_bounds__(256) k_map_counts(const argus_interval_t* intervals, const u64* interval_offsets,
                                                     u32 num_streams, u32 exec_region, u32 num_pcs, u64* counts,
                                                     argus_status_t* status, int use_cache) {
+  argus_kernel_begin_long();
   __shared__ u32 keys[kMapSlots];
   __shared__ u64 sums[kMapSlots];
   for (u32 i = threadIdx.x; i < kMapSlots; i += blockDim.x) { keys[i] = kMapEmpty; sums[i] = 0; }
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(256) k_map_counts(const argus_interval_t* inte
 // One thread per PC: column total (kept for the row pass), alpha, entropy.
 __global__ void __launch_bounds__(kAttrThreads) k_attr_columns(const u64* counts, u32 num_rows, u32 num_pcs,
                                                                double* entropy, double* alpha, u64* totals) {
+  argus_kernel_begin_long();
   const u32 p = blockIdx.x * kAttrThreads + threadIdx.x;
   if (p >= num_pcs) return;
   u64 total = 0;
@@ -83,6 +85,7 @@ __global__ void __launch_bounds__(kAttrThreads) k_attr_columns(const u64* counts
 // threads by a fixed tree: the same bits every run.
 __global__ void __launch_bounds__(kAttrThreads) k_attr_rows(const u64* counts, const u64* totals, u32 num_rows, u32 num_pcs,
                                                             const double* metric, u32 num_chunks, double* partial) {
+  argus_kernel_begin();
   __shared__ double sh[kAttrThreads / 32];
   const u32 r = blockIdx.y, c = blockIdx.x;
   const u32 p0 = c * kAttrChunk, p1 = p0 + kAttrChunk < num_pcs ? p0 + kAttrChunk : num_pcs;
@@ -103,6 +106,7 @@ __global__ void __launch_bounds__(kAttrThreads) k_attr_rows(const u64* counts, c
 }
 
 __global__ void __launch_bounds__(256) k_attr_finish(const double* partial, u32 num_chunks, u32 num_rows, double* mhat) {
+  argus_kernel_begin();
   const u32 r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= num_rows) return;
   double s = 0.0;
@@ -133,9 +137,8 @@ extern "C" int argus_map_pc_counts(const argus_interval_t* intervals, const uint
   ARGUS_CUDA_TRY(cudaMemsetAsync(counts, 0, ((size_t)exec_region + 1) * num_pcs * sizeof(uint64_t), stream));
   if (num_streams == 0) return ARGUS_OK;
   const int use_cache = ((uint64_t)exec_region + 1) * num_pcs < 0xffffffffull;  // cell indices must fit the 32-bit keys
-  k_map_counts<<<148 * 8, 256, 0, stream>>>(intervals, (const u64*)interval_offsets, num_streams, exec_region, num_pcs,
-                                            (u64*)counts, status, use_cache);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_map_counts, 148 * 8, 256, 0, stream, intervals, (const u64*)interval_offsets, num_streams, exec_region,
+               num_pcs, (u64*)counts, status, use_cache);
   return ARGUS_OK;
 }
 
@@ -156,13 +159,10 @@ extern "C" int argus_attribute(const uint64_t* counts, uint32_t num_rows, uint32
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   u64* totals = (u64*)((char*)workspace + L.totals);
   double* partial = (double*)((char*)workspace + L.partial);
-  k_attr_columns<<<(num_pcs + kAttrThreads - 1) / kAttrThreads, kAttrThreads, 0, stream>>>((const u64*)counts, num_rows, num_pcs,
-                                                                                            entropy, alpha, totals);
-  ARGUS_CHECK_LAUNCH();
-  k_attr_rows<<<dim3(L.chunks, num_rows), kAttrThreads, 0, stream>>>((const u64*)counts, totals, num_rows, num_pcs, metric,
-                                                                     L.chunks, partial);
-  ARGUS_CHECK_LAUNCH();
-  k_attr_finish<<<(num_rows + 255) / 256, 256, 0, stream>>>(partial, L.chunks, num_rows, mhat);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_attr_columns, (num_pcs + kAttrThreads - 1) / kAttrThreads, kAttrThreads, 0, stream, (const u64*)counts, num_rows,
+               num_pcs, entropy, alpha, totals);
+  ARGUS_LAUNCH(k_attr_rows, dim3(L.chunks, num_rows), kAttrThreads, 0, stream, (const u64*)counts, totals, num_rows, num_pcs, metric,
+               L.chunks, partial);
+  ARGUS_LAUNCH(k_attr_finish, (num_rows + 255) / 256, 256, 0, stream, partial, L.chunks, num_rows, mhat);
   return ARGUS_OK;
 }

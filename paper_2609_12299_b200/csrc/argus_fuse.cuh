@@ -52,6 +52,7 @@ struct ArgusFuseArgs {    // selection inside the pass over the digests
   u64* entries;           // the digest array: a warp writes the entries of its slice over the digests it has consumed
   u64* starts;            // begin times of the entries' intervals, same positions
   ArgusOvPiece* pieces;   // [S][slices]
+  ArgusOvCtl* ctl;        // cleared by the pass
 };
 
 struct ArgusFuseCtx {     // per CTA, for the stream it is aggregating

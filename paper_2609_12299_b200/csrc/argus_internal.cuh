@@ -4,6 +4,9 @@
 
 #include "argus_fuse.cuh"
 
+// argus_api.cu — one small kernel that clears a status block and/or `bytes` (a multiple of 8) at `extra` (both nullable).
+int argus_internal_clear(argus_status_t* status, void* extra, size_t bytes, void* cuda_stream);
+
 // argus_pair.cu — the whole pairing pipeline. kernel_choice: 0 = automatic, 1 = one thread per stream, 2 = tiled.
 // `digest` (nullable): one 8-byte digest per interval record, at the record's position (see argus_fuse.cuh).
 // `ring_written` (nullable): `events` is a ring container (one slot of ring_capacity records per stream, written[s] records

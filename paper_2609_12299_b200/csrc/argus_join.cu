@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(kJoinThreads) k_join(const argus_interval_t* r
                                                        const argus_interval_t* samples, u64 num_samples,
                                                        const u64* sample_offsets, u32 num_runs, u32 num_streams,
                                                        argus_join_t* out, argus_status_t* status) {
+  argus_kernel_begin_long();
   __shared__ u64 vals[ARGUS_JOIN_MAX_SAMPLES];
   __shared__ u64 warp_sum[kJoinThreads / 32];
   __shared__ u32 cnt;
@@ -141,6 +142,7 @@ __device__ __forceinline__ void join_key(const argus_interval_t* rec, u32* strea
 // Every query claims the slot of its key, or finds the query that already has. A slot's key is the key of the
 // query that owns it (read through the reference record), so claiming is one compare-and-swap and nothing waits.
 __global__ void __launch_bounds__(256) k_join_claim(JoinHashArgs g) {
+  argus_kernel_begin();
   const u32 q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.num_queries) return;
   g.count[q] = 0; g.sum[q] = 0;
@@ -164,6 +166,7 @@ __global__ void __launch_bounds__(256) k_join_claim(JoinHashArgs g) {
 }
 
 __global__ void __launch_bounds__(256) k_join_fill(JoinHashArgs g) {
+  argus_kernel_begin();
   const u32 slot = blockIdx.x * blockDim.x + threadIdx.x;
   if (slot > g.cap_mask) return;
   const u32 o = g.table[slot].owner;
@@ -174,6 +177,7 @@ __global__ void __launch_bounds__(256) k_join_fill(JoinHashArgs g) {
 }
 
 __global__ void __launch_bounds__(256) k_join_scan(JoinHashArgs g) {
+  argus_kernel_begin_long();
   const uint4* tab = reinterpret_cast<const uint4*>(g.table);
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < g.num_samples; i += (u64)gridDim.x * blockDim.x) {
     const uint4* p = reinterpret_cast<const uint4*>(g.samples + i);
@@ -196,6 +200,7 @@ __global__ void __launch_bounds__(256) k_join_scan(JoinHashArgs g) {
 }
 
 __global__ void __launch_bounds__(kJoinThreads) k_join_rank(JoinHashArgs g) {
+  argus_kernel_begin();
   __shared__ u64 vals[ARGUS_JOIN_MAX_SAMPLES];
   const u32 tid = threadIdx.x;
   for (u32 q = blockIdx.x; q < g.num_queries; q += gridDim.x) {
@@ -274,10 +279,8 @@ static int join_impl(const argus_interval_t* reference, uint64_t num_reference, 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
   if (num_queries == 0) return ARGUS_OK;
-  k_join<<<num_queries < 148u * 8u ? num_queries : 148u * 8u, kJoinThreads, 0, stream>>>(
-      reference, num_reference, (const u64*)ref_index, num_queries, samples, num_samples, (const u64*)sample_offsets, num_runs,
-      num_streams, out, status);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_join, num_queries < 148u * 8u ? num_queries : 148u * 8u, kJoinThreads, 0, stream, reference, num_reference,
+               (const u64*)ref_index, num_queries, samples, num_samples, (const u64*)sample_offsets, num_runs, num_streams, out, status);
   return ARGUS_OK;
 }
 
@@ -325,20 +328,16 @@ extern "C" int argus_join_samples_hashed(const argus_interval_t* reference, uint
   g.key_of_query = (u32*)(ws + L.key_of_query); g.count = (u64*)(ws + L.count); g.sum = (u64*)(ws + L.sum);
   g.vals = (u64*)(ws + L.vals); g.out = out; g.status = status;
   ARGUS_CUDA_TRY(cudaMemsetAsync(ws + L.table, 0, (size_t)L.cap * sizeof(JoinSlot), stream));
-  k_join_claim<<<(num_queries + 255) / 256, 256, 0, stream>>>(g);
-  ARGUS_CHECK_LAUNCH();
-  k_join_fill<<<(L.cap + 255) / 256, 256, 0, stream>>>(g);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_join_claim, (num_queries + 255) / 256, 256, 0, stream, g);
+  ARGUS_LAUNCH(k_join_fill, (L.cap + 255) / 256, 256, 0, stream, g);
   if (num_samples) {
     int dev = 0, sms = 0;
     ARGUS_CUDA_TRY(cudaGetDevice(&dev));
     ARGUS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const u64 want = (num_samples + 255) / 256;
     const u64 cap_blocks = (u64)sms * 16;
-    k_join_scan<<<(unsigned)(want < cap_blocks ? want : cap_blocks), 256, 0, stream>>>(g);
-    ARGUS_CHECK_LAUNCH();
+    ARGUS_LAUNCH(k_join_scan, (unsigned)(want < cap_blocks ? want : cap_blocks), 256, 0, stream, g);
   }
-  k_join_rank<<<num_queries < 2368u ? num_queries : 2368u, kJoinThreads, 0, stream>>>(g);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_join_rank, num_queries < 2368u ? num_queries : 2368u, kJoinThreads, 0, stream, g);
   return ARGUS_OK;
 }

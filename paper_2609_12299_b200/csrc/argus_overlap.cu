@@ -52,6 +52,7 @@ __device__ __forceinline__ bool ov_mask_bit(const u32* mask, u32 i) { return !ma
 // Where the workspace has a place for every interval the entries go straight to their slice's; else the warp collects them
 // and appends about 100 at a time, exactly as many places as it needs, as pieces of a chain.
 __global__ void __launch_bounds__(kSelThreads) k_ov_select(OvSelectArgs a) {
+  argus_kernel_begin_long();
   __shared__ u32 filter[kSelFilter / 32];
   __shared__ u32 sh_pairs[2 * ARGUS_MAX_PAIRS];
   __shared__ u64 stage[kSelWarps][kSelStage];
@@ -290,7 +291,8 @@ __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratc
 // Sort of both roles together, up to kTile spans (in0[0..n0), in1[0..n1); a role that is in order already comes with n = 0),
 // into out0 and out1: spans are spread over buckets of equal width in start time, about one for a span, and a span's place is
 // the number of earlier ones in its bucket. Elements are 8 bytes, start time relative to the role's earliest (50 bits) and place (14
-// bits); the spans follow once (4,096 spans a role: 20 us; merging runs pairwise took 50 us). Returns false, the same for all threads and with nothing written, when a bucket would hold
+// bits); the spans follow once (4,096 spans a role: 20 us; merging runs pairwise took 50 us). Returns false, the same for
+// all threads and with nothing written, when a bucket would hold
 // more than kBucketMost (starts that crowd) or a role's starts spread over 2^50 ticks: the caller then merges.
 constexpr u32 kBuckets = 8192, kBucketMost = 32;  // buckets of a role at most
 __host__ __device__ constexpr u32 bucket_word(u32 b) { return b + (b >> 5); }  // padded: threads sum up runs of counters without bank conflicts
@@ -424,6 +426,7 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
 // DIGEST: entries as the pass over the digests leaves them (argus_fuse.cuh); else {index in the stream, region}.
 template <bool DIGEST>
 __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
+  argus_kernel_begin_long();
   extern __shared__ __align__(16) unsigned char pair_raw[];
   ulonglong2* const tile = reinterpret_cast<ulonglong2*>(pair_raw);
   __shared__ u32 sh_hit[kPairThreads];             // CTAs of this SM among the ones just looked at
@@ -439,7 +442,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
   const u32 P = a.pairs[2 * k], C = a.pairs[2 * k + 1];
   const u32 num_ctas = a.num_streams / a.warps_per_cta, per_cta = a.warps_per_cta * a.slices;
   if (tid == 0) {
-    sh_u = a.status->code;
+    sh_u = __ldcg(&a.status->code);
     if (a.ctl->num_entries > a.entry_capacity) {  // the selection ran out of room
       sh_u = ARGUS_ERR_CAPACITY;
       if (blockIdx.x == 0) {
@@ -741,8 +744,7 @@ int launch_pair(const OvPairArgs& a, cudaStream_t stream) {
     opted_in[dev].store(true, std::memory_order_release);
   }
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);
-  k_ov_pair<DIGEST><<<a.blocks, kPairThreads, kPairSmem, stream>>>(a);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_ov_pair<DIGEST>, a.blocks, kPairThreads, kPairSmem, stream, a);
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 1);
   return ARGUS_OK;
 }
@@ -795,10 +797,13 @@ static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_interv
     return ARGUS_ERR_INVALID_ARG;
   if ((uint64_t)num_pairs * num_sms * 2 > 0x7fffffffull) return ARGUS_ERR_INVALID_ARG;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  if (reset_status) ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
-  if (num_pairs == 0) return ARGUS_OK;
   const size_t fixed = ov_fixed_bytes(num_streams);
-  if (workspace_bytes < fixed) return ARGUS_ERR_WORKSPACE;
+  if (num_pairs && workspace_bytes < fixed) return ARGUS_ERR_WORKSPACE;
+  if (reset_status || num_pairs) {
+    const int rc = argus_internal_clear(reset_status ? status : nullptr, num_pairs ? workspace : nullptr, sizeof(ArgusOvCtl), cuda_stream);
+    if (rc != ARGUS_OK) return rc;
+  }
+  if (num_pairs == 0) return ARGUS_OK;
   const u64 cap = (workspace_bytes - fixed) / kBytesPerSpan;
   const u32 slices = select_slices(num_streams), heads = num_streams * slices;
   // control block, spans, scratch, entries, pieces
@@ -810,7 +815,6 @@ static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_interv
   uint64_t* const entries = (uint64_t*)w;
   w += argus_align_up((size_t)cap * 8, 16);
   ArgusOvPiece* const pieces = (ArgusOvPiece*)w;
-  ARGUS_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(ArgusOvCtl), stream));
   if (num_streams) {
     OvSelectArgs o;
     o.intervals = intervals; o.interval_offsets = (const u64*)interval_offsets; o.max_intervals = max_intervals;
@@ -824,8 +828,7 @@ static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_interv
     o.ctx_lo = scope ? scope->ctx_lo : 0; o.ctx_hi = scope ? scope->ctx_hi : 0xffffffffu; o.warp_mask = scope ? scope->warp_mask : ~0ull;
     o.sm_mask = scope ? scope->sm_mask : nullptr; o.region_mask = scope ? scope->region_mask : nullptr;
     const u64 items = (u64)num_streams * (slices / kSelWarps);
-    k_ov_select<<<(unsigned)(items < kSelGrid ? items : kSelGrid), kSelThreads, 0, stream>>>(o);
-    ARGUS_CHECK_LAUNCH();
+    ARGUS_LAUNCH(k_ov_select, (unsigned)(items < kSelGrid ? items : kSelGrid), kSelThreads, 0, stream, o);
   }
   return launch_pair<false>(pair_args(intervals, interval_offsets, entries, cap, pieces, slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs,
                                       num_pairs, out, status, ctl, spans, cap), stream);

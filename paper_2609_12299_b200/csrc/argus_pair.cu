@@ -1,13 +1,13 @@
 // argus_pair.cu — argus_pair_intervals: marker events -> nested intervals + ambiguity records.
 //
 // Pipeline enqueued on the caller's stream (no host synchronisation):
-//   memset(control block, event bitmap)
-//   pair pass 1   : intervals written at provisional bases floor((off[s]-off[0])/2), exact for
-//                   well-formed traces; per-stream counts; ambiguity notes + bitmap bits
-//   offsets       : scan of counts -> interval_offsets; sets `redo` when a base was provisional-wrong
-//   pair pass 2   : only does work when `redo` is set (malformed traces): rewrites intervals at the
-//                   final bases
-//   ambiguity     : popcount prefix over the bitmap -> rank of every note -> ordered records, offsets
+//   init, order   : control block and event bitmap cleared; the count of every stream foretold, and from their sum the
+//                   provisional base of its intervals; the order in which streams start
+//   pair pass 1   : intervals written at the provisional bases; per-stream counts; ambiguity notes + bitmap bits
+//   offsets       : scan of counts -> interval_offsets; sets `redo` when a count came out other than foretold;
+//                   popcount prefix over the bitmap if there are notes
+//   pair pass 2   : only does work when `redo` is set: rewrites the intervals of the streams behind at the final bases
+//   ambiguity     : rank of every note in the bitmap -> ordered records, offsets
 #include "argus_internal.cuh"
 #include "argus_pair_common.cuh"
 
@@ -26,9 +26,10 @@ std::atomic<u32> g_poll_limit{1u << 19};  // see argus_testing_set_poll_limit
 // Exact for any input; used for small traces and as the arbiter the tiled kernel falls back to.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_pair_thread_per_stream(ArgusPairArgs a) {
+  argus_kernel_begin_long();
   const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= a.num_streams) return;
-  if (a.redo && !a.ctl->redo) return;
+  if (a.redo && !__ldcg(&a.ctl->redo)) return;
   const u64 off0 = a.stream_offsets[0];
   const u64 lo = a.stream_offsets[s], hi = a.stream_offsets[s + 1];
   if (hi < lo || hi > a.num_events || lo < off0 || (hi - lo) >> 32) {
@@ -36,9 +37,8 @@ __global__ void __launch_bounds__(128) k_pair_thread_per_stream(ArgusPairArgs a)
     if (!a.redo) a.counts[s] = 0;
     return;
   }
-  const u64 base = a.redo ? a.interval_offsets[s] : ((lo - off0) >> 1);
-  // second pass: intervals that already lie where they belong (same position, all of them fitted) stay
-  if (a.redo && base == ((lo - off0) >> 1) && base + a.counts[s] <= a.interval_capacity) return;
+  const u64 base = a.redo ? a.interval_offsets[s] : a.bases[s];
+  if (a.redo && s < __ldcg(&a.ctl->redo_from)) return;  // second pass: these intervals already lie where they belong
   ArgusFrame stk[ARGUS_MAX_DEPTH];
   ArgusSeqState st;
   st.h = 0; st.n_int = 0; st.n_ctx = st.n_rev = st.n_clamp = 0; st.failed = false;
@@ -55,25 +55,168 @@ __global__ void __launch_bounds__(128) k_pair_thread_per_stream(ArgusPairArgs a)
 }
 
 // ---------------------------------------------------------------------------------------------
-// order: streams sorted by length class (floor(log2(events))), longest first. A stream is a chain of chunks that
-// one CTA at a time walks, so when lengths differ (producer and consumer warps of one kernel) the long chains must
-// start first or they end last, alone. Counting sort in one block; the order inside a class does not matter.
+// Foretelling a stream's interval count. Intervals are written before anybody knows how many the streams before theirs
+// hold, and a wrong guess costs the second pass. A stream whose markers nest has (events - unmatched ends - unmatched
+// begins) / 2 intervals; unmatched ends lie at its front (a ring slot that has wrapped) and unmatched begins at its back (a
+// stream that was cut short), so a look at both ends tells them. A stream that starts with begin(r) and stops with end(r) is
+// taken to be whole. Otherwise, if its last marker is an end(b), b is taken to be an outermost region and the front is read
+// until an unmatched end(b), which tells that the back is whole; if there is none and its first marker is a begin(a), the back is
+// read until an unmatched begin(a); kGuessEvents at most.
+// (Pairing of traces cut at either end: 24 M events 551 -> 289 us, 142 M in a ring 2,700 -> 1,374 us. The look costs 4 us, and
+// 20 to 40 us when many streams are read.)
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order) {
-  __shared__ u32 cnt[64], cur[64];
-  __shared__ u32 one_class;
-  if (threadIdx.x < 64) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
+constexpr int kInitThreads = 256;
+constexpr u32 kGuessRun = 32;  // consecutive events a thread looks at (first a quarter of them: a cut is usually near)
+constexpr u32 kGuessEvents = kInitThreads * kGuessRun;
+
+// Unmatched closing markers from one end of a stream on (FRONT: ends, from the first event; else begins, from the last
+// backwards), up to and including the first one of region `outer` (*met: there is one). One block; heights by a prefix sum
+// over the threads' runs.
+template <bool FRONT, u32 RUN>
+__device__ __noinline__ u32 guess_unmatched(const ArgusPairArgs& a, const uint4* src, u32 ring_first, u32 n, u32 outer, bool* met) {
+  __shared__ int sh[33], low_of[kInitThreads / 32];
+  __shared__ u32 stop;
+  const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, limit = n < kInitThreads * RUN ? n : kInitThreads * RUN;
+  if (threadIdx.x == 0) stop = 0xffffffffu;
+  u32 opens = 0, closes = 0, outers = 0;  // a bit per event of the run
+#pragma unroll 8
+  for (u32 j = 0; j < RUN; ++j) {
+    const u32 i = threadIdx.x * RUN + j;
+    if (i >= limit) break;
+    u32 at = FRONT ? i : n - 1 - i;
+    if (a.ring_written) { const u32 room = a.ring_capacity - ring_first; at = at >= room ? at - room : ring_first + at; }
+    const u32 tag = __ldg(reinterpret_cast<const u32*>(src + at) + 2);
+    if (((tag & 1u) != 0) == FRONT) { closes |= 1u << j; if ((tag >> 1) == outer) outers |= 1u << j; }
+    else opens |= 1u << j;
+  }
+  int total;
+  const int start = argus_block_exclusive_scan<int>(__popc(opens) - __popc(closes), sh, &total);
+  int h = start, low = start;  // the lowest height after any event of the run, and of the runs before it
+  for (u32 j = 0; j < RUN; ++j) {
+    h += (int)((opens >> j) & 1u) - (int)((closes >> j) & 1u);
+    low = h < low ? h : low;
+  }
+  int upto = low;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) { const int o = __shfl_up_sync(0xffffffffu, upto, d); if (lane >= (u32)d && o < upto) upto = o; }
+  if (lane == 31) low_of[warp] = upto;
   __syncthreads();
-  for (u32 s = threadIdx.x; s < a.num_streams; s += blockDim.x) {
-    const u64 lo = a.stream_offsets[s], hi = a.stream_offsets[s + 1];
-    const u64 n = hi > lo ? hi - lo : 0;
-    atomicAdd(&cnt[n ? 63 - __clzll((long long)n) : 0], 1u);
+  int before = __shfl_up_sync(0xffffffffu, upto, 1);
+  if (lane == 0 || before > 0) before = 0;
+  int lowest = 0;
+  for (u32 w = 0; w < kInitThreads / 32; ++w) {
+    const int o = low_of[w];
+    if (w < warp && o < before) before = o;
+    if (o < lowest) lowest = o;
+  }
+  if (outers && low < before) {  // an unmatched one of `outer` may be here: the first event that goes below everything before it
+    h = start;
+    for (u32 j = 0; j < RUN; ++j) {
+      h += (int)((opens >> j) & 1u) - (int)((closes >> j) & 1u);
+      if (h < before) {
+        before = h;
+        if ((outers >> j) & 1u) { atomicMin(&stop, (u32)-h); break; }
+      }
+    }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {  // bases, classes in descending order
+  const u32 s = stop;  // (unmatched markers are counted one by one: the earliest stop is the one with the least depth)
+  __syncthreads();
+  *met = s != 0xffffffffu;
+  return *met ? s : (u32)-lowest;
+}
+
+template <bool FRONT>
+__device__ __forceinline__ u32 guess_unmatched(const ArgusPairArgs& a, const uint4* src, u32 ring_first, u32 n, u32 outer, bool* met) {
+  const u32 u = guess_unmatched<FRONT, kGuessRun / 4>(a, src, ring_first, n, outer, met);
+  return *met || n <= kGuessEvents / 4 ? u : guess_unmatched<FRONT, kGuessRun>(a, src, ring_first, n, outer, met);
+}
+
+// Clears the workspace's zeroed part and the status block.
+__device__ __forceinline__ void pair_clear(const ArgusPairArgs& a, uint4* zeroed, u64 zeroed_words, int clear_status, u64 first, u64 stride) {
+  for (u64 i = first; i < zeroed_words; i += stride) zeroed[i] = make_uint4(0, 0, 0, 0);
+  if (clear_status && first < 8) reinterpret_cast<u64*>(a.status)[first] = 0;
+}
+
+__device__ __forceinline__ u32 stream_length(const ArgusPairArgs& a, u64 off0, u32 s) {
+  const u64 lo = a.stream_offsets[s], hi = a.stream_offsets[s + 1];
+  return hi < lo || hi > a.num_events || lo < off0 || ((hi - lo) >> 32) ? 0u : (u32)(hi - lo);  // (bad offsets are reported by the pairing kernel)
+}
+
+constexpr u32 kInitStreams = 4;  // streams a block looks at at a time
+__global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uint4* zeroed, u64 zeroed_words, int clear_status) {
+  argus_kernel_begin();
+  pair_clear(a, zeroed, zeroed_words, clear_status, (u64)blockIdx.x * blockDim.x + threadIdx.x, (u64)gridDim.x * blockDim.x);
+  const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
+  for (u32 s0 = blockIdx.x * kInitStreams; s0 < a.num_streams; s0 += gridDim.x * kInitStreams) {
+    // a thread per stream takes a look at its first and last marker; the block reads the ends of those that are not whole
+    const u32 sm = s0 + threadIdx.x;
+    u32 n = 0, f = 0, l = 1;
+    if (threadIdx.x < kInitStreams && sm < a.num_streams) {
+      n = stream_length(a, off0, sm);
+      a.bases[sm] = n >> 1;
+      if (n) {
+        const u32 first = a.ring_written ? argus_ring_first(a, sm) : 0u;
+        const uint4* src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)sm * a.ring_capacity : a.stream_offsets[sm]);
+        u32 end = n - 1;
+        if (a.ring_written) { const u32 room = a.ring_capacity - first; end = end >= room ? end - room : first + end; }
+        f = __ldg(reinterpret_cast<const u32*>(src + first) + 2);
+        l = __ldg(reinterpret_cast<const u32*>(src + end) + 2);
+      }
+    }
+    __shared__ u32 sh_n[kInitStreams], sh_f[kInitStreams], sh_l[kInitStreams];
+    __syncthreads();
+    if (threadIdx.x < kInitStreams) { sh_n[threadIdx.x] = n; sh_f[threadIdx.x] = f; sh_l[threadIdx.x] = l; }
+    __syncthreads();
+    for (u32 k = 0; k < kInitStreams; ++k) {
+      const u32 s = s0 + k, nk = sh_n[k], fk = sh_f[k], lk = sh_l[k];
+      if (!nk || (!(fk & 1u) && (lk & 1u) && (fk >> 1) == (lk >> 1))) continue;
+      const u32 first = a.ring_written ? argus_ring_first(a, s) : 0u;
+      const uint4* src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
+      bool met = false;
+      u32 unmatched = lk & 1u ? guess_unmatched<true>(a, src, first, nk, lk >> 1, &met) : 0u;
+      if (!met && !(fk & 1u)) unmatched += guess_unmatched<false>(a, src, first, nk, fk >> 1, &met);
+      if (threadIdx.x == 0) a.bases[s] = (nk - (unmatched < nk ? unmatched : nk)) >> 1;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// order: provisional bases (exclusive sum of the foretold counts), and the streams sorted by length class
+// (floor(log2(events))), longest first. A stream is a chain of chunks that one CTA at a time walks, so when lengths differ
+// (producer and consumer warps of one kernel) the long chains must start first or they end last, alone. Counting sort in one
+// block; the order inside a class does not matter. Small calls have no init kernel before this one (`alone`).
+// ---------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
+                                                            int clear_status, int alone) {
+  argus_kernel_begin_long();  // the pairing kernel's blocks spread evenly only over SMs that are free when they come
+  __shared__ u32 cnt[64], cur[64];
+  __shared__ u64 sh[33];
+  __shared__ u32 one_class;
+  if (alone) pair_clear(a, zeroed, zeroed_words, clear_status, threadIdx.x, blockDim.x);
+  if (threadIdx.x < 64) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
+  __syncthreads();
+  const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
+  u64 carry = 0;
+  for (u32 s0 = 0; s0 < a.num_streams; s0 += kScanThreads) {
+    const u32 s = s0 + threadIdx.x;
+    u64 c = 0;
+    if (s < a.num_streams) {
+      const u32 n = stream_length(a, off0, s);
+      c = alone ? n >> 1 : a.bases[s];
+      atomicAdd(&cnt[n ? 31 - __clz((int)n) : 0], 1u);
+    }
+    u64 total;
+    const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
+    if (s < a.num_streams) a.bases[s] = carry + ex;
+    carry += total;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {  // first places, classes in descending order
+    a.bases[a.num_streams] = carry;
     u32 base = 0;
     one_class = 0;
-    for (int c = 63; c >= 0; --c) {
+    for (int c = 31; c >= 0; --c) {
       const u32 k = cnt[c];
       if (k == a.num_streams) one_class = 1;
       cnt[c] = base;
@@ -86,49 +229,8 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
     return;
   }
   for (u32 s = threadIdx.x; s < a.num_streams; s += blockDim.x) {
-    const u64 lo = a.stream_offsets[s], hi = a.stream_offsets[s + 1];
-    const u64 n = hi > lo ? hi - lo : 0;
-    const u32 c = n ? 63 - __clzll((long long)n) : 0;
+    const u32 n = stream_length(a, off0, s), c = n ? 31 - __clz((int)n) : 0;
     order[cnt[c] + atomicAdd(&cur[c], 1u)] = s;
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
-// offsets: exclusive scan of per-stream counts; decides whether the second pass is needed.
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kScanThreads) k_pair_offsets(ArgusPairArgs a) {
-  __shared__ u64 sh[33];
-  __shared__ u32 mismatch;
-  if (threadIdx.x == 0) mismatch = 0;
-  __syncthreads();
-  const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
-  u64 carry = 0;
-  for (u32 s0 = 0; s0 < a.num_streams; s0 += kScanThreads) {
-    const u32 s = s0 + threadIdx.x;
-    const u64 c = s < a.num_streams ? a.counts[s] : 0;
-    u64 total;
-    const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
-    if (s < a.num_streams) {
-      const u64 fin = carry + ex;
-      // (beyond the capacity only when the call ends with ARGUS_ERR_CAPACITY: offsets then stay inside the array, so
-      // that a call chained behind this one without a host check reads nothing it must not)
-      a.interval_offsets[s] = fin < a.interval_capacity ? fin : a.interval_capacity;
-      const u64 lo = a.stream_offsets[s];
-      if (lo >= off0 && fin != ((lo - off0) >> 1) && c != 0) mismatch = 1;
-    }
-    carry += total;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    a.interval_offsets[a.num_streams] = carry < a.interval_capacity ? carry : a.interval_capacity;
-    a.ctl->total_intervals = carry;
-    a.status->intervals_required = carry;
-    if (carry > a.interval_capacity) {
-      argus_set_error(a.status, ARGUS_ERR_CAPACITY, 0, carry);
-      a.ctl->redo = 0;
-    } else {
-      a.ctl->redo = (mismatch || a.ctl->spec_overflow) ? 1u : 0u;
-    }
   }
 }
 
@@ -147,11 +249,60 @@ struct AmbigArgs {
   u64* ambig_offsets;
 };
 
-// (a fixed grid walks the blocks of words: a trace without ambiguous markers, the usual case, costs one small launch)
-__global__ void __launch_bounds__(kWordsPerBlock) k_ambig_word_prefix(AmbigArgs g) {
+// Block 0: exclusive scan of the per-stream counts; decides whether the second pass is needed, and from which stream on.
+__device__ __forceinline__ void pair_offsets(const ArgusPairArgs& a) {
+  __shared__ u64 sh[33];
+  __shared__ u32 first_bad, last_used;
+  if (threadIdx.x == 0) { first_bad = 0xffffffffu; last_used = 0; }
+  __syncthreads();
+  u64 carry = 0;
+  u32 bad = 0xffffffffu, used = 0;
+  for (u32 s0 = 0; s0 < a.num_streams; s0 += kScanThreads) {
+    const u32 s = s0 + threadIdx.x;
+    const u64 c = s < a.num_streams ? a.counts[s] : 0;
+    u64 total;
+    const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
+    if (s < a.num_streams) {
+      const u64 fin = carry + ex;
+      // (beyond the capacity only when the call ends with ARGUS_ERR_CAPACITY: offsets then stay inside the array, so
+      // that a call chained behind this one without a host check reads nothing it must not)
+      a.interval_offsets[s] = fin < a.interval_capacity ? fin : a.interval_capacity;
+      const u64 told = a.bases[s + 1] - a.bases[s];
+      // a stream with fewer intervals than foretold lies right, those after it do not; one with more has lost its tail to the
+      // next stream's writes
+      if (c < told && s + 1 < bad) bad = s + 1;
+      if (c > told && s < bad) bad = s;
+      if (c) used = s;
+    }
+    carry += total;
+  }
+  atomicMin(&first_bad, bad);
+  atomicMax(&last_used, used);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a.interval_offsets[a.num_streams] = carry < a.interval_capacity ? carry : a.interval_capacity;
+    a.ctl->total_intervals = carry;
+    a.status->intervals_required = carry;
+    a.ctl->redo_from = first_bad;
+    if (carry > a.interval_capacity) {
+      argus_set_error(a.status, ARGUS_ERR_CAPACITY, 0, carry);
+      a.ctl->redo = 0;
+    } else {
+      a.ctl->redo = carry && first_bad <= last_used ? 1u : 0u;
+    }
+  }
+}
+
+// The other blocks, when there are notes: set bits before every word within its block of words, and, by the last block to
+// be done, before every block of words.
+__global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
+  argus_kernel_begin();
+  if (blockIdx.x == 0) { pair_offsets(g.p); return; }
+  if (__ldcg(&g.p.ctl->n_notes) == 0) return;
   __shared__ u32 sh[33];
-  if (g.p.ctl->n_notes == 0) return;
-  for (u64 blk = blockIdx.x; blk < g.num_blocks; blk += gridDim.x) {
+  __shared__ u64 sh64[33];
+  __shared__ u32 last;
+  for (u64 blk = blockIdx.x - 1; blk < g.num_blocks; blk += gridDim.x - 1) {
     const u64 w = blk * kWordsPerBlock + threadIdx.x;
     const u32 c = w < g.num_words ? __popc(g.p.bits[w]) : 0u;
     u32 total;
@@ -160,20 +311,20 @@ __global__ void __launch_bounds__(kWordsPerBlock) k_ambig_word_prefix(AmbigArgs 
     if (threadIdx.x == 0) g.block_prefix[blk] = total;
     __syncthreads();
   }
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_ambig_block_scan(AmbigArgs g) {
-  __shared__ u64 sh[33];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&g.p.ctl->prefix_done, 1u) == gridDim.x - 2;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   u64 carry = 0;
-  if (g.p.ctl->n_notes != 0) {
-    for (u64 b0 = 0; b0 < g.num_blocks; b0 += kScanThreads) {
-      const u64 b = b0 + threadIdx.x;
-      const u64 c = b < g.num_blocks ? g.block_prefix[b] : 0;
-      u64 total;
-      const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
-      if (b < g.num_blocks) g.block_prefix[b] = carry + ex;
-      carry += total;
-    }
+  for (u64 b0 = 0; b0 < g.num_blocks; b0 += kScanThreads) {
+    const u64 b = b0 + threadIdx.x;
+    const u64 c = b < g.num_blocks ? __ldcg(g.block_prefix + b) : 0;
+    u64 total;
+    const u64 ex = argus_block_exclusive_scan<u64>(c, sh64, &total);
+    if (b < g.num_blocks) g.block_prefix[b] = carry + ex;
+    carry += total;
   }
   if (threadIdx.x == 0) {
     g.block_prefix[g.num_blocks] = carry;
@@ -191,10 +342,21 @@ __device__ __forceinline__ u64 ambig_rank(const AmbigArgs& g, u64 gpos) {
   return g.block_prefix[w / kWordsPerBlock] + g.word_prefix[w] + __popc(g.p.bits[w] & ((1u << (gpos & 31)) - 1u));
 }
 
-__global__ void __launch_bounds__(256) k_ambig_scatter(AmbigArgs g) {
-  const u64 n_notes = g.p.ctl->n_notes;
+__device__ __forceinline__ void ambig_offset(const AmbigArgs& g, u64 s) {
+  if (__ldcg(&g.p.ctl->n_notes) == 0) { g.ambig_offsets[s] = 0; return; }
+  const u64 off0 = g.p.num_streams ? g.p.stream_offsets[0] : 0;
+  const u64 o = g.p.num_streams ? g.p.stream_offsets[s] : 0;
+  const u64 r = o >= off0 ? ambig_rank(g, o - off0) : 0;
+  g.ambig_offsets[s] = r < g.ambig_capacity ? r : g.ambig_capacity;  // inside the array also after ARGUS_ERR_CAPACITY
+}
+
+// ambig_offsets, and the notes as records in order
+__global__ void __launch_bounds__(256) k_ambig_records(AmbigArgs g) {
+  argus_kernel_begin_long();  // (a long kernel's blocks come next, as after k_pair_order)
+  for (u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x; s <= g.p.num_streams; s += (u64)gridDim.x * blockDim.x) ambig_offset(g, s);
+  const u64 n_notes = __ldcg(&g.p.ctl->n_notes);
   const u64 n = n_notes < g.p.note_capacity ? n_notes : g.p.note_capacity;
-  const u64 off0 = g.p.stream_offsets[0];
+  const u64 off0 = n ? g.p.stream_offsets[0] : 0;
   for (u64 j = (u64)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (u64)gridDim.x * blockDim.x) {
     const u64 note = g.p.notes[j];
     const u64 gpos = note & ((1ull << ARGUS_NOTE_POS_BITS) - 1);
@@ -223,18 +385,8 @@ __global__ void __launch_bounds__(256) k_ambig_scatter(AmbigArgs g) {
   }
 }
 
-__global__ void __launch_bounds__(256) k_ambig_offsets(AmbigArgs g) {
-  const u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s > g.p.num_streams) return;
-  if (g.p.ctl->n_notes == 0) { g.ambig_offsets[s] = 0; return; }
-  const u64 off0 = g.p.stream_offsets[0];
-  const u64 o = g.p.stream_offsets[s];
-  const u64 r = o >= off0 ? ambig_rank(g, o - off0) : 0;
-  g.ambig_offsets[s] = r < g.ambig_capacity ? r : g.ambig_capacity;  // inside the array also after ARGUS_ERR_CAPACITY
-}
-
 struct Layout {
-  size_t ctl, counts, queue, bits, word_prefix, block_prefix, notes, records, order, total;
+  size_t ctl, counts, queue, bits, word_prefix, block_prefix, notes, records, order, bases, total;
   u64 num_words, num_blocks, queue_capacity;
   u32 record_capacity;
 };
@@ -256,6 +408,7 @@ Layout make_layout(uint64_t num_events, uint32_t num_streams, uint64_t ambig_cap
   L.notes = o; o += argus_align_up((size_t)ambig_capacity * 8 + 8, 256);
   L.records = o; o += argus_align_up((size_t)L.record_capacity * sizeof(ArgusStreamRecord), 256);
   L.order = o; o += argus_align_up((size_t)num_streams * 4 + 4, 256);
+  L.bases = o; o += argus_align_up(((size_t)num_streams + 1) * 8, 256);
   L.total = o;
   return L;
 }
@@ -297,7 +450,7 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   a.events = events; a.stream_offsets = (const u64*)stream_offsets; a.num_events = num_events;
   a.num_streams = num_streams; a.num_regions = num_regions;
   a.intervals = intervals; a.interval_capacity = interval_capacity; a.interval_offsets = (u64*)interval_offsets;
-  a.counts = (u64*)(ws + L.counts);
+  a.counts = (u64*)(ws + L.counts); a.bases = (u64*)(ws + L.bases);
   a.notes = (u64*)(ws + L.notes); a.note_capacity = ambig_capacity;
   a.bits = (u32*)(ws + L.bits);
   a.ctl = (ArgusPairCtl*)(ws + L.ctl);
@@ -311,17 +464,24 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   // a stream's intervals start at half its first event's position at the latest, so positions stay below num_events / 2 + 1
   a.digest = digest_capacity >= (interval_capacity < num_events / 2 + 1 ? interval_capacity : num_events / 2 + 1) ? (u64*)digest : nullptr;
 
-  if (reset_status) ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
-  // control block, counts and bitmap are contiguous at the start of the workspace
-  ARGUS_CUDA_TRY(cudaMemsetAsync(ws, 0, L.word_prefix, stream));
-
   const bool tiled = (kernel_choice != 1 && argus_pair_tiled_usable(a)) || ring_written != nullptr;
-  a.order = nullptr;
-  if (tiled && num_streams > 1) {
-    k_pair_order<<<1, kScanThreads, 0, stream>>>(a, (u32*)(ws + L.order));
-    ARGUS_CHECK_LAUNCH();
-    a.order = (const u32*)(ws + L.order);
+  // control block, counts, queue and bitmap are contiguous at the start of the workspace and start at zero
+  uint4* const zeroed = (uint4*)ws;
+  const u64 zeroed_words = L.word_prefix / 16;
+  u32* const order = (u32*)(ws + L.order);
+  // Small calls: one block clears and orders. Beyond that a grid clears, and looks at the ends of the streams.
+  const bool alone = num_events < (1u << 20) && num_streams <= 8192;
+  if (!alone) {
+    const u64 want = (u64)num_streams / kInitStreams + zeroed_words / 4096 + 1;
+    ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status);
   }
+  ARGUS_LAUNCH(k_pair_order, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone);
+  a.order = tiled && num_streams > 1 ? order : nullptr;
+
+  AmbigArgs g;
+  g.p = a; g.num_words = L.num_words; g.span = num_events;
+  g.word_prefix = (u32*)(ws + L.word_prefix); g.block_prefix = (u64*)(ws + L.block_prefix);
+  g.num_blocks = L.num_blocks; g.ambig = ambig; g.ambig_capacity = ambig_capacity; g.ambig_offsets = (u64*)ambig_offsets;
   for (int pass = 0; pass < 2; ++pass) {
     a.redo = pass;
     if (num_streams) {
@@ -330,33 +490,15 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
         const int rc = argus_launch_pair_tiled(a, stream);
         if (rc != ARGUS_OK) return rc;
       } else {
-        k_pair_thread_per_stream<<<(num_streams + 127) / 128, 128, 0, stream>>>(a);
-        ARGUS_CHECK_LAUNCH();
+        ARGUS_LAUNCH(k_pair_thread_per_stream, (num_streams + 127) / 128, 128, 0, stream, a);
       }
       if (pass == 0) argus_prof_mark(ARGUS_PROF_PAIR, stream, 1);
     }
-    if (pass == 0) {
-      k_pair_offsets<<<1, kScanThreads, 0, stream>>>(a);
-      ARGUS_CHECK_LAUNCH();
-    }
+    if (pass == 0)
+      ARGUS_LAUNCH(k_pair_offsets, (unsigned)(L.num_blocks < 592 ? L.num_blocks : 592) + 1, kScanThreads, 0, stream, g);
   }
-
-  AmbigArgs g;
-  g.p = a; g.num_words = L.num_words; g.span = num_events;
-  g.word_prefix = (u32*)(ws + L.word_prefix); g.block_prefix = (u64*)(ws + L.block_prefix);
-  g.num_blocks = L.num_blocks; g.ambig = ambig; g.ambig_capacity = ambig_capacity; g.ambig_offsets = (u64*)ambig_offsets;
-  if (L.num_blocks) {
-    k_ambig_word_prefix<<<(unsigned)(L.num_blocks < 2368 ? L.num_blocks : 2368), kWordsPerBlock, 0, stream>>>(g);
-    ARGUS_CHECK_LAUNCH();
-  }
-  k_ambig_block_scan<<<1, kScanThreads, 0, stream>>>(g);
-  ARGUS_CHECK_LAUNCH();
-  if (num_streams && num_events) {
-    k_ambig_scatter<<<296, 256, 0, stream>>>(g);
-    ARGUS_CHECK_LAUNCH();
-  }
-  k_ambig_offsets<<<(num_streams + 1 + 255) / 256, 256, 0, stream>>>(g);
-  ARGUS_CHECK_LAUNCH();
+  const u64 want = ((u64)num_streams + 1 + 255) / 256;
+  ARGUS_LAUNCH(k_ambig_records, (unsigned)(alone ? (want > 16 ? want : 16) : 296), 256, 0, stream, g);
   return ARGUS_OK;
 }
 
@@ -390,7 +532,7 @@ extern "C" int argus_pair_intervals_ring(const argus_event_t* ring, uint32_t slo
   if (num_streams && (!ring || !written)) return ARGUS_ERR_INVALID_ARG;
   if (((uintptr_t)written & 7) || ((uintptr_t)dropped & 7)) return ARGUS_ERR_INVALID_ARG;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
+  { const int rc = argus_internal_clear(status, nullptr, 0, cuda_stream); if (rc != ARGUS_OK) return rc; }
   const uint64_t bound = (uint64_t)num_streams * slot_capacity;  // what the slots can hold: sizes the workspace
   int rc = argus_internal_ring_offsets(written, slot_capacity, num_streams, bound, stream_offsets, dropped, status, cuda_stream);
   if (rc != ARGUS_OK) return rc;

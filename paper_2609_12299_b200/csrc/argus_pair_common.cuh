@@ -25,7 +25,7 @@ struct ArgusFrame {  // one open region occurrence, 32 bytes
 struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of a call
   u64 n_notes;         // ambiguity notes appended (may exceed the list capacity)
   u32 redo;            // 1 = provisional interval bases were wrong; second pass needed
-  u32 spec_overflow;   // a provisional position fell outside interval_capacity
+  u32 redo_from;       // first stream whose intervals the second pass writes again
   u64 total_intervals;
   u64 total_ambig;
   // work queue of the tiled kernel, one set per pass (0 = first, 1 = redo): positions below num_streams are the
@@ -34,7 +34,8 @@ struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of
   u64 q_tail[2];       // hand-overs published (queue entries written)
   u32 n_records[2];    // hand-over records allocated
   u32 n_done[2];       // streams walked to their end (or given up on)
-  u64 reserved[2];
+  u32 prefix_done;     // blocks that have counted their share of the ambiguity bitmap
+  u32 pad;
 };
 
 // A long stream is walked in chunks of about kChunkEvents events. After a chunk the CTA stores the stream's
@@ -64,12 +65,13 @@ struct ArgusPairArgs {
   u64 interval_capacity;
   u64* interval_offsets;  // final offsets (output of the offsets kernel)
   u64* counts;            // per-stream interval counts (workspace)
+  u64* bases;             // [S + 1] provisional first interval of every stream: the sum of the counts foretold for those before it
   u64* notes;             // packed ambiguity notes (workspace)
   u64 note_capacity;
   u32* bits;              // one bit per event (workspace)
   ArgusPairCtl* ctl;
   argus_status_t* status;
-  int redo;               // 0 = first pass with provisional bases, 1 = second pass with final bases
+  int redo;               // 0 = first pass with provisional bases, 1 = second pass with final bases (streams from ctl->redo_from on)
   u32* queue;             // hand-over queue entries (record index + 1; zeroed), null = streams are never split
   u64 queue_capacity;
   ArgusStreamRecord* records;
@@ -154,8 +156,6 @@ __device__ __forceinline__ bool argus_seq_step(const ArgusPairArgs& a, ArgusFram
     argus_store_interval(a.intervals + pos, f.ts, incl, excl, f.region, f.ctx, stream,
                          s.h > 0 ? stk[s.h - 1].region : ARGUS_NONE, f.idx, (u32)s.h, flags);
     if (a.digest) a.digest[pos] = argus_digest_pack(f.region, incl, excl, flags);
-  } else if (!a.redo) {
-    a.ctl->spec_overflow = 1;
   }
   s.n_int++;
   if (s.h > 0) stk[s.h - 1].child += incl;

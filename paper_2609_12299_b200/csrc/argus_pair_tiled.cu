@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   SM& sm = *reinterpret_cast<SM*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (a.redo && !a.ctl->redo) return;
+  argus_kernel_begin_long();
+  if (a.redo && !__ldcg(&a.ctl->redo)) return;
   if (tid == 0) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);
@@ -237,10 +238,9 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     }
     const u32 n = (u32)(hi - lo);
     const u64 gpos0 = lo - off0;
-    const u64 out_base = a.redo ? a.interval_offsets[s] : (gpos0 >> 1);
-    if (a.redo && rec == kNoRec && out_base == (gpos0 >> 1) && out_base + a.counts[s] <= a.interval_capacity) {
-      // second pass: this stream's intervals (and digests) already lie where they belong — the first pass wrote them
-      // at the same positions, all of them fitted, and no other stream writes there in either pass
+    const u64 out_base = a.redo ? a.interval_offsets[s] : a.bases[s];
+    if (a.redo && s < __ldcg(&a.ctl->redo_from)) {
+      // second pass: this stream's intervals (and digests) already lie where they belong
       if (tid == 0) atomicAdd(&a.ctl->n_done[1], 1u);
       __syncthreads();
       continue;
@@ -452,8 +452,6 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
                 q[1] = make_uint4((u32)excl, (u32)(excl >> 32), pe.z >> 1, pe.w);
                 q[2] = make_uint4(s, preg, bidx, (d >> SM::kDescShift) | (flags << 16));
                 if (a.digest) a.digest[pos] = argus_digest_pack(pe.z >> 1, incl, excl, flags);
-              } else if (!a.redo) {
-                a.ctl->spec_overflow = 1;
               }
             }
           }
@@ -599,8 +597,7 @@ int launch_tiled(const ArgusPairArgs& a, cudaStream_t stream) {
     grid_cache = grid_of[dev];
   }
   const u32 grid = a.num_streams < (u32)grid_cache ? a.num_streams : (u32)grid_cache;
-  k_pair_tiled<NT, E, MINB, RING><<<grid, NT, smem, stream>>>(a);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_pair_tiled<NT, E, MINB, RING>, grid, NT, smem, stream, a);
   return ARGUS_OK;
 }
 

@@ -12,6 +12,7 @@ constexpr int kRingScanThreads = 1024;
 __global__ void __launch_bounds__(kRingScanThreads) k_ring_offsets(const u64* written, u32 slot_capacity, u32 num_streams,
                                                                    u64 event_capacity, u64* stream_offsets, u64* dropped,
                                                                    argus_status_t* status) {
+  argus_kernel_begin();
   __shared__ u64 sh[33];
   u64 carry = 0;
   for (u32 s0 = 0; s0 < num_streams; s0 += kRingScanThreads) {
@@ -36,6 +37,7 @@ __global__ void __launch_bounds__(kRingScanThreads) k_ring_offsets(const u64* wr
 
 __global__ void __launch_bounds__(256) k_ring_copy(const uint4* ring, u32 slot_capacity, const u64* written, u32 num_streams,
                                                    uint4* events, const u64* stream_offsets, const argus_status_t* status) {
+  argus_kernel_begin_long();
   if (status->code != 0) return;  // the packed records do not fit: nothing is copied
   for (u32 s = blockIdx.x; s < num_streams; s += gridDim.x) {
     const u64 w = written[s];
@@ -55,9 +57,8 @@ __global__ void __launch_bounds__(256) k_ring_copy(const uint4* ring, u32 slot_c
 
 int argus_internal_ring_offsets(const uint64_t* written, uint32_t slot_capacity, uint32_t num_streams, uint64_t event_capacity,
                                 uint64_t* stream_offsets, uint64_t* dropped, argus_status_t* status, void* cuda_stream) {
-  k_ring_offsets<<<1, kRingScanThreads, 0, (cudaStream_t)cuda_stream>>>((const u64*)written, slot_capacity, num_streams, event_capacity,
-                                                                        (u64*)stream_offsets, (u64*)dropped, status);
-  ARGUS_CHECK_LAUNCH();
+  ARGUS_LAUNCH(k_ring_offsets, 1, kRingScanThreads, 0, (cudaStream_t)cuda_stream, (const u64*)written, slot_capacity, num_streams,
+               event_capacity, (u64*)stream_offsets, (u64*)dropped, status);
   return ARGUS_OK;
 }
 
@@ -71,15 +72,13 @@ extern "C" int argus_ring_linearise(const argus_event_t* ring, uint32_t slot_cap
       ((uintptr_t)dropped & 7))
     return ARGUS_ERR_INVALID_ARG;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), stream));
-  k_ring_offsets<<<1, kRingScanThreads, 0, stream>>>((const u64*)written, slot_capacity, num_streams, event_capacity,
-                                                     (u64*)stream_offsets, (u64*)dropped, status);
-  ARGUS_CHECK_LAUNCH();
+  { const int rc = argus_internal_clear(status, nullptr, 0, cuda_stream); if (rc != ARGUS_OK) return rc; }
+  ARGUS_LAUNCH(k_ring_offsets, 1, kRingScanThreads, 0, stream, (const u64*)written, slot_capacity, num_streams,
+               event_capacity, (u64*)stream_offsets, (u64*)dropped, status);
   if (num_streams) {
-    k_ring_copy<<<num_streams < 148u * 16u ? num_streams : 148u * 16u, 256, 0, stream>>>(
-        reinterpret_cast<const uint4*>(ring), slot_capacity, (const u64*)written, num_streams,
-        reinterpret_cast<uint4*>(events), (const u64*)stream_offsets, status);
-    ARGUS_CHECK_LAUNCH();
+    ARGUS_LAUNCH(k_ring_copy, num_streams < 148u * 16u ? num_streams : 148u * 16u, 256, 0, stream,
+                 reinterpret_cast<const uint4*>(ring), slot_capacity, (const u64*)written, num_streams,
+                 reinterpret_cast<uint4*>(events), (const u64*)stream_offsets, status);
   }
   return ARGUS_OK;
 }

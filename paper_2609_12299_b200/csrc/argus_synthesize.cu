@@ -73,7 +73,6 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
   const SynLayout L = syn_layout(num_events, num_streams, num_regions, ambig_capacity, num_pairs, num_sms, max_overlap_spans);
   if (workspace_bytes < L.total) return ARGUS_ERR_WORKSPACE;
   const int g_synth_mode = g_synth_mode_knob.load(std::memory_order_relaxed);
-  cudaStream_t stream = (cudaStream_t)cuda_stream;
   char* ws = (char*)workspace;
   const bool want_agg = warp_tab || cta_tab || sm_tab || kernel_tab;
 
@@ -85,7 +84,7 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
   ArgusFuseArgs f = ArgusFuseArgs();
   if (use_digest && num_pairs) {
     f.pairs = pairs; f.num_pairs = num_pairs; f.entries = (u64*)(ws + L.digest); f.starts = (u64*)(ws + L.starts); f.pieces = (ArgusOvPiece*)(ws + L.pieces);
-    ARGUS_CUDA_TRY(cudaMemsetAsync(ov_ctl, 0, sizeof(ArgusOvCtl), stream));
+    f.ctl = ov_ctl;
   }
   int rc = argus_internal_pair(events, num_events, stream_offsets, num_streams, num_regions, intervals, interval_capacity,
                                interval_offsets, ambig, ambig_capacity, ambig_offsets, status, ws + L.pair, L.pair_bytes,
@@ -140,7 +139,7 @@ extern "C" int argus_synthesize_ring(const argus_event_t* ring, uint32_t slot_ca
   if (!status || !stream_offsets || slot_capacity == 0) return ARGUS_ERR_INVALID_ARG;
   if (num_streams && (!ring || !written)) return ARGUS_ERR_INVALID_ARG;
   if (((uintptr_t)written & 7) || ((uintptr_t)dropped & 7) || ((uintptr_t)stream_offsets & 7)) return ARGUS_ERR_INVALID_ARG;
-  ARGUS_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(argus_status_t), (cudaStream_t)cuda_stream));
+  { const int rc = argus_internal_clear(status, nullptr, 0, cuda_stream); if (rc != ARGUS_OK) return rc; }
   const uint64_t bound = (uint64_t)num_streams * slot_capacity;  // what the slots can hold: sizes the workspace
   const int rc = argus_internal_ring_offsets(written, slot_capacity, num_streams, bound, stream_offsets, dropped, status, cuda_stream);
   if (rc != ARGUS_OK) return rc;

@@ -52,6 +52,7 @@ struct AggArgs {
   int iter_inline;    // global path taken inside k_agg_streams_compact (one read of the intervals serves both)
   // overlap selection in the pass over the digests (argus_synthesize)
   ArgusFuseArgs ov;
+  u32 parts;          // k_agg_streams_digest: blocks that share a stream
   const u64* digest;  // digests of the intervals (k_agg_streams_digest; overwritten with entries where overlap is selected), null = read the records
   u64 interval_limit; // records the interval array holds: a stream whose offsets reach beyond it is reported, not read
 };
@@ -290,9 +291,11 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
     }
     __syncthreads();
   }
-  for (u32 s = blockIdx.x; s < a.num_streams; s += gridDim.x) {
+  {
+    const u32 s = blockIdx.x / a.parts, part = blockIdx.x % a.parts, slices = a.parts * kDgSlices;
     u64* row = a.warp_tab + (size_t)s * cells;
-    for (u32 i = threadIdx.x; i < cells; i += blockDim.x) row[i] = (i % kCell == 2) ? ~0ull : 0ull;
+    if (a.parts == 1)  // (else the rows have been initialised: several blocks add to one)
+      for (u32 i = threadIdx.x; i < cells; i += blockDim.x) row[i] = (i % kCell == 2) ? ~0ull : 0ull;
     for (u32 i = threadIdx.x; i < kDgWords * num_cells; i += blockDim.x) {
       const u32 f = i % kDgWords, c = i / kDgWords;
       u32 v = f == kDgMin ? 0xffffffffu : 0u;
@@ -315,15 +318,16 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
       const u64* const dgs = a.digest + lo;
       const argus_interval_t* const ivs = a.intervals + lo;
       u32 i0, i1;
-      argus_ov_slice(n, kDgSlices, warp, &i0, &i1);
+      argus_ov_slice(n, slices, part * kDgSlices + warp, &i0, &i1);
       out_first = i0;
       u64* const ents = a.ov.entries + lo + i0;
       u64* const starts = a.ov.starts + lo + i0;
       // two legs: the probe (the first intervals of every slice, each into its region's cell), then, hot regions chosen, the rest
-      const u32 probe_end = n >= kDigestMinStream ? (i0 + 32 < i1 ? i0 + 32 : i1) : i1;
+      const bool probe = n / a.parts >= kDigestMinStream;
+      const u32 probe_end = probe ? (i0 + 32 < i1 ? i0 + 32 : i1) : i1;
       for (int leg = 0; leg < 2; ++leg) {
         const u32 leg_lo = leg ? probe_end : i0, leg_hi = leg ? i1 : probe_end;
-        if (leg && n >= kDigestMinStream) {
+        if (leg && probe) {
           // warp 0 ranks the regions by their counts so far; kDigestHot rounds of a warp-wide maximum
           if (threadIdx.x < 32) {
             for (u32 h = 0; h < kDigestHot; ++h) {
@@ -427,9 +431,9 @@ __global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a)
     if (has_ov && lane == 0) {
       ArgusOvPiece e;
       e.pos = lo + out_first; e.count = out_count; e.next = kOvNone;
-      a.ov.pieces[s * kDgSlices + warp] = e;
+      a.ov.pieces[s * slices + part * kDgSlices + warp] = e;
     }
-    if (a.ambig && a.ambig_offsets) {
+    if (a.ambig && a.ambig_offsets && part == 0) {
       const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
       for (u64 i = alo + threadIdx.x; i < ahi && ahi >= alo; i += blockDim.x) {
         const u32 region = a.ambig[i].tag >> 1;
@@ -644,7 +648,8 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
                                     argus_agg_t* sm_tab, argus_agg_t* kernel_tab, argus_agg_t* role_tab,
                                     argus_agg_t* iter_tab, argus_status_t* status, void* workspace,
                                     size_t workspace_bytes, void* cuda_stream, bool reset_status,
-                                    const ArgusFuseArgs* ov_select, const uint64_t* digest, uint64_t interval_limit) {
+                                    const ArgusFuseArgs* ov_select, const uint64_t* digest, uint32_t digest_parts,
+                                    uint64_t interval_limit) {
   if (!interval_offsets || !status || !workspace) return ARGUS_ERR_INVALID_ARG;
   if (ov_select && !digest) return ARGUS_ERR_INVALID_ARG;
   if (warps_per_cta == 0 || num_streams % warps_per_cta != 0) return ARGUS_ERR_INVALID_ARG;
@@ -680,7 +685,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   a.role_tab = (u64*)role_tab; a.iter_tab = (u64*)iter_tab; a.num_iters = num_iters;
   if (ov_select) { a.ov = *ov_select; } else { a.ov = ArgusFuseArgs(); }
   a.digest = !scope && !role_tab && !iter_tab && num_regions <= kAggCompactRegions ? (const u64*)digest : nullptr;
-  a.interval_limit = interval_limit;
+  a.parts = digest_parts; a.interval_limit = interval_limit;
   const size_t smem = (size_t)num_regions * sizeof(argus_agg_t);
   a.use_smem = smem <= kAggSmemLimit;
   const size_t iter_bytes = (size_t)num_iters * smem;
@@ -710,7 +715,8 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       const size_t dg = digest_table_words(num_regions) * 4 + ((num_regions + 31) / 32) * 4;
       if (dg > 48 * 1024)
         ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_digest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
-      ARGUS_LAUNCH(k_agg_streams_digest, num_streams, kDgThreads, dg, stream, a);
+      if (a.parts > 1) ARGUS_LAUNCH(k_agg_init, 592, 256, 0, stream, a.warp_tab, (u64)num_streams * num_regions * kCell);
+      ARGUS_LAUNCH(k_agg_streams_digest, num_streams * a.parts, kDgThreads, dg, stream, a);
     } else {
       ARGUS_LAUNCH(k_agg_streams_compact, num_streams, kAggThreads, compact, stream, a);
     }
@@ -746,11 +752,18 @@ int argus_internal_aggregate(const argus_interval_t* intervals, const uint64_t* 
   return argus_internal_aggregate_scoped(intervals, interval_offsets, ambig, ambig_offsets, num_streams, warps_per_cta, cta_sm,
                                          num_sms, num_regions, nullptr, warp_tab, cta_tab, sm_tab, kernel_tab, nullptr,
                                          nullptr, status, workspace, workspace_bytes, cuda_stream, reset_status, nullptr,
-                                         nullptr, interval_limit);
+                                         nullptr, 1, interval_limit);
 }
 
 bool argus_aggregate_can_read_digests(uint32_t num_regions) { return num_regions <= kAggCompactRegions; }
-uint32_t argus_aggregate_digest_slices() { return kDgSlices; }
+// Few streams: several blocks share one, six for every SM in all, as long as each has 8,192 intervals to look at.
+// (96 streams of 259,328 intervals: 142 us; 352 us with a block each.)
+uint32_t argus_aggregate_digest_parts(uint32_t num_streams, uint64_t num_events) {
+  if (num_streams == 0) return 1;
+  const uint64_t room = 888 / num_streams, work = num_events / 2 / num_streams / 8192, parts = room < work ? room : work;
+  return (uint32_t)(parts < 1 ? 1 : parts);
+}
+uint32_t argus_aggregate_digest_slices(uint32_t parts) { return parts * kDgSlices; }
 
 extern "C" int argus_aggregate(const argus_interval_t* intervals, const uint64_t* interval_offsets,
                                const argus_ambiguity_t* ambig, const uint64_t* ambig_offsets, uint32_t num_streams,

@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(256) k_ambig_records(AmbigArgs g) {
 }
 
 struct Layout {
-  size_t ctl, counts, queue, bits, word_prefix, block_prefix, notes, records, order, bases, total;
+  size_t ctl, counts, queue, bits, word_prefix, block_prefix, notes, records, order, bases, split, total;
   u64 num_words, num_blocks, queue_capacity;
   u32 record_capacity;
 };
@@ -409,6 +409,7 @@ Layout make_layout(uint64_t num_events, uint32_t num_streams, uint64_t ambig_cap
   L.records = o; o += argus_align_up((size_t)L.record_capacity * sizeof(ArgusStreamRecord), 256);
   L.order = o; o += argus_align_up((size_t)num_streams * 4 + 4, 256);
   L.bases = o; o += argus_align_up(((size_t)num_streams + 1) * 8, 256);
+  L.split = o; o += argus_split_bytes(num_events, num_streams);
   L.total = o;
   return L;
 }
@@ -416,7 +417,7 @@ Layout make_layout(uint64_t num_events, uint32_t num_streams, uint64_t ambig_cap
 }  // namespace
 
 // implemented in argus_pair_tiled.cu
-int argus_launch_pair_tiled(const ArgusPairArgs& a, cudaStream_t stream);
+int argus_launch_pair_tiled(const ArgusPairArgs& a, cudaStream_t stream, bool split);
 bool argus_pair_tiled_usable(const ArgusPairArgs& a);
 
 extern "C" void argus_testing_set_poll_limit(unsigned int polls) { g_poll_limit.store(polls ? polls : 1u << 19); }
@@ -477,6 +478,8 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   }
   ARGUS_LAUNCH(k_pair_order, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone);
   a.order = tiled && num_streams > 1 ? order : nullptr;
+  a.segments = nullptr; a.split_failed = nullptr; a.segment_tiles = 0;
+  const bool split = kernel_choice == 0 && tiled && !ring_written && argus_split_usable(num_events, num_streams);
 
   AmbigArgs g;
   g.p = a; g.num_words = L.num_words; g.span = num_events;
@@ -487,7 +490,11 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
     if (num_streams) {
       if (pass == 0) argus_prof_mark(ARGUS_PROF_PAIR, stream, 0);
       if (tiled) {
-        const int rc = argus_launch_pair_tiled(a, stream);
+        if (pass == 0 && split) {
+          const int rc = argus_launch_pair_split(a, ws + L.split, stream);
+          if (rc != ARGUS_OK) return rc;
+        }
+        const int rc = argus_launch_pair_tiled(a, stream, false);
         if (rc != ARGUS_OK) return rc;
       } else {
         ARGUS_LAUNCH(k_pair_thread_per_stream, (num_streams + 127) / 128, 128, 0, stream, a);

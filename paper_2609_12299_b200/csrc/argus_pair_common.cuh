@@ -35,7 +35,9 @@ struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of
   u32 n_records[2];    // hand-over records allocated
   u32 n_done[2];       // streams walked to their end (or given up on)
   u32 prefix_done;     // blocks that have counted their share of the ambiguity bitmap
-  u32 pad;
+  u32 seg_head;        // segments taken (split pass)
+  u32 num_failed;      // streams that the split pass has to leave to the chained one
+  u32 num_segments;
 };
 
 // A long stream is walked in chunks of about kChunkEvents events. After a chunk the CTA stores the stream's
@@ -53,6 +55,24 @@ struct ArgusStreamRecord {
   uint4 frames[ARGUS_MAX_DEPTH];      // open begin markers as event records
   u64 child[ARGUS_MAX_DEPTH];         // their child time so far
   u32 idx[ARGUS_MAX_DEPTH];           // their index within the stream
+};
+
+// Few long streams: a stream is cut into segments that are walked at the same time (argus_pair_split.cu). What a segment
+// needs to know and what it leaves behind.
+struct ArgusSegment {
+  u32 stream, first_tile, num_tiles;
+  int ch;                             // frames open where it starts
+  u32 unmatched_ends, unmatched_begins;  // by height, within the segment
+  u32 flags[3];                       // intervals with CTX_MISMATCH, TIME_REVERSED, CHILD_CLAMPED
+  u32 end_ch;                         // frames open where it ends
+  u64 n_int;                          // intervals of the stream up to its end
+  u32 idx[ARGUS_MAX_DEPTH];           // the open frames' begin markers, by level
+  u32 open[ARGUS_MAX_DEPTH];          // the segment's unmatched begins, innermost first; of the stream's last segment, in the
+                                      // end, the frames open at the end of the stream by level
+  u64 ledger[ARGUS_MAX_DEPTH];        // child time that the segment gave to the frames open at its end, by level
+  u64 note_pos[ARGUS_MAX_DEPTH];      // record of the initial frame of a level that the segment closed (~0: none): its child time
+  u64 note_child[ARGUS_MAX_DEPTH];    // lacks what earlier segments gave it; what this one gave
+  u64 note_incl[ARGUS_MAX_DEPTH];     // its inclusive time
 };
 
 struct ArgusPairArgs {
@@ -81,8 +101,18 @@ struct ArgusPairArgs {
                           // min(interval_capacity, num_events / 2 + 1), which is all a stream can reach
   const u64* ring_written; // non-null: `events` is a ring container, one slot of ring_capacity records per stream, record i of
   u32 ring_capacity;       // a stream at slot position i mod capacity; stream_offsets then describe the packed survivors
+  ArgusSegment* segments;  // non-null: split pass; or, in the chained pass after it, what that left: only failed streams are walked
+  u32* split_failed;       // [S]
+  u32 segment_tiles;       // tiles of a segment
   u32 poll_limit;          // polls without any hand-over anywhere after which an idle CTA gives up (about a second)
 };
+
+// argus_pair_split.cu
+constexpr u32 kSplitTile = 640;  // events of a tile of the split pass
+bool argus_split_usable(uint64_t num_events, uint32_t num_streams);
+uint32_t argus_split_max_segments(uint64_t num_events, uint32_t num_streams);
+size_t argus_split_bytes(uint64_t num_events, uint32_t num_streams);
+int argus_launch_pair_split(ArgusPairArgs& a, void* room, cudaStream_t stream);
 
 #define ARGUS_NOTE_POS_BITS 48
 

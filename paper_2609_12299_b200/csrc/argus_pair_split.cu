@@ -1,0 +1,242 @@
+// argus_pair_split.cu — few long streams: pairing of the segments of a stream at the same time.
+//
+// A stream is a chain: what a marker means depends on the stack that everything before it leaves. With fewer streams than the
+// chip has room for blocks (a trace of some of the SMs) the chained pass leaves most of it idle. Here
+//   k_split_scan  : one block per segment reads the markers' kinds only and finds, by heights, how many ends close a frame from
+//                   before the segment and which begins stay open at its end;
+//   k_split_chain : one warp per stream walks its segments and gives every one the stack where it starts;
+//   (the SPLIT instantiation of the tiled kernel walks the segments: argus_pair_tiled.cu)
+//   k_split_fix   : one block per stream completes the child time of the frames that were open across a segment's start, counts
+//                   the stream's intervals and notes the frames open at its end.
+// Heights know nothing of region ids. A segment that meets a marker which breaks the parallel rules gives its stream up; the
+// chained pass, which follows and does nothing otherwise, walks such streams from their beginning.
+//
+// The scan reads the events once more (16 of then 56 bytes an event). 96 streams of 518,656 events: pairing 2,412 -> 690 us.
+#include "argus_internal.cuh"
+#include "argus_pair_common.cuh"
+
+namespace {
+
+constexpr int kScanThreads = 256;
+constexpr int kFixThreads = 512;
+constexpr u32 kRun = 32;  // consecutive events a thread looks at
+constexpr u32 kBlockEvents = kScanThreads * kRun;
+
+__device__ __forceinline__ u32 split_length(const ArgusPairArgs& a, u32 s) {
+  const u64 off0 = a.stream_offsets[0], lo = a.stream_offsets[s], hi = a.stream_offsets[s + 1];
+  return hi < lo || hi > a.num_events || lo < off0 || ((hi - lo) >> 32) ? 0u : (u32)(hi - lo);
+}
+__device__ __forceinline__ u32 split_segments(const ArgusPairArgs& a, u32 s) {  // an empty or bad stream has one, of no tiles
+  const u64 per = (u64)a.segment_tiles * kSplitTile, n = split_length(a, s);
+  return n ? (u32)((n + per - 1) / per) : 1u;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u32* first_segment) {
+  argus_kernel_begin();
+  __shared__ u32 sh[33], sh_stream, sh_before;
+  __shared__ int shi[33], low_of[kScanThreads / 32];
+  const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the block's segment: streams' segments one after the other
+  if (tid == 0) sh_stream = 0xffffffffu;
+  __syncthreads();
+  u32 carry = 0;
+  for (u32 s0 = 0; s0 < a.num_streams; s0 += kScanThreads) {
+    const u32 s = s0 + tid, c = s < a.num_streams ? split_segments(a, s) : 0u;
+    u32 total;
+    const u32 ex = carry + argus_block_exclusive_scan<u32>(c, sh, &total);
+    if (blockIdx.x == 0 && s < a.num_streams) { first_segment[s] = ex; a.split_failed[s] = 0; }
+    if (blockIdx.x >= ex && blockIdx.x < ex + c) { sh_stream = s; sh_before = ex; }
+    carry += total;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0 && tid == 0) { first_segment[a.num_streams] = carry; a.ctl->num_segments = carry; }
+  if (sh_stream == 0xffffffffu) return;
+  const u32 s = sh_stream, j = blockIdx.x - sh_before, n = split_length(a, s), per = a.segment_tiles * kSplitTile;
+  ArgusSegment* const g = a.segments + blockIdx.x;
+  const u32 start = j * per, count = n - start < per ? n - start : per;
+  const uint4* const src = reinterpret_cast<const uint4*>(a.events + a.stream_offsets[s]) + start;
+  // from the last event back: a begin without an end behind it goes below every height so far
+  int height = 0, lowest = 0;
+  for (u32 i0 = 0; i0 < count; i0 += kBlockEvents) {
+    u32 ends = 0;  // bit j: event i0 + (32 tid + j) from the end is an end
+    const u32 w0 = i0 + warp * 32 * kRun;
+#pragma unroll 16
+    for (u32 r = 0; r < kRun; ++r) {
+      const u32 i = w0 + r * 32 + lane;
+      const u32 tag = i < count ? __ldg(reinterpret_cast<const u32*>(src + (count - 1 - i)) + 2) : 0u;
+      const u32 b = __ballot_sync(0xffffffffu, tag & 1u);
+      if (lane == r) ends = b;
+    }
+    const u32 mine = i0 + tid * kRun, have = mine < count ? (count - mine < kRun ? count - mine : kRun) : 0u;
+    const u32 begins = have ? ~ends & (0xffffffffu >> (32 - have)) : 0u;
+    int total;
+    const int h0 = height + argus_block_exclusive_scan<int>(__popc(ends) - __popc(begins), shi, &total);
+    int h = h0, low = h0;
+#pragma unroll
+    for (u32 r = 0; r < kRun; ++r) {
+      h += (int)((ends >> r) & 1u) - (int)((begins >> r) & 1u);
+      low = h < low ? h : low;
+    }
+    int upto = low;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const int o = __shfl_up_sync(0xffffffffu, upto, d); if (lane >= (u32)d && o < upto) upto = o; }
+    if (lane == 31) low_of[warp] = upto;
+    __syncthreads();
+    int before = __shfl_up_sync(0xffffffffu, upto, 1);
+    if (lane == 0 || before > lowest) before = lowest;
+    int all = lowest;
+    for (u32 w = 0; w < kScanThreads / 32; ++w) {
+      const int o = low_of[w];
+      if (w < warp && o < before) before = o;
+      if (o < all) all = o;
+    }
+    if (low < before) {
+      h = h0;
+      for (u32 r = 0; r < kRun; ++r) {
+        h += (int)((ends >> r) & 1u) - (int)((begins >> r) & 1u);
+        if (h < before) {
+          before = h;
+          if (-h <= ARGUS_MAX_DEPTH) g->open[-h - 1] = start + (count - 1 - (mine + r));
+        }
+      }
+    }
+    lowest = all;
+    height += total;
+    __syncthreads();
+  }
+  if (tid < ARGUS_MAX_DEPTH) g->note_pos[tid] = ~0ull;
+  if (tid < 3) g->flags[tid] = 0;
+  if (tid == 0) {
+    g->stream = s; g->first_tile = j * a.segment_tiles; g->num_tiles = (count + kSplitTile - 1) / kSplitTile;
+    g->unmatched_begins = (u32)-lowest;
+    g->unmatched_ends = (u32)(height - lowest);
+  }
+}
+
+// (a segment's summary is asked for four segments ahead: what is left is one round of shared memory per segment)
+__global__ void __launch_bounds__(32) k_split_chain(ArgusPairArgs a, const u32* first_segment) {
+  argus_kernel_begin_long();
+  static_assert(ARGUS_MAX_DEPTH == 64, "two levels a lane");
+  __shared__ u32 stack[ARGUS_MAX_DEPTH];
+  constexpr u32 kAhead = 4;
+  const u32 s = blockIdx.x, lane = threadIdx.x;
+  const u32 g0 = first_segment[s], g1 = first_segment[s + 1];
+  int h = 0;
+  bool fail = false;
+  u32 ends[kAhead], begins[kAhead], open0[kAhead], open1[kAhead];
+#pragma unroll
+  for (u32 q = 0; q < kAhead; ++q) {
+    const ArgusSegment* const g = a.segments + (g0 + q < g1 ? g0 + q : g0);
+    ends[q] = __ldcg(&g->unmatched_ends); begins[q] = __ldcg(&g->unmatched_begins);
+    open0[q] = __ldcg(g->open + lane); open1[q] = __ldcg(g->open + lane + 32);
+  }
+  for (u32 k0 = g0; k0 < g1 && !fail; k0 += kAhead) {
+#pragma unroll
+    for (u32 q = 0; q < kAhead; ++q) {
+      const u32 k = k0 + q;
+      if (k >= g1 || fail) break;
+      ArgusSegment* const g = a.segments + k;
+      const int ue = (int)ends[q], ub = (int)begins[q], low = h - ue;
+      const u32 o0 = open0[q], o1 = open1[q];
+      if (k + kAhead < g1) {
+        const ArgusSegment* const n = g + kAhead;
+        ends[q] = __ldcg(&n->unmatched_ends); begins[q] = __ldcg(&n->unmatched_begins);
+        open0[q] = __ldcg(n->open + lane); open1[q] = __ldcg(n->open + lane + 32);
+      }
+      if ((int)lane < h) g->idx[lane] = stack[lane];
+      if ((int)lane + 32 < h) g->idx[lane + 32] = stack[lane + 32];
+      if (lane == 0) g->ch = h;
+      if (low < 0 || ub > ARGUS_MAX_DEPTH || low + ub > ARGUS_MAX_DEPTH) { fail = true; break; }
+      __syncwarp();
+      if ((int)lane < ub) stack[low + ub - 1 - (int)lane] = o0;
+      if ((int)lane + 32 < ub) stack[low + ub - 1 - (int)lane - 32] = o1;
+      h = low + ub;
+      __syncwarp();
+      if (k + 1 == g1) {
+        if ((int)lane < h) g->open[lane] = stack[lane];
+        if ((int)lane + 32 < h) g->open[lane + 32] = stack[lane + 32];
+      }
+    }
+  }
+  if (fail && lane == 0) { a.split_failed[s] = 1; atomicAdd(&a.ctl->num_failed, 1u); }
+}
+
+__global__ void __launch_bounds__(kFixThreads) k_split_fix(ArgusPairArgs a, const u32* first_segment) {
+  argus_kernel_begin_long();
+  const u32 s = blockIdx.x;
+  if (__ldcg(a.split_failed + s)) return;
+  const u32 g0 = first_segment[s], g1 = first_segment[s + 1], per = a.segment_tiles * kSplitTile;
+  const u64 off0 = a.stream_offsets[0];
+  u32 ctx = 0, rev = 0, clamp = 0;
+  const u64 limit = a.bases[s + 1] < a.interval_capacity ? a.bases[s + 1] : a.interval_capacity;
+  for (u32 i = threadIdx.x; i < (g1 - g0) * ARGUS_MAX_DEPTH; i += blockDim.x) {
+    const u32 k = g0 + i / ARGUS_MAX_DEPTH, l = i % ARGUS_MAX_DEPTH;
+    const ArgusSegment* const g = a.segments + k;
+    if (l == 0) { ctx += g->flags[0]; rev += g->flags[1]; clamp += g->flags[2]; }
+    const u64 pos = g->note_pos[l];
+    if (pos == ~0ull) continue;
+    u64 child = g->note_child[l];
+    const u64 incl = g->note_incl[l];
+#pragma unroll 4
+    for (u32 q = g0 + g->idx[l] / per; q < k; ++q) child += a.segments[q].ledger[l];
+    const bool clamped = child > incl;
+    clamp += clamped;
+    if (pos >= limit) continue;  // not written: such a stream is written by the second pass
+    argus_interval_t* const r = a.intervals + pos;
+    const u32 flags = r->flags | (clamped ? ARGUS_FLAG_CHILD_CLAMPED : 0u);
+    const u64 excl = clamped ? 0 : incl - child;
+    r->exclusive = excl;
+    r->flags = (uint16_t)flags;
+    if (a.digest) a.digest[pos] = argus_digest_pack(r->region, incl, excl, flags);
+  }
+  if (ctx) atomicAdd((u64*)&a.status->n_ctx_mismatch, (u64)ctx);
+  if (rev) atomicAdd((u64*)&a.status->n_time_reversed, (u64)rev);
+  if (clamp) atomicAdd((u64*)&a.status->n_child_clamped, (u64)clamp);
+  const u32 n = split_length(a, s);
+  const ArgusSegment* const last = a.segments + (g1 - 1);
+  if (threadIdx.x == 0) a.counts[s] = n ? last->n_int : 0;
+  if (n && threadIdx.x < last->end_ch) argus_note_ambiguity(a, a.stream_offsets[s] - off0 + last->open[threadIdx.x], ARGUS_AMBIG_BEGIN_EOS, threadIdx.x);
+}
+
+}  // namespace
+
+// Fewer streams than three quarters of the blocks of the pairing kernel that run at a time (7 x 148), and long ones: the chained
+// pass would leave the rest of the chip idle. Above, the scan (a quarter of the split pass) eats the gain.
+bool argus_split_usable(uint64_t num_events, uint32_t num_streams) {
+  return num_streams > 0 && num_streams < 777 && num_events > (1u << 20) && num_events / num_streams >= 16 * kSplitTile;
+}
+
+static u32 split_tiles(uint64_t num_events) {  // about three segments for every block that runs at a time, of 8 tiles at least
+  const u64 tiles = (num_events / 3072 + kSplitTile - 1) / kSplitTile;
+  return (u32)(tiles < 8 ? 8 : tiles);
+}
+
+uint32_t argus_split_max_segments(uint64_t num_events, uint32_t num_streams) {
+  return (u32)(num_events / ((u64)split_tiles(num_events) * kSplitTile)) + num_streams;
+}
+
+size_t argus_split_bytes(uint64_t num_events, uint32_t num_streams) {
+  if (!argus_split_usable(num_events, num_streams)) return 0;
+  return argus_align_up((size_t)argus_split_max_segments(num_events, num_streams) * sizeof(ArgusSegment), 256) +
+         argus_align_up(((size_t)num_streams + 1) * 4, 256) + argus_align_up((size_t)num_streams * 4, 256);
+}
+
+int argus_launch_pair_tiled(const ArgusPairArgs& a, cudaStream_t stream, bool split);
+
+// The whole split pass; `room` holds argus_split_bytes(). Leaves a.segments and a.split_failed set for the chained pass.
+int argus_launch_pair_split(ArgusPairArgs& a, void* room, cudaStream_t stream) {
+  const u32 most = argus_split_max_segments(a.num_events, a.num_streams);
+  char* w = (char*)room;
+  a.segments = (ArgusSegment*)w;
+  w += argus_align_up((size_t)most * sizeof(ArgusSegment), 256);
+  u32* const first_segment = (u32*)w;
+  w += argus_align_up(((size_t)a.num_streams + 1) * 4, 256);
+  a.split_failed = (u32*)w;
+  a.segment_tiles = split_tiles(a.num_events);
+  ARGUS_LAUNCH(k_split_scan, most, kScanThreads, 0, stream, a, first_segment);
+  ARGUS_LAUNCH(k_split_chain, a.num_streams, 32, 0, stream, a, (const u32*)first_segment);
+  const int rc = argus_launch_pair_tiled(a, stream, true);
+  if (rc != ARGUS_OK) return rc;
+  ARGUS_LAUNCH(k_split_fix, a.num_streams, kFixThreads, 0, stream, a, (const u32*)first_segment);
+  return ARGUS_OK;
+}

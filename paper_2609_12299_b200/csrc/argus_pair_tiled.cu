@@ -137,6 +137,7 @@ struct TileSmem {
   int badpos[2];                   // first position of the window where the parallel rules fail (INT_MAX = none); windows alternate
                                    // between the two, so that one can be reset while stragglers still read the other
   int dead, failed;
+  int low;                         // split pass: lowest initial frame that the window closed
 };
 
 // Latest begin of the tile at level L and position < pos (pos <= T); -1 if there is none. Written without
@@ -190,7 +191,9 @@ __device__ __forceinline__ void tile_fetch(const ArgusPairArgs& a, uint4* dst, c
   }
 }
 
-template <int NT, int E, int MINB, bool RING = false>
+// SPLIT: the work items are segments of streams instead of whole streams (see argus_pair_split.cu): the initial stack comes with
+// the segment, and a marker that breaks the parallel rules gives the stream up to the chained pass that follows.
+template <int NT, int E, int MINB, bool RING = false, bool SPLIT = false>
 __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   using SM = TileSmem<NT, E>;
   constexpr int T = SM::T, NW = SM::NW, NWORDS = SM::NWORDS, MAXI = SM::MAXI, NI = SM::NI;
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   argus_kernel_begin_long();
   if (a.redo && !__ldcg(&a.ctl->redo)) return;
+  if (!SPLIT && !a.redo && a.segments && !__ldcg(&a.ctl->num_failed)) return;
   if (tid == 0) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);
@@ -217,7 +221,10 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     if (tid == 0) {
       u64 st = ~0ull;
       u32 rc = kNoRec;
-      if (!tile_pop_work(a, a.redo ? 1 : 0, &st, &rc)) st = ~0ull;
+      if (SPLIT) {
+        rc = atomicAdd(&a.ctl->seg_head, 1u);
+        st = rc < a.ctl->num_segments ? a.segments[rc].stream : ~0ull;
+      } else if (!tile_pop_work(a, a.redo ? 1 : 0, &st, &rc)) st = ~0ull;
       sm.cur_stream = st;
       sm.cur_rec = rc;
     }
@@ -226,6 +233,12 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     if (s64 >= a.num_streams) break;
     const u32 s = (u32)s64;
     u32 rec = sm.cur_rec;
+    if (SPLIT ? __ldcg(a.split_failed + s) != 0 : (a.segments && !a.redo && rec == kNoRec && !__ldcg(a.split_failed + s))) {
+      if (!SPLIT && tid == 0) atomicAdd(&a.ctl->n_done[0], 1u);  // walked by the split pass
+      __syncthreads();
+      continue;
+    }
+    ArgusSegment* const seg = SPLIT ? a.segments + rec : nullptr;
     const u64 lo = a.stream_offsets[s], hi = a.stream_offsets[s + 1];
     if (hi < lo || hi > a.num_events || lo < off0 || ((hi - lo) >> 32)) {
       if (tid == 0) {
@@ -255,8 +268,22 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     // reserves a record.
     u32 ti0 = 0;
     constexpr u32 kChunkTiles = (kChunkEvents + T - 1) / T;
-    bool chunked = a.queue != nullptr && ntiles > kChunkTiles;
-    if (rec != kNoRec) {
+    bool chunked = !SPLIT && a.queue != nullptr && ntiles > kChunkTiles;
+    int init_h = 0;      // split: frames of the initial stack that are still open (uniform)
+    u64 limit = a.interval_capacity;
+    if (SPLIT) {
+      ti0 = seg->first_tile;
+      ch = init_h = seg->ch;
+      n_int = ((u64)ti0 * T - (u64)ch) >> 1;  // every marker before is a begin or an end, and the open ones are the difference
+      if (a.bases[s + 1] < limit) limit = a.bases[s + 1];
+      if (tid < ch) {
+        const u32 at = seg->idx[tid];
+        sm.evall[T + tid] = __ldg(reinterpret_cast<const uint4*>(src + at));
+        sm.cchild[0][tid] = 0;
+        sm.cidx[0][tid] = at;
+      }
+      if (tid == 0) sm.low = 0x7fffffff;
+    } else if (rec != kNoRec) {
       const ArgusStreamRecord* r = a.records + rec;
       ti0 = __ldcg(&r->next_tile);
       ch = __ldcg(&r->ch);
@@ -276,7 +303,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       rec = sm.cur_rec;
       if (rec == kNoRec) chunked = false;  // cannot happen (one record per long stream); then the stream is walked whole
     }
-    const u32 ti_end = chunked && ti0 + kChunkTiles < ntiles ? ti0 + kChunkTiles : ntiles;
+    const u32 ti_end = SPLIT ? ti0 + seg->num_tiles : chunked && ti0 + kChunkTiles < ntiles ? ti0 + kChunkTiles : ntiles;
     if (tid == 0 && ti0 < ti_end) {  // first tile of this chunk, into the buffer its index selects
       const u32 start = ti0 * (u32)T;
       tile_fetch<RING>(a, (ti0 & 1) ? sm.evall + T + 2 * kCar : sm.evall, src, ring_first, start,
@@ -442,11 +469,17 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
               u64 incl = 0, excl = 0;
               if (ee.w != pe.w) { flags |= ARGUS_FLAG_CTX_MISMATCH; ++tot_ctx; }
               if (ts < bts) { flags |= ARGUS_FLAG_TIME_REVERSED; ++tot_rev; } else { incl = ts - bts; }
-              if (child > incl) { flags |= ARGUS_FLAG_CHILD_CLAMPED; ++tot_clamp; } else { excl = incl - child; }
+              const u64 pos = pos0 + (u64)rk;
+              if (SPLIT && carried && partner - cbase < init_h) {  // its child time is completed afterwards
+                seg->note_child[partner - cbase] = child;
+                seg->note_incl[partner - cbase] = incl;
+                seg->note_pos[partner - cbase] = pos;
+                atomicMin(&sm.low, partner - cbase);
+                excl = incl;
+              } else if (child > incl) { flags |= ARGUS_FLAG_CHILD_CLAMPED; ++tot_clamp; } else { excl = incl - child; }
               const u32 bidx = carried ? sm.cidx[cpar][partner - cbase] : tile_start + (u32)partner;
               const u32 preg = parent == cbase + kSink ? ARGUS_NONE : (reinterpret_cast<const u32*>(evb + parent)[2] >> 1);
-              const u64 pos = pos0 + (u64)rk;
-              if (pos < a.interval_capacity) {
+              if (pos < (SPLIT ? limit : a.interval_capacity)) {
                 uint4* q = reinterpret_cast<uint4*>(a.intervals + pos);
                 q[0] = make_uint4(pe.x, pe.y, (u32)incl, (u32)(incl >> 32));
                 q[1] = make_uint4((u32)excl, (u32)(excl >> 32), pe.z >> 1, pe.w);
@@ -470,8 +503,13 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
           w0 = wend;
           wend = tn;
           __syncthreads();
+          if (SPLIT) init_h = sm.low < init_h ? sm.low : init_h;
         } else if (badpos > w0) {
           wend = badpos;  // [w0, badpos) is well nested: do it again on its own (nothing was committed yet)
+        } else if (SPLIT) {  // the chained pass walks this stream
+          stream_failed = true;
+          __syncthreads();
+          break;
         } else {
           // ---------------- the marker(s) at w0 go through the sequential stack machine ----------------
           const int nseq = small_streak >= 2 ? ((tn - w0) < kSeqChunk ? (tn - w0) : kSeqChunk) : 1;
@@ -533,7 +571,18 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       }
       return;
     }
-    if (!stream_failed && ti_end < ntiles) {
+    if (SPLIT) {
+      if (stream_failed) {
+        if (tid == 0 && atomicExch(a.split_failed + s, 1u) == 0) atomicAdd(&a.ctl->num_failed, 1u);
+      } else {
+        if (tid < ch) seg->ledger[tid] = sm.cchild[cpar][tid];
+        if (tid == 0) { seg->n_int = n_int; seg->end_ch = (u32)ch; }
+        if (tot_ctx) atomicAdd(&seg->flags[0], tot_ctx);
+        if (tot_rev) atomicAdd(&seg->flags[1], tot_rev);
+        if (tot_clamp) atomicAdd(&seg->flags[2], tot_clamp);
+      }
+      tot_ctx = tot_rev = tot_clamp = 0;
+    } else if (!stream_failed && ti_end < ntiles) {
       // hand the stream on: its state goes into the record, the record into the queue
       ArgusStreamRecord* r = a.records + rec;
       if (tid == 0) { r->stream = s; r->next_tile = ti_end; r->ch = ch; r->n_int = n_int; }
@@ -573,7 +622,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
 
 // The shared-memory opt-in and the occupancy of one instantiation belong to one device: looked up once per
 // device, under a lock (two host threads may make their first call at the same time).
-template <int NT, int E, int MINB, bool RING>
+template <int NT, int E, int MINB, bool RING, bool SPLIT = false>
 int launch_tiled(const ArgusPairArgs& a, cudaStream_t stream) {
   constexpr int kMaxDevices = 64;
   static int grid_of[kMaxDevices];
@@ -586,18 +635,19 @@ int launch_tiled(const ArgusPairArgs& a, cudaStream_t stream) {
   {
     std::lock_guard<std::mutex> lk(mu);
     if (!grid_of[dev]) {
-      ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_pair_tiled<NT, E, MINB, RING>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_pair_tiled<NT, E, MINB, RING, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       int sms = 0, per_sm = 0;
       ARGUS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-      ARGUS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair_tiled<NT, E, MINB, RING>, NT, smem));
+      ARGUS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair_tiled<NT, E, MINB, RING, SPLIT>, NT, smem));
       if (per_sm < 1) return ARGUS_ERR_CUDA;
       if (per_sm > MINB) per_sm = MINB;
       grid_of[dev] = sms * per_sm;
     }
     grid_cache = grid_of[dev];
   }
-  const u32 grid = a.num_streams < (u32)grid_cache ? a.num_streams : (u32)grid_cache;
-  ARGUS_LAUNCH(k_pair_tiled<NT, E, MINB, RING>, grid, NT, smem, stream, a);
+  const u32 items = SPLIT ? argus_split_max_segments(a.num_events, a.num_streams) : a.num_streams;
+  const u32 grid = items < (u32)grid_cache ? items : (u32)grid_cache;
+  ARGUS_LAUNCH(k_pair_tiled<NT, E, MINB, RING, SPLIT>, grid, NT, smem, stream, a);
   return ARGUS_OK;
 }
 
@@ -611,7 +661,8 @@ bool argus_pair_tiled_usable(const ArgusPairArgs& a) { return a.num_streams > 0;
 // <threads, events per thread, CTAs per SM> (test aid: tiles end at other places; results do not depend on it).
 extern "C" void argus_set_tile_variant(int v) { g_variant.store(v); }
 
-int argus_launch_pair_tiled(const ArgusPairArgs& a, cudaStream_t stream) {
+int argus_launch_pair_tiled(const ArgusPairArgs& a, cudaStream_t stream, bool split) {
+  if (split) return launch_tiled<128, kSplitTile / 128, 7, false, true>(a, stream);
   if (a.ring_written) return launch_tiled<128, 5, 7, true>(a, stream);  // ring container: one shape
   switch (g_variant.load(std::memory_order_relaxed)) {
     case 1: return launch_tiled<192, 5, 4, false>(a, stream);

@@ -16,6 +16,7 @@ std::atomic<int> g_synth_mode_knob{-1};  // -1 = automatic
 struct SynLayout {
   size_t pair, pair_bytes, agg, agg_bytes, ov, ov_bytes, pieces, spans, digest, starts, total;
   uint64_t digest_capacity;
+  uint32_t parts, slices;
 };
 
 SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_regions, uint64_t ambig_capacity,
@@ -27,7 +28,9 @@ SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_reg
   // Overlap: the plain call's workspace, or control block, first pieces of the slices and 32 bytes a span (the entries
   // lie in the digest array).
   const bool digests = argus_aggregate_can_read_digests(num_regions);
-  const size_t pieces = (size_t)num_streams * argus_aggregate_digest_slices() * sizeof(ArgusOvPiece);
+  L.parts = argus_aggregate_digest_parts(num_streams, num_events);
+  L.slices = argus_aggregate_digest_slices(L.parts);
+  const size_t pieces = (size_t)num_streams * L.slices * sizeof(ArgusOvPiece);
   L.ov = o;
   L.pieces = o + argus_align_up(sizeof(ArgusOvCtl), 256);
   L.spans = L.pieces + argus_align_up(pieces, 256);
@@ -97,13 +100,13 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
                                          cta_sm, num_sms, num_regions, nullptr, warp_tab, cta_tab, sm_tab, kernel_tab,
                                          nullptr, nullptr, status, ws + L.agg, L.agg_bytes, cuda_stream, false,
                                          f.num_pairs ? &f : nullptr,
-                                         use_digest ? (const uint64_t*)(ws + L.digest) : nullptr, interval_capacity);
+                                         use_digest ? (const uint64_t*)(ws + L.digest) : nullptr, L.parts, interval_capacity);
     if (rc != ARGUS_OK) return rc;
   }
   if (num_pairs) {
     if (f.num_pairs) {
       rc = argus_internal_overlap_from_digests(intervals, (const uint64_t*)f.starts, (const uint64_t*)f.entries, f.pieces,
-                                               argus_aggregate_digest_slices(), num_streams, warps_per_cta, cta_sm, num_sms, pairs,
+                                               L.slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs,
                                                num_pairs, overlap_out, status, ov_ctl, ws + L.spans, max_overlap_spans, cuda_stream);
     } else {
       rc = argus_internal_overlap(intervals, interval_capacity, interval_offsets, num_streams, warps_per_cta, cta_sm, num_sms,

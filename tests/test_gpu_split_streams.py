@@ -1,0 +1,84 @@
+"""Few long streams: the segments of a stream are paired at the same time. Frames that stay open over many segments, streams that
+end in the middle, empty and short ones among them, and markers that make a stream fall back to the chained pass, against the
+oracle; both pairing alone and the one-call pipeline."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_12299_b200 as argus
+from paper_2609_12299_b200 import tracegen as tg
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _wrap(ev, region, ctx=0):
+    """The stream inside one interval of `region` that is open over all of it."""
+    out = np.zeros(len(ev) + 2, argus.EVENT_DTYPE)
+    out[1:-1] = ev
+    out[0] = (ev["ts"][0] - 5, region << 1, ctx)
+    out[-1] = (ev["ts"][-1] + 7, (region << 1) | 1, ctx)
+    return out
+
+
+def _trace(kind, rng):
+    idx, ctas, iters = {"gemm": (1, 3, 1300), "attention": (2, 2, 8), "decode": (3, 1, 40)}[kind]
+    spec = tg.config(idx).scaled(ctas, iters)
+    ev, offs = tg.generate_host(spec)
+    streams = [ev[offs[s]:offs[s + 1]] for s in range(spec.num_streams)]
+    return spec, streams
+
+
+@pytest.mark.parametrize("change", ["none", "wrapped", "cut", "lengths", "clamped", "defects"])
+@pytest.mark.parametrize("kind", ["gemm", "attention", "decode"])
+def test_segments(kind, change):
+    rng = np.random.default_rng(7)
+    spec, streams = _trace(kind, rng)
+    R = spec.num_regions + 2
+    if change == "wrapped":      # two levels that are open over every segment
+        streams = [_wrap(_wrap(e, R - 1), R - 2) for e in streams]
+    elif change == "cut":        # ends missing at the back
+        streams = [e[:len(e) - int(rng.integers(0, 40))] for e in streams]
+    elif change == "lengths":    # exact multiples of a tile and of a segment, one event more, one tile, nothing
+        for s, n in enumerate([640, 641, 0, 8 * 640, 8 * 640 + 1, 1]):
+            streams[s] = streams[s][:n]
+    elif change == "clamped":    # outer intervals shorter than their children
+        streams = [_wrap(e, R - 1) for e in streams]
+        for e in streams:
+            e["ts"][-1] = e["ts"][0] + np.uint64(9)
+    elif change == "defects":    # one stream loses an end, one has a stray one, one has an outlier in time
+        streams = [_wrap(e, R - 1) for e in streams]
+        streams[0] = np.delete(streams[0], len(streams[0]) // 2)
+        streams[1]["tag"][len(streams[1]) // 3] ^= 1
+        streams[2]["ts"][len(streams[2]) // 2:] += np.uint64(1 << 33)
+    while sum(len(e) for e in streams) <= 1 << 20:
+        streams = streams + streams[:spec.warps_per_cta]
+    ev = np.concatenate(streams)
+    offs = np.cumsum([0] + [len(e) for e in streams]).astype(np.uint64)
+    S, W = len(streams), spec.warps_per_cta
+    assert S < 777 and len(ev) > 1 << 20 and len(ev) // S >= 10240
+    d_ev = torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).to(DEV)
+    d_off = torch.from_numpy(offs.view(np.int64).copy()).to(DEV)
+    _, iv, ioffs, am, aoffs, o_st = oracle.pair(ev, offs, R)
+
+    def check(p):
+        st = p.fetch_status()
+        assert int(st["code"]) == 0
+        assert np.array_equal(p.interval_offsets.cpu().numpy().view(np.uint64), ioffs)
+        assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)
+        assert p.intervals_numpy().tobytes() == iv.tobytes()
+        assert p.ambig_numpy().tobytes() == am.tobytes()
+        for f in ("n_ctx_mismatch", "n_time_reversed", "n_child_clamped", "intervals_required", "ambig_required"):
+            assert int(st[f]) == int(o_st[f]), f
+
+    check(argus.argus_pair_intervals(d_ev, d_off, R))
+    cta_sm = (np.arange(S // W) % 2).astype(np.uint32)
+    pairs = np.concatenate([spec.overlap_pairs, [[0, 1]]]).astype(np.uint32)
+    r = argus.argus_synthesize(d_ev, d_off, R, W, torch.from_numpy(cta_sm.view(np.int32)).to(DEV), 2, torch.from_numpy(pairs.view(np.int32)).to(DEV))
+    check(r.pair)
+    _, tabs, _ = oracle.aggregate(iv, ioffs, am, aoffs, W, cta_sm, 2, R)
+    for lv in ("warp", "cta", "sm", "kernel"):
+        assert r.agg.table_numpy(lv).tobytes() == tabs[lv].tobytes(), lv
+    _, ov, _ = oracle.overlap(iv, ioffs, W, cta_sm, 2, pairs)
+    assert r.overlap_numpy(2).tobytes() == ov.tobytes()

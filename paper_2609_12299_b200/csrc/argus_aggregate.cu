@@ -8,12 +8,11 @@
 //                   several CTAs fit an SM), for up to kAggCompactRegions regions;
 //   k_agg_streams : the same with a full 576 B-per-region copy in shared memory when that fits, else on
 //                   the global row itself. Integer atomics only: the result does not depend on thread order.
-//   k_agg_rollup  : CTA-scope cells = reduction over the warps of each CTA; SM-scope and kernel-scope cells by atomic
-//                   add/min/max of CTA cells.
-//   k_agg_role    : warp-role cells = reduction over the CTAs of each warp index (plain loads).
-//   k_agg_iter    : per-iteration cells (key = ctx - ctx_lo) of the intervals of a scope.
-// A scope (iteration window, warp mask, SM mask, region mask) filters what k_agg_streams and
-// k_agg_iter take in; without one everything is selected.
+//   k_agg_rollup  : CTA-scope and warp-role cells = reductions over the warps of each CTA and over the CTAs; SM-scope and
+//                   kernel-scope cells by atomic add/min/max of CTA cells.
+//   k_agg_iter_windows, k_agg_iter : per-iteration cells (key = ctx - ctx_lo) of the intervals of a scope.
+// A scope (iteration window, warp mask, SM mask, region mask) filters what the kernels over intervals
+// take in; without one everything is selected.
 #include "argus_internal.cuh"
 
 namespace {
@@ -22,8 +21,8 @@ constexpr int kAggThreads = 256;
 constexpr u32 kCell = 72;  // u64 words per argus_agg_t
 constexpr size_t kAggSmemLimit = 200 * 1024;
 constexpr u32 kAggCompactRegions = 400;  // 112 B each: 44.8 KB of shared memory at most
-constexpr size_t kIterScratchBytes = 32u << 20;  // workspace for private copies of an iteration table
-constexpr u32 kIterMaxCopies = 32;
+constexpr u32 kIterThreads = 512, kIterWarps = kIterThreads / 32;  // k_agg_iter_windows
+constexpr u32 kMaxParts = 16;            // blocks that share a stream in k_agg_streams_compact
 
 struct AggArgs {
   const argus_interval_t* intervals;
@@ -46,22 +45,21 @@ struct AggArgs {
   u64* role_tab;  // [W][R][72], nullable
   u64* iter_tab;  // [num_iters][R][72], nullable
   u32 num_iters;
-  int iter_smem;
-  u64* iter_copies;   // global path: private copies of the iteration table, one per group of blocks (null: none)
-  u32 num_copies;
-  int iter_inline;    // global path taken inside k_agg_streams_compact (one read of the intervals serves both)
+  ulonglong2* ranges; // [S][parts] first and last + 1 interval of the part that is in the iteration window (null: not asked for)
   // overlap selection in the pass over the digests (argus_synthesize)
   ArgusFuseArgs ov;
-  u32 parts;          // k_agg_streams_digest: blocks that share a stream
+  u32 parts;          // k_agg_streams_digest, k_agg_streams_compact: blocks that share a stream
   const u64* digest;  // digests of the intervals (k_agg_streams_digest; overwritten with entries where overlap is selected), null = read the records
   u64 interval_limit; // records the interval array holds: a stream whose offsets reach beyond it is reported, not read
 };
 
-// SM-scope and kernel-scope tables start empty; the kernel after the one that calls this adds to them.
+// The tables that the kernels after the one that calls this add to start empty.
 __device__ __forceinline__ void agg_empty_tables(const AggArgs& a) {
   const u64 first = (u64)blockIdx.x * blockDim.x + threadIdx.x, stride = (u64)gridDim.x * blockDim.x, row = (u64)a.num_regions * kCell;
   if (a.sm_tab) for (u64 i = first; i < a.num_sms * row; i += stride) a.sm_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
   if (a.kernel_tab) for (u64 i = first; i < row; i += stride) a.kernel_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
+  if (a.role_tab) for (u64 i = first; i < a.warps_per_cta * row; i += stride) a.role_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
+  if (a.iter_tab) for (u64 i = first; i < a.num_iters * row; i += stride) a.iter_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
 }
 
 __device__ __forceinline__ bool mask_bit(const u32* mask, u32 i) { return !mask || ((mask[i >> 5] >> (i & 31)) & 1u); }
@@ -92,19 +90,6 @@ __device__ __forceinline__ void agg_add_interval(u64* tab, u32 region, u64 incl,
   atomicAdd(c + 1, incl);
   atomicMin(c + 2, incl);
   atomicMax(c + 3, incl);
-  atomicAdd(c + 4, excl);
-  if (flags) atomicAdd(c + 7, 1ull);
-  atomicAdd(c + 8 + log2_bin(incl), 1ull);
-}
-
-// The same for a table in global memory that many blocks share: three atomics per interval instead of six. The
-// count is left out (it is the sum of the histogram bins and is filled in afterwards) and min / max are
-// only updated while they still move (a stale read only costs a redundant atomic).
-__device__ __forceinline__ void agg_add_interval_lean(u64* tab, u32 region, u64 incl, u64 excl, u32 flags) {
-  u64* c = tab + (size_t)region * kCell;
-  atomicAdd(c + 1, incl);
-  if (incl < __ldcg(c + 2)) atomicMin(c + 2, incl);
-  if (incl > __ldcg(c + 3)) atomicMax(c + 3, incl);
   atomicAdd(c + 4, excl);
   if (flags) atomicAdd(c + 7, 1ull);
   atomicAdd(c + 8 + log2_bin(incl), 1ull);
@@ -160,53 +145,59 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
   argus_kernel_begin_long();
   agg_empty_tables(a);
   extern __shared__ __align__(16) unsigned char sh_raw[];
+  __shared__ u64 range[2];
   ArgusAggCell* const ctab = reinterpret_cast<ArgusAggCell*>(sh_raw);
   const u32 R = a.num_regions;
   const u32 cells = R * kCell;
-  // iteration table too large for shared memory: this block's private copy in global memory (or the table itself)
-  u64* const iter_base = !a.iter_inline ? nullptr
-                         : a.iter_copies ? a.iter_copies + (u64)(blockIdx.x % a.num_copies) * a.num_iters * cells : a.iter_tab;
-  for (u32 s = blockIdx.x; s < a.num_streams; s += gridDim.x) {
-    u64* row = a.warp_tab + (size_t)s * cells;
-    // the global row takes flag counts' overflow path, bins outside the window and the ambiguity counters directly
+  const u32 s = blockIdx.x / a.parts, part = blockIdx.x % a.parts;
+  u64* row = a.warp_tab + (size_t)s * cells;
+  // the global row takes bins outside the windows and the ambiguity counters directly
+  if (a.parts == 1)  // (else the rows have been initialised: several blocks add to one)
     for (u32 i = threadIdx.x; i < cells; i += blockDim.x) row[i] = (i % kCell == 2) ? ~0ull : 0ull;
-    argus_fuse_init(ctab, R, threadIdx.x, blockDim.x);
-    __threadfence();
-    __syncthreads();
-    ArgusFuseCtx fx;
-    fx.tab = ctab; fx.row = row;
-    const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
-    const int sel = stream_in_scope(a, s);
-    if (sel == 2 && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, a.cta_sm[s / a.warps_per_cta]);
-    if (hi < lo || hi > a.interval_limit) {
-      if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
-    } else if (sel == 1) {
-      for (u64 i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
-        const uint4 q0 = __ldg(p), q1 = __ldg(p + 1), q2 = __ldg(p + 2);
-        const u32 region = q1.z;
-        if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
-        if (!record_in_scope(a, q1.w, region)) continue;
-        const u64 incl = (u64)q0.z | ((u64)q0.w << 32), excl = (u64)q1.x | ((u64)q1.y << 32);
-        argus_fuse_aggregate(fx, region, incl, excl, q2.w >> 16);
-        if (a.iter_inline) agg_add_interval_lean(iter_base + (u64)(q1.w - a.ctx_lo) * cells, region, incl, excl, q2.w >> 16);
-      }
+  argus_fuse_init(ctab, R, threadIdx.x, blockDim.x);
+  if (threadIdx.x == 0) { range[0] = ~0ull; range[1] = 0; }
+  __threadfence();
+  __syncthreads();
+  ArgusFuseCtx fx;
+  fx.tab = ctab; fx.row = row;
+  u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
+  const int sel = stream_in_scope(a, s);
+  if (sel == 2 && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, a.cta_sm[s / a.warps_per_cta]);
+  if (hi < lo || hi > a.interval_limit) {
+    if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
+  } else if (sel == 1) {
+    if (a.parts > 1) {
+      const u64 per = (hi - lo + a.parts - 1) / a.parts;
+      const u64 from = lo + per * part;
+      lo = from < hi ? from : hi;
+      hi = lo + per < hi ? lo + per : hi;
     }
-    if (a.ambig && a.ambig_offsets && sel == 1) {
-      const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
-      for (u64 i = alo + threadIdx.x; i < ahi && ahi >= alo; i += blockDim.x) {
-        const u32 region = a.ambig[i].tag >> 1;
-        if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
-        if (!record_in_scope(a, a.ambig[i].ctx, region)) continue;
-        const u32 which = a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5;
-        atomicAdd(row + (size_t)region * kCell + which, 1ull);
-        if (a.iter_inline) atomicAdd(iter_base + ((u64)(a.ambig[i].ctx - a.ctx_lo) * R + region) * kCell + which, 1ull);
-      }
+    u64 first = ~0ull, last = 0;
+    for (u64 i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+      const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
+      const uint4 q0 = __ldg(p), q1 = __ldg(p + 1), q2 = __ldg(p + 2);
+      const u32 region = q1.z;
+      if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
+      if (!record_in_scope(a, q1.w, region)) continue;
+      const u64 incl = (u64)q0.z | ((u64)q0.w << 32), excl = (u64)q1.x | ((u64)q1.y << 32);
+      argus_fuse_aggregate(fx, region, incl, excl, q2.w >> 16);
+      if (first == ~0ull) first = i;
+      last = i + 1;
     }
-    __syncthreads();
-    argus_fuse_flush(ctab, row, R, threadIdx.x, blockDim.x);
-    __syncthreads();
+    if (a.ranges && last) { atomicMin(&range[0], first); atomicMax(&range[1], last); }
   }
+  if (a.ambig && a.ambig_offsets && sel == 1 && part == 0) {
+    const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
+    for (u64 i = alo + threadIdx.x; i < ahi && ahi >= alo; i += blockDim.x) {
+      const u32 region = a.ambig[i].tag >> 1;
+      if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
+      if (!record_in_scope(a, a.ambig[i].ctx, region)) continue;
+      atomicAdd(row + (size_t)region * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
+    }
+  }
+  __syncthreads();
+  if (a.ranges && threadIdx.x == 0) a.ranges[blockIdx.x] = make_ulonglong2(range[0], range[1]);
+  argus_fuse_flush(ctab, row, R, threadIdx.x, blockDim.x);
 }
 
 // ---- the pass over the intervals' 8-byte digests (what argus_synthesize's pairing wrote beside the records) ----
@@ -506,63 +497,148 @@ __global__ void __launch_bounds__(256) k_agg_init(u64* tab, u64 n) {
     tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
 }
 
-// CTA cells = reduction over the warps of each CTA (written if asked for), added to the SM-scope and kernel-scope cells (atomic
-// add / min / max on integers). Bound by the read of the warp-scope table; eight warps' words are asked for at a time.
+// One word of the cells of kGroup CTAs: CTA cells = reduction over the warps of each (written if asked for), warp-role cells over
+// the CTAs; CTA cells go to the SM-scope cells, their reduction over the group to the kernel-scope cells (atomic add / min / max
+// on integers; empty words add nothing). Bound by the one read of the warp-scope table, of which a thread has kGroup words in
+// flight: 64 us for 275 MB; 77 us a CTA a thread, and 288 us more for the roles by themselves.
+__device__ __forceinline__ void cell_add(u64* d, u32 field, u64 v) {
+  if (field == 2 ? v == ~0ull : v == 0ull) return;  // identity element: nothing to add
+  if (field == 2) atomicMin(d, v); else if (field == 3) atomicMax(d, v); else atomicAdd(d, v);
+}
+template <u32 kGroup>
 __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
   argus_kernel_begin_long();
-  const u64 per_cta = (u64)a.num_regions * kCell, n = (u64)a.num_ctas * per_cta;
+  const u64 per_cta = (u64)a.num_regions * kCell, n = (u64)((a.num_ctas + kGroup - 1) / kGroup) * per_cta;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-    const u64 c = i / per_cta, rem = i % per_cta;
+    const u32 c0 = (u32)(i / per_cta) * kGroup, have = a.num_ctas - c0 < kGroup ? a.num_ctas - c0 : kGroup;
+    const u64 rem = i % per_cta;
     const u32 field = (u32)(rem % kCell);
-    const u64* src = a.warp_tab + c * a.warps_per_cta * per_cta + rem;
-    u64 v = src[0];
-#pragma unroll 8
-    for (u32 w = 1; w < a.warps_per_cta; ++w) v = combine(field, v, src[(u64)w * per_cta]);
-    if (cta_out) cta_out[i] = v;
-    if (field == 2 ? v == ~0ull : v == 0ull) continue;  // identity element: nothing to add
-    if (a.sm_tab) {
-      const u32 m = a.cta_sm[c];
-      if (m >= a.num_sms) { argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, (u32)c, m); continue; }
-      u64* d = a.sm_tab + (u64)m * per_cta + rem;
-      if (field == 2) atomicMin(d, v); else if (field == 3) atomicMax(d, v); else atomicAdd(d, v);
+    const u64 none = field == 2 ? ~0ull : 0ull;
+    const u64* src = a.warp_tab + (u64)c0 * a.warps_per_cta * per_cta + rem;
+    u64 v[kGroup];
+#pragma unroll
+    for (u32 q = 0; q < kGroup; ++q) v[q] = none;
+#pragma unroll kGroup == 1 ? 8 : 2
+    for (u32 w = 0; w < a.warps_per_cta; ++w) {
+      u64 x[kGroup];
+#pragma unroll
+      for (u32 q = 0; q < kGroup; ++q) x[q] = q < have ? src[((u64)q * a.warps_per_cta + w) * per_cta] : none;
+      u64 all = none;
+#pragma unroll
+      for (u32 q = 0; q < kGroup; ++q) { v[q] = combine(field, v[q], x[q]); all = combine(field, all, x[q]); }
+      if (a.role_tab) cell_add(a.role_tab + w * per_cta + rem, field, all);
     }
-    if (a.kernel_tab) {
-      u64* d = a.kernel_tab + rem;
-      if (field == 2) atomicMin(d, v); else if (field == 3) atomicMax(d, v); else atomicAdd(d, v);
+    u64 all = none;
+#pragma unroll
+    for (u32 q = 0; q < kGroup; ++q) {
+      if (q >= have) break;
+      all = combine(field, all, v[q]);
+      if (cta_out) cta_out[(u64)(c0 + q) * per_cta + rem] = v[q];
+      if (a.sm_tab && v[q] != none) {
+        const u32 m = a.cta_sm[c0 + q];
+        if (m >= a.num_sms) { argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, c0 + q, m); continue; }
+        cell_add(a.sm_tab + (u64)m * per_cta + rem, field, v[q]);
+      }
     }
+    if (a.kernel_tab) cell_add(a.kernel_tab + rem, field, all);
   }
 }
 
-// role_tab[w][r][j] = reduce over c of warp_tab[c*W + w][r][j]
-__global__ void __launch_bounds__(256) k_agg_role(AggArgs a) {
+// iter_tab[ctx - ctx_lo][r] with the compact cells. A block walks a few streams side by side (kIterWarps warps, shared out
+// among them) and holds the cells of two neighbouring iterations in shared memory; a warp that comes to a later one waits until
+// all have, then the older cells are added to the table. (38 M intervals in 16 iterations of 202 regions: 551 us.) Iterations come in order in a stream, so each is gathered once for all of
+// the block's streams, where an atomic on the table for every field of an interval took
+// 2.0 ms for 38 M of them. An interval of an earlier iteration than the two is added to the table directly. Only the part of a
+// stream that the pass before found to be in the window is read.
+__global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u32 streams_per_block) {
   argus_kernel_begin_long();
-  const u64 per_row = (u64)a.num_regions * kCell;
-  const u64 n = (u64)a.warps_per_cta * per_row;
-  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-    const u64 w = i / per_row, rem = i % per_row;
-    const u32 field = (u32)(rem % kCell);
-    const u64* src = a.warp_tab + w * per_row + rem;
-    u64 acc = src[0];
-    for (u32 c = 1; c < a.num_ctas; ++c) acc = combine(field, acc, src[(u64)c * a.warps_per_cta * per_row]);
-    a.role_tab[i] = acc;
+  extern __shared__ __align__(16) unsigned char sh_raw[];
+  __shared__ u32 need;
+  const u32 R = a.num_regions, cells = R * kCell, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  ArgusAggCell* const tab0 = reinterpret_cast<ArgusAggCell*>(sh_raw);
+  ArgusAggCell* const tab1 = tab0 + R;
+  constexpr u32 kNone = 0xffffffffu;
+  const u32 m = kIterWarps / streams_per_block;  // warps of a stream
+  const u32 s = blockIdx.x * streams_per_block + warp / m, mine = warp % m;
+  u64 lo = ~0ull, hi = 0;
+  if (s < a.num_streams && stream_in_scope(a, s) == 1) {  // (a bad cta_sm entry has been reported)
+    for (u32 q = 0; q < a.parts; ++q) {
+      const ulonglong2 r = a.ranges[(u64)s * a.parts + q];
+      lo = r.x < lo ? r.x : lo;
+      hi = r.y > hi ? r.y : hi;
+    }
+    if (mine == 0 && a.ambig && a.ambig_offsets) {
+      const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
+      for (u64 i = alo + lane; i < ahi && ahi >= alo; i += 32) {
+        const u32 region = a.ambig[i].tag >> 1, ctx = a.ambig[i].ctx;
+        if (region >= R || !record_in_scope(a, ctx, region)) continue;
+        atomicAdd(a.iter_tab + ((u64)(ctx - a.ctx_lo) * R + region) * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
+      }
+    }
   }
-}
-
-// iter_tab[ctx - ctx_lo][r]: selected intervals and ambiguity records keyed by iteration. A block gathers its
-// streams in a shared-memory copy of the table when that fits and adds the non-empty cells to the global
-// table (initialised by k_agg_init) at the end; otherwise it updates the global table record by record.
-__global__ void __launch_bounds__(kAggThreads) k_agg_iter(AggArgs a) {
-  argus_kernel_begin_long();
-  extern __shared__ __align__(16) u64 sh_tab[];
-  const u32 R = a.num_regions;
-  const u64 cells = (u64)a.num_iters * R * kCell;
-  // too large for shared memory: blocks add to one of a few private copies in global memory, which spreads the
-  // atomics over more addresses; k_agg_iter_reduce combines the copies afterwards
-  u64* tab = a.iter_smem ? sh_tab : a.iter_copies ? a.iter_copies + (u64)(blockIdx.x % a.num_copies) * cells : a.iter_tab;
-  if (a.iter_smem) {
-    for (u64 i = threadIdx.x; i < cells; i += blockDim.x) sh_tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
+  argus_fuse_init(tab0, 2 * R, threadIdx.x, kIterThreads);
+  if (threadIdx.x == 0) need = kNone;
+  __syncthreads();
+  u64 at = lo < hi ? lo + mine * 32 : ~0ull;
+  const u64 end = lo < hi ? hi : 0ull;
+  u32 cur = 0;         // the two iterations at hand: cur (in table `odd`) and cur + 1
+  u32 odd = 0, want = kNone;
+  bool fresh = true;   // the round at `at` has not been loaded
+  uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
+  u32 flags = 0;
+  for (;;) {
+    // take what belongs to the two iterations
+    while (at < end) {
+      if (fresh) {
+        const u64 i = at + lane;
+        want = kNone;
+        if (i < end) {
+          const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
+          q0 = __ldg(p); q1 = __ldg(p + 1);
+          flags = __ldg(reinterpret_cast<const u32*>(p + 2) + 3) >> 16;
+          if (q1.z < R && record_in_scope(a, q1.w, q1.z)) want = q1.w - a.ctx_lo;
+        }
+        fresh = false;
+      }
+      if (want != kNone && want <= cur + 1) {
+        const u64 incl = (u64)q0.z | ((u64)q0.w << 32), excl = (u64)q1.x | ((u64)q1.y << 32);
+        u64* const row = a.iter_tab + (u64)want * cells;
+        if (want < cur) {
+          agg_add_interval(row, q1.z, incl, excl, flags);
+        } else {
+          ArgusFuseCtx fx;
+          fx.tab = ((want - cur) ^ odd) ? tab1 : tab0;
+          fx.row = row;
+          argus_fuse_aggregate(fx, q1.z, incl, excl, flags);
+        }
+        want = kNone;
+      }
+      if (__any_sync(0xffffffffu, want != kNone)) break;
+      at += (u64)m * 32;
+      fresh = true;
+    }
+    const u32 least = __reduce_min_sync(0xffffffffu, at < end ? want : kNone);
+    if (lane == 0 && least != kNone) atomicMin(&need, least);
+    __syncthreads();
+    const u32 next = need;
+    __syncthreads();
+    if (threadIdx.x == 0) need = kNone;
+    ArgusAggCell* const older = odd ? tab1 : tab0;
+    argus_fuse_flush(older, a.iter_tab + (u64)cur * cells, R, threadIdx.x, kIterThreads);
+    if (next != cur + 2 && cur + 1 < a.num_iters) argus_fuse_flush(odd ? tab0 : tab1, a.iter_tab + (u64)(cur + 1) * cells, R, threadIdx.x, kIterThreads);
+    if (next == kNone) return;
+    __syncthreads();
+    argus_fuse_init(older, R, threadIdx.x, kIterThreads);
+    if (next != cur + 2) argus_fuse_init(odd ? tab0 : tab1, R, threadIdx.x, kIterThreads);
+    if (next == cur + 2) { cur += 1; odd ^= 1; } else { cur = next; }
     __syncthreads();
   }
+}
+
+// The same for more regions than the compact cells are kept for: every interval straight into the table.
+__global__ void __launch_bounds__(kAggThreads) k_agg_iter(AggArgs a) {
+  argus_kernel_begin_long();
+  const u32 R = a.num_regions;
   for (u32 s = blockIdx.x; s < a.num_streams; s += gridDim.x) {
     if (stream_in_scope(a, s) != 1) continue;  // a bad cta_sm entry is reported by k_agg_streams
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
@@ -572,66 +648,28 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_iter(AggArgs a) {
       const u32 region = q1.z, ctx = q1.w;
       if (region >= R || !record_in_scope(a, ctx, region)) continue;
       const uint4 q0 = __ldg(p), q2 = __ldg(p + 2);
-      u64* row = tab + (u64)(ctx - a.ctx_lo) * R * kCell;
-      const u64 incl = (u64)q0.z | ((u64)q0.w << 32), excl = (u64)q1.x | ((u64)q1.y << 32);
-      if (a.iter_smem) agg_add_interval(row, region, incl, excl, q2.w >> 16);
-      else agg_add_interval_lean(row, region, incl, excl, q2.w >> 16);
+      agg_add_interval(a.iter_tab + (u64)(ctx - a.ctx_lo) * R * kCell, region, (u64)q0.z | ((u64)q0.w << 32), (u64)q1.x | ((u64)q1.y << 32), q2.w >> 16);
     }
     if (a.ambig && a.ambig_offsets) {
       const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
       for (u64 i = alo + threadIdx.x; i < ahi && ahi >= alo; i += blockDim.x) {
         const u32 region = a.ambig[i].tag >> 1, ctx = a.ambig[i].ctx;
         if (region >= R || !record_in_scope(a, ctx, region)) continue;
-        atomicAdd(tab + ((u64)(ctx - a.ctx_lo) * R + region) * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
+        atomicAdd(a.iter_tab + ((u64)(ctx - a.ctx_lo) * R + region) * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
       }
     }
   }
-  if (a.iter_smem) {
-    __syncthreads();
-    for (u64 i = threadIdx.x; i < cells; i += blockDim.x) {
-      const u32 field = (u32)(i % kCell);
-      const u64 v = sh_tab[i];
-      if (field == 2 ? v == ~0ull : v == 0ull) continue;
-      u64* d = a.iter_tab + i;
-      if (field == 2) atomicMin(d, v); else if (field == 3) atomicMax(d, v); else atomicAdd(d, v);
-    }
-  }
 }
 
-// iter_tab[i] = combination of cell word i over the private copies (none: iter_tab holds the sums already);
-// the interval count of a cell, which the global path leaves out, is the sum of its histogram bins.
-__global__ void __launch_bounds__(256) k_agg_iter_reduce(AggArgs a) {
-  argus_kernel_begin();
-  const u64 cells = (u64)a.num_iters * a.num_regions * kCell;
-  if (a.iter_copies) {
-    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < cells; i += (u64)gridDim.x * blockDim.x) {
-      const u32 field = (u32)(i % kCell);
-      if (field == 0) continue;
-      u64 acc = a.iter_copies[i];
-      for (u32 c = 1; c < a.num_copies; ++c) acc = combine(field, acc, a.iter_copies[(u64)c * cells + i]);
-      a.iter_tab[i] = acc;
-    }
-  }
-  for (u64 cell = (u64)blockIdx.x * blockDim.x + threadIdx.x; cell < cells / kCell; cell += (u64)gridDim.x * blockDim.x) {
-    u64 n = 0;
-    for (u32 b = 0; b < 64; ++b) {
-      u64 v = 0;
-      if (a.iter_copies) for (u32 c = 0; c < a.num_copies; ++c) v += a.iter_copies[(u64)c * cells + cell * kCell + 8 + b];
-      else v = a.iter_tab[cell * kCell + 8 + b];
-      n += v;
-    }
-    a.iter_tab[cell * kCell] = n;
-  }
-}
-
-struct AggLayout { size_t warp, iter, total; };
+struct AggLayout { size_t warp, ranges, total; };
 
 AggLayout agg_layout(uint32_t num_streams, uint32_t num_regions) {
   AggLayout L;
   const size_t row = (size_t)num_regions * sizeof(argus_agg_t);
   L.warp = 0;
-  L.iter = argus_align_up((size_t)num_streams * row, 256);
-  L.total = L.iter + kIterScratchBytes;
+  L.ranges = argus_align_up((size_t)num_streams * row, 256);
+  L.total = L.ranges + argus_align_up((size_t)num_streams * kMaxParts * sizeof(ulonglong2), 256);
+  if (L.total < 2 * L.ranges) L.total = 2 * L.ranges;  // two tables of the warp scope's size have always fitted
   return L;
 }
 
@@ -688,24 +726,17 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   a.parts = digest_parts; a.interval_limit = interval_limit;
   const size_t smem = (size_t)num_regions * sizeof(argus_agg_t);
   a.use_smem = smem <= kAggSmemLimit;
-  const size_t iter_bytes = (size_t)num_iters * smem;
-  a.iter_smem = iter_tab && iter_bytes <= kAggSmemLimit;
-  a.iter_copies = nullptr; a.num_copies = 0;
-  if (iter_tab && !a.iter_smem && 2 * iter_bytes <= kIterScratchBytes) {
-    a.num_copies = (u32)(kIterScratchBytes / iter_bytes < kIterMaxCopies ? kIterScratchBytes / iter_bytes : kIterMaxCopies);
-    a.iter_copies = (u64*)((char*)workspace + L.iter);
-  }
-  const size_t need = a.use_smem ? smem : 0, need_iter = a.iter_smem ? iter_bytes : 0;
+  const size_t need = a.use_smem ? smem : 0;
   if (need > 48 * 1024)
     ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
-  if (need_iter > 48 * 1024)
-    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_iter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_iter));
-  const u64 iter_cells = (u64)num_iters * num_regions * kCell;
-  a.iter_inline = iter_tab && !a.iter_smem && num_regions <= kAggCompactRegions;
-  if (iter_tab) {
-    if (a.iter_copies) ARGUS_LAUNCH(k_agg_init, 592, 256, 0, stream, a.iter_copies, iter_cells * a.num_copies);
-    else ARGUS_LAUNCH(k_agg_init, 296, 256, 0, stream, (u64*)iter_tab, iter_cells);
+  const bool windows = iter_tab && num_regions <= kAggCompactRegions;
+  a.ranges = windows ? (ulonglong2*)((char*)workspace + L.ranges) : nullptr;
+  if (!a.digest) {  // few streams: several blocks share one (how many intervals there are is not known here)
+    const u32 room = 888 / num_streams;
+    a.parts = num_regions > kAggCompactRegions || room < 1 ? 1 : room < kMaxParts ? room : kMaxParts;
   }
+  if (num_regions <= kAggCompactRegions && a.parts > 1)
+    ARGUS_LAUNCH(k_agg_init, 592, 256, 0, stream, a.warp_tab, (u64)num_streams * num_regions * kCell);
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 0);
   if (num_regions <= kAggCompactRegions) {
     const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell);
@@ -715,30 +746,31 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       const size_t dg = digest_table_words(num_regions) * 4 + ((num_regions + 31) / 32) * 4;
       if (dg > 48 * 1024)
         ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_digest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
-      if (a.parts > 1) ARGUS_LAUNCH(k_agg_init, 592, 256, 0, stream, a.warp_tab, (u64)num_streams * num_regions * kCell);
       ARGUS_LAUNCH(k_agg_streams_digest, num_streams * a.parts, kDgThreads, dg, stream, a);
     } else {
-      ARGUS_LAUNCH(k_agg_streams_compact, num_streams, kAggThreads, compact, stream, a);
+      ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
     }
   } else {
     ARGUS_LAUNCH(k_agg_streams, num_streams, kAggThreads, need, stream, a);
   }
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 1);
-  if (iter_tab) {
-    if (!a.iter_inline) {
-      const unsigned iter_grid = a.iter_smem ? 296u : 148u * 8u;
-      ARGUS_LAUNCH(k_agg_iter, num_streams < iter_grid ? num_streams : iter_grid, kAggThreads, need_iter, stream, a);
-    }
-    if (!a.iter_smem) {
-      ARGUS_LAUNCH(k_agg_iter_reduce, 296, 256, 0, stream, a);
-    }
+  if (iter_tab && windows) {
+    u32 per = kIterWarps;  // streams of a block: at least two blocks for every SM where the streams allow it
+    while (per > 1 && num_streams / per < 296) per >>= 1;
+    const size_t two = 2 * (size_t)num_regions * sizeof(ArgusAggCell);
+    if (two > 48 * 1024)
+      ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_iter_windows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)two));
+    ARGUS_LAUNCH(k_agg_iter_windows, (num_streams + per - 1) / per, kIterThreads, two, stream, a, per);
+  } else if (iter_tab) {
+    ARGUS_LAUNCH(k_agg_iter, num_streams < 1184u ? num_streams : 1184u, kAggThreads, 0, stream, a);
   }
-  if (role_tab) {
-    ARGUS_LAUNCH(k_agg_role, 296, 256, 0, stream, a);
-  }
-  if (cta_tab || sm_tab || kernel_tab) {
-    const u64 want = ((u64)a.num_ctas * num_regions * kCell + 255) / 256;
-    ARGUS_LAUNCH(k_agg_rollup, (unsigned)(want < 2368 ? want : 2368), 256, 0, stream, a, (u64*)cta_tab);
+  if (cta_tab || sm_tab || kernel_tab || role_tab) {
+    // groups of CTAs where that leaves enough threads to fill the chip (148 x 2,048)
+    const u64 words = (u64)num_regions * kCell, groups = ((u64)a.num_ctas + 7) / 8;
+    if (groups * words >= 148 * 1024)
+      ARGUS_LAUNCH(k_agg_rollup<8>, (unsigned)((groups * words + 255) / 256 < 4736 ? (groups * words + 255) / 256 : 4736), 256, 0, stream, a, (u64*)cta_tab);
+    else
+      ARGUS_LAUNCH(k_agg_rollup<1>, (unsigned)((a.num_ctas * words + 255) / 256 < 4736 ? (a.num_ctas * words + 255) / 256 : 4736), 256, 0, stream, a, (u64*)cta_tab);
   }
   return ARGUS_OK;
 }

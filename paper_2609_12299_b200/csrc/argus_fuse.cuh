@@ -135,28 +135,30 @@ __device__ __forceinline__ void argus_fuse_aggregate(const ArgusFuseCtx& fx, u32
   argus_fuse_agg_rest(c, fx.row, region, incl, flags);
 }
 
+// Adds the cells to a global row, which may hold something already (bins outside the windows, ambiguity counters, what other
+// blocks have added).
 __device__ __forceinline__ void argus_fuse_flush(const ArgusAggCell* tab, u64* row, u32 num_regions, u32 tid, u32 nthreads) {
-  constexpr u32 kItems = 8 + kAggWindow;
+  constexpr u32 kItems = 6 + kAggWindow;
   for (u32 i = tid; i < num_regions * kItems; i += nthreads) {
     const u32 r = i / kItems, f = i % kItems;
     const ArgusAggCell& c = tab[r];
+    if (c.hbase == kAggUnset) continue;  // the first interval of a region chooses its window
     u64* cell = row + (size_t)r * kAggCellWords;
     switch (f) {
       case 0: {
         u64 n = c.count_out;
 #pragma unroll
         for (u32 j = 0; j < kAggWindow; ++j) n += c.h[j];
-        cell[0] = n;
+        atomicAdd(cell + 0, n);
         break;
       }
-      case 1: cell[1] = c.sum_incl; break;
-      case 2: cell[2] = c.min_incl; break;
-      case 3: cell[3] = c.max_incl; break;
-      case 4: cell[4] = c.sum_excl; break;
-      case 5: case 6: break;  // ambiguity counters are added later from the ambiguity records
-      case 7: cell[7] = c.nflag; break;
+      case 1: atomicAdd(cell + 1, c.sum_incl); break;
+      case 2: atomicMin(cell + 2, c.min_incl); break;
+      case 3: atomicMax(cell + 3, c.max_incl); break;
+      case 4: atomicAdd(cell + 4, c.sum_excl); break;
+      case 5: if (c.nflag) atomicAdd(cell + 7, (u64)c.nflag); break;
       default: {
-        const u32 j = f - 8;
+        const u32 j = f - 6;
         if (c.h[j]) atomicAdd(cell + 8 + c.hbase + j, (u64)c.h[j]);
       }
     }

@@ -532,13 +532,13 @@ __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
 #pragma unroll
     for (u32 q = 0; q < kGroup; ++q) {
       if (q >= have) break;
-      all = combine(field, all, v[q]);
       if (cta_out) cta_out[(u64)(c0 + q) * per_cta + rem] = v[q];
       if (a.sm_tab && v[q] != none) {
         const u32 m = a.cta_sm[c0 + q];
         if (m >= a.num_sms) { argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, c0 + q, m); continue; }
         cell_add(a.sm_tab + (u64)m * per_cta + rem, field, v[q]);
       }
+      all = combine(field, all, v[q]);
     }
     if (a.kernel_tab) cell_add(a.kernel_tab + rem, field, all);
   }
@@ -546,9 +546,9 @@ __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
 
 // iter_tab[ctx - ctx_lo][r] with the compact cells. A block walks a few streams side by side (kIterWarps warps, shared out
 // among them) and holds the cells of two neighbouring iterations in shared memory; a warp that comes to a later one waits until
-// all have, then the older cells are added to the table. (38 M intervals in 16 iterations of 202 regions: 551 us.) Iterations come in order in a stream, so each is gathered once for all of
-// the block's streams, where an atomic on the table for every field of an interval took
-// 2.0 ms for 38 M of them. An interval of an earlier iteration than the two is added to the table directly. Only the part of a
+// all have, then the older cells are added to the table. Iterations come in order in a stream, so each is gathered once for
+// all of the block's streams: 551 us for 38 M intervals in 16 iterations of 202 regions, where atomics on the table for every
+// interval took 2.0 ms. An interval of an earlier iteration than the two is added to the table directly. Only the part of a
 // stream that the pass before found to be in the window is read.
 __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u32 streams_per_block) {
   argus_kernel_begin_long();

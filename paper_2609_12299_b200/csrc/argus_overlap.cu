@@ -453,7 +453,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
   }
   __syncthreads();
   // (a capacity error that another block of this launch reports is not waited for: such a block has no room itself or is done)
-  if (sh_u != 0) return;
+  if (sh_u != 0) {  // nothing measured: zeros
+    if (tid == 0) a.out[blockIdx.x] = argus_overlap_t{};
+    return;
+  }
 
   // ---- gather: round 0 counts, round 1 places, in stream and slice order ----
   // With one pair every entry is in a role of it, and round 0 only adds up the pieces.
@@ -630,7 +633,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
         }
       }
       base = sh64[0];
-      if (base + sh64[1] > a.capacity) return;
+      if (base + sh64[1] > a.capacity) {
+        if (tid == 0) a.out[blockIdx.x] = argus_overlap_t{};
+        return;
+      }
       if (sh64[1] == 0) break;
     }
   }

@@ -55,3 +55,23 @@ def test_overlap_sizes_and_orders(order, per_stream):
             out, st = argus.argus_overlap(d_iv, len(iv), d_off, W, d_sm, M, d_pairs, workspace_bytes=ws)
             assert int(argus.argus_status_fetch(st)["code"]) == 0
             assert out.cpu().numpy().view(argus.OVERLAP_DTYPE).reshape(want.shape).tobytes() == want.tobytes()
+
+
+def test_sm_index_out_of_range_leaves_zeros_and_the_other_tables():
+    """A CTA mapped to an SM that does not exist: the call reports it; the overlap is all zeros, and the tables hold every other
+    CTA's intervals."""
+    spec_sm = np.array([0, 1, 2], np.uint32)      # num_sms = 2
+    S, W, R = 6, 2, 3
+    ev = np.zeros((S, 4), argus.EVENT_DTYPE)
+    ev["ts"] = np.arange(4) * 10
+    ev["tag"] = [0, 2, 3, 1]
+    offs = (np.arange(S + 1) * 4).astype(np.uint64)
+    d_ev = torch.from_numpy(ev.reshape(-1).view(np.uint8).copy()).to(DEV)
+    d_off = torch.from_numpy(offs.view(np.int64).copy()).to(DEV)
+    d_pairs = torch.tensor([[0, 1]], dtype=torch.int32, device=DEV)
+    r = argus.argus_synthesize(d_ev, d_off, R, W, torch.from_numpy(spec_sm.view(np.int32)).to(DEV), 2, d_pairs)
+    st = r.fetch_status()
+    assert int(st["code"]) == 1
+    assert not r.overlap.cpu().numpy().any()
+    assert int(r.agg.table_numpy("cta")["count"].sum()) == 12
+    assert int(r.agg.table_numpy("sm")["count"].sum()) == int(r.agg.table_numpy("kernel")["count"].sum()) == 8

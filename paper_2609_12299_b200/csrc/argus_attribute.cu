@@ -3,125 +3,153 @@
 //   k_map_counts   : exec records of a mapping-run trace arrive as intervals of the extra region id R whose
 //                    parent_region is the innermost active region (pairing did the stack work); this pass adds
 //                    their execution counts into counts[owner][pc] (integer atomics: order does not matter).
-//   k_attr_columns : one thread per PC: column total, alpha, entropy;
-//   k_attr_rows    : one block per (row, chunk of PCs): the lifted metric summed in a fixed order;
-//   k_attr_finish  : mhat[row] = sum of the chunk partials, in chunk order.
+//   k_attr_tile    : one block per 32 PCs and all rows: column totals, alpha, entropy, and the block's share of the lifted
+//                    metric of every row;
+//   k_attr_finish  : mhat[row] = sum of the blocks' shares, in a fixed order.
 #include "argus_common.cuh"
 
 namespace {
 
 constexpr int kAttrThreads = 256;
-constexpr u32 kAttrChunk = 8192;      // PCs one block of the row pass covers
+constexpr u32 kAttrWarps = kAttrThreads / 32;
+constexpr u32 kAttrRows = 400;        // rows of 32 counts a block keeps in shared memory (100 KB)
 constexpr u32 kMapSlots = 2048;       // shared-memory cache of (owner, pc) cells per block
 constexpr u32 kMapEmpty = 0xffffffffu;
-
-// 64-bit add as native 32-bit shared atomics; each carry is propagated exactly once
-__device__ __forceinline__ void shared_add64(u64* p64, u64 v) {
-  u32* p = reinterpret_cast<u32*>(p64);
-  const u32 lo = (u32)v, hi = (u32)(v >> 32);
-  if (lo) {
-    const u32 old = atomicAdd(p, lo);
-    if (old + lo < old) atomicAdd(p + 1, 1u);
-  }
-  if (hi) atomicAdd(p + 1, hi);
-}
+constexpr u32 kMapSmall = 1u << 12;   // executions a cache slot takes at a time ...
+constexpr u32 kMapFlush = 1u << 19;   // ... and records after which the cache is emptied: their product stays below 2^32
 
 // A mapping run touches few of the (R + 1) x P cells and touches them very often, so each block gathers
-// its additions in a small direct-mapped table in shared memory (cell index -> sum) and adds the table
-// to the global counts at the end; a cell whose slot is taken by another cell goes to the global counts directly.
+// its additions in a small direct-mapped table in shared memory (cell index -> 32-bit sum) and adds the table
+// to the global counts at the end; a cell whose slot is taken by another cell, or a count of kMapSmall and more, goes to the
+// global counts directly. A slot's key is looked at before it is claimed and the add returns nothing: a warp's lanes hit few
+// cells, and what they do to one is done one lane after the other. 57.6 M intervals, 808 cells: 682 us with a compare-and-swap
+// and a returning 64-bit add per record, 433 us this way (6.4 TB/s of records).
 __global__ void __launch_bounds__(256) k_map_counts(const argus_interval_t* intervals, const u64* interval_offsets,
                                                     u32 num_streams, u32 exec_region, u32 num_pcs, u64* counts,
                                                     argus_status_t* status, int use_cache) {
   argus_kernel_begin_long();
   __shared__ u32 keys[kMapSlots];
-  __shared__ u64 sums[kMapSlots];
+  __shared__ u32 sums[kMapSlots];
   for (u32 i = threadIdx.x; i < kMapSlots; i += blockDim.x) { keys[i] = kMapEmpty; sums[i] = 0; }
   __syncthreads();
   const u64 lo = interval_offsets[0], hi = interval_offsets[num_streams];
-  for (u64 i = lo + (u64)blockIdx.x * blockDim.x + threadIdx.x; i < hi; i += (u64)gridDim.x * blockDim.x) {
-    const uint4* p = reinterpret_cast<const uint4*>(intervals + i);
-    const uint4 q1 = __ldg(p + 1);
-    if (q1.z != exec_region) continue;
-    const u32 pc = q1.w;
-    if (pc >= num_pcs) { argus_set_error(status, ARGUS_ERR_INVALID_ARG, 0, i); continue; }
-    const uint4 q0 = __ldg(p), q2 = __ldg(p + 2);
-    const u64 k = (u64)q0.z | ((u64)q0.w << 32);
-    if (!k) continue;
-    const u32 owner = q2.y < exec_region ? q2.y : exec_region;  // no parent, or a malformed nesting of exec records
-    const u64 cell = (u64)owner * num_pcs + pc;
-    if (use_cache) {
-      const u32 key = (u32)cell;
-      const u32 slot = (key * 2654435761u) >> 21;  // 11 bits
-      const u32 old = atomicCAS(&keys[slot], kMapEmpty, key);
-      if (old == kMapEmpty || old == key) { shared_add64(&sums[slot], k); continue; }
+  u32 seen = 0;  // records of this block since the cache was emptied
+  for (u64 base = lo + (u64)blockIdx.x * blockDim.x; base < hi; base += (u64)gridDim.x * blockDim.x) {
+    const u64 i = base + threadIdx.x;
+    if (i < hi) {
+      const uint4* p = reinterpret_cast<const uint4*>(intervals + i);
+      const uint2 k2 = __ldg(reinterpret_cast<const uint2*>(p) + 1), rc = __ldg(reinterpret_cast<const uint2*>(p + 1) + 1);
+      const u32 parent = __ldg(reinterpret_cast<const u32*>(p + 2) + 1);
+      const u64 k = (u64)k2.x | ((u64)k2.y << 32);
+      const u32 pc = rc.y;
+      if (rc.x != exec_region) {
+      } else if (pc >= num_pcs) {
+        argus_set_error(status, ARGUS_ERR_INVALID_ARG, 0, i);
+      } else if (k) {
+        const u32 owner = parent < exec_region ? parent : exec_region;  // no parent, or a malformed nesting of exec records
+        const u64 cell = (u64)owner * num_pcs + pc;
+        bool cached = false;
+        if (use_cache && k < kMapSmall) {
+          const u32 key = (u32)cell;
+          const u32 slot = (key * 2654435761u) >> 21;  // 11 bits
+          u32 have = *reinterpret_cast<volatile u32*>(&keys[slot]);
+          if (have == kMapEmpty) { have = atomicCAS(&keys[slot], kMapEmpty, key); if (have == kMapEmpty) have = key; }
+          cached = have == key;
+          if (cached) atomicAdd(&sums[slot], (u32)k);
+        }
+        if (!cached) atomicAdd(counts + cell, k);
+      }
     }
-    atomicAdd(counts + cell, k);
+    seen += blockDim.x;
+    if (seen >= kMapFlush) {  // uniform
+      __syncthreads();
+      for (u32 j = threadIdx.x; j < kMapSlots; j += blockDim.x)
+        if (sums[j]) { atomicAdd(counts + keys[j], (u64)sums[j]); sums[j] = 0; }
+      seen = 0;
+      __syncthreads();
+    }
   }
   __syncthreads();
   for (u32 i = threadIdx.x; i < kMapSlots; i += blockDim.x)
-    if (keys[i] != kMapEmpty && sums[i]) atomicAdd(counts + keys[i], sums[i]);
+    if (sums[i]) atomicAdd(counts + keys[i], (u64)sums[i]);
 }
 
-// One thread per PC: column total (kept for the row pass), alpha, entropy.
-__global__ void __launch_bounds__(kAttrThreads) k_attr_columns(const u64* counts, u32 num_rows, u32 num_pcs,
-                                                               double* entropy, double* alpha, u64* totals) {
+// One lane per PC, rows shared out among the warps. The block's counts are read once and kept (kAttrRows rows at most, else read
+// again): bound by HBM, counts in and alpha out (203 rows x 70,560 PCs: 63 us with the sums, 222 us in three kernels that read the
+// counts three times). Sums over rows and over PCs are taken in an order that the shape alone fixes, so the
+// same bits come out every run.
+__global__ void __launch_bounds__(kAttrThreads) k_attr_tile(const u64* counts, u32 num_rows, u32 num_pcs, const double* metric,
+                                                            double* entropy, double* alpha, u32 num_blocks, double* partial) {
   argus_kernel_begin_long();
-  const u32 p = blockIdx.x * kAttrThreads + threadIdx.x;
-  if (p >= num_pcs) return;
+  extern __shared__ __align__(16) u64 held[];  // [num_rows][32]
+  __shared__ u64 total_of[kAttrWarps][32];
+  __shared__ double entropy_of[kAttrWarps][32];
+  const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+  const bool in = p < num_pcs, keep = num_rows <= kAttrRows;
   u64 total = 0;
-  for (u32 r = 0; r < num_rows; ++r) total += counts[(size_t)r * num_pcs + p];
-  totals[p] = total;
-  double h = 0.0;
-  for (u32 r = 0; r < num_rows; ++r) {
-    const u64 n = counts[(size_t)r * num_pcs + p];
-    const double a = (total == 0 || n == 0) ? 0.0 : (double)n / (double)total;
-    if (alpha) alpha[(size_t)r * num_pcs + p] = a;
-    if (a > 0.0) h -= a * log(a);
+#pragma unroll 8
+  for (u32 r = warp; r < num_rows; r += kAttrWarps) {
+    const u64 n = in ? __ldg(counts + (size_t)r * num_pcs + p) : 0ull;
+    if (keep) held[r * 32 + lane] = n;
+    total += n;
   }
-  entropy[p] = h;
+  total_of[warp][lane] = total;
+  __syncthreads();
+  total = 0;
+#pragma unroll
+  for (u32 w = 0; w < kAttrWarps; ++w) total += total_of[w][lane];
+  const double m = in ? metric[p] : 0.0;
+  double h = 0.0;
+#pragma unroll 4
+  for (u32 r = warp; r < num_rows; r += kAttrWarps) {
+    const u64 n = keep ? held[r * 32 + lane] : in ? __ldg(counts + (size_t)r * num_pcs + p) : 0ull;
+    const bool some = n != 0 && total != 0;
+    double a = 0.0, part = 0.0;
+    if (some) {
+      a = (double)n / (double)total;
+      if (a > 0.0) h -= a * log(a);
+      part = a * m;
+    }
+    if (alpha && in) __stcs(alpha + (size_t)r * num_pcs + p, a);
+    if (__any_sync(0xffffffffu, some)) {
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) part += __shfl_down_sync(0xffffffffu, part, d);
+    }
+    if (lane == 0) partial[(size_t)r * num_blocks + blockIdx.x] = part;
+  }
+  entropy_of[warp][lane] = h;
+  __syncthreads();
+  if (warp == 0 && in) {
+    h = 0.0;
+#pragma unroll
+    for (u32 w = 0; w < kAttrWarps; ++w) h += entropy_of[w][lane];
+    entropy[p] = h;
+  }
 }
 
-// Block (chunk c, row r): sum over the chunk's PCs of alpha * metric, every thread in index order, then the
-// threads by a fixed tree: the same bits every run.
-__global__ void __launch_bounds__(kAttrThreads) k_attr_rows(const u64* counts, const u64* totals, u32 num_rows, u32 num_pcs,
-                                                            const double* metric, u32 num_chunks, double* partial) {
-  argus_kernel_begin();
-  __shared__ double sh[kAttrThreads / 32];
-  const u32 r = blockIdx.y, c = blockIdx.x;
-  const u32 p0 = c * kAttrChunk, p1 = p0 + kAttrChunk < num_pcs ? p0 + kAttrChunk : num_pcs;
-  double acc = 0.0;
-  for (u32 p = p0 + threadIdx.x; p < p1; p += kAttrThreads) {
-    const u64 n = counts[(size_t)r * num_pcs + p], total = totals[p];
-    if (n && total) acc += ((double)n / (double)total) * metric[p];
-  }
+__global__ void __launch_bounds__(kAttrThreads) k_attr_finish(const double* partial, u32 num_blocks, double* mhat) {
+  argus_kernel_begin_long();
+  __shared__ double sh[kAttrWarps];
+  const u32 r = blockIdx.x;
+  double s = 0.0;
+  for (u32 b = threadIdx.x; b < num_blocks; b += kAttrThreads) s += partial[(size_t)r * num_blocks + b];
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < kAttrThreads / 32; ++w) s += sh[w];
-    partial[(size_t)r * num_chunks + c] = s;
+    s = 0.0;
+    for (u32 w = 0; w < kAttrWarps; ++w) s += sh[w];
+    mhat[r] = s;
   }
 }
 
-__global__ void __launch_bounds__(256) k_attr_finish(const double* partial, u32 num_chunks, u32 num_rows, double* mhat) {
-  argus_kernel_begin();
-  const u32 r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= num_rows) return;
-  double s = 0.0;
-  for (u32 c = 0; c < num_chunks; ++c) s += partial[(size_t)r * num_chunks + c];
-  mhat[r] = s;
-}
-
-struct AttrLayout { size_t totals, partial, total; u32 chunks; };
+struct AttrLayout { size_t total; u32 blocks; };
 
 AttrLayout attr_layout(uint32_t num_rows, uint32_t num_pcs) {
   AttrLayout L;
-  L.chunks = (num_pcs + kAttrChunk - 1) / kAttrChunk;
-  L.totals = 0;
-  L.partial = argus_align_up((size_t)num_pcs * 8, 256);
-  L.total = L.partial + argus_align_up((size_t)num_rows * L.chunks * 8 + 8, 256);
+  L.blocks = (num_pcs + 31) / 32;
+  L.total = argus_align_up((size_t)num_rows * L.blocks * 8 + 8, 256);
   return L;
 }
 
@@ -157,12 +185,12 @@ extern "C" int argus_attribute(const uint64_t* counts, uint32_t num_rows, uint32
   const AttrLayout L = attr_layout(num_rows, num_pcs);
   if (workspace_bytes < L.total) return ARGUS_ERR_WORKSPACE;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  u64* totals = (u64*)((char*)workspace + L.totals);
-  double* partial = (double*)((char*)workspace + L.partial);
-  ARGUS_LAUNCH(k_attr_columns, (num_pcs + kAttrThreads - 1) / kAttrThreads, kAttrThreads, 0, stream, (const u64*)counts, num_rows,
-               num_pcs, entropy, alpha, totals);
-  ARGUS_LAUNCH(k_attr_rows, dim3(L.chunks, num_rows), kAttrThreads, 0, stream, (const u64*)counts, totals, num_rows, num_pcs, metric,
-               L.chunks, partial);
-  ARGUS_LAUNCH(k_attr_finish, (num_rows + 255) / 256, 256, 0, stream, partial, L.chunks, num_rows, mhat);
+  double* partial = (double*)workspace;
+  const size_t smem = num_rows <= kAttrRows ? (size_t)num_rows * 32 * 8 : 0;
+  if (smem > 48 * 1024)
+    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_attr_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ARGUS_LAUNCH(k_attr_tile, L.blocks, kAttrThreads, smem, stream, (const u64*)counts, num_rows, num_pcs, metric, entropy, alpha, L.blocks,
+               partial);
+  ARGUS_LAUNCH(k_attr_finish, num_rows, kAttrThreads, 0, stream, (const double*)partial, L.blocks, mhat);
   return ARGUS_OK;
 }

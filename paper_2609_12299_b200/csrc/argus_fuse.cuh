@@ -75,6 +75,12 @@ __device__ __forceinline__ u64 argus_digest_pack(u32 region, u64 incl, u64 excl,
   return (u64)lo | ((u64)hi << 32);
 }
 
+// The same for durations that fit 32 bits, excl <= incl.
+__device__ __forceinline__ u64 argus_digest_pack32(u32 region, u32 incl, u32 excl, u32 flags) {
+  const u32 lo = region | (flags ? 1u << 16 : 0u) | (incl >> kDigestBits ? 1u << 17 : 0u) | (incl << 18);
+  return (u64)lo | ((u64)(((incl >> 14) & 0x1ffu) | (excl << 9)) << 32);
+}
+
 __device__ __forceinline__ u64 argus_entry_pack(u64 digest, u32 place) {
   if (((u32)digest & kDigestWide) || place >> (64 - kEntryIndexShift)) return ((u64)place << 18) | kDigestWide | ((u32)digest & 0xffffu);
   return (digest & ((1ull << kEntryIndexShift) - 1ull)) | ((u64)place << kEntryIndexShift);

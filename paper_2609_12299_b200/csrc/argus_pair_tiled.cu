@@ -18,10 +18,9 @@
 // This is exact when the tile is well nested (every end meets the frame on top with the same region
 // id). A tile is consumed in windows: the first position where a rule fails (region mismatch, negative
 // height, bad region id, depth overflow, level window exceeded, 2^32 ticks of child time in one
-// window) cuts the window there; the prefix is
-// redone on its own (its records come out the same again), the offending marker goes through the
-// sequential stack machine on the carried stack, and a new window starts after it, so the result is
-// always the sequential definition's.
+// window) cuts the window there; what lies before it counts (what ends behind it have added to their
+// parents is taken back), the offending marker goes through the sequential stack machine on the carried
+// stack, and a new window starts after it, so the result is always the sequential definition's.
 //
 // Bound by instruction issue and the latency of the phases (7 blocks = 28 warps per SM, capped by shared memory and registers
 // alike), next by the way of shared-memory accesses through the load/store pipe. Looking an end up and writing its record in one
@@ -335,9 +334,10 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       }
 
       // The tile is consumed in windows [w0, wend). A well-nested tile is one window. When the parallel
-      // rules fail first at position p, the window is cut there: [w0, p) is redone in parallel (it is well
-      // nested), the marker at p goes through the sequential stack machine, and a new window starts after it.
-      int w0 = 0, wend = tn, small_streak = 0;
+      // rules fail first at position p, the window is cut there: [w0, p) counts (it is well nested), the
+      // marker at p goes through the sequential stack machine, and a new window starts after it.
+      int w0 = 0, small_streak = 0;
+      const int wend = tn;
       while (w0 < tn) {
         const int cbase = carlo + cpar * kCar;           // carried level L -> reference cbase + L
         uint4* const car_next = sm.evall + T + (cpar ^ 1) * kCar;
@@ -385,7 +385,6 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
           }
         }
         const u32 ex = before + incl_cnt - mine_cnt;
-        const int win_nb = (int)(tot & 0xffffu);
         const int win_ne = (int)(tot >> 16) < MAXI ? (int)(tot >> 16) : MAXI;  // more ends than that means a violation earlier
         const int h0 = ch + (int)(ex & 0xffffu) - (int)(ex >> 16);
         const int lbase = ch > kLevelWindow / 2 ? ch - kLevelWindow / 2 : 0;
@@ -420,8 +419,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
 
         // ---------------- ends, one thread each, NT at a time in output order ----------------
         // A round looks up begin and parent and feeds the parent's child time; then, after a barrier, it writes its records:
-        // a child ends before its parent, so what this round and those before it have added is all there will be. Records of
-        // ends before a cut are the final ones already (a cut window writes them again).
+        // a child ends before its parent, so what this round and those before it have added is all there will be.
         const u64 pos0 = out_base + n_int, room = SPLIT ? limit : a.interval_capacity;
         const int fit = pos0 + (u64)win_ne <= room ? win_ne : pos0 < room ? (int)(room - pos0) : 0;  // records that fit the output
         uint4* const rec0 = reinterpret_cast<uint4*>(a.intervals + pos0);
@@ -510,42 +508,55 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
               q[2] = make_uint4(s, preg, bidx, (d >> SM::kDescShift) | (flags << 16));
               if (dig0) dig0[rk] = argus_digest_pack32(btag >> 1, incl, excl, flags);
             }
+          } else if (incl) {
+            atomicSub(&accb[parent], incl);  // an end at or after a cut
           }
         }
         const int badpos = sm.badpos[bp];  // every round's barrier has passed
         bp ^= 1;
         if (tid == 0) sm.badpos[bp] = 0x7fffffff;  // nobody reads or reports into it before the next window's barriers
 
-        if (badpos >= wend) {
-          // ---------------- the window counts: the stack it leaves behind ----------------
+        if (SPLIT && badpos < wend) {  // the chained pass walks this stream
+          stream_failed = true;
+          __syncthreads();
+          break;
+        }
+        // the window counts up to `upto`: the stack it leaves behind, in the next window's index space (`pos`: events before it
+        // are looked at)
+        auto count_window = [&](int upto, int ne, int pos) {
           if (win_flags) { tot_ctx += win_flags & 1023u; tot_rev += (win_flags >> 10) & 1023u; tot_clamp += win_flags >> 20; }
-          const int new_ch = ch + win_nb - win_ne;
-          if (tid < new_ch) {  // the stack this window leaves behind, in the next window's index space
-            const int e = tile_latest_begin<NT, E, false>(sm, tid, lbase, T);
+          const int new_ch = ch + (upto - w0) - 2 * ne;  // every marker is a begin or an end
+          if (tid < new_ch) {
+            const int e = tile_latest_begin<NT, E, false>(sm, tid, lbase, pos);
             const int from = e >= 0 ? e : cbase + tid;
             car_next[tid] = evb[from];
             sm.cchild[cpar ^ 1][tid] = (e >= 0 ? 0ull : sm.cchild[cpar][tid]) + accb[from];
             sm.cidx[cpar ^ 1][tid] = e >= 0 ? tile_start + (u32)e : sm.cidx[cpar][tid];
           }
-          small_streak = (wend - w0 < 32) ? small_streak + 1 : 0;
+          small_streak = (upto - w0 < 32) ? small_streak + 1 : 0;
           ch = new_ch;
-          n_int += (u64)win_ne;
+          n_int += (u64)ne;
           cpar ^= 1;
-          w0 = wend;
-          wend = tn;
+          w0 = upto;
           __syncthreads();
+        };
+        if (badpos >= wend) {
+          count_window(wend, win_ne, T);
           if (SPLIT) init_h = sm.low < init_h ? sm.low : init_h;
-        } else if (badpos > w0) {
-          wend = badpos;  // [w0, badpos) is well nested: do it again on its own (nothing was committed yet)
-        } else if (SPLIT) {  // the chained pass walks this stream
-          stream_failed = true;
-          __syncthreads();
-          break;
         } else {
+          if (badpos > w0) {  // the ends before the cut (also a barrier for what the ends after it have taken back)
+            int ne = 0;
+            for (int rk = tid; rk - tid < win_ne; rk += NT)
+              ne += __syncthreads_count(rk < win_ne && (int)(sm.desc[rk] & ((1u << SM::kDescShift) - 1u)) < badpos);
+            __syncthreads();
+            count_window(badpos, ne, badpos);
+          }
           // ---------------- the marker(s) at w0 go through the sequential stack machine ----------------
           const int nseq = small_streak >= 2 ? ((tn - w0) < kSeqChunk ? (tn - w0) : kSeqChunk) : 1;
+          const int base = carlo + cpar * kCar;
+          uint4* const seq_next = sm.evall + T + (cpar ^ 1) * kCar;
           if (tid < ch) {
-            const uint4 f = evb[cbase + tid];
+            const uint4 f = evb[base + tid];
             ArgusFrame& o = sm.fstk[tid];
             o.ts = (u64)f.x | ((u64)f.y << 32); o.child = sm.cchild[cpar][tid]; o.region = f.z >> 1; o.ctx = f.w;
             o.idx = sm.cidx[cpar][tid]; o.pad = 0;
@@ -571,13 +582,12 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
           if (sm.failed) stream_failed = true;
           if (tid < ch) {
             const ArgusFrame f = sm.fstk[tid];
-            car_next[tid] = make_uint4((u32)f.ts, (u32)(f.ts >> 32), f.region << 1, f.ctx);
+            seq_next[tid] = make_uint4((u32)f.ts, (u32)(f.ts >> 32), f.region << 1, f.ctx);
             sm.cchild[cpar ^ 1][tid] = f.child;
             sm.cidx[cpar ^ 1][tid] = f.idx;
           }
           cpar ^= 1;
           w0 += nseq;
-          wend = tn;
           ++small_streak;
           __syncthreads();
           if (stream_failed) break;

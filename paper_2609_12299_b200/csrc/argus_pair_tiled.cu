@@ -19,8 +19,9 @@
 // id). A tile is consumed in windows: the first position where a rule fails (region mismatch, negative
 // height, bad region id, depth overflow, level window exceeded, 2^32 ticks of child time in one
 // window) cuts the window there; what lies before it counts (what ends behind it have added to their
-// parents is taken back), the offending marker goes through the sequential stack machine on the carried
-// stack, and a new window starts after it, so the result is always the sequential definition's.
+// parents is taken back; if a sum wrapped, it is done again, up to the cut), the offending marker goes through the
+// sequential stack machine on the carried stack, and a new window starts after it, so the result is always the
+// sequential definition's.
 //
 // Bound by instruction issue and the latency of the phases (7 blocks = 28 warps per SM, capped by shared memory and registers
 // alike), next by the way of shared-memory accesses through the load/store pipe. Looking an end up and writing its record in one
@@ -140,6 +141,7 @@ struct TileSmem {
   u32 cur_rec;                     // hand-over record of the stream being walked (kNoRec: none)
   u64 n_int;                       // written by the sequential redo path
   int ch;
+  u32 wrapped;                     // a sum of 32-bit child time wrapped in this window
   int badpos[2];                   // first position of the window where the parallel rules fail (INT_MAX = none); windows alternate
                                    // between the two, so that one can be reset while stragglers still read the other
   int dead, failed;
@@ -336,8 +338,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       // The tile is consumed in windows [w0, wend). A well-nested tile is one window. When the parallel
       // rules fail first at position p, the window is cut there: [w0, p) counts (it is well nested), the
       // marker at p goes through the sequential stack machine, and a new window starts after it.
-      int w0 = 0, small_streak = 0;
-      const int wend = tn;
+      int w0 = 0, wend = tn, small_streak = 0;
       while (w0 < tn) {
         const int cbase = carlo + cpar * kCar;           // carried level L -> reference cbase + L
         uint4* const car_next = sm.evall + T + (cpar ^ 1) * kCar;
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         for (int i = tid; i < (kLevelWindow + 1) * NWORDS / 4; i += NT) reinterpret_cast<uint4*>(&sm.bm[0][0])[i] = make_uint4(0, 0, 0, 0);
         if (tid <= kLevelWindow) sm.summ[tid] = 0;
         if (tid < ch) accb[cbase + tid] = 0;  // what this window adds to the carried frames (a cut window starts clean again)
-        if (tid == 0) { sm.failed = 0; accb[cbase + kSink] = 0; }
+        if (tid == 0) { sm.failed = 0; sm.wrapped = 0; accb[cbase + kSink] = 0; }
         if (whole) {
 #pragma unroll
           for (int k = 0; k < E; ++k) mine_cnt += tags[k] & 1u;
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
                 // the parent gathers what this window adds to its child time in 32 bits; an interval or a sum of 2^32 ticks
                 // cuts the window here, and the sequential machine (64-bit throughout) takes this marker
                 const u32 old = atomicAdd(&accb[parent], incl);
-                live = live && old + incl >= old;
+                if (old + incl < old) { live = false; sm.wrapped = 1; }
               } else {
                 live = false;
               }
@@ -538,11 +539,17 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
           n_int += (u64)ne;
           cpar ^= 1;
           w0 = upto;
+          wend = tn;
           __syncthreads();
         };
         if (badpos >= wend) {
           count_window(wend, win_ne, T);
           if (SPLIT) init_h = sm.low < init_h ? sm.low : init_h;
+        } else if (badpos > w0 && sm.wrapped) {
+          // which of the ends that share a parent makes its sum wrap depends on their order, and so one before the cut may have
+          // wrapped it unseen: [w0, badpos) is done again on its own (nothing was counted yet)
+          wend = badpos;
+          __syncthreads();
         } else {
           if (badpos > w0) {  // the ends before the cut (also a barrier for what the ends after it have taken back)
             int ne = 0;
@@ -588,6 +595,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
           }
           cpar ^= 1;
           w0 += nseq;
+          wend = tn;
           ++small_streak;
           __syncthreads();
           if (stream_failed) break;

@@ -2,7 +2,7 @@
 //
 //   k_agg_streams_digest : argus_synthesize's pass: one CTA per stream reads the 8-byte digests the pairing
 //                   kernel wrote beside the interval records (not the records) and gathers the stream's row
-//                   in 100-byte shared-memory cells, with per-lane copies of the most frequent regions' cells;
+//                   in 124-byte shared-memory cells, with per-lane copies of the most frequent regions' cells;
 //   k_agg_streams_compact : the same over the 48-byte records, with an optional scope: that stream's row in
 //                   a compact shared-memory form (112 B per region: sums, min, max, a 16-bin window, so
 //                   several CTAs fit an SM), for up to kAggCompactRegions regions;
@@ -49,6 +49,7 @@ struct AggArgs {
   // overlap selection in the pass over the digests (argus_synthesize)
   ArgusFuseArgs ov;
   u32 parts;          // k_agg_streams_digest, k_agg_streams_compact: blocks that share a stream
+  u32 slices;         // k_agg_streams_digest: slices of a stream, one per warp of its blocks
   const u64* digest;  // digests of the intervals (k_agg_streams_digest; overwritten with entries where overlap is selected), null = read the records
   u64 interval_limit; // records the interval array holds: a stream whose offsets reach beyond it is reported, not read
 };
@@ -201,25 +202,27 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
 }
 
 // ---- the pass over the intervals' 8-byte digests (what argus_synthesize's pairing wrote beside the records) ----
-// One CTA per stream, no scope. The stream's row is gathered in shared memory in cells of kDgWords = 25 32-bit
-// words (an odd size: the cells of 32 different regions start in 32 different banks). A few regions usually own
-// most intervals of a stream, and 32 lanes adding to one address serialise; so after a probe of the stream's
-// first intervals the kDigestHot most frequent regions get 32 copies of their cell, one per lane (consecutive
-// cells: never a bank conflict), which are folded into the region's cell when the stream ends. The last word of
-// a region's cell (meta) holds what a lane needs to know about its region: histogram window base, copy slot,
-// whether the region appears in an overlap pair. A digest marked wide (a duration of 2^23 ticks or more) sends
-// its lane to the record and to 64-bit atomics on the global row. Every warp walks a slice of the stream, so that overlap
-// candidates stay in order; their entries replace digests that the warp has consumed: no list, no atomics. The table is
-// addressed with 32-bit shared-memory addresses and the fields by constant offsets.
+// One block per stream (or several), no scope. The stream's row is gathered in shared memory in cells of kDgWords = 31 32-bit
+// words (an odd size: the cells of 32 different regions start in 32 different banks) that hold all the 23 histogram bins a
+// digest can fall into. All words start at zero: the minimum is kept as the maximum of the complement. A few regions usually
+// own most intervals of a stream, and 32 lanes adding to one address serialise; so after a count of the regions in the first
+// round of every warp the kDigestHot most frequent ones get 32 copies of their cell, one per lane (consecutive cells: never a
+// bank conflict), which are folded into the region's cell when the stream ends. meta[region] holds the byte address of the
+// cell to add to, whether it is one of 32 copies, and whether the region appears in an overlap pair. What does not count (past
+// the end, a bad region, a digest marked wide) goes to a cell of its own that nobody reads, so that the common case has no
+// selects. Every warp walks a slice of the stream, so that overlap candidates stay in order; their entries replace digests that
+// the warp has consumed: no list, no atomics. The row is written once, with plain stores; wide intervals (a duration of 2^23
+// ticks or more) are added to it afterwards, from their records, by the warps that saw one.
 constexpr u32 kDigestHot = 4;
-constexpr u32 kDgSumInclLo = 0, kDgSumInclHi = 1, kDgSumExclLo = 2, kDgSumExclHi = 3, kDgMin = 4, kDgMax = 5, kDgFlag = 6,
-              kDgCountOut = 7, kDgBins = 8, kDgMeta = kDgBins + kAggWindow, kDgWords = kDgMeta + 1;
+constexpr u32 kDgSumInclLo = 0, kDgSumInclHi = 1, kDgSumExclLo = 2, kDgSumExclHi = 3, kDgNotMin = 4, kDgMax = 5, kDgFlag = 6,
+              kDgBins = 7, kDgCount = kDgBins + kDigestBits, kDgWords = kDgCount + 1;
 static_assert(kDgWords % 2 == 1, "an odd cell size keeps the cells of different regions in different banks");
-constexpr u32 kDgNone = 0xffu;                 // meta: bits 0-7 window base, 8-15 copy slot (kDgNone = unset), bit 16 in a pair
-constexpr u32 kDigestProbe = 512;              // intervals looked at before the hot regions are chosen
-constexpr u32 kDigestMinStream = 2048;         // shorter streams are gathered without copies
+constexpr u32 kDgHot = 1u << 31, kDgInPair = 1u << 30, kDgAddr = (1u << 18) - 1;  // meta
+constexpr u64 kDgPad = 0xffffull;              // what a lane past the end looks at: no such region
 
-__host__ __device__ constexpr size_t digest_table_words(u32 R) { return (size_t)kDgWords * (R + kDigestHot * 32); }
+// cells of the regions, the cell that nobody reads, copies; then meta for each region and for no region
+__host__ __device__ constexpr u32 digest_cell_words(u32 R, u32 copies) { return (kDgWords * (R + 1 + kDigestHot * copies) + 3) & ~3u; }
+__host__ __device__ constexpr size_t digest_table_bytes(u32 R, u32 copies) { return 4 * ((size_t)digest_cell_words(R, copies) + R + 1 + (R + 31) / 32); }
 
 template <u32 F> __device__ __forceinline__ u32 dg_add(u32 cell, u32 v) {  // returns the old value
   u32 old;
@@ -229,261 +232,230 @@ template <u32 F> __device__ __forceinline__ u32 dg_add(u32 cell, u32 v) {  // re
 template <u32 F> __device__ __forceinline__ void dg_inc(u32 cell, u32 v) {
   asm volatile("red.shared.add.u32 [%0+%2], %1;" :: "r"(cell), "r"(v), "n"(F * 4) : "memory");
 }
-template <u32 F> __device__ __forceinline__ void dg_min(u32 cell, u32 v) {
-  asm volatile("red.shared.min.u32 [%0+%2], %1;" :: "r"(cell), "r"(v), "n"(F * 4) : "memory");
-}
 template <u32 F> __device__ __forceinline__ void dg_max(u32 cell, u32 v) {
   asm volatile("red.shared.max.u32 [%0+%2], %1;" :: "r"(cell), "r"(v), "n"(F * 4) : "memory");
 }
 
-// The histogram bin of an interval whose bin is not inside the region's window as the lane saw it: the window
-// may not be chosen yet (then this lane tries to), or the bin really lies outside (then it is counted here).
-// Returns the bin's place in the window, or kAggWindow and beyond when it has been dealt with.
-__device__ __noinline__ u32 digest_bin_rare(u32* meta_word, u32 bin, u32 cell, u64* row_bins) {
-  const u32 m = *reinterpret_cast<volatile u32*>(meta_word);
-  u32 hb = m & 0xffu;
-  if (hb == kDgNone) {
-    const u32 want = bin > 6u ? bin - 6u : 0u;   // bin <= 22: the window never passes bin 63
-    const u32 prev = atomicCAS(meta_word, m, (m & ~0xffu) | want);  // only the window base changes while intervals are added
-    hb = (prev & 0xffu) == kDgNone ? want : (prev & 0xffu);
-  }
-  const u32 rel = bin - hb;
-  if (rel < kAggWindow) return rel;
-  dg_inc<kDgCountOut>(cell, 1u);
-  atomicAdd(row_bins + bin, 1ull);
-  return 0xffffffffu;
+// A wide interval, from its record, with atomics on the global row.
+__device__ __noinline__ void digest_wide(u64* row, u32 R, uint4 q0, uint4 q1, u32 flags) {
+  if (q1.z >= R) return;
+  u64* const c = row + (size_t)q1.z * kCell;
+  const u64 span = (u64)q0.z | ((u64)q0.w << 32);
+  atomicAdd(c + 0, 1ull);
+  atomicAdd(c + 1, span);
+  atomicMin(c + 2, span);
+  atomicMax(c + 3, span);
+  atomicAdd(c + 4, (u64)q1.x | ((u64)q1.y << 32));
+  if (flags) atomicAdd(c + 7, 1ull);
+  atomicAdd(c + 8 + log2_bin(span), 1ull);
 }
 
-// (512 threads, three blocks per SM: the same 48 warps as six blocks of 256, but a stream's set-up, the choice of its hot
-// regions and the write-back of its row are shared by twice the threads; measured 2.33 ms against 2.45 ms on trace 3)
-constexpr int kDgThreads = 512;
-constexpr u32 kDgSlices = kDgThreads / 32;     // slices of a stream, one per warp (also the slices of the overlap entries)
-__global__ void __launch_bounds__(kDgThreads, 3) k_agg_streams_digest(AggArgs a) {
+//
+// Bound by instruction issue and the atomics' way through the load/store pipe. Bins that need no window, a trash cell instead of
+// selects, a row written once instead of emptied, added to and read back, and a loop of two rounds (the digests asked for
+// ahead change places without moves): decode trace (307 M intervals) 1,215 -> 903 us = 2.7 TB/s of digests, attention 400 -> 323,
+// GEMM 234 -> 188. Unrolled once 1,017, three times 898 (GEMM 191), four times 913. What a stream costs before its first
+// interval and after its last one (85 us of the decode trace's 903) decides for short ones: fewer threads for them and eight
+// copies instead of 32, so that more streams are on the chip (see argus_aggregate_digest_slices).
+template <u32 kThreads, u32 kCopies, u32 kBlocks>
+__global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArgs a) {
+  constexpr u32 kMinProbe = 4 * kThreads;    // shorter streams are gathered without copies
+  constexpr u32 kSlices = kThreads / 32;   // slices of a stream, one per warp (also the slices of the overlap entries)
+  extern __shared__ __align__(16) unsigned char sh_raw[];
+  const u32 R = a.num_regions;
+  u32* const tab = reinterpret_cast<u32*>(sh_raw);
+  u32* const meta = tab + digest_cell_words(R, kCopies);
+  u32* const pairbits = meta + R + 1;
+  __shared__ u32 hot_region[kDigestHot], often[64], num_often;
+  const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 tab_addr = (u32)__cvta_generic_to_shared(tab);
+  const bool has_ov = a.ov.num_pairs != 0;
+  const u32 s = blockIdx.x / a.parts, part = blockIdx.x % a.parts;
+  for (u32 i = tid; i < digest_cell_words(R, kCopies) / 4; i += kThreads) reinterpret_cast<uint4*>(tab)[i] = make_uint4(0, 0, 0, 0);
+  for (u32 i = tid; i < (R + 31) / 32; i += kThreads) pairbits[i] = 0;
+  if (tid < kDigestHot) hot_region[tid] = 0xffffffffu;
+  if (tid == 0) num_often = 0;
   argus_kernel_begin_long();
   agg_empty_tables(a);
-  if (a.ov.num_pairs && blockIdx.x == 0 && threadIdx.x == 0) *a.ov.ctl = ArgusOvCtl{};
-  extern __shared__ __align__(16) unsigned char sh_raw[];
-  u32* const tab = reinterpret_cast<u32*>(sh_raw);
-  const u32 R = a.num_regions;
-  const u32 num_cells = R + kDigestHot * 32;
-  u32* const pairbits = tab + (size_t)kDgWords * num_cells;
-  __shared__ u32 hot_region[kDigestHot];
-  const u32 tab_addr = (u32)__cvta_generic_to_shared(tab);
-  const u32 cells = R * kCell;
-  const u32 lane = threadIdx.x & 31;
-  const u32 warp = threadIdx.x >> 5;
-  const bool has_ov = a.ov.num_pairs != 0;
-  for (u32 i = threadIdx.x; i < (R + 31) / 32; i += blockDim.x) pairbits[i] = 0;
+  if (has_ov && blockIdx.x == 0 && tid == 0) *a.ov.ctl = ArgusOvCtl{};
+  const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
+  u64* const row = a.warp_tab + (size_t)s * R * kCell;
   __syncthreads();
   if (has_ov) {
-    for (u32 i = threadIdx.x; i < 2 * a.ov.num_pairs; i += blockDim.x) {
+    for (u32 i = tid; i < 2 * a.ov.num_pairs; i += kThreads) {
       const u32 r = a.ov.pairs[i];
       if (r < R) atomicOr(&pairbits[r >> 5], 1u << (r & 31));
     }
     __syncthreads();
   }
+  for (u32 r = tid; r <= R; r += kThreads)
+    meta[r] = (tab_addr + r * (kDgWords * 4)) | (r < R && ((pairbits[r >> 5] >> (r & 31)) & 1u) ? kDgInPair : 0u);
+  if (has_ov && tid == 0) {
+    const u32 m = a.cta_sm[s / a.warps_per_cta];
+    if (m >= a.num_sms) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, m);
+  }
+  const bool good = hi >= lo && hi <= a.interval_limit && !((hi - lo) >> 32);
+  if (!good && tid == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
+  const u32 n = good ? (u32)(hi - lo) : 0u;
+  const u64* const dgs = a.digest + lo;
+  const argus_interval_t* const ivs = a.intervals + lo;
+  u32 i0, i1;
+  argus_ov_slice(n, a.slices, part * kSlices + warp, &i0, &i1);
+  u64* const ents = a.ov.entries + lo + i0;
+  u64* const starts = a.ov.starts + lo + i0;
+  // digests are asked for two rounds ahead (one round is shorter than a loaded DRAM access)
+  u32 i = i0 + lane;
+  u64 dg_next = i < i1 ? dgs[i] : kDgPad;
+  u64 dg_next2 = i + 32 < i1 ? dgs[i + 32] : kDgPad;
+  __syncthreads();
+  if (n / a.parts >= kMinProbe) {  // the regions that the first round of every warp sees most
+    const u32 region = (u32)dg_next & 0xffffu;
+    if (region < R) dg_inc<kDgCount>(tab_addr + region * (kDgWords * 4), 1u);
+    __syncthreads();
+    for (u32 r = tid; r < R; r += kThreads) {
+      const u32 cnt = tab[r * kDgWords + kDgCount];
+      if (cnt >= kThreads / 64) often[atomicAdd(&num_often, 1u)] = (cnt << 16) | r;  // at most 64 of them
+    }
+    __syncthreads();
+    if (tid < num_often) {
+      const u32 key = often[tid], r = key & 0xffffu;
+      u32 rank = 0;
+      for (u32 k = 0; k < num_often; ++k) rank += often[k] > key;
+      if (rank < kDigestHot) {
+        hot_region[rank] = r;
+        meta[r] = (tab_addr + (R + 1 + rank * kCopies) * (kDgWords * 4)) | kDgHot | (meta[r] & kDgInPair);
+      }
+    }
+    __syncthreads();
+  }
+  // every lane of a warp runs the same number of rounds, so that entries can be appended a warp at a time
+  const u32 own_copy = lane % kCopies * (kDgWords * 4);
+  u32 out_count = 0;  // warp-uniform: entries of the warp's slice
+  bool wide = false;  // the lane met a wide digest
+  bool late = false;  // the lane's candidate of the round before: its begin time may still be on its way
+  u64 late_t0 = 0;
+  u64* late_start = nullptr;
+#pragma unroll 2
+  for (u32 b = i0; b < i1; b += 32, i += 32) {
+    const u64 dg = dg_next;
+    dg_next = dg_next2;
+    dg_next2 = i + 64 < i1 ? dgs[i + 64] : kDgPad;
+    const u32 dlo = (u32)dg, dhi = (u32)(dg >> 32);
+    const u32 region = dlo & 0xffffu;
+    const u32 m = meta[region < R ? region : R];
+    const u32 incl = __funnelshift_r(dlo, dhi, 18) & ((1u << kDigestBits) - 1), excl = dhi >> (32 - kDigestBits);
+    const u32 normal = (m & kDgAddr) + (m >> 31) * own_copy;
+    const u32 cell = dlo & kDigestWide ? tab_addr + R * (kDgWords * 4) : normal;
+    const u32 old_i = dg_add<kDgSumInclLo>(cell, incl);
+    const u32 old_e = dg_add<kDgSumExclLo>(cell, excl);
+    dg_max<kDgNotMin>(cell, ~incl);
+    dg_max<kDgMax>(cell, incl);
+    dg_inc<kDgBins>(cell + (31u - (u32)__clz((int)(incl | 1u))) * 4, 1u);
+    bool cand = (m & kDgInPair) && incl;
+    // whatever is rare (a carry, a flag, a wide digest, no such region) is settled in one place
+    if (old_i > ~incl || old_e > ~excl || (dlo & (kDigestFlag | kDigestWide)) || region >= R) {
+      if (region >= R) {
+        if (i < i1) argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, lo + i);
+      } else if (dlo & kDigestWide) {
+        wide = true;
+        cand = m & kDgInPair;  // (its inclusive duration is not 0: the exclusive one is never longer)
+      } else {
+        if (old_i > ~incl) dg_inc<kDgSumInclHi>(cell, 1u);
+        if (old_e > ~excl) dg_inc<kDgSumExclHi>(cell, 1u);
+        if (dlo & kDigestFlag) dg_inc<kDgFlag>(cell, 1u);
+      }
+    }
+    const u32 bal = __ballot_sync(0xffffffffu, cand);
+    if (late) late_start[0] = late_t0;  // asked for a round ago
+    late = cand;
+    if (bal) {  // (the entries of a slice never reach the digests that are still to be read)
+      if (cand) {
+        const u32 at = out_count + __popc(bal & ((1u << lane) - 1u));
+        ents[at] = argus_entry_pack(dg, i - i0);
+        late_start = starts + at;
+        late_t0 = __ldg(reinterpret_cast<const u64*>(ivs + i));
+      }
+      out_count += __popc(bal);
+    }
+  }
+  if (late) late_start[0] = late_t0;
+  if (has_ov && lane == 0) {
+    ArgusOvPiece e;
+    e.pos = lo + (good ? i0 : 0u); e.count = out_count; e.next = kOvNone;
+    a.ov.pieces[s * a.slices + part * kSlices + warp] = e;
+  }
+  __syncthreads();
+  // the copies into their region's cell (which nobody added to): a thread per (hot region, field)
+  if (tid < kDigestHot * kDgCount) {
+    const u32 h = tid / kDgCount, f = tid % kDgCount, r = hot_region[h];
+    if (r != 0xffffffffu && f != kDgSumInclHi && f != kDgSumExclHi) {
+      const u32* src = tab + (R + 1 + h * kCopies) * kDgWords + f;
+      u32* dst = tab + r * kDgWords + f;
+      const bool sum = f == kDgSumInclLo || f == kDgSumExclLo, most = f == kDgNotMin || f == kDgMax;
+      u64 acc = 0;
+#pragma unroll 8
+      for (u32 l = 0; l < kCopies; ++l) {
+        const u32 v = src[l * kDgWords];
+        if (sum) acc += (u64)v | ((u64)src[l * kDgWords + 1] << 32);
+        else acc = most ? (v > acc ? v : acc) : acc + v;
+      }
+      dst[0] = (u32)acc;
+      if (sum) dst[1] = (u32)(acc >> 32);
+    }
+  }
+  __syncthreads();
+  for (u32 r = tid; r < R; r += kThreads) {
+    u32* c = tab + r * kDgWords;
+    u32 cnt = 0;
+#pragma unroll
+    for (u32 j = 0; j < kDigestBits; ++j) cnt += c[kDgBins + j];
+    c[kDgCount] = cnt;
+  }
+  __syncthreads();
+  // the regions' cells into the global row; a thread keeps to one field
+  const bool alone = a.parts == 1;  // (else the rows have been initialised: several blocks add to one)
+  auto put = [&](u64* p, u32 field, u64 v) {
+    if (alone) *p = v;
+    else if (field == 2) { if (v != ~0ull) atomicMin(p, v); }
+    else if (field == 3) { if (v) atomicMax(p, v); }
+    else if (v) atomicAdd(p, v);
+  };
   {
-    const u32 s = blockIdx.x / a.parts, part = blockIdx.x % a.parts, slices = a.parts * kDgSlices;
-    u64* row = a.warp_tab + (size_t)s * cells;
-    if (a.parts == 1)  // (else the rows have been initialised: several blocks add to one)
-      for (u32 i = threadIdx.x; i < cells; i += blockDim.x) row[i] = (i % kCell == 2) ? ~0ull : 0ull;
-    for (u32 i = threadIdx.x; i < kDgWords * num_cells; i += blockDim.x) {
-      const u32 f = i % kDgWords, c = i / kDgWords;
-      u32 v = f == kDgMin ? 0xffffffffu : 0u;
-      if (f == kDgMeta && c < R) v = kDgNone | (kDgNone << 8) | (((pairbits[c >> 5] >> (c & 31)) & 1u) << 16);
-      tab[i] = v;
+    const u32 f = tid % 64;
+    for (u32 r = tid / 64; r < R; r += kThreads / 64) put(row + (size_t)r * kCell + 8 + f, 8 + f, f < kDigestBits ? tab[r * kDgWords + kDgBins + f] : 0u);
+  }
+  {
+    const u32 f = tid % 8;
+    const u32 w = f == 0 ? kDgCount : f == 1 ? kDgSumInclLo : f == 2 ? kDgNotMin : f == 3 ? kDgMax : f == 4 ? kDgSumExclLo : kDgFlag;
+    for (u32 r = tid / 8; r < R; r += kThreads / 8) {
+      const u32* c = tab + r * kDgWords + w;
+      u64 v = c[0];
+      if (f == 1 || f == 4) v |= (u64)c[1] << 32;
+      if (f == 2) v = v ? (u64)(u32)~(u32)v : ~0ull;
+      if (f == 5 || f == 6) v = 0;  // ambiguity records: below
+      put(row + (size_t)r * kCell + f, f, v);
     }
-    if (threadIdx.x < kDigestHot) hot_region[threadIdx.x] = 0xffffffffu;
-    __threadfence();
-    __syncthreads();
-    const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
-    if (has_ov && threadIdx.x == 0) {
-      const u32 m = a.cta_sm[s / a.warps_per_cta];
-      if (m >= a.num_sms) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, m);
+  }
+  u64 alo = 0, ahi = 0;
+  if (a.ambig && a.ambig_offsets && part == 0) { alo = a.ambig_offsets[s]; ahi = a.ambig_offsets[s + 1]; }
+  wide = __any_sync(0xffffffffu, wide);
+  if (!__syncthreads_or(wide || alo < ahi)) return;
+  __threadfence();
+  __syncthreads();
+  if (wide) {  // (where entries have replaced the digests, the records tell)
+    for (u32 k = i0 + lane; k < i1; k += 32) {
+      const bool gone = k - i0 < out_count;
+      if (!gone && !((u32)dgs[k] & kDigestWide)) continue;
+      const uint4* p = reinterpret_cast<const uint4*>(ivs + k);
+      const uint4 q0 = __ldg(p), q1 = __ldg(p + 1), q2 = __ldg(p + 2);
+      const u32 too_long = ((q0.z | q1.x) >> kDigestBits) | q0.w | q1.y;
+      if (too_long) digest_wide(row, R, q0, q1, q2.w >> 16);
     }
-    u32 out_count = 0, out_first = 0;  // warp-uniform: entries of the warp's slice, where they start in the stream
-    if (hi < lo || hi > a.interval_limit || ((hi - lo) >> 32)) {
-      if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
-    } else {
-      const u32 n = (u32)(hi - lo);
-      const u64* const dgs = a.digest + lo;
-      const argus_interval_t* const ivs = a.intervals + lo;
-      u32 i0, i1;
-      argus_ov_slice(n, slices, part * kDgSlices + warp, &i0, &i1);
-      out_first = i0;
-      u64* const ents = a.ov.entries + lo + i0;
-      u64* const starts = a.ov.starts + lo + i0;
-      // two legs: the probe (the first intervals of every slice, each into its region's cell), then, hot regions chosen, the rest
-      const bool probe = n / a.parts >= kDigestMinStream;
-      const u32 probe_end = probe ? (i0 + 32 < i1 ? i0 + 32 : i1) : i1;
-      for (int leg = 0; leg < 2; ++leg) {
-        const u32 leg_lo = leg ? probe_end : i0, leg_hi = leg ? i1 : probe_end;
-        if (leg && probe) {
-          // warp 0 ranks the regions by their counts so far; kDigestHot rounds of a warp-wide maximum
-          if (threadIdx.x < 32) {
-            for (u32 h = 0; h < kDigestHot; ++h) {
-              u32 best = 0;
-              for (u32 r = lane; r < R; r += 32) {
-                const u32* c = tab + r * kDgWords;
-                if (((c[kDgMeta] >> 8) & 0xffu) != kDgNone) continue;
-                u32 cnt = c[kDgCountOut];
-#pragma unroll
-                for (u32 j = 0; j < kAggWindow; ++j) cnt += c[kDgBins + j];
-                const u32 key = ((cnt > 0xffffu ? 0xffffu : cnt) << 16) | r;
-                best = key > best ? key : best;
-              }
-              const u32 top = __reduce_max_sync(0xffffffffu, best);
-              if ((top >> 16) < kDigestProbe / 64) break;  // not worth a set of copies
-              if (lane == 0) { atomicAnd(&tab[(top & 0xffffu) * kDgWords + kDgMeta], ~0xff00u | (h << 8)); hot_region[h] = top & 0xffffu; }
-              __syncwarp();
-            }
-          }
-          __syncthreads();
-        }
-        // every lane of a warp runs the same number of rounds, so that entries can be appended a warp at a time
-        u32 b = leg_lo;
-        bool late = false;  // the lane's candidate of the round before: its begin time may still be on its way
-        u64 late_t0 = 0;
-        u64* late_start = nullptr;
-        // digests are asked for two rounds ahead (one round is shorter than a loaded DRAM access)
-        u64 dg_next = b + lane < leg_hi ? dgs[b + lane] : 0ull;
-        u64 dg_next2 = b + lane + 32 < leg_hi ? dgs[b + lane + 32] : 0ull;
-        for (; b < leg_hi; b += 32) {
-          const u32 i = b + lane;
-          const u64 dg = dg_next;
-          dg_next = dg_next2;
-          dg_next2 = i + 64 < leg_hi ? dgs[i + 64] : 0ull;
-          const u32 dlo = (u32)dg, dhi = (u32)(dg >> 32);
-          const bool in = i < leg_hi;
-          const u32 region = dlo & 0xffffu;
-          const bool ok = in && region < R;
-          const u32 rsafe = ok ? region : 0u;
-          const u32 incl = (dlo >> 18) | ((dhi & 0x1ffu) << 14), excl = dhi >> 9;
-          const u32 meta = tab[rsafe * kDgWords + kDgMeta];
-          const u32 slot = (meta >> 8) & 0xffu;
-          const u32 cell = tab_addr + (slot != kDgNone ? R + slot * 32 + lane : rsafe) * (kDgWords * 4);
-          // the common case without a branch: a lane that does not take part (past the end, wide, bad region)
-          // adds nothing; whatever is rare (a carry, a flag, a bin outside the window, ...) is settled in one place
-          const bool take = ok && !(dlo & (1u << 17));
-          const u32 vi = take ? incl : 0u, ve = take ? excl : 0u;
-          const u32 old_i = dg_add<kDgSumInclLo>(cell, vi);
-          const u32 old_e = dg_add<kDgSumExclLo>(cell, ve);
-          dg_min<kDgMin>(cell, take ? incl : 0xffffffffu);
-          dg_max<kDgMax>(cell, vi);
-          const u32 bin = 31u - (u32)__clz((int)(incl | 1u));
-          const u32 rel = bin - (meta & 0xffu);
-          const bool in_win = take && rel < kAggWindow;
-          dg_inc<kDgBins>(cell + (in_win ? rel : 0u) * 4, in_win ? 1u : 0u);
-          u64 span = vi;
-          const bool rare = in && ((dlo & (3u << 16)) || !ok || old_i + vi < old_i || old_e + ve < old_e || !in_win);
-          if (rare) {
-            if (!ok) {
-              argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, lo + i);
-            } else if (!take) {
-              u64* const row_cell = row + (size_t)region * kCell;
-              const uint4* p = reinterpret_cast<const uint4*>(ivs + i);
-              const uint4 q0 = __ldg(p), q1 = __ldg(p + 1);
-              span = (u64)q0.z | ((u64)q0.w << 32);
-              atomicAdd(row_cell + 0, 1ull);
-              atomicAdd(row_cell + 1, span);
-              atomicMin(row_cell + 2, span);
-              atomicMax(row_cell + 3, span);
-              atomicAdd(row_cell + 4, (u64)q1.x | ((u64)q1.y << 32));
-              if (dlo & (1u << 16)) atomicAdd(row_cell + 7, 1ull);
-              atomicAdd(row_cell + 8 + log2_bin(span), 1ull);
-            } else {
-              if (old_i + vi < old_i) dg_inc<kDgSumInclHi>(cell, 1u);
-              if (old_e + ve < old_e) dg_inc<kDgSumExclHi>(cell, 1u);
-              if (dlo & (1u << 16)) dg_inc<kDgFlag>(cell, 1u);
-              if (!in_win) {
-                const u32 r2 = digest_bin_rare(tab + region * kDgWords + kDgMeta, bin, cell, row + (size_t)region * kCell + 8);
-                if (r2 < kAggWindow) dg_inc<kDgBins>(cell + r2 * 4, 1u);
-              }
-            }
-          }
-          const bool cand = ok && ((meta >> 16) & 1u) && span;
-          const u32 bal = __ballot_sync(0xffffffffu, cand);
-          if (late) late_start[0] = late_t0;  // asked for a round ago
-          late = cand;
-          if (bal) {  // (the entries of a slice never reach the digests that are still to be read)
-            const u32 at = out_count + __popc(bal & ((1u << lane) - 1u));
-            if (cand) {
-              ents[at] = argus_entry_pack(dg, i - i0);
-              late_start = starts + at;
-              late_t0 = __ldg(reinterpret_cast<const u64*>(ivs + i));
-            }
-            out_count += __popc(bal);
-          }
-        }
-        if (late) late_start[0] = late_t0;
-        __syncthreads();
-      }
-    }
-    if (has_ov && lane == 0) {
-      ArgusOvPiece e;
-      e.pos = lo + out_first; e.count = out_count; e.next = kOvNone;
-      a.ov.pieces[s * slices + part * kDgSlices + warp] = e;
-    }
-    if (a.ambig && a.ambig_offsets && part == 0) {
-      const u64 alo = a.ambig_offsets[s], ahi = a.ambig_offsets[s + 1];
-      for (u64 i = alo + threadIdx.x; i < ahi && ahi >= alo; i += blockDim.x) {
-        const u32 region = a.ambig[i].tag >> 1;
-        if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
-        atomicAdd(row + (size_t)region * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
-      }
-    }
-    __syncthreads();
-    // fold the lanes' copies into their region's cell: one thread per (hot region, field)
-    if (threadIdx.x < kDigestHot * kDgMeta) {
-      const u32 h = threadIdx.x / kDgMeta, f = threadIdx.x % kDgMeta;
-      const u32 r = hot_region[h];
-      if (r != 0xffffffffu && f != kDgSumInclHi && f != kDgSumExclHi) {
-        const u32* src = tab + (R + h * 32) * kDgWords + f;
-        u32* dst = tab + r * kDgWords + f;
-        if (f == kDgSumInclLo || f == kDgSumExclLo) {
-          u64 sum = (u64)dst[0] | ((u64)dst[1] << 32);
-          for (u32 l = 0; l < 32; ++l) sum += (u64)src[l * kDgWords] | ((u64)src[l * kDgWords + 1] << 32);
-          dst[0] = (u32)sum;
-          dst[1] = (u32)(sum >> 32);
-        } else {
-          u32 acc = dst[0];
-          for (u32 l = 0; l < 32; ++l) {
-            const u32 v = src[l * kDgWords];
-            acc = f == kDgMin ? (v < acc ? v : acc) : f == kDgMax ? (v > acc ? v : acc) : acc + v;
-          }
-          dst[0] = acc;
-        }
-      }
-    }
-    __syncthreads();
-    // the regions' cells into the global row, which already holds the wide intervals, the bins outside the
-    // windows and the ambiguity counters: everything is combined, nothing overwritten
-    constexpr u32 kItems = 6 + kAggWindow;
-    for (u32 i = threadIdx.x; i < R * kItems; i += blockDim.x) {
-      const u32 r = i % R, f = i / R;
-      const u32* c = tab + r * kDgWords;
-      u64* cell = row + (size_t)r * kCell;
-      switch (f) {
-        case 0: {
-          u64 cnt = c[kDgCountOut];
-#pragma unroll
-          for (u32 j = 0; j < kAggWindow; ++j) cnt += c[kDgBins + j];
-          if (cnt) atomicAdd(cell + 0, cnt);
-          break;
-        }
-        case 1: { const u64 v = (u64)c[kDgSumInclLo] | ((u64)c[kDgSumInclHi] << 32); if (v) atomicAdd(cell + 1, v); break; }
-        case 2: { const u32 v = c[kDgMin]; if (v != 0xffffffffu) atomicMin(cell + 2, (u64)v); break; }
-        case 3: { const u32 v = c[kDgMax]; if (v) atomicMax(cell + 3, (u64)v); break; }
-        case 4: { const u64 v = (u64)c[kDgSumExclLo] | ((u64)c[kDgSumExclHi] << 32); if (v) atomicAdd(cell + 4, v); break; }
-        case 5: { const u32 v = c[kDgFlag]; if (v) atomicAdd(cell + 7, (u64)v); break; }
-        default: {
-          const u32 j = f - 6;
-          const u32 v = c[kDgBins + j];
-          if (v) atomicAdd(cell + 8 + (c[kDgMeta] & 0xffu) + j, (u64)v);
-        }
-      }
-    }
-    __syncthreads();
+  }
+  for (u64 k = alo + tid; k < ahi; k += kThreads) {
+    const u32 region = a.ambig[k].tag >> 1;
+    if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, k); continue; }
+    atomicAdd(row + (size_t)region * kCell + (a.ambig[k].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
   }
 }
 
@@ -686,7 +658,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
                                     argus_agg_t* sm_tab, argus_agg_t* kernel_tab, argus_agg_t* role_tab,
                                     argus_agg_t* iter_tab, argus_status_t* status, void* workspace,
                                     size_t workspace_bytes, void* cuda_stream, bool reset_status,
-                                    const ArgusFuseArgs* ov_select, const uint64_t* digest, uint32_t digest_parts,
+                                    const ArgusFuseArgs* ov_select, const uint64_t* digest, uint32_t digest_parts, uint32_t digest_slices,
                                     uint64_t interval_limit) {
   if (!interval_offsets || !status || !workspace) return ARGUS_ERR_INVALID_ARG;
   if (ov_select && !digest) return ARGUS_ERR_INVALID_ARG;
@@ -723,7 +695,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   a.role_tab = (u64*)role_tab; a.iter_tab = (u64*)iter_tab; a.num_iters = num_iters;
   if (ov_select) { a.ov = *ov_select; } else { a.ov = ArgusFuseArgs(); }
   a.digest = !scope && !role_tab && !iter_tab && num_regions <= kAggCompactRegions ? (const u64*)digest : nullptr;
-  a.parts = digest_parts; a.interval_limit = interval_limit;
+  a.parts = digest_parts; a.slices = digest_slices; a.interval_limit = interval_limit;
   const size_t smem = (size_t)num_regions * sizeof(argus_agg_t);
   a.use_smem = smem <= kAggSmemLimit;
   const size_t need = a.use_smem ? smem : 0;
@@ -743,10 +715,11 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
     if (compact > 48 * 1024)
       ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_compact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)compact));
     if (a.digest) {
-      const size_t dg = digest_table_words(num_regions) * 4 + ((num_regions + 31) / 32) * 4;
-      if (dg > 48 * 1024)
-        ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_digest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
-      ARGUS_LAUNCH(k_agg_streams_digest, num_streams * a.parts, kDgThreads, dg, stream, a);
+      const u32 warps = a.slices / a.parts;
+      const size_t dg = digest_table_bytes(num_regions, warps == 16 ? 32 : 8);
+      const auto kernel = warps == 16 ? k_agg_streams_digest<512, 32, 3> : warps == 8 ? k_agg_streams_digest<256, 8, 6> : k_agg_streams_digest<128, 8, 12>;
+      if (dg > 48 * 1024) ARGUS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
+      ARGUS_LAUNCH(kernel, num_streams * a.parts, warps * 32, dg, stream, a);
     } else {
       ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
     }
@@ -784,18 +757,25 @@ int argus_internal_aggregate(const argus_interval_t* intervals, const uint64_t* 
   return argus_internal_aggregate_scoped(intervals, interval_offsets, ambig, ambig_offsets, num_streams, warps_per_cta, cta_sm,
                                          num_sms, num_regions, nullptr, warp_tab, cta_tab, sm_tab, kernel_tab, nullptr,
                                          nullptr, status, workspace, workspace_bytes, cuda_stream, reset_status, nullptr,
-                                         nullptr, 1, interval_limit);
+                                         nullptr, 1, 0, interval_limit);
 }
 
 bool argus_aggregate_can_read_digests(uint32_t num_regions) { return num_regions <= kAggCompactRegions; }
 // Few streams: several blocks share one, six for every SM in all, as long as each has 8,192 intervals to look at.
-// (96 streams of 259,328 intervals: 142 us; 352 us with a block each.)
+// (96 streams of 259,328 intervals: 104 us; 352 us with a block each.)
 uint32_t argus_aggregate_digest_parts(uint32_t num_streams, uint64_t num_events) {
   if (num_streams == 0) return 1;
   const uint64_t room = 888 / num_streams, work = num_events / 2 / num_streams / 8192, parts = room < work ? room : work;
   return (uint32_t)(parts < 1 ? 1 : parts);
 }
-uint32_t argus_aggregate_digest_slices(uint32_t parts) { return parts * kDgSlices; }
+// A warp for each slice. By the streams' average length: 128 threads below 1,024 intervals, 256 below 8,192, else 512. Measured
+// with 4 / 8 / 16 warps (148 CTAs, us): 350 intervals a stream 20 / 22 / 31, 870: 27 / 39 / 43, 1,700: 41 / 41 / 60, 3,500:
+// 66 / 61 / 69, 6,100: 120 / 99 / 115 (202 regions), 130,000: 2,065 / 1,175 / 1,002.
+uint32_t argus_aggregate_digest_slices(uint32_t num_streams, uint64_t num_events) {
+  const uint32_t parts = argus_aggregate_digest_parts(num_streams, num_events);
+  const uint64_t length = num_streams ? num_events / 2 / num_streams : 0;
+  return parts * (length < 1024 ? 4 : length < 8192 ? 8 : 16);
+}
 
 extern "C" int argus_aggregate(const argus_interval_t* intervals, const uint64_t* interval_offsets,
                                const argus_ambiguity_t* ambig, const uint64_t* ambig_offsets, uint32_t num_streams,

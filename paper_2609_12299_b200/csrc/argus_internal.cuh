@@ -37,11 +37,11 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
                                     argus_agg_t* sm_tab, argus_agg_t* kernel_tab, argus_agg_t* role_tab,
                                     argus_agg_t* iter_tab, argus_status_t* status, void* workspace,
                                     size_t workspace_bytes, void* cuda_stream, bool reset_status,
-                                    const ArgusFuseArgs* ov_select, const uint64_t* digest = nullptr, uint32_t digest_parts = 1,
+                                    const ArgusFuseArgs* ov_select, const uint64_t* digest = nullptr, uint32_t digest_parts = 1, uint32_t digest_slices = 0,
                                     uint64_t interval_limit = ~0ull);
 bool argus_aggregate_can_read_digests(uint32_t num_regions);
 uint32_t argus_aggregate_digest_parts(uint32_t num_streams, uint64_t num_events);  // blocks of the pass over the digests that share a stream
-uint32_t argus_aggregate_digest_slices(uint32_t parts);  // slices per stream in which that pass selects overlap candidates
+uint32_t argus_aggregate_digest_slices(uint32_t num_streams, uint64_t num_events);  // slices per stream in which that pass selects overlap candidates
 
 // argus_ring.cu — stream_offsets (and dropped) of the records that survive in the slots of a ring container;
 // status->code = ARGUS_ERR_CAPACITY if they exceed event_capacity. The status block is not cleared.

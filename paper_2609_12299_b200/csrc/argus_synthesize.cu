@@ -29,7 +29,7 @@ SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_reg
   // lie in the digest array).
   const bool digests = argus_aggregate_can_read_digests(num_regions);
   L.parts = argus_aggregate_digest_parts(num_streams, num_events);
-  L.slices = argus_aggregate_digest_slices(L.parts);
+  L.slices = argus_aggregate_digest_slices(num_streams, num_events);
   const size_t pieces = (size_t)num_streams * L.slices * sizeof(ArgusOvPiece);
   L.ov = o;
   L.pieces = o + argus_align_up(sizeof(ArgusOvCtl), 256);
@@ -100,7 +100,7 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
                                          cta_sm, num_sms, num_regions, nullptr, warp_tab, cta_tab, sm_tab, kernel_tab,
                                          nullptr, nullptr, status, ws + L.agg, L.agg_bytes, cuda_stream, false,
                                          f.num_pairs ? &f : nullptr,
-                                         use_digest ? (const uint64_t*)(ws + L.digest) : nullptr, L.parts, interval_capacity);
+                                         use_digest ? (const uint64_t*)(ws + L.digest) : nullptr, L.parts, L.slices, interval_capacity);
     if (rc != ARGUS_OK) return rc;
   }
   if (num_pairs) {

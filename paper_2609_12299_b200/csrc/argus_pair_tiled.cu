@@ -27,8 +27,11 @@
 // alike), next by the way of shared-memory accesses through the load/store pipe. Looking an end up and writing its record in one
 // go, with one barrier between, instead of two sweeps over all ends that each read both event records: a quarter fewer
 // shared-memory wavefronts; together with a window that needs no bounds checks as the usual case and look-ups without range
-// selects (decode trace, 614 M events: 5.42 -> 5.01 ms = 4.9 TB/s of 16 B read + 24 B written an event, 75 % of the copy rate; 5.4
-// TB/s with the digests).
+// selects (decode trace, 614 M events: 5.42 -> 5.01 ms); then heights by vote over 32 markers in a row instead of a scan over the
+// threads' own five, and a word of a level's bitmap stored at once, by the lowest lane of those that match in level, instead of
+// a bit at a time (4.90 ms = 5.0 TB/s of 16 B read + 24 B written an event, 77 % of the copy rate, 5.5 TB/s with the digests;
+// attention 1.50 -> 1.45 ms; with votes but a bit at a time 5.08 and 1.57). Tiles of 512 events with 8 blocks: GEMM 638 -> 707
+// us, 160 threads with four events each and 6 blocks: 674.
 #include "argus_internal.cuh"
 #include "argus_pair_common.cuh"
 
@@ -345,13 +348,12 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
 
         // ---------------- phase A: heights by prefix sum; begins into per-level bitmaps; ends into `desc` ----------
         const bool whole = w0 == 0 && wend == T;  // the usual window: no marker needs a look at the window's bounds
-        u32 tags[E];
-        u32 mine_cnt = 0;  // begins, ends: 16 bits each
+        // a warp looks at 32 E markers in a row, 32 at a time: what lies before a marker is a vote and a count of bits
+        const int e0 = w0 + warp * (32 * E) + lane;
+        u32 tags[E], begins[E], ends[E];
+        u32 mine_cnt = 0;  // the warp's begins, ends: 16 bits each
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-          const int e = w0 + tid * E + k;
-          tags[k] = whole || e < wend ? reinterpret_cast<const u32*>(evb + e)[2] : 0xffffffffu;
-        }
+        for (int k = 0; k < E; ++k) tags[k] = whole || e0 + 32 * k < wend ? reinterpret_cast<const u32*>(evb + e0 + 32 * k)[2] : 0xffffffffu;
         for (int i = tid; i < T / 4; i += NT) reinterpret_cast<uint4*>(accb)[i] = make_uint4(0, 0, 0, 0);
         for (int i = tid; i < (kLevelWindow + 1) * NWORDS / 4; i += NT) reinterpret_cast<uint4*>(&sm.bm[0][0])[i] = make_uint4(0, 0, 0, 0);
         if (tid <= kLevelWindow) sm.summ[tid] = 0;
@@ -359,20 +361,23 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         if (tid == 0) { sm.failed = 0; sm.wrapped = 0; accb[cbase + kSink] = 0; }
         if (whole) {
 #pragma unroll
-          for (int k = 0; k < E; ++k) mine_cnt += tags[k] & 1u;
-          mine_cnt = (mine_cnt << 16) + (E - mine_cnt);
+          for (int k = 0; k < E; ++k) {
+            ends[k] = __ballot_sync(0xffffffffu, tags[k] & 1u);
+            begins[k] = ~ends[k];
+            mine_cnt += __popc(ends[k]);
+          }
+          mine_cnt = (mine_cnt << 16) + (32 * E - mine_cnt);
         } else {
 #pragma unroll
-          for (int k = 0; k < E; ++k) mine_cnt += w0 + tid * E + k < wend ? ((tags[k] & 1u) ? 0x10000u : 1u) : 0u;
+          for (int k = 0; k < E; ++k) {
+            const bool valid = e0 + 32 * k < wend;
+            ends[k] = __ballot_sync(0xffffffffu, valid && (tags[k] & 1u));
+            begins[k] = __ballot_sync(0xffffffffu, valid && !(tags[k] & 1u));
+            mine_cnt += (__popc(ends[k]) << 16) + __popc(begins[k]);
+          }
         }
         // block prefix sum: one barrier
-        u32 incl_cnt = mine_cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const u32 o = __shfl_up_sync(0xffffffffu, incl_cnt, d);
-          if (lane >= d) incl_cnt += o;
-        }
-        if (lane == 31) sm.warp_tot[warp] = incl_cnt;
+        if (lane == 0) sm.warp_tot[warp] = mine_cnt;
         __syncthreads();
         u32 before = 0, tot = 0;
 #pragma unroll
@@ -385,7 +390,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
             tot += t[q];
           }
         }
-        const u32 ex = before + incl_cnt - mine_cnt;
+        const u32 ex = before;
         const int win_ne = (int)(tot >> 16) < MAXI ? (int)(tot >> 16) : MAXI;  // more ends than that means a violation earlier
         const int h0 = ch + (int)(ex & 0xffffu) - (int)(ex >> 16);
         const int lbase = ch > kLevelWindow / 2 ? ch - kLevelWindow / 2 : 0;
@@ -395,25 +400,35 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         // id, height never negative, levels as above; the first marker that breaks one is reported, later ones (whose heights may
         // mean nothing) at most leave bits and descriptors behind it.
         auto place = [&](auto WHOLE) {
-          int h = h0, rank = (int)(ex >> 16);
+          int h_base = h0, rank_base = (int)(ex >> 16);
+          const u32 lower = (1u << lane) - 1u;
           u32 viol = 0;
 #pragma unroll
           for (int k = 0; k < E; ++k) {
-            const int e = w0 + tid * E + k;
+            const int e = e0 + 32 * k;
             const bool valid = decltype(WHOLE)::value || e < wend;  // (not "tag != all ones": that is a marker too, with a region id out of range)
             const bool is_e = valid && (tags[k] & 1u), is_b = valid && !(tags[k] & 1u);
+            const int nb = __popc(begins[k] & lower);
+            const int ne = decltype(WHOLE)::value ? lane - nb : __popc(ends[k] & lower);
+            const int h = h_base + nb - ne, rank = rank_base + ne;
             const u32 l = (u32)(h - lbase);  // level of the frame a begin opens, inside the window
             const bool ok_b = l < levels;
             if ((valid && (tags[k] >> 1) >= a.num_regions) || (is_e && h < 1) || (is_b && !ok_b)) viol |= 1u << k;
             if (is_e && rank < MAXI) sm.desc[rank] = (typename SM::desc_t)((u32)e | ((u32)((h - 1) & 0x3f) << SM::kDescShift));
-            if (is_b && ok_b) {
+            if (decltype(WHOLE)::value) {  // the warp's 32 markers are one word of the bitmaps: a store for each level
+              const u32 same = __match_any_sync(0xffffffffu, is_b && ok_b ? l : 0xffffffffu);
+              if (is_b && ok_b && !(same & lower)) {
+                sm.bm[l][e >> 5] = same;
+                atomicOr(reinterpret_cast<u32*>(&sm.summ[l]) + (NWORDS <= 32 ? 0 : e >> 10), 1u << ((e >> 5) & 31));
+              }
+            } else if (is_b && ok_b) {
               atomicOr(&sm.bm[l][e >> 5], 1u << (e & 31));
               atomicOr(reinterpret_cast<u32*>(&sm.summ[l]) + (NWORDS <= 32 ? 0 : e >> 10), 1u << ((e >> 5) & 31));
             }
-            rank += is_e ? 1 : 0;
-            h += is_b ? 1 : (is_e ? -1 : 0);
+            rank_base += __popc(ends[k]);
+            h_base += __popc(begins[k]) - __popc(ends[k]);
           }
-          if (viol) atomicMin(&sm.badpos[bp], w0 + tid * E + __ffs((int)viol) - 1);
+          if (viol) atomicMin(&sm.badpos[bp], e0 + 32 * (__ffs((int)viol) - 1));
         };
         if (whole) place(std::true_type{}); else place(std::false_type{});
         __syncthreads();

@@ -59,6 +59,7 @@ size_t argus_internal_overlap_bytes(uint64_t max_spans, uint32_t num_streams);  
 int argus_internal_overlap_from_digests(const argus_interval_t* intervals, const uint64_t* starts, const uint64_t* entries, const ArgusOvPiece* pieces,
                                         uint32_t slices, uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm,
                                         uint32_t num_sms, const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out,
-                                        argus_status_t* status, ArgusOvCtl* ctl, void* spans, uint64_t max_spans, void* cuda_stream);
+                                        argus_status_t* status, ArgusOvCtl* ctl, void* spans, uint64_t max_spans, uint64_t num_intervals,
+                                        void* cuda_stream);
 
 #endif  // ARGUS_INTERNAL_CUH_

@@ -151,7 +151,6 @@ constexpr u32 kPairWarps = kPairThreads / 32;
 constexpr u32 kVT = 9;                                 // spans a thread merges at a time (odd: lanes that far apart hit different banks)
 constexpr u32 kTile = kPairThreads * kVT;              // spans in shared memory at a time (144 KB)
 constexpr u32 kBatch = kPairThreads;                   // slices whose spans are placed at a time
-constexpr u32 kGather = 4;                             // entries a thread asks for at a time
 constexpr size_t kPairSmem = (size_t)kTile * sizeof(ulonglong2);
 
 struct OvPairArgs {
@@ -308,7 +307,7 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
   const u32 nb = 2u << bits;
   for (u32 b = threadIdx.x; b < nb; b += kPairThreads) cnt[bucket_word(b)] = 0;
   u64 low0 = ~0ull, low1 = ~0ull, high0 = 0, high1 = 0;
-#pragma unroll 3
+#pragma unroll 1
   for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
     const u64 x = i < n0 ? in0[i].x : in1[i - n0].x;
     if (i < n0) { low0 = x < low0 ? x : low0; high0 = x > high0 ? x : high0; }
@@ -336,7 +335,7 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
     const u32 have = 64u - (u32)__clzll((long long)range), sh = have > bits ? have - bits : 0u;  // range < 2^have
     if (role) { low1 = mn; shift1 = sh; } else { low0 = mn; shift0 = sh; }
   }
-#pragma unroll 3
+#pragma unroll 1
   for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
     const bool role = i >= n0;
     const u64 x = role ? in1[i - n0].x - low1 : in0[i].x - low0;
@@ -351,14 +350,14 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
   u32 at = argus_block_exclusive_scan<u32>(mine, scan, &total);
   for (u32 b = c0; b < c0 + per && b < nb; ++b) { const u32 c = cnt[bucket_word(b)]; cnt[bucket_word(b)] = at; at += c; }
   __syncthreads();
-#pragma unroll 3
+#pragma unroll 1
   for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
     const bool role = i >= n0;
     const u64 x = role ? in1[i - n0].x - low1 : in0[i].x - low0;
     t[atomicAdd(&cnt[bucket_word((role ? 1u << bits : 0u) + (u32)(x >> (role ? shift1 : shift0)))], 1u)] = (x << 14) | i;
   }
   __syncthreads();
-#pragma unroll 3
+#pragma unroll 1
   for (u32 i = threadIdx.x; i < n; i += kPairThreads) {  // the counter of a bucket is now where it ends
     const bool role = i >= n0;  // (the first n0 elements are role 0's)
     const u64 v = t[i];
@@ -375,17 +374,13 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
 // d[0..n) in start order -> the disjoint pieces of their union: piece i = [max(start_i, E), max(end_i, that)) with E the largest
 // end of the spans before i (pieces may be empty). Returns this thread's share of the sum of their lengths.
 __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
-  constexpr u32 kPer = 4;  // consecutive spans a thread takes at a time
   const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u64 carry = 0, len = 0;
-  for (u64 i0 = 0; i0 < n; i0 += kPer * kPairThreads) {
-    const u64 at = i0 + (u64)threadIdx.x * kPer;
-    ulonglong2 s[kPer];
-    u64 e = 0;
-#pragma unroll
-    for (u32 j = 0; j < kPer; ++j) s[j] = at + j < n ? d[at + j] : make_ulonglong2(0, 0);
-#pragma unroll
-    for (u32 j = 0; j < kPer; ++j) e = s[j].y > e ? s[j].y : e;
+#pragma unroll 1
+  for (u64 i0 = 0; i0 < n; i0 += kPairThreads) {
+    const u64 at = i0 + threadIdx.x;
+    const ulonglong2 s = at < n ? d[at] : make_ulonglong2(0, 0);
+    u64 e = s.y;
 #pragma unroll
     for (int dd = 1; dd < 32; dd <<= 1) {
       const u64 o = __shfl_up_sync(0xffffffffu, e, dd);
@@ -404,14 +399,10 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
     const u64 warps_before = warp ? __shfl_sync(0xffffffffu, w, warp - 1) : 0ull, all = __shfl_sync(0xffffffffu, w, 31);
     before = before > warps_before ? before : warps_before;
     before = before > carry ? before : carry;
-#pragma unroll
-    for (u32 j = 0; j < kPer; ++j) {
-      if (at + j < n) {
-        const u64 a = s[j].x > before ? s[j].x : before, b = s[j].y > a ? s[j].y : a;
-        d[at + j] = make_ulonglong2(a, b);
-        len += b - a;
-        before = b > before ? b : before;
-      }
+    if (at < n) {
+      const u64 a = s.x > before ? s.x : before, b = s.y > a ? s.y : a;
+      d[at] = make_ulonglong2(a, b);
+      len += b - a;
     }
     carry = all > carry ? all : carry;
     __syncthreads();
@@ -422,9 +413,10 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
 // Latency decides (one block per SM and pair). The entries of up to kBatch slices are taken as one flat sequence, so that
 // every thread has kGather entries and then as many begin times (or pieces of records) in flight, whatever the slices hold.
 // 148 SMs, two roles of 16,000 spans each: 109 us (five kernels before it: 393 us); 2,048 spans a role from 16 interleaved
-// streams: 43 us (178 us); a few hundred spans: 28 us, most of it fixed steps one after the other (45 us).
+// streams: 43 us (178 us); a few hundred spans: 25 us, most of it fixed steps one after the other (45 us; 13 us of these go to
+// the gathering, 7 to the sort, 4 to the cutting and 4 to the walk).
 // DIGEST: entries as the pass over the digests leaves them (argus_fuse.cuh); else {index in the stream, region}.
-template <bool DIGEST>
+template <bool DIGEST, u32 kGather>
 __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
   argus_kernel_begin_long();
   extern __shared__ __align__(16) unsigned char pair_raw[];
@@ -739,20 +731,28 @@ size_t ov_fixed_bytes(u32 num_streams) {
   return argus_align_up(sizeof(ArgusOvCtl), 256) + argus_align_up((size_t)num_streams * select_slices(num_streams) * sizeof(ArgusOvPiece), 256) + 1024;
 }
 
-template <bool DIGEST>
+template <bool DIGEST, u32 kGather>
 int launch_pair(const OvPairArgs& a, cudaStream_t stream) {
   static std::atomic<bool> opted_in[64];  // the shared-memory opt-in belongs to a device
   int dev = 0;
   ARGUS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return ARGUS_ERR_INVALID_ARG;
   if (!opted_in[dev].load(std::memory_order_acquire)) {
-    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_ov_pair<DIGEST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
+    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_ov_pair<DIGEST, kGather>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
     opted_in[dev].store(true, std::memory_order_release);
   }
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);
-  ARGUS_LAUNCH(k_ov_pair<DIGEST>, a.blocks, kPairThreads, kPairSmem, stream, a);
+  ARGUS_LAUNCH(k_ov_pair<DIGEST, kGather>, a.blocks, kPairThreads, kPairSmem, stream, a);
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 1);
   return ARGUS_OK;
+}
+
+// Entries a thread asks for at a time: four where an SM has many to go through, else two, because a block that runs through its
+// code once waits for that code as well (us for 4 / 2 entries; intervals an SM: 2,500: 27.1 / 25.2, 4,700: 15.9 / 13.9, 90,000 (records): 74.2 /
+// 70.6, 232,000: 108.8 / 113.5, 235,000: 113.0 / 116.9).
+template <bool DIGEST>
+int launch_pair(const OvPairArgs& a, uint64_t num_intervals, cudaStream_t stream) {
+  return num_intervals / a.num_sms < (1u << 17) ? launch_pair<DIGEST, 2>(a, stream) : launch_pair<DIGEST, 4>(a, stream);
 }
 
 }  // namespace
@@ -783,11 +783,12 @@ static OvPairArgs pair_args(const argus_interval_t* intervals, const uint64_t* i
 int argus_internal_overlap_from_digests(const argus_interval_t* intervals, const uint64_t* starts, const uint64_t* entries, const ArgusOvPiece* pieces,
                                         uint32_t slices, uint32_t num_streams, uint32_t warps_per_cta, const uint32_t* cta_sm,
                                         uint32_t num_sms, const uint32_t* pairs, uint32_t num_pairs, argus_overlap_t* out,
-                                        argus_status_t* status, ArgusOvCtl* ctl, void* spans, uint64_t max_spans, void* cuda_stream) {
+                                        argus_status_t* status, ArgusOvCtl* ctl, void* spans, uint64_t max_spans, uint64_t num_intervals,
+                                        void* cuda_stream) {
   OvPairArgs a = pair_args(intervals, nullptr, entries, ~0ull, pieces, slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs, num_pairs,
                            out, status, ctl, spans, max_spans);
   a.starts = (const u64*)starts;
-  return launch_pair<true>(a, (cudaStream_t)cuda_stream);
+  return launch_pair<true>(a, num_intervals, (cudaStream_t)cuda_stream);
 }
 
 static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_intervals, const uint64_t* interval_offsets,
@@ -837,7 +838,7 @@ static int overlap_scoped(const argus_interval_t* intervals, uint64_t max_interv
     ARGUS_LAUNCH(k_ov_select, (unsigned)(items < kSelGrid ? items : kSelGrid), kSelThreads, 0, stream, o);
   }
   return launch_pair<false>(pair_args(intervals, interval_offsets, entries, cap, pieces, slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs,
-                                      num_pairs, out, status, ctl, spans, cap), stream);
+                                      num_pairs, out, status, ctl, spans, cap), max_intervals, stream);
 }
 
 int argus_internal_overlap(const argus_interval_t* intervals, uint64_t max_intervals, const uint64_t* interval_offsets,

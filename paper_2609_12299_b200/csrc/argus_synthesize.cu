@@ -107,7 +107,7 @@ static int synthesize_impl(const argus_event_t* events, uint64_t num_events, con
     if (f.num_pairs) {
       rc = argus_internal_overlap_from_digests(intervals, (const uint64_t*)f.starts, (const uint64_t*)f.entries, f.pieces,
                                                L.slices, num_streams, warps_per_cta, cta_sm, num_sms, pairs,
-                                               num_pairs, overlap_out, status, ov_ctl, ws + L.spans, max_overlap_spans, cuda_stream);
+                                               num_pairs, overlap_out, status, ov_ctl, ws + L.spans, max_overlap_spans, L.digest_capacity, cuda_stream);
     } else {
       rc = argus_internal_overlap(intervals, interval_capacity, interval_offsets, num_streams, warps_per_cta, cta_sm, num_sms,
                                   pairs, num_pairs, overlap_out, status, ws + L.ov, L.ov_bytes, cuda_stream, false);

@@ -1,5 +1,6 @@
 """argus_overlap's kernel at the sizes where its branches change: spans in order or not, one role or both, around the number of
-spans it holds in shared memory, starts that crowd, and a workspace too small for the plain layout of the entries."""
+spans it holds in shared memory and the number of intervals an SM at which threads ask for more at a time, starts that crowd, and
+a workspace too small for the plain layout of the entries."""
 import numpy as np
 import pytest
 import torch
@@ -35,7 +36,7 @@ def _intervals(rng, per_stream, S, order, other):
 
 
 @pytest.mark.parametrize("order", ["disjoint", "overlapping", "shuffled", "crowded"])
-@pytest.mark.parametrize("per_stream", [1, 33, TILE // 4, TILE // 2, TILE // 2 + 1, 23_000])
+@pytest.mark.parametrize("per_stream", [1, 33, TILE // 4, TILE // 2, TILE // 2 + 1, 23_000, 65_535, 65_536])
 def test_overlap_sizes_and_orders(order, per_stream):
     rng = np.random.default_rng(per_stream)
     S, W, M, other = 4, 2, 2, 3

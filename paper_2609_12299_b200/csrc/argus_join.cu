@@ -100,7 +100,11 @@ __device__ __forceinline__ void join_ranks(const u64* vals, u32 n, JoinRanks& sh
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kJoinThreads) k_join(const argus_interval_t* reference, u64 num_reference,
+// Bound by the keys in flight (few blocks where queries are few; five per SM, by shared memory, where they are many), so a
+// thread asks for eight at a time: 8 queries against 614 M samples 1,298 -> 430 ms (four: 539), 2,000 queries with a stream of
+// 259,328 samples each 4.98 -> 4.29 ms (four: 4.45).
+constexpr u32 kJoinAhead = 8;
+__global__ void __launch_bounds__(kJoinThreads, 5) k_join(const argus_interval_t* reference, u64 num_reference,
                                                        const u64* ref_index, u32 num_queries,
                                                        const argus_interval_t* samples, u64 num_samples,
                                                        const u64* sample_offsets, u32 num_runs, u32 num_streams,
@@ -139,16 +143,24 @@ __global__ void __launch_bounds__(kJoinThreads) k_join(const argus_interval_t* r
           continue;
         }
       }
-      for (u64 i = lo + tid; i < hi; i += kJoinThreads) {
-        const uint4* p = reinterpret_cast<const uint4*>(samples + i);
-        const uint4 q1 = __ldg(p + 1);
-        if (q1.z != key_region || q1.w != key_ctx) continue;
-        if (__ldg(reinterpret_cast<const u32*>(p + 2)) != key_stream) continue;
-        const uint4 q0 = __ldg(p);
-        const u64 v = (u64)q0.z | ((u64)q0.w << 32);
-        sum += v;
-        const u32 slot = atomicAdd(&cnt, 1u);
-        if (slot < ARGUS_JOIN_MAX_SAMPLES) vals[slot] = v;
+      for (u64 i0 = lo + tid; i0 < hi; i0 += (u64)kJoinThreads * kJoinAhead) {
+        uint2 key[kJoinAhead];  // region, ctx
+#pragma unroll
+        for (u32 j = 0; j < kJoinAhead; ++j) {
+          const u64 i = i0 + j * kJoinThreads;
+          key[j] = i < hi ? __ldg(reinterpret_cast<const uint2*>(samples + i) + 3) : make_uint2(~key_region, 0u);
+        }
+#pragma unroll
+        for (u32 j = 0; j < kJoinAhead; ++j) {
+          if (key[j].x != key_region || key[j].y != key_ctx) continue;
+          const uint4* p = reinterpret_cast<const uint4*>(samples + i0 + j * kJoinThreads);
+          if (__ldg(reinterpret_cast<const u32*>(p + 2)) != key_stream) continue;
+          const uint4 q0 = __ldg(p);
+          const u64 v = (u64)q0.z | ((u64)q0.w << 32);
+          sum += v;
+          const u32 slot = atomicAdd(&cnt, 1u);
+          if (slot < ARGUS_JOIN_MAX_SAMPLES) vals[slot] = v;
+        }
       }
     }
 #pragma unroll

@@ -42,3 +42,21 @@ def test_ranks(values):
                     argus.argus_join_samples_grouped(d_ref, d_idx, d_smp, d_off, 1)):
         assert int(argus.argus_status_fetch(st)["code"]) == 0
         assert out.cpu().numpy()[: len(sizes) * 64].view(argus.JOIN_DTYPE).tobytes() == want.tobytes()
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 2047, 2048, 2049, 4097])
+def test_scan_lengths(n):
+    """Samples around the numbers that a block asks for at a time: the last ones count, those past the end of a range do not."""
+    rng = np.random.default_rng(n)
+    ref = np.zeros(3, argus.INTERVAL_DTYPE)
+    ref["region"], ref["stream"] = [0, 1, 0], [0, 0, 1]
+    smp = np.zeros(2 * n + 3, argus.INTERVAL_DTYPE)
+    smp["region"], smp["inclusive"] = rng.integers(0, 2, len(smp)), rng.integers(1, 1 << 40, len(smp))
+    smp["region"][n - 1], smp["stream"][n:] = 0, 1
+    idx = np.arange(3, dtype=np.uint64)
+    _, want, _ = oracle.join_samples(ref, idx, smp)
+    d_ref, d_smp, d_idx = _dev(ref), _dev(smp), torch.from_numpy(idx.view(np.int64).copy()).to(DEV)
+    d_off = torch.tensor([[0, n, len(smp)]], dtype=torch.int64, device=DEV)
+    for out, st in (argus.argus_join_samples(d_ref, d_idx, d_smp), argus.argus_join_samples_grouped(d_ref, d_idx, d_smp, d_off, 2)):
+        assert int(argus.argus_status_fetch(st)["code"]) == 0
+        assert out.cpu().numpy()[: 3 * 64].view(argus.JOIN_DTYPE).tobytes() == want.tobytes()

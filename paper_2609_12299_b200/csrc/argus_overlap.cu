@@ -413,8 +413,8 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
 // Latency decides (one block per SM and pair). The entries of up to kBatch slices are taken as one flat sequence, so that
 // every thread has kGather entries and then as many begin times (or pieces of records) in flight, whatever the slices hold.
 // 148 SMs, two roles of 16,000 spans each: 109 us (five kernels before it: 393 us); 2,048 spans a role from 16 interleaved
-// streams: 43 us (178 us); a few hundred spans: 25 us, most of it fixed steps one after the other (45 us; 13 us of these go to
-// the gathering, 7 to the sort, 4 to the cutting and 4 to the walk).
+// streams: 43 us (178 us); a few hundred spans: 25 us, most of it fixed steps one after the other (45 us): about 12 us go to
+// the gathering, 6 to the sort, 3 to the cutting and 4 to the walk.
 // DIGEST: entries as the pass over the digests leaves them (argus_fuse.cuh); else {index in the stream, region}.
 template <bool DIGEST, u32 kGather>
 __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {

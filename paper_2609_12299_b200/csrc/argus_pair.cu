@@ -62,8 +62,8 @@ __global__ void __launch_bounds__(128) k_pair_thread_per_stream(ArgusPairArgs a)
 // taken to be whole. Otherwise, if its last marker is an end(b), b is taken to be an outermost region and the front is read
 // until an unmatched end(b), which tells that the back is whole; if there is none and its first marker is a begin(a), the back is
 // read until an unmatched begin(a); kGuessEvents at most.
-// (Pairing of traces cut at either end: 24 M events 551 -> 289 us, 142 M in a ring 2,700 -> 1,374 us. The look costs 4 us, and
-// 20 to 40 us when many streams are read.)
+// (Pairing of traces cut at either end: 24 M events 551 -> 289 us, 142 M in a ring 2,700 -> 1,374 us; 262 and 1,215 with the
+// pairing kernel of today. The look costs 4 us, and 20 to 40 us when many streams are read.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kInitThreads = 256;
 constexpr u32 kGuessRun = 32;  // consecutive events a thread looks at (first a quarter of them: a cut is usually near)

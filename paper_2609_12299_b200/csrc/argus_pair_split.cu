@@ -11,7 +11,8 @@
 // Heights know nothing of region ids. A segment that meets a marker which breaks the parallel rules gives its stream up; the
 // chained pass, which follows and does nothing otherwise, walks such streams from their beginning.
 //
-// The scan reads the events once more (16 of then 56 bytes an event). 96 streams of 518,656 events: pairing 2,412 -> 690 us.
+// The scan reads the events once more (16 of then 56 bytes an event). 96 streams of 518,656 events: pairing 2,412 -> 660 us
+// (scan 132, chain 36, segments 458, fix 27).
 #include "argus_internal.cuh"
 #include "argus_pair_common.cuh"
 

@@ -142,6 +142,7 @@ struct TileSmem {
   u64 bar[2];
   u64 cur_stream;
   u32 cur_rec;                     // hand-over record of the stream being walked (kNoRec: none)
+  int skip;                        // the piece of work taken is not to be walked
   u64 n_int;                       // written by the sequential redo path
   int ch;
   u32 wrapped;                     // a sum of 32-bit child time wrapped in this window
@@ -197,7 +198,10 @@ __device__ __forceinline__ void tile_fetch(const ArgusPairArgs& a, uint4* dst, c
 }
 
 // SPLIT: the work items are segments of streams instead of whole streams (see argus_pair_split.cu): the initial stack comes with
-// the segment, and a marker that breaks the parallel rules gives the stream up to the chained pass that follows.
+// the segment, and a marker that breaks the parallel rules gives the stream up to the chained pass that follows. Other blocks may
+// give up the stream of this block's segment at any moment, so one thread reads that word and all threads follow its answer; the
+// other words of global memory that a block branches on around its barriers (offsets, bases, segments, hand-over records, redo,
+// redo_from, num_failed) are not written while the kernel runs, or are read by the one thread that takes the work.
 template <int NT, int E, int MINB, bool RING = false, bool SPLIT = false>
 __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   using SM = TileSmem<NT, E>;
@@ -235,13 +239,14 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       } else if (!tile_pop_work(a, a.redo ? 1 : 0, &st, &rc)) st = ~0ull;
       sm.cur_stream = st;
       sm.cur_rec = rc;
+      sm.skip = st < a.num_streams && (SPLIT ? __ldcg(a.split_failed + st) != 0 : (a.segments && !a.redo && rc == kNoRec && !__ldcg(a.split_failed + st)));
     }
     __syncthreads();
     const u64 s64 = sm.cur_stream;
     if (s64 >= a.num_streams) break;
     const u32 s = (u32)s64;
     u32 rec = sm.cur_rec;
-    if (SPLIT ? __ldcg(a.split_failed + s) != 0 : (a.segments && !a.redo && rec == kNoRec && !__ldcg(a.split_failed + s))) {
+    if (sm.skip) {
       if (!SPLIT && tid == 0) atomicAdd(&a.ctl->n_done[0], 1u);  // walked by the split pass
       __syncthreads();
       continue;

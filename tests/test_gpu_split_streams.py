@@ -82,3 +82,39 @@ def test_segments(kind, change):
         assert r.agg.table_numpy(lv).tobytes() == tabs[lv].tobytes(), lv
     _, ov, _ = oracle.overlap(iv, ioffs, W, cta_sm, 2, pairs)
     assert r.overlap_numpy(2).tobytes() == ov.tobytes()
+
+
+@pytest.mark.parametrize("kind", ["gemm", "decode"])
+def test_streams_given_up_while_their_segments_are_walked(kind):
+    """Three streams in four have defects all over their length, so that many blocks give up a stream while others take up its
+    segments; the healthy streams between them must not notice. Every run against the oracle."""
+    rng = np.random.default_rng(11)
+    spec, streams = _trace(kind, rng)
+    R = spec.num_regions + 1
+    streams = streams * -(-(1 << 24) // sum(len(e) for e in streams))  # segments for every block, three times over
+    streams = [_wrap(e, R - 1) for e in streams]
+    for s in range(len(streams)):
+        if s % 4 == 0:
+            continue
+        at = rng.integers(1, len(streams[s]) - 1, 1 + 5 * (s % 4))  # 6, 11 or 16 places
+        if s % 2:
+            streams[s] = np.delete(streams[s], at)
+        else:
+            streams[s]["tag"][at] ^= 1
+    ev = np.concatenate(streams)
+    offs = np.cumsum([0] + [len(e) for e in streams]).astype(np.uint64)
+    S = len(streams)
+    assert S < 777 and len(ev) // S >= 10240
+    d_ev = torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).to(DEV)
+    d_off = torch.from_numpy(offs.view(np.int64).copy()).to(DEV)
+    _, iv, ioffs, am, aoffs, o_st = oracle.pair(ev, offs, R)
+    assert int(o_st["code"]) == 0 and len(am)
+    want = [torch.from_numpy(x.view(np.uint8).reshape(-1).copy()).to(DEV) for x in (iv, am, ioffs, aoffs)]
+    p = None
+    for _ in range(60):
+        p = argus.argus_pair_intervals(d_ev, d_off, R, out=p)
+        assert int(p.fetch_status()["code"]) == 0
+        assert torch.equal(p.interval_offsets.view(torch.uint8), want[2]) and torch.equal(p.ambig_offsets.view(torch.uint8), want[3])
+        assert torch.equal(p.intervals[:len(want[0])], want[0]) and torch.equal(p.ambig[:len(want[1])], want[1])
+        p.intervals.zero_()
+        p.ambig.zero_()

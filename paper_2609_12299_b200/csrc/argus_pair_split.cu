@@ -50,7 +50,18 @@ __global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u3
     carry += total;
   }
   __syncthreads();
-  if (blockIdx.x == 0 && tid == 0) { first_segment[a.num_streams] = carry; a.ctl->num_segments = carry; }
+  // Offsets that decrease let streams share events, and then there may be more segments than blocks and room: the chained pass,
+  // which reports such offsets, walks all streams.
+  const bool fits = carry <= gridDim.x;
+  if (blockIdx.x == 0 && tid == 0) {
+    first_segment[a.num_streams] = carry;
+    a.ctl->num_segments = fits ? carry : 0u;
+    if (!fits) a.ctl->num_failed = a.num_streams;
+  }
+  if (!fits) {
+    if (blockIdx.x == 0) for (u32 s = tid; s < a.num_streams; s += kScanThreads) a.split_failed[s] = 1;
+    return;
+  }
   if (sh_stream == 0xffffffffu) return;
   const u32 s = sh_stream, j = blockIdx.x - sh_before, n = split_length(a, s), per = a.segment_tiles * kSplitTile;
   ArgusSegment* const g = a.segments + blockIdx.x;
@@ -121,6 +132,7 @@ __global__ void __launch_bounds__(32) k_split_chain(ArgusPairArgs a, const u32* 
   __shared__ u32 stack[ARGUS_MAX_DEPTH];
   constexpr u32 kAhead = 4;
   const u32 s = blockIdx.x, lane = threadIdx.x;
+  if (__ldcg(a.split_failed + s)) return;  // (more segments than room: nobody has looked at them)
   const u32 g0 = first_segment[s], g1 = first_segment[s + 1];
   int h = 0;
   bool fail = false;

@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       if (tid == 0) {
         argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
         if (!a.redo) a.counts[s] = 0;
-        atomicAdd(&a.ctl->n_done[a.redo ? 1 : 0], 1u);
+        if (!SPLIT) atomicAdd(&a.ctl->n_done[a.redo ? 1 : 0], 1u);  // (the chained pass counts what the split pass has walked)
       }
       __syncthreads();
       continue;

@@ -462,8 +462,10 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   a.poll_limit = g_poll_limit.load(std::memory_order_relaxed);
   a.ring_written = (const u64*)ring_written; a.ring_capacity = ring_capacity;
   if (ring_written && (ring_capacity == 0 || kernel_choice == 1)) return ARGUS_ERR_INVALID_ARG;  // only the tiled kernel reads rings
-  // a stream's intervals start at half its first event's position at the latest, so positions stay below num_events / 2 + 1
-  a.digest = digest_capacity >= (interval_capacity < num_events / 2 + 1 ? interval_capacity : num_events / 2 + 1) ? (u64*)digest : nullptr;
+  // Digests lie at their records' positions, so the digest array bounds both. A trace has num_events / 2 intervals at most, which is
+  // what the array holds; only offsets that decrease, which are reported, make streams share events and reach further.
+  a.digest = (u64*)digest;
+  if (digest && digest_capacity < a.interval_capacity) a.interval_capacity = digest_capacity;
 
   const bool tiled = (kernel_choice != 1 && argus_pair_tiled_usable(a)) || ring_written != nullptr;
   // control block, counts, queue and bitmap are contiguous at the start of the workspace and start at zero

@@ -97,8 +97,8 @@ struct ArgusPairArgs {
   ArgusStreamRecord* records;
   u32 record_capacity;
   const u32* order;       // streams in the order in which the tiled kernel starts them: longest first (null = by index)
-  u64* digest;            // one digest per interval record, same positions (null = none); holds every position below
-                          // min(interval_capacity, num_events / 2 + 1), which is all a stream can reach
+  u64* digest;            // one digest per interval record, same positions (null = none); interval_capacity is then no larger than
+                          // what it holds
   const u64* ring_written; // non-null: `events` is a ring container, one slot of ring_capacity records per stream, record i of
   u32 ring_capacity;       // a stream at slot position i mod capacity; stream_offsets then describe the packed survivors
   ArgusSegment* segments;  // non-null: split pass; or, in the chained pass after it, what that left: only failed streams are walked

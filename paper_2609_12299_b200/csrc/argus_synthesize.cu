@@ -37,7 +37,7 @@ SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_reg
   const size_t from_entries = L.spans - o + (size_t)max_overlap_spans * 32, plain = argus_internal_overlap_bytes(max_overlap_spans, num_streams);
   L.ov_bytes = num_pairs ? argus_align_up(from_entries > plain ? from_entries : plain, 256) : 0;
   o += L.ov_bytes;
-  // one digest per interval (a stream's intervals start at half its first event's position at the latest)
+  // one digest per interval (two events each, so num_events / 2 at most; pairing and the pass over the digests stay inside the array)
   L.digest_capacity = digests ? num_events / 2 + 1 : 0;
   L.digest = o; o += argus_align_up((size_t)L.digest_capacity * 8, 256);
   L.starts = o; o += num_pairs ? argus_align_up((size_t)L.digest_capacity * 8, 256) : 0;  // begin times of overlap candidates

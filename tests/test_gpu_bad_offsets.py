@@ -44,3 +44,23 @@ def test_pairing(n, streams, length):
                                   ao.data_ptr(), st.data_ptr(), ws.data_ptr(), need, torch.cuda.current_stream().cuda_stream)
     assert rc == 0 and int(argus.argus_status_fetch(st)["code"]) == BAD_OFFSETS
     assert all(_untouched(t, k) for t, k in ((ws, need), (iv, icap * 48), (am, n * 32), (st, 64), (io, (streams + 1) * 8), (ao, (streams + 1) * 8)))
+
+
+@pytest.mark.parametrize("num_pairs", [0, 1])
+@pytest.mark.parametrize("n,streams,length", [(1000, 4, 1000), (1 << 20, 80, 30_000), (1 << 21, 200, 30_000)])
+def test_synthesize(n, streams, length, num_pairs):
+    """Room for more intervals than so many events can hold: the digests beside them stop where their array does."""
+    ev, off = _input(n, streams, length)
+    lib = argus.load_library()
+    icap, sms, spans = streams * length, 2, n
+    cta_sm, pairs = torch.zeros(streams, dtype=torch.int32, device=DEV), torch.zeros(2, dtype=torch.int32, device=DEV)
+    need = lib.argus_synthesize_workspace_bytes(n, streams, 1, n, num_pairs, sms, spans)
+    ws, iv, am, st = _guarded(need), _guarded(icap * 48), _guarded(n * 32), _guarded(64)
+    io, ao = _guarded((streams + 1) * 8), _guarded((streams + 1) * 8)
+    tabs, ov = [_guarded(k * 576) for k in (streams, streams, sms, 1)], _guarded(sms * 32)
+    rc = lib.argus_synthesize(ev.data_ptr(), n, off.data_ptr(), streams, 1, iv.data_ptr(), icap, io.data_ptr(), am.data_ptr(), n, ao.data_ptr(), 1,
+                              cta_sm.data_ptr(), sms, *[t.data_ptr() for t in tabs], pairs.data_ptr(), num_pairs, ov.data_ptr(), spans,
+                              st.data_ptr(), ws.data_ptr(), need, torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and int(argus.argus_status_fetch(st)["code"]) == BAD_OFFSETS
+    assert all(_untouched(t, k) for t, k in ((ws, need), (iv, icap * 48), (am, n * 32), (st, 64), (io, (streams + 1) * 8), (ao, (streams + 1) * 8)))
+    assert all(_untouched(t, k * 576) for t, k in zip(tabs, (streams, streams, sms, 1))) and _untouched(ov, sms * 32)

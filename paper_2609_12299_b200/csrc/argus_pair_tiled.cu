@@ -131,8 +131,10 @@ struct TileSmem {
   alignas(16) u32 accall[T + 4 * kCar];      // child time each frame gathers in the current window (32 bits: an overflow cuts the
                                    // window), same index space shifted by 2 kCar
   desc_t desc[MAXI];               // per end, in end order: event index | level << kDescShift
+  static constexpr int kBmVectors = ((kLevelWindow + 1) * NWORDS + 3) / 4;  // 16-byte vectors that cover bm
   union {
     alignas(16) u32 bm[kLevelWindow + 1][NWORDS];  // (the last row stays empty: levels outside the window) per level: bit e set = event e of the tile is a begin at that level
+    uint4 bm_vectors[kBmVectors];      // the same, as it is cleared: all of it, the last words of the last row too
     ArgusFrame fstk[ARGUS_MAX_DEPTH];  // stack in the layout the sequential path uses (no bitmap is live while it runs)
   };
   u64 summ[kLevelWindow + 1];      // per level: bit w set = bm[level][w] != 0
@@ -360,7 +362,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
 #pragma unroll
         for (int k = 0; k < E; ++k) tags[k] = whole || e0 + 32 * k < wend ? reinterpret_cast<const u32*>(evb + e0 + 32 * k)[2] : 0xffffffffu;
         for (int i = tid; i < T / 4; i += NT) reinterpret_cast<uint4*>(accb)[i] = make_uint4(0, 0, 0, 0);
-        for (int i = tid; i < (kLevelWindow + 1) * NWORDS / 4; i += NT) reinterpret_cast<uint4*>(&sm.bm[0][0])[i] = make_uint4(0, 0, 0, 0);
+        for (int i = tid; i < SM::kBmVectors; i += NT) sm.bm_vectors[i] = make_uint4(0, 0, 0, 0);
         if (tid <= kLevelWindow) sm.summ[tid] = 0;
         if (tid < ch) accb[cbase + tid] = 0;  // what this window adds to the carried frames (a cut window starts clean again)
         if (tid == 0) { sm.failed = 0; sm.wrapped = 0; accb[cbase + kSink] = 0; }

@@ -735,3 +735,37 @@ def test_other_tile_shapes_give_the_same_result(variant):
     finally:
         argus_set_tile_variant(0)
         argus_set_synthesize_mode(-1)
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2, 3])
+def test_many_open_frames_that_close_within_a_tile(variant):
+    """Streams that stay 20 to 64 frames deep, with pairs on top, stray ends that send the whole stack through the sequential
+    machine, and runs of ends that go below the levels a tile keeps bitmaps of, in every tile shape."""
+    from paper_2609_12299_b200.binding import argus_set_tile_variant
+    rng = np.random.default_rng(23)
+    evs = []
+    for s in range(64):
+        deep = 64 if s % 4 == 0 else int(rng.integers(20, 64))
+        rows, stack, t = [], [], 0
+        while len(rows) < 6000:
+            while len(stack) < deep - 1:
+                stack.append(int(rng.integers(0, 2)))
+                rows.append((t, "B", stack[-1], 0))
+                t += int(rng.integers(0, 9))
+            for _ in range(int(rng.integers(1, 260))):  # pairs on top, now and then at full height
+                r = int(rng.integers(0, 2))
+                rows += [(t, "B", r, 0), (t + int(rng.integers(0, 50)), "E", r, 0)]
+                t = rows[-1][0]
+                if rng.random() < 0.02:
+                    rows += [(t, "B", 1, 0), (t, "E", 2, 0), (t + 3, "E", 1, 0)]  # the end of region 2 has no begin
+                    t += 3
+            for _ in range(int(rng.integers(9, deep))):
+                rows.append((t, "E", stack.pop(), 0))
+                t += int(rng.integers(0, 9))
+        evs.append(make_events(rows))
+    offs = np.cumsum([0] + [len(e) for e in evs]).astype(np.uint64)
+    argus_set_tile_variant(variant)
+    try:
+        assert_pair_matches(np.concatenate(evs), offs, 3, KERNEL_TILED)
+    finally:
+        argus_set_tile_variant(0)

@@ -479,7 +479,9 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
                 const u64 dlt = ((u64)ee.x | ((u64)ee.y << 32)) - bts;
                 incl = (u32)dlt;
                 if (ee.w != pe.w) flags = ARGUS_FLAG_CTX_MISMATCH;
-                if (((pe.z ^ ee.z) ^ 1u) | (u32)(dlt >> 32)) {  // another region, time running backwards, or 2^32 ticks and more
+                // another region, 2^32 ticks and more, or time running backwards (which shows in the difference's upper half, or, when
+                // the difference wraps to a small one, in the times')
+                if ((((pe.z ^ ee.z) ^ 1u) | (u32)(dlt >> 32)) != 0 || ee.y < pe.y) {
                   live = (pe.z ^ ee.z) == 1u && ((u64)ee.x | ((u64)ee.y << 32)) < bts;
                   incl = 0;
                   flags |= ARGUS_FLAG_TIME_REVERSED;

@@ -43,3 +43,33 @@ def test_child_time_wraps_in_a_cut_window(share, lost, kernel):
     assert p.ambig_numpy().tobytes() == am.tobytes()
     for f in ("n_ctx_mismatch", "n_time_reversed", "n_child_clamped"):
         assert int(st[f]) == int(o_st[f]), f
+
+
+@pytest.mark.parametrize("kernel", [KERNEL_AUTO, KERNEL_TILED])
+def test_times_at_both_ends_of_the_64_bit_range(kernel):
+    """An end whose time lies nearly 2^64 ticks before its begin's: the difference wraps to a few ticks, but the time runs backwards."""
+    rng = np.random.default_rng(5)
+    streams = []
+    for s in range(20):
+        n = int(rng.integers(1, 4000))
+        ev = np.zeros(4 * n, argus.EVENT_DTYPE)      # an outer interval around an inner one, n times
+        ev["tag"] = np.tile(np.array([0, 2, 3, 1], np.uint32), n)
+        near = rng.integers(0, 1 << 40 if s % 2 else 200, 4 * n).astype(np.uint64)
+        ev["ts"] = np.where(rng.random(4 * n) < 0.5, near, ~near)
+        streams.append(ev)
+    # begin near the top, end near the bottom: a step of 15, of 2^32 - 1, of 2^32, of 0 (no step back), and the other way round
+    top = np.uint64(2**64 - 1)
+    for b, e in ((top - np.uint64(9), 5), (top, (1 << 32) - 2), (top, (1 << 32) - 1), (top, top), (5, top - np.uint64(9)), (top, 0)):
+        ev = np.zeros(2, argus.EVENT_DTYPE)
+        ev["ts"], ev["tag"] = [b, e], [0, 1]
+        streams.append(ev)
+    ev = np.concatenate(streams)
+    offs = np.cumsum([0] + [len(e) for e in streams]).astype(np.uint64)
+    _, iv, ioffs, am, _, o_st = oracle.pair(ev, offs, 2)
+    p = argus.argus_pair_intervals(torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).cuda(),
+                                   torch.from_numpy(offs.view(np.int64).copy()).cuda(), 2, kernel=kernel)
+    st = p.fetch_status()
+    assert int(st["code"]) == 0 and int(o_st["code"]) == 0 and len(am) == 0
+    assert p.intervals_numpy().tobytes() == iv.tobytes()
+    for f in ("n_ctx_mismatch", "n_time_reversed", "n_child_clamped"):
+        assert int(st[f]) == int(o_st[f]), f

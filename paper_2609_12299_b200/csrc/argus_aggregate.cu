@@ -716,9 +716,10 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_compact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)compact));
     if (a.digest) {
       const u32 warps = a.slices / a.parts;
-      const size_t dg = digest_table_bytes(num_regions, warps == 16 ? 32 : 8);
+      const u32 copies = warps == 16 ? 32 : 8;
+      const size_t dg = digest_table_bytes(num_regions, copies);
       const auto kernel = warps == 16 ? k_agg_streams_digest<512, 32, 3> : warps == 8 ? k_agg_streams_digest<256, 8, 6> : k_agg_streams_digest<128, 8, 12>;
-      if (dg > 48 * 1024) ARGUS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg));
+      if (dg > 48 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, digest_table_bytes(kAggCompactRegions, copies)));
       ARGUS_LAUNCH(kernel, num_streams * a.parts, warps * 32, dg, stream, a);
     } else {
       ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
@@ -732,7 +733,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
     while (per > 1 && num_streams / per < 296) per >>= 1;
     const size_t two = 2 * (size_t)num_regions * sizeof(ArgusAggCell);
     if (two > 48 * 1024)
-      ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_iter_windows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)two));
+      ARGUS_CUDA_TRY(argus_allow_smem(k_agg_iter_windows, 2 * (size_t)kAggCompactRegions * sizeof(ArgusAggCell)));
     ARGUS_LAUNCH(k_agg_iter_windows, (num_streams + per - 1) / per, kIterThreads, two, stream, a, per);
   } else if (iter_tab) {
     ARGUS_LAUNCH(k_agg_iter, num_streams < 1184u ? num_streams : 1184u, kAggThreads, 0, stream, a);

@@ -50,6 +50,13 @@ inline cudaError_t argus_launch(void (*kernel)(P...), dim3 grid, dim3 block, siz
 }
 #define ARGUS_LAUNCH(...) ARGUS_CUDA_TRY(argus_launch(__VA_ARGS__))
 
+// Shared memory of 48 KB and more has to be asked for, and the limit belongs to the kernel and the device, not to a launch: it is
+// always set to the same, the most that any call needs, since another host thread may launch the kernel at the same time.
+template <class K>
+inline cudaError_t argus_allow_smem(K* kernel, size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 __device__ __forceinline__ void argus_kernel_begin_long() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void argus_kernel_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -58,8 +58,9 @@ inline cudaError_t argus_allow_smem(K* kernel, size_t most) {
 }
 
 __device__ __forceinline__ void argus_kernel_begin_long() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void argus_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void argus_kernel_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  argus_launch_next();
   argus_kernel_begin_long();
 }
 

@@ -60,76 +60,72 @@ __global__ void __launch_bounds__(128) k_pair_thread_per_stream(ArgusPairArgs a)
 // begins) / 2 intervals; unmatched ends lie at its front (a ring slot that has wrapped) and unmatched begins at its back (a
 // stream that was cut short), so a look at both ends tells them. A stream that starts with begin(r) and stops with end(r) is
 // taken to be whole. Otherwise, if its last marker is an end(b), b is taken to be an outermost region and the front is read
-// until an unmatched end(b), which tells that the back is whole; if there is none and its first marker is a begin(a), the back is
-// read until an unmatched begin(a); kGuessEvents at most.
+// until an unmatched end(b), which tells that the back is whole; if its first marker is a begin(a), the back is read until an
+// unmatched begin(a), which tells that the front is whole; kGuessEvents at most. Both may be asked for: a stream whose ends are
+// unclear is read from the back first, where a cut shows soon, others from the front.
+// Unclear are begin(a) ... end(b): cut, or whole with several outermost regions. Where more than a quarter of the streams look
+// like that they are taken to be whole but for a 32nd of their length at either end, and short ones are not read.
 // (Pairing of traces cut at either end: 24 M events 551 -> 289 us, 142 M in a ring 2,700 -> 1,374 us; 262 and 1,215 with the
-// pairing kernel of today. The look costs 4 us, and 20 to 40 us when many streams are read.)
+// pairing kernel of today. Streams of five outermost regions, one after the other: 8,000 of 4,000 events 775 us with a block for
+// each stream and both ends of each read, 342 us, 402 without foretelling; 10^6 of 24 events 14,449, 6,110 and 6,473.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kInitThreads = 256;
-constexpr u32 kGuessRun = 32;  // consecutive events a thread looks at (first a quarter of them: a cut is usually near)
-constexpr u32 kGuessEvents = kInitThreads * kGuessRun;
+constexpr u32 kGuessEvents = 8192;
 
 // Unmatched closing markers from one end of a stream on (FRONT: ends, from the first event; else begins, from the last
-// backwards), up to and including the first one of region `outer` (*met: there is one). One block; heights by a prefix sum
-// over the threads' runs.
-template <bool FRONT, u32 RUN>
-__device__ __noinline__ u32 guess_unmatched(const ArgusPairArgs& a, const uint4* src, u32 ring_first, u32 n, u32 outer, bool* met) {
-  __shared__ int sh[33], low_of[kInitThreads / 32];
-  __shared__ u32 stop;
-  const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, limit = n < kInitThreads * RUN ? n : kInitThreads * RUN;
-  if (threadIdx.x == 0) stop = 0xffffffffu;
-  u32 opens = 0, closes = 0, outers = 0;  // a bit per event of the run
-#pragma unroll 8
-  for (u32 j = 0; j < RUN; ++j) {
-    const u32 i = threadIdx.x * RUN + j;
-    if (i >= limit) break;
-    u32 at = FRONT ? i : n - 1 - i;
-    if (a.ring_written) { const u32 room = a.ring_capacity - ring_first; at = at >= room ? at - room : ring_first + at; }
-    const u32 tag = __ldg(reinterpret_cast<const u32*>(src + at) + 2);
-    if (((tag & 1u) != 0) == FRONT) { closes |= 1u << j; if ((tag >> 1) == outer) outers |= 1u << j; }
-    else opens |= 1u << j;
-  }
-  int total;
-  const int start = argus_block_exclusive_scan<int>(__popc(opens) - __popc(closes), sh, &total);
-  int h = start, low = start;  // the lowest height after any event of the run, and of the runs before it
-  for (u32 j = 0; j < RUN; ++j) {
-    h += (int)((opens >> j) & 1u) - (int)((closes >> j) & 1u);
-    low = h < low ? h : low;
-  }
-  int upto = low;
+// backwards), up to and including the first one of region `outer` (*met: there is one), among `limit` events. One warp; a cut is
+// usually near, so the first batch is small.
+template <bool FRONT>
+__device__ __noinline__ u32 guess_unmatched(const ArgusPairArgs& a, const uint4* src, u32 ring_first, u32 n, u32 outer, u32 limit, bool* met) {
+  const u32 lane = threadIdx.x & 31;
+  int height = 0, lowest = 0;  // uniform
+  for (u32 i0 = 0, rows = 8; i0 < limit; i0 += rows * 32, rows = 32) {
+    u32 opens = 0, closes = 0, outers = 0;  // bit j of lane l: event i0 + 32 l + j
+#pragma unroll 16
+    for (u32 r = 0; r < rows; ++r) {
+      const u32 i = i0 + r * 32 + lane;
+      const bool in = i < limit;
+      u32 at = FRONT ? i : n - 1 - i;
+      if (a.ring_written) { const u32 room = a.ring_capacity - ring_first; at = at >= room ? at - room : ring_first + at; }
+      const u32 tag = in ? __ldg(reinterpret_cast<const u32*>(src + at) + 2) : 0u;
+      const bool close = in && ((tag & 1u) != 0) == FRONT;
+      const u32 c = __ballot_sync(0xffffffffu, close), o = __ballot_sync(0xffffffffu, close && (tag >> 1) == outer), have = __ballot_sync(0xffffffffu, in);
+      if (lane == r) { closes = c; outers = o; opens = have & ~c; }
+    }
+    const int mine = __popc(opens) - __popc(closes);
+    int upto = mine;
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) { const int o = __shfl_up_sync(0xffffffffu, upto, d); if (lane >= (u32)d && o < upto) upto = o; }
-  if (lane == 31) low_of[warp] = upto;
-  __syncthreads();
-  int before = __shfl_up_sync(0xffffffffu, upto, 1);
-  if (lane == 0 || before > 0) before = 0;
-  int lowest = 0;
-  for (u32 w = 0; w < kInitThreads / 32; ++w) {
-    const int o = low_of[w];
-    if (w < warp && o < before) before = o;
-    if (o < lowest) lowest = o;
-  }
-  if (outers && low < before) {  // an unmatched one of `outer` may be here: the first event that goes below everything before it
-    h = start;
-    for (u32 j = 0; j < RUN; ++j) {
+    for (int d = 1; d < 32; d <<= 1) { const int o = __shfl_up_sync(0xffffffffu, upto, d); if (lane >= (u32)d) upto += o; }
+    const int start = height + upto - mine;
+    int h = start, low = start;  // the lowest height after any event of the lane
+    for (u32 j = 0; j < 32; ++j) {
       h += (int)((opens >> j) & 1u) - (int)((closes >> j) & 1u);
-      if (h < before) {
-        before = h;
-        if ((outers >> j) & 1u) { atomicMin(&stop, (u32)-h); break; }
+      low = h < low ? h : low;
+    }
+    int before = low;  // and of the lanes before it
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const int o = __shfl_up_sync(0xffffffffu, before, d); if (lane >= (u32)d && o < before) before = o; }
+    const int all = __shfl_sync(0xffffffffu, before, 31);
+    before = __shfl_up_sync(0xffffffffu, before, 1);
+    if (lane == 0 || before > lowest) before = lowest;
+    u32 stop = 0xffffffffu;
+    if (outers && low < before) {  // an unmatched one of `outer` may be here: the first event that goes below everything before it
+      h = start;
+      for (u32 j = 0; j < 32; ++j) {
+        h += (int)((opens >> j) & 1u) - (int)((closes >> j) & 1u);
+        if (h < before) {
+          before = h;
+          if ((outers >> j) & 1u) { stop = (u32)-h; break; }
+        }
       }
     }
+    stop = __reduce_min_sync(0xffffffffu, stop);  // (unmatched markers are counted one by one: the earliest stop is the one with the least depth)
+    if (stop != 0xffffffffu) { *met = true; return stop; }
+    lowest = all < lowest ? all : lowest;
+    height += __shfl_sync(0xffffffffu, upto, 31);
   }
-  __syncthreads();
-  const u32 s = stop;  // (unmatched markers are counted one by one: the earliest stop is the one with the least depth)
-  __syncthreads();
-  *met = s != 0xffffffffu;
-  return *met ? s : (u32)-lowest;
-}
-
-template <bool FRONT>
-__device__ __forceinline__ u32 guess_unmatched(const ArgusPairArgs& a, const uint4* src, u32 ring_first, u32 n, u32 outer, bool* met) {
-  const u32 u = guess_unmatched<FRONT, kGuessRun / 4>(a, src, ring_first, n, outer, met);
-  return *met || n <= kGuessEvents / 4 ? u : guess_unmatched<FRONT, kGuessRun>(a, src, ring_first, n, outer, met);
+  *met = false;
+  return (u32)-lowest;
 }
 
 // Clears the workspace's zeroed part and the status block.
@@ -143,40 +139,63 @@ __device__ __forceinline__ u32 stream_length(const ArgusPairArgs& a, u64 off0, u
   return hi < lo || hi > a.num_events || lo < off0 || ((hi - lo) >> 32) ? 0u : (u32)(hi - lo);  // (bad offsets are reported by the pairing kernel)
 }
 
-constexpr u32 kInitStreams = 4;  // streams a block looks at at a time
-__global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uint4* zeroed, u64 zeroed_words, int clear_status) {
+// First and last marker's tag of a stream; false when it is empty.
+__device__ __forceinline__ bool stream_ends(const ArgusPairArgs& a, u32 s, u32 n, u32* first, u32* last) {
+  if (!n) return false;
+  const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u;
+  const uint4* src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
+  u32 end = n - 1;
+  if (a.ring_written) { const u32 room = a.ring_capacity - head; end = end >= room ? end - room : head + end; }
+  *first = __ldg(reinterpret_cast<const u32*>(src + head) + 2);
+  *last = __ldg(reinterpret_cast<const u32*>(src + end) + 2);
+  return true;
+}
+// begin(a) ... end(b), and not a ring slot that has wrapped
+__device__ __forceinline__ bool ends_unclear(const ArgusPairArgs& a, u32 s, u32 first, u32 last) {
+  return !(first & 1u) && (last & 1u) && (first >> 1) != (last >> 1) && !(a.ring_written && a.ring_written[s] > a.ring_capacity);
+}
+
+// A warp takes `per` streams at a time: their first and last markers, a lane each, then a look at those that are not whole.
+__global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uint4* zeroed, u64 zeroed_words, int clear_status, u32 per) {
   argus_kernel_begin();
   pair_clear(a, zeroed, zeroed_words, clear_status, (u64)blockIdx.x * blockDim.x + threadIdx.x, (u64)gridDim.x * blockDim.x);
-  const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
-  for (u32 s0 = blockIdx.x * kInitStreams; s0 < a.num_streams; s0 += gridDim.x * kInitStreams) {
-    // a thread per stream takes a look at its first and last marker; the block reads the ends of those that are not whole
-    const u32 sm = s0 + threadIdx.x;
+  const u32 lane = threadIdx.x & 31;
+  const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0, warps = (u64)gridDim.x * (kInitThreads / 32);
+  int many = -1;  // whether more than a quarter of the streams have unclear ends (a sample of 32 tells, when it is asked for)
+  for (u64 s0 = ((u64)blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5)) * per; s0 < a.num_streams; s0 += warps * per) {
     u32 n = 0, f = 0, l = 1;
-    if (threadIdx.x < kInitStreams && sm < a.num_streams) {
+    if (lane < per && s0 + lane < a.num_streams) {
+      const u32 sm = (u32)(s0 + lane);
       n = stream_length(a, off0, sm);
       a.bases[sm] = n >> 1;
-      if (n) {
-        const u32 first = a.ring_written ? argus_ring_first(a, sm) : 0u;
-        const uint4* src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)sm * a.ring_capacity : a.stream_offsets[sm]);
-        u32 end = n - 1;
-        if (a.ring_written) { const u32 room = a.ring_capacity - first; end = end >= room ? end - room : first + end; }
-        f = __ldg(reinterpret_cast<const u32*>(src + first) + 2);
-        l = __ldg(reinterpret_cast<const u32*>(src + end) + 2);
-      }
+      stream_ends(a, sm, n, &f, &l);
     }
-    __shared__ u32 sh_n[kInitStreams], sh_f[kInitStreams], sh_l[kInitStreams];
-    __syncthreads();
-    if (threadIdx.x < kInitStreams) { sh_n[threadIdx.x] = n; sh_f[threadIdx.x] = f; sh_l[threadIdx.x] = l; }
-    __syncthreads();
-    for (u32 k = 0; k < kInitStreams; ++k) {
-      const u32 s = s0 + k, nk = sh_n[k], fk = sh_f[k], lk = sh_l[k];
-      if (!nk || (!(fk & 1u) && (lk & 1u) && (fk >> 1) == (lk >> 1))) continue;
-      const u32 first = a.ring_written ? argus_ring_first(a, s) : 0u;
+    for (u32 todo = __ballot_sync(0xffffffffu, n && ((f & 1u) || !(l & 1u) || (f >> 1) != (l >> 1))); todo; todo &= todo - 1) {
+      const int k = __ffs((int)todo) - 1;
+      const u32 s = (u32)s0 + k, nk = __shfl_sync(0xffffffffu, n, k), fk = __shfl_sync(0xffffffffu, f, k), lk = __shfl_sync(0xffffffffu, l, k);
+      u32 limit = nk < kGuessEvents ? nk : kGuessEvents;
+      const bool unclear = ends_unclear(a, s, fk, lk);
+      if (unclear) {
+        if (many < 0) {
+          const u32 si = (u32)((u64)lane * a.num_streams / 32);
+          u32 fi = 0, li = 0;
+          many = __popc(__ballot_sync(0xffffffffu, stream_ends(a, si, stream_length(a, off0, si), &fi, &li) && ends_unclear(a, si, fi, li))) > 8;
+        }
+        if (many && nk / 32 < limit) limit = nk / 32;
+        if (many && limit < 32) continue;
+      }
+      const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u;
       const uint4* src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
       bool met = false;
-      u32 unmatched = lk & 1u ? guess_unmatched<true>(a, src, first, nk, lk >> 1, &met) : 0u;
-      if (!met && !(fk & 1u)) unmatched += guess_unmatched<false>(a, src, first, nk, fk >> 1, &met);
-      if (threadIdx.x == 0) a.bases[s] = (nk - (unmatched < nk ? unmatched : nk)) >> 1;
+      u32 unmatched = 0;
+      if (unclear) {
+        unmatched = guess_unmatched<false>(a, src, head, nk, fk >> 1, limit, &met);
+        if (!met) unmatched += guess_unmatched<true>(a, src, head, nk, lk >> 1, limit, &met);
+      } else {
+        if (lk & 1u) unmatched = guess_unmatched<true>(a, src, head, nk, lk >> 1, limit, &met);
+        if (!met && !(fk & 1u)) unmatched += guess_unmatched<false>(a, src, head, nk, fk >> 1, limit, &met);
+      }
+      if (lane == 0) a.bases[s] = (nk - (unmatched < nk ? unmatched : nk)) >> 1;
     }
   }
 }
@@ -480,8 +499,10 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   // Small calls: one block clears and orders. Beyond that a grid clears, and looks at the ends of the streams.
   const bool alone = num_events < (1u << 20) && num_streams <= 8192;
   if (!alone) {
-    const u64 want = (u64)num_streams / kInitStreams + zeroed_words / 4096 + 1;
-    ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status);
+    // a stream a warp, up to what the chip holds of them
+    const u32 per = num_streams <= 148u * 64u ? 1u : num_streams < 32u * 148u * 64u ? (num_streams + 148u * 64u - 1) / (148u * 64u) : 32u;
+    const u64 want = ((u64)num_streams / per + kInitThreads / 32 - 1) / (kInitThreads / 32) + zeroed_words / 4096 + 1;
+    ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status, per);
   }
   ARGUS_LAUNCH(k_pair_order, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone);
   a.order = tiled && num_streams > 1 ? order : nullptr;

@@ -71,3 +71,35 @@ def test_wrapped_ring(slot):
     assert p.intervals_numpy().tobytes() == iv.tobytes()
     assert p.ambig_numpy().tobytes() == am.tobytes()
     assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)
+
+
+@pytest.mark.parametrize("S,length,cut", [(1025, 1200, 0.0), (1500, 9000, 0.3), (1500, 9000, 0.02), (11_000, 200, 0.5), (40_000, 30, 0.1), (300_001, 6, 0.1)])
+def test_streams_of_several_outermost_regions(S, length, cut):
+    """Streams that begin and end with different regions although they are whole, and streams among them that lack some of their
+    front or back; more streams than a block, and than all warps, take at a time."""
+    rng = np.random.default_rng(S)
+    n = 3 * rng.integers(length // 6, length // 3 + 2, S)
+    offs = np.concatenate([[0], np.cumsum(2 * n)])
+    inner = np.arange(offs[-1]) - np.repeat(offs[:-1], 2 * n)      # index within the stream: a pair around another, then a pair
+    ev = np.zeros(offs[-1], argus.EVENT_DTYPE)
+    ev["ts"] = np.arange(len(ev)) * 3
+    six = inner % 6
+    region = np.where((six == 1) | (six == 2), 6, (inner // 6 * 2 + (six >= 4)) % 5)
+    ev["tag"] = region * 2 + np.isin(six, (2, 3, 5))
+    keep = np.ones(len(ev), bool)
+    for s in np.nonzero(rng.random(S) < cut)[0]:
+        k = int(rng.integers(1, 2 * n[s] + 1))
+        if rng.random() < 0.5:
+            keep[offs[s]:offs[s] + k // 4] = False
+        else:
+            keep[offs[s + 1] - k:offs[s + 1]] = False
+    kept = np.concatenate([[0], np.cumsum(keep)])
+    ev, offs = ev[keep], kept[offs].astype(np.uint64)
+    assert len(ev) > 1 << 20
+    _, iv, ioffs, am, aoffs, _ = oracle.pair(ev, offs, 7)
+    p = argus.argus_pair_intervals(torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).to(DEV), torch.from_numpy(offs.view(np.int64).copy()).to(DEV), 7)
+    assert int(p.fetch_status()["code"]) == 0
+    assert np.array_equal(p.interval_offsets.cpu().numpy().view(np.uint64), ioffs)
+    assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)
+    assert p.intervals_numpy().tobytes() == iv.tobytes()
+    assert p.ambig_numpy().tobytes() == am.tobytes()

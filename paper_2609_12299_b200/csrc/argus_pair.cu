@@ -18,6 +18,9 @@
 namespace {
 
 constexpr int kScanThreads = 1024;
+// Streams a thread of the one-block scans over all streams takes at a time: four where there are many (10^6 streams: 1,690 -> 1,325 us
+// and 1,640 -> 860), one where a block holds them all (16 streams: a call of 45 us is 1 to 2 us longer with four).
+constexpr u32 kScanRun = 4;
 constexpr u32 kWordsPerBlock = 1024;  // bitmap words per prefix block (32768 events)
 std::atomic<u32> g_poll_limit{1u << 19};  // see argus_testing_set_poll_limit
 
@@ -206,6 +209,41 @@ __global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uin
 // (producer and consumer warps of one kernel) the long chains must start first or they end last, alone. Counting sort in one
 // block; the order inside a class does not matter. Small calls have no init kernel before this one (`alone`).
 // ---------------------------------------------------------------------------------------------
+// Returns the sum of the foretold counts.
+template <u32 RUN>
+__device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int alone, u32* cnt, u64* sh) {
+  u64 carry = 0;
+  for (u64 s0 = 0; s0 < a.num_streams; s0 += kScanThreads * RUN) {
+    const u64 s = s0 + threadIdx.x * RUN;
+    u64 c[RUN], sum = 0, total;
+#pragma unroll
+    for (u32 j = 0; j < RUN; ++j) {
+      u32 cls = 64;
+      c[j] = 0;
+      if (s + j < a.num_streams) {
+        const u32 n = stream_length(a, off0, (u32)s + j);
+        c[j] = alone ? n >> 1 : a.bases[s + j];
+        cls = n ? 31 - __clz((int)n) : 0;
+        if (RUN == 1) atomicAdd(&cnt[cls], 1u);
+      }
+      sum += c[j];
+      if (RUN > 1) {
+        const u32 same = __match_any_sync(0xffffffffu, cls);  // a warp's streams are mostly of one class
+        if (cls < 64 && !(same & ((1u << (threadIdx.x & 31)) - 1u))) atomicAdd(&cnt[cls], (u32)__popc(same));
+      }
+    }
+    u64 at = carry + argus_block_exclusive_scan<u64>(sum, sh, &total);
+#pragma unroll
+    for (u32 j = 0; j < RUN; ++j) {
+      if (s + j < a.num_streams) a.bases[s + j] = at;
+      at += c[j];
+    }
+    carry += total;
+  }
+  return carry;
+}
+
+template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
                                                             int clear_status, int alone) {
   argus_kernel_begin_long();  // the pairing kernel's blocks spread evenly only over SMs that are free when they come
@@ -216,20 +254,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
   if (threadIdx.x < 64) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
   __syncthreads();
   const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
-  u64 carry = 0;
-  for (u32 s0 = 0; s0 < a.num_streams; s0 += kScanThreads) {
-    const u32 s = s0 + threadIdx.x;
-    u64 c = 0;
-    if (s < a.num_streams) {
-      const u32 n = stream_length(a, off0, s);
-      c = alone ? n >> 1 : a.bases[s];
-      atomicAdd(&cnt[n ? 31 - __clz((int)n) : 0], 1u);
-    }
-    u64 total;
-    const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
-    if (s < a.num_streams) a.bases[s] = carry + ex;
-    carry += total;
-  }
+  const u64 carry = order_bases<RUN>(a, off0, alone, cnt, sh);
   __syncthreads();
   if (threadIdx.x == 0) {  // first places, classes in descending order
     a.bases[a.num_streams] = carry;
@@ -268,33 +293,47 @@ struct AmbigArgs {
   u64* ambig_offsets;
 };
 
+// interval_offsets; returns the sum of the counts. *bad: first stream that does not lie right, *used: last one that has any.
+template <u32 RUN>
+__device__ __forceinline__ u64 final_offsets(const ArgusPairArgs& a, u64* sh, u32* bad, u32* used) {
+  u64 carry = 0;
+  for (u64 s0 = 0; s0 < a.num_streams; s0 += kScanThreads * RUN) {
+    const u64 s = s0 + threadIdx.x * RUN;
+    u64 c[RUN], sum = 0, total;
+#pragma unroll
+    for (u32 j = 0; j < RUN; ++j) { c[j] = s + j < a.num_streams ? a.counts[s + j] : 0; sum += c[j]; }
+    u64 fin = carry + argus_block_exclusive_scan<u64>(sum, sh, &total);
+    u64 base = s < a.num_streams ? a.bases[s] : 0;
+#pragma unroll
+    for (u32 j = 0; j < RUN; ++j) {
+      if (s + j >= a.num_streams) break;
+      const u32 sj = (u32)s + j;
+      // (beyond the capacity only when the call ends with ARGUS_ERR_CAPACITY: offsets then stay inside the array, so
+      // that a call chained behind this one without a host check reads nothing it must not)
+      a.interval_offsets[sj] = fin < a.interval_capacity ? fin : a.interval_capacity;
+      const u64 next = a.bases[s + j + 1], told = next - base;
+      // a stream with fewer intervals than foretold lies right, those after it do not; one with more has lost its tail to the
+      // next stream's writes
+      if (c[j] < told && sj + 1 < *bad) *bad = sj + 1;
+      if (c[j] > told && sj < *bad) *bad = sj;
+      if (c[j]) *used = sj;
+      fin += c[j];
+      base = next;
+    }
+    carry += total;
+  }
+  return carry;
+}
+
 // Block 0: exclusive scan of the per-stream counts; decides whether the second pass is needed, and from which stream on.
+template <u32 RUN>
 __device__ __forceinline__ void pair_offsets(const ArgusPairArgs& a) {
   __shared__ u64 sh[33];
   __shared__ u32 first_bad, last_used;
   if (threadIdx.x == 0) { first_bad = 0xffffffffu; last_used = 0; }
   __syncthreads();
-  u64 carry = 0;
   u32 bad = 0xffffffffu, used = 0;
-  for (u32 s0 = 0; s0 < a.num_streams; s0 += kScanThreads) {
-    const u32 s = s0 + threadIdx.x;
-    const u64 c = s < a.num_streams ? a.counts[s] : 0;
-    u64 total;
-    const u64 ex = argus_block_exclusive_scan<u64>(c, sh, &total);
-    if (s < a.num_streams) {
-      const u64 fin = carry + ex;
-      // (beyond the capacity only when the call ends with ARGUS_ERR_CAPACITY: offsets then stay inside the array, so
-      // that a call chained behind this one without a host check reads nothing it must not)
-      a.interval_offsets[s] = fin < a.interval_capacity ? fin : a.interval_capacity;
-      const u64 told = a.bases[s + 1] - a.bases[s];
-      // a stream with fewer intervals than foretold lies right, those after it do not; one with more has lost its tail to the
-      // next stream's writes
-      if (c < told && s + 1 < bad) bad = s + 1;
-      if (c > told && s < bad) bad = s;
-      if (c) used = s;
-    }
-    carry += total;
-  }
+  const u64 carry = final_offsets<RUN>(a, sh, &bad, &used);
   atomicMin(&first_bad, bad);
   atomicMax(&last_used, used);
   __syncthreads();
@@ -314,6 +353,7 @@ __device__ __forceinline__ void pair_offsets(const ArgusPairArgs& a) {
 
 // The other blocks, when there are notes: set bits before every word within its block of words, and, by the last block to
 // be done, before every block of words.
+template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   // The second pass comes next, and its blocks spread evenly only over SMs that are free when they come (96 streams with a lost end
   // each: 5,993 us when they came beside this kernel's blocks, 4,111 us after them). Without notes it has nothing to do, and a few
@@ -321,7 +361,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   if (gridDim.x <= 37) argus_launch_next();
   argus_kernel_begin_long();
   if (gridDim.x > 37 && __ldcg(&g.p.ctl->n_notes) == 0) argus_launch_next();
-  if (blockIdx.x == 0) { pair_offsets(g.p); return; }
+  if (blockIdx.x == 0) { pair_offsets<RUN>(g.p); return; }
   if (__ldcg(&g.p.ctl->n_notes) == 0) return;
   __shared__ u32 sh[33];
   __shared__ u64 sh64[33];
@@ -504,7 +544,8 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
     const u64 want = ((u64)num_streams / per + kInitThreads / 32 - 1) / (kInitThreads / 32) + zeroed_words / 4096 + 1;
     ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status, per);
   }
-  ARGUS_LAUNCH(k_pair_order, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone);
+  const bool many = num_streams > kScanThreads;
+  ARGUS_LAUNCH(many ? k_pair_order<kScanRun> : k_pair_order<1>, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone);
   a.order = tiled && num_streams > 1 ? order : nullptr;
   a.segments = nullptr; a.split_failed = nullptr; a.segment_tiles = 0;
   const bool split = kernel_choice == 0 && tiled && !ring_written && argus_split_usable(num_events, num_streams);
@@ -530,7 +571,7 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
       if (pass == 0) argus_prof_mark(ARGUS_PROF_PAIR, stream, 1);
     }
     if (pass == 0)
-      ARGUS_LAUNCH(k_pair_offsets, (unsigned)(L.num_blocks < 592 ? L.num_blocks : 592) + 1, kScanThreads, 0, stream, g);
+      ARGUS_LAUNCH(many ? k_pair_offsets<kScanRun> : k_pair_offsets<1>, (unsigned)(L.num_blocks < 592 ? L.num_blocks : 592) + 1, kScanThreads, 0, stream, g);
   }
   const u64 want = ((u64)num_streams + 1 + 255) / 256;
   ARGUS_LAUNCH(k_ambig_records, (unsigned)(alone ? (want > 16 ? want : 16) : 296), 256, 0, stream, g);

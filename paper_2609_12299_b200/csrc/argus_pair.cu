@@ -209,9 +209,9 @@ __global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uin
 // (producer and consumer warps of one kernel) the long chains must start first or they end last, alone. Counting sort in one
 // block; the order inside a class does not matter. Small calls have no init kernel before this one (`alone`).
 // ---------------------------------------------------------------------------------------------
-// Returns the sum of the foretold counts.
+// Returns the sum of the foretold counts; *longest: events of the longest stream of this thread.
 template <u32 RUN>
-__device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int alone, u32* cnt, u64* sh) {
+__device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int alone, u32* cnt, u64* sh, u32* longest) {
   u64 carry = 0;
   for (u64 s0 = 0; s0 < a.num_streams; s0 += kScanThreads * RUN) {
     const u64 s = s0 + threadIdx.x * RUN;
@@ -224,6 +224,7 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
         const u32 n = stream_length(a, off0, (u32)s + j);
         c[j] = alone ? n >> 1 : a.bases[s + j];
         cls = n ? 31 - __clz((int)n) : 0;
+        *longest = n > *longest ? n : *longest;
         if (RUN == 1) atomicAdd(&cnt[cls], 1u);
       }
       sum += c[j];
@@ -245,19 +246,26 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
 
 template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
-                                                            int clear_status, int alone) {
+                                                            int clear_status, int alone, int ask_split) {
   argus_kernel_begin_long();  // the pairing kernel's blocks spread evenly only over SMs that are free when they come
   __shared__ u32 cnt[64], cur[64];
   __shared__ u64 sh[33];
-  __shared__ u32 one_class;
+  __shared__ u32 one_class, longest_of;
+  if (threadIdx.x == 0) longest_of = 0;
   if (alone) pair_clear(a, zeroed, zeroed_words, clear_status, threadIdx.x, blockDim.x);
   if (threadIdx.x < 64) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
   __syncthreads();
   const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
-  const u64 carry = order_bases<RUN>(a, off0, alone, cnt, sh);
+  u32 longest = 0;
+  const u64 carry = order_bases<RUN>(a, off0, alone, cnt, sh, &longest);
+  if (ask_split) {
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    if ((threadIdx.x & 31) == 0) atomicMax(&longest_of, longest);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {  // first places, classes in descending order
     a.bases[a.num_streams] = carry;
+    if (ask_split) a.ctl->split = argus_split_pays(longest_of, a.num_events, a.num_streams);
     u32 base = 0;
     one_class = 0;
     for (int c = 31; c >= 0; --c) {
@@ -545,10 +553,10 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
     ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status, per);
   }
   const bool many = num_streams > kScanThreads;
-  ARGUS_LAUNCH(many ? k_pair_order<kScanRun> : k_pair_order<1>, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone);
+  const bool split = kernel_choice == 0 && tiled && !ring_written && argus_split_usable(num_events, num_streams);
+  ARGUS_LAUNCH(many ? k_pair_order<kScanRun> : k_pair_order<1>, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone, (int)split);
   a.order = tiled && num_streams > 1 ? order : nullptr;
   a.segments = nullptr; a.split_failed = nullptr; a.segment_tiles = 0;
-  const bool split = kernel_choice == 0 && tiled && !ring_written && argus_split_usable(num_events, num_streams);
 
   AmbigArgs g;
   g.p = a; g.num_words = L.num_words; g.span = num_events;

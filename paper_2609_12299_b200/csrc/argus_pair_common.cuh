@@ -38,6 +38,7 @@ struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of
   u32 seg_head;        // segments taken (split pass)
   u32 num_failed;      // streams that the split pass has to leave to the chained one
   u32 num_segments;
+  u32 split;           // the split pass is worth it (argus_split_pays)
 };
 
 // A long stream is walked in chunks of about kChunkEvents events. After a chunk the CTA stores the stream's
@@ -113,6 +114,17 @@ bool argus_split_usable(uint64_t num_events, uint32_t num_streams);
 uint32_t argus_split_max_segments(uint64_t num_events, uint32_t num_streams);
 size_t argus_split_bytes(uint64_t num_events, uint32_t num_streams);
 int argus_launch_pair_split(ArgusPairArgs& a, void* room, cudaStream_t stream);
+// Is the split pass the faster one for streams of which the longest has `longest` events? The chained pass takes 4.05 ns an event of the
+// longest stream with a stream on an SM and 0.75 ns more for each further one; the split pass 85 events a ns and 35 us more than the
+// chained one with the split kernels launched for nothing (12 us). Measured (us, split / chained by itself; streams x events): decode
+// trace, equal lengths, 96 x 12,156 71 / 66, 96 x 32,416 89 / 143, 320 x 12,156 103 / 90, 320 x 32,416 183 / 197, 448 x 32,416 239 /
+// 209, 448 x 129,664 689 / 762, 512 x 32,416 259 / 211, 512 x 518,656 2,739 / 2,923, 592 x 518,656 3,231 / 3,005, 768 x 32,416 359 / 271;
+// GEMM trace, two of twelve streams 2.3 times as long as the others, longest 25,200 of 288 99 / 140, of 768 181 / 213, longest 72,000 of
+// 768 390 / 443.
+__host__ __device__ __forceinline__ bool argus_split_pays(u32 longest, u64 num_events, u32 num_streams) {
+  const u32 per_sm = (num_streams + 147) / 148;
+  return (u64)longest * (280 + 64 * per_sm) > num_events + 3000000;  // both sides in 1 / 85 ns
+}
 
 #define ARGUS_NOTE_POS_BITS 48
 

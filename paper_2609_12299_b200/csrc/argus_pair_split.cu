@@ -32,8 +32,18 @@ __device__ __forceinline__ u32 split_segments(const ArgusPairArgs& a, u32 s) {  
   return n ? (u32)((n + per - 1) / per) : 1u;
 }
 
+// Every stream is left to the chained pass. One block.
+__device__ __forceinline__ void leave_all(const ArgusPairArgs& a) {
+  for (u32 s = threadIdx.x; s < a.num_streams; s += kScanThreads) a.split_failed[s] = 1;
+  if (threadIdx.x == 0) { a.ctl->num_segments = 0; a.ctl->num_failed = a.num_streams; }
+}
+
 __global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u32* first_segment) {
   argus_kernel_begin();
+  if (!__ldcg(&a.ctl->split)) {  // the chained pass is the faster one
+    if (blockIdx.x == 0) leave_all(a);
+    return;
+  }
   __shared__ u32 sh[33], sh_stream, sh_before;
   __shared__ int shi[33], low_of[kScanThreads / 32];
   const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -52,16 +62,11 @@ __global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u3
   __syncthreads();
   // Offsets that decrease let streams share events, and then there may be more segments than blocks and room: the chained pass,
   // which reports such offsets, walks all streams.
-  const bool fits = carry <= gridDim.x;
-  if (blockIdx.x == 0 && tid == 0) {
-    first_segment[a.num_streams] = carry;
-    a.ctl->num_segments = fits ? carry : 0u;
-    if (!fits) a.ctl->num_failed = a.num_streams;
-  }
-  if (!fits) {
-    if (blockIdx.x == 0) for (u32 s = tid; s < a.num_streams; s += kScanThreads) a.split_failed[s] = 1;
+  if (carry > gridDim.x) {
+    if (blockIdx.x == 0) leave_all(a);
     return;
   }
+  if (blockIdx.x == 0 && tid == 0) { first_segment[a.num_streams] = carry; a.ctl->num_segments = carry; }
   if (sh_stream == 0xffffffffu) return;
   const u32 s = sh_stream, j = blockIdx.x - sh_before, n = split_length(a, s), per = a.segment_tiles * kSplitTile;
   ArgusSegment* const g = a.segments + blockIdx.x;
@@ -132,7 +137,7 @@ __global__ void __launch_bounds__(32) k_split_chain(ArgusPairArgs a, const u32* 
   __shared__ u32 stack[ARGUS_MAX_DEPTH];
   constexpr u32 kAhead = 4;
   const u32 s = blockIdx.x, lane = threadIdx.x;
-  if (__ldcg(a.split_failed + s)) return;  // (more segments than room: nobody has looked at them)
+  if (__ldcg(a.split_failed + s)) return;  // (all streams are left: there are no segments)
   const u32 g0 = first_segment[s], g1 = first_segment[s + 1];
   int h = 0;
   bool fail = false;
@@ -214,7 +219,7 @@ __global__ void __launch_bounds__(kFixThreads) k_split_fix(ArgusPairArgs a, cons
 }  // namespace
 
 // Fewer streams than three quarters of the blocks of the pairing kernel that run at a time (7 x 148), and long ones: the chained
-// pass would leave the rest of the chip idle. Above, the scan (a quarter of the split pass) eats the gain.
+// pass would leave the rest of the chip idle. Whether that outweighs the scan is decided on the device, by the longest stream.
 bool argus_split_usable(uint64_t num_events, uint32_t num_streams) {
   return num_streams > 0 && num_streams < 777 && num_events > (1u << 20) && num_events / num_streams >= 16 * kSplitTile;
 }

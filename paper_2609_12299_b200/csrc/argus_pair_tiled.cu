@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   argus_kernel_begin_long();
   if (a.redo && !__ldcg(&a.ctl->redo)) return;
   if (!SPLIT && !a.redo && a.segments && !__ldcg(&a.ctl->num_failed)) return;
+  if (SPLIT && !__ldcg(&a.ctl->num_segments)) return;
   if (tid == 0) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);

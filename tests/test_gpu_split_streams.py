@@ -118,3 +118,19 @@ def test_streams_given_up_while_their_segments_are_walked(kind):
         assert torch.equal(p.intervals[:len(want[0])], want[0]) and torch.equal(p.ambig[:len(want[1])], want[1])
         p.intervals.zero_()
         p.ambig.zero_()
+
+
+@pytest.mark.parametrize("S,n", [(110, 11_000), (320, 12_000), (592, 12_000), (776, 10_250)])
+def test_few_streams_that_the_chained_pass_walks(S, n):
+    """Streams of equal length, too short or too many for their segments to pay: the split kernels are launched and leave them all."""
+    i = np.arange(S * n) % n
+    ev = np.zeros(S * n, argus.EVENT_DTYPE)
+    ev["ts"] = np.arange(S * n) * 5
+    ev["tag"] = np.array([0, 2, 3, 1], np.uint32)[i % 4]
+    ev["tag"][(i >= n // 2) & (i < n // 2 + 4)] = 2          # four begins without an end in the middle of every stream
+    offs = (np.arange(S + 1) * n).astype(np.uint64)
+    _, iv, ioffs, am, aoffs, _ = oracle.pair(ev, offs, 2)
+    p = argus.argus_pair_intervals(torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).to(DEV), torch.from_numpy(offs.view(np.int64).copy()).to(DEV), 2)
+    assert int(p.fetch_status()["code"]) == 0 and len(am)
+    assert np.array_equal(p.interval_offsets.cpu().numpy().view(np.uint64), ioffs)
+    assert p.intervals_numpy().tobytes() == iv.tobytes() and p.ambig_numpy().tobytes() == am.tobytes()

@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
   __syncthreads();
   if (threadIdx.x == 0) {  // first places, classes in descending order
     a.bases[a.num_streams] = carry;
-    if (ask_split) a.ctl->split = argus_split_pays(longest_of, a.num_events, a.num_streams);
+    if (ask_split) { a.ctl->split = argus_split_pays(longest_of, a.num_events, a.num_streams); a.ctl->longest = longest_of; }
     u32 base = 0;
     one_class = 0;
     for (int c = 31; c >= 0; --c) {

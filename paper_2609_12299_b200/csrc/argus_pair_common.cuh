@@ -36,9 +36,11 @@ struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of
   u32 n_done[2];       // streams walked to their end (or given up on)
   u32 prefix_done;     // blocks that have counted their share of the ambiguity bitmap
   u32 seg_head;        // segments taken (split pass)
-  u32 num_failed;      // streams that the split pass has to leave to the chained one
-  u32 num_segments;
-  u32 split;           // the split pass is worth it (argus_split_pays)
+  u32 longest;         // events of the longest stream
+  alignas(16) u32 num_failed;  // streams that the split pass has to leave to the chained one (read together with the next two)
+  u32 num_segments;    // 0 where the segments do not fit their room, too
+  u32 split;           // the split pass is worth it (argus_split_pays), and no long stream has been given up
+  u32 pad;
 };
 
 // A long stream is walked in chunks of about kChunkEvents events. After a chunk the CTA stores the stream's
@@ -124,6 +126,21 @@ int argus_launch_pair_split(ArgusPairArgs& a, void* room, cudaStream_t stream);
 __host__ __device__ __forceinline__ bool argus_split_pays(u32 longest, u64 num_events, u32 num_streams) {
   const u32 per_sm = (num_streams + 147) / 148;
   return (u64)longest * (280 + 64 * per_sm) > num_events + 3000000;  // both sides in 1 / 85 ns
+}
+
+// After the split pass: are its segments what counts, or is everything left to the chained pass? *failed: has a stream been given up?
+__device__ __forceinline__ bool argus_split_in_force(const ArgusPairArgs& a, bool* failed) {
+  const uint4 w = __ldcg(reinterpret_cast<const uint4*>(&a.ctl->num_failed));
+  *failed = w.x != 0;
+  return w.y && w.z;
+}
+
+// Gives a stream of `length` events up. The chained pass takes about as long for one long stream as for all of them, so one
+// that is about as long as the longest takes all others with it. One thread.
+__device__ __forceinline__ void argus_split_give_up(const ArgusPairArgs& a, u32 s, u32 length) {
+  if (atomicExch(a.split_failed + s, 1u)) return;
+  if (argus_split_pays(__ldcg(&a.ctl->longest) - length, a.num_events, a.num_streams)) atomicAdd(&a.ctl->num_failed, 1u);
+  else atomicExch(&a.ctl->split, 0u);
 }
 
 #define ARGUS_NOTE_POS_BITS 48

@@ -9,7 +9,10 @@
 //   k_split_fix   : one block per stream completes the child time of the frames that were open across a segment's start, counts
 //                   the stream's intervals and notes the frames open at its end.
 // Heights know nothing of region ids. A segment that meets a marker which breaks the parallel rules gives its stream up; the
-// chained pass, which follows and does nothing otherwise, walks such streams from their beginning.
+// chained pass, which follows and does nothing otherwise, walks such streams from their beginning. A stream about as long as the
+// longest takes all others with it, and the blocks stop within eight tiles (384 streams of 129,664 events with a lost or doubled
+// marker in two of three: 1,922 us when they went on, 1,582 us; 1,385 in the chained
+// passes by themselves).
 //
 // The scan reads the events once more (16 of then 56 bytes an event). 96 streams of 518,656 events: pairing 2,412 -> 660 us
 // (scan 132, chain 36, segments 458, fix 27).
@@ -32,18 +35,9 @@ __device__ __forceinline__ u32 split_segments(const ArgusPairArgs& a, u32 s) {  
   return n ? (u32)((n + per - 1) / per) : 1u;
 }
 
-// Every stream is left to the chained pass. One block.
-__device__ __forceinline__ void leave_all(const ArgusPairArgs& a) {
-  for (u32 s = threadIdx.x; s < a.num_streams; s += kScanThreads) a.split_failed[s] = 1;
-  if (threadIdx.x == 0) { a.ctl->num_segments = 0; a.ctl->num_failed = a.num_streams; }
-}
-
 __global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u32* first_segment) {
   argus_kernel_begin();
-  if (!__ldcg(&a.ctl->split)) {  // the chained pass is the faster one
-    if (blockIdx.x == 0) leave_all(a);
-    return;
-  }
+  const u32 split = __ldcg(&a.ctl->split);
   __shared__ u32 sh[33], sh_stream, sh_before;
   __shared__ int shi[33], low_of[kScanThreads / 32];
   const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -60,12 +54,9 @@ __global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u3
     carry += total;
   }
   __syncthreads();
-  // Offsets that decrease let streams share events, and then there may be more segments than blocks and room: the chained pass,
-  // which reports such offsets, walks all streams.
-  if (carry > gridDim.x) {
-    if (blockIdx.x == 0) leave_all(a);
-    return;
-  }
+  // No segments where the chained pass is the faster one. Offsets that decrease let streams share events, and then there may be more
+  // segments than blocks and room: the chained pass, which reports such offsets, walks all streams.
+  if (!split || carry > gridDim.x) return;
   if (blockIdx.x == 0 && tid == 0) { first_segment[a.num_streams] = carry; a.ctl->num_segments = carry; }
   if (sh_stream == 0xffffffffu) return;
   const u32 s = sh_stream, j = blockIdx.x - sh_before, n = split_length(a, s), per = a.segment_tiles * kSplitTile;
@@ -137,7 +128,7 @@ __global__ void __launch_bounds__(32) k_split_chain(ArgusPairArgs a, const u32* 
   __shared__ u32 stack[ARGUS_MAX_DEPTH];
   constexpr u32 kAhead = 4;
   const u32 s = blockIdx.x, lane = threadIdx.x;
-  if (__ldcg(a.split_failed + s)) return;  // (all streams are left: there are no segments)
+  if (!__ldcg(&a.ctl->num_segments)) return;  // all streams are left
   const u32 g0 = first_segment[s], g1 = first_segment[s + 1];
   int h = 0;
   bool fail = false;
@@ -176,13 +167,14 @@ __global__ void __launch_bounds__(32) k_split_chain(ArgusPairArgs a, const u32* 
       }
     }
   }
-  if (fail && lane == 0) { a.split_failed[s] = 1; atomicAdd(&a.ctl->num_failed, 1u); }
+  if (fail && lane == 0) argus_split_give_up(a, s, split_length(a, s));
 }
 
 __global__ void __launch_bounds__(kFixThreads) k_split_fix(ArgusPairArgs a, const u32* first_segment) {
   argus_kernel_begin_long();
   const u32 s = blockIdx.x;
-  if (__ldcg(a.split_failed + s)) return;
+  bool any_failed;
+  if (!argus_split_in_force(a, &any_failed) || (any_failed && __ldcg(a.split_failed + s))) return;
   const u32 g0 = first_segment[s], g1 = first_segment[s + 1], per = a.segment_tiles * kSplitTile;
   const u64 off0 = a.stream_offsets[0];
   u32 ctx = 0, rev = 0, clamp = 0;

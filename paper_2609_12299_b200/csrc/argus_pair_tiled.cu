@@ -145,6 +145,7 @@ struct TileSmem {
   u64 cur_stream;
   u32 cur_rec;                     // hand-over record of the stream being walked (kNoRec: none)
   int skip;                        // the piece of work taken is not to be walked
+  int stop;                        // split pass: everything is left to the chained pass
   u64 n_int;                       // written by the sequential redo path
   int ch;
   u32 wrapped;                     // a sum of 32-bit child time wrapped in this window
@@ -203,7 +204,8 @@ __device__ __forceinline__ void tile_fetch(const ArgusPairArgs& a, uint4* dst, c
 // the segment, and a marker that breaks the parallel rules gives the stream up to the chained pass that follows. Other blocks may
 // give up the stream of this block's segment at any moment, so one thread reads that word and all threads follow its answer; the
 // other words of global memory that a block branches on around its barriers (offsets, bases, segments, hand-over records, redo,
-// redo_from, num_failed) are not written while the kernel runs, or are read by the one thread that takes the work.
+// redo_from, and after the split pass its outcome) are not written while the kernel runs, or are read by the one thread that takes the
+// work, as is the word that calls the split pass off.
 template <int NT, int E, int MINB, bool RING = false, bool SPLIT = false>
 __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   using SM = TileSmem<NT, E>;
@@ -214,8 +216,9 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   argus_kernel_begin_long();
   if (a.redo && !__ldcg(&a.ctl->redo)) return;
-  if (!SPLIT && !a.redo && a.segments && !__ldcg(&a.ctl->num_failed)) return;
-  if (SPLIT && !__ldcg(&a.ctl->num_segments)) return;
+  bool failed = false;
+  const bool segments = !SPLIT && !a.redo && a.segments && argus_split_in_force(a, &failed);  // the chained pass after a split one
+  if (segments && !failed) return;
   if (tid == 0) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);
@@ -236,13 +239,18 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     if (tid == 0) {
       u64 st = ~0ull;
       u32 rc = kNoRec;
+      bool skip = false;
       if (SPLIT) {
+        const uint4 w = __ldcg(reinterpret_cast<const uint4*>(&a.ctl->num_failed));  // num_failed, num_segments, split
         rc = atomicAdd(&a.ctl->seg_head, 1u);
-        st = rc < a.ctl->num_segments ? a.segments[rc].stream : ~0ull;
+        st = w.z && rc < w.y ? a.segments[rc].stream : ~0ull;
+        skip = w.x && st < a.num_streams && __ldcg(a.split_failed + st);
       } else if (!tile_pop_work(a, a.redo ? 1 : 0, &st, &rc)) st = ~0ull;
       sm.cur_stream = st;
       sm.cur_rec = rc;
-      sm.skip = st < a.num_streams && (SPLIT ? __ldcg(a.split_failed + st) != 0 : (a.segments && !a.redo && rc == kNoRec && !__ldcg(a.split_failed + st)));
+      if (!SPLIT && segments) skip = st < a.num_streams && rc == kNoRec && !__ldcg(a.split_failed + st);
+      sm.skip = skip;
+      sm.stop = 0;
     }
     __syncthreads();
     const u64 s64 = sm.cur_stream;
@@ -341,9 +349,11 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         tile_fetch<RING>(a, b ? ev0 : ev1, src, ring_first, nstart, (n - nstart) < (u32)T ? (n - nstart) : (u32)T, &sm.bar[b ^ 1]);
       }
       {
+        const u32 go_on = SPLIT && tid == 0 && (ti & 7u) == 7u ? __ldcg(&a.ctl->split) : 1u;
         const bool ok = mbar_wait_bounded(&sm.bar[b], b ? ph1 : ph0);
         if (b) ph1 ^= 1; else ph0 ^= 1;
         if (!ok) sm.dead = 1;
+        if (SPLIT && !go_on) sm.stop = 1;
       }
 
       // The tile is consumed in windows [w0, wend). A well-nested tile is one window. When the parallel
@@ -542,7 +552,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         bp ^= 1;
         if (tid == 0) sm.badpos[bp] = 0x7fffffff;  // nobody reads or reports into it before the next window's barriers
 
-        if (SPLIT && badpos < wend) {  // the chained pass walks this stream
+        if (SPLIT && (badpos < wend || sm.stop)) {  // the chained pass walks this stream
           stream_failed = true;
           __syncthreads();
           break;
@@ -647,7 +657,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     }
     if (SPLIT) {
       if (stream_failed) {
-        if (tid == 0 && atomicExch(a.split_failed + s, 1u) == 0) atomicAdd(&a.ctl->num_failed, 1u);
+        if (tid == 0) argus_split_give_up(a, s, n);
       } else {
         if (tid < ch) seg->ledger[tid] = sm.cchild[cpar][tid];
         if (tid == 0) { seg->n_int = n_int; seg->end_ch = (u32)ch; }

@@ -364,11 +364,12 @@ __device__ __forceinline__ void pair_offsets(const ArgusPairArgs& a) {
 template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   // The second pass comes next, and its blocks spread evenly only over SMs that are free when they come (96 streams with a lost end
-  // each: 5,993 us when they came beside this kernel's blocks, 4,111 us after them). Without notes it has nothing to do, and a few
-  // blocks leave most SMs free (the smallest calls are 0.5 us shorter).
-  if (gridDim.x <= 37) argus_launch_next();
+  // each: 5,993 us when they came beside this kernel's blocks, 4,111 us after them). Not so where there are enough of them to fill the
+  // chip or few blocks here; and without notes it has nothing to do (coming early saves 0.5 us of the smallest call, 2 us of others).
+  const bool early = gridDim.x <= 37 || g.p.num_streams >= 1036;
+  if (early) argus_launch_next();
   argus_kernel_begin_long();
-  if (gridDim.x > 37 && __ldcg(&g.p.ctl->n_notes) == 0) argus_launch_next();
+  if (!early && __ldcg(&g.p.ctl->n_notes) == 0) argus_launch_next();
   if (blockIdx.x == 0) { pair_offsets<RUN>(g.p); return; }
   if (__ldcg(&g.p.ctl->n_notes) == 0) return;
   __shared__ u32 sh[33];

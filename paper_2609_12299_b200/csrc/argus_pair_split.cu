@@ -11,8 +11,7 @@
 // Heights know nothing of region ids. A segment that meets a marker which breaks the parallel rules gives its stream up; the
 // chained pass, which follows and does nothing otherwise, walks such streams from their beginning. A stream about as long as the
 // longest takes all others with it, and the blocks stop within eight tiles (384 streams of 129,664 events with a lost or doubled
-// marker in two of three: 1,922 us when they went on, 1,582 us; 1,385 in the chained
-// passes by themselves).
+// marker in two of three: 1,922 us when they went on, 1,582 us; 1,385 in the chained passes by themselves).
 //
 // The scan reads the events once more (16 of then 56 bytes an event). 96 streams of 518,656 events: pairing 2,412 -> 660 us
 // (scan 132, chain 36, segments 458, fix 27).

@@ -39,8 +39,7 @@ void argus_profile_enable(int on);
 int argus_profile_read(double* ms_total /*host [4]*/, unsigned long long* launches /*host [4]*/);
 
 /* argus_set_synthesize_mode: where argus_synthesize aggregates and selects overlap spans: -1 automatic,
- * 1 in one pass over the intervals' digests, 2 the three plain operations, 3 the three operations with the
- * aggregation over the interval records. A mode the inputs do not allow falls back to the automatic choice.
+ * 1 in one pass over the intervals' digests, 2 and 3 the three plain operations. A mode the inputs do not allow falls back to the automatic choice.
  * argus_set_tile_variant: shape of the tiled pairing kernel, 0 = the default <128 threads, 5 events per
  * thread, 7 blocks per SM>, 1..3 = <192,5,4>, <64,5,8>, <256,7,2> (tiles end at other places).
  * argus_testing_set_poll_limit: polls after which a block of the tiled pairing kernel that waits for a

@@ -18,7 +18,7 @@ def _stale(out: str, deps: list[str]) -> bool:
 def build_library(force: bool = False, verbose: bool = False) -> str:
     csrc = os.path.join(_HERE, "csrc")
     srcs = sorted(glob.glob(os.path.join(csrc, "*.cu")))
-    deps = srcs + glob.glob(os.path.join(csrc, "*.cuh")) + [os.path.join(_ROOT, "include", "argus.h")]
+    deps = srcs + glob.glob(os.path.join(csrc, "*.cuh")) + glob.glob(os.path.join(_ROOT, "include", "*.h"))
     out = os.path.join(_HERE, "libargus.so")
     if force or _stale(out, deps):
         cmd = [NVCC, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-I", os.path.join(_ROOT, "include"), "-shared",

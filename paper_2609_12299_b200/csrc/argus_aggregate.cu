@@ -6,8 +6,8 @@
 //   k_agg_streams_compact : the same over the 48-byte records, with an optional scope: that stream's row in
 //                   a compact shared-memory form (112 B per region: sums, min, max, a 16-bin window, so
 //                   several CTAs fit an SM), for up to kAggCompactRegions regions;
-//   k_agg_streams : the same with a full 576 B-per-region copy in shared memory when that fits, else on
-//                   the global row itself. Integer atomics only: the result does not depend on thread order.
+//   k_agg_streams : the same on the global row itself, for more regions than that. Integer atomics only: the
+//                   result does not depend on thread order.
 //   k_agg_rollup  : CTA-scope and warp-role cells = reductions over the warps of each CTA and over the CTAs; SM-scope and
 //                   kernel-scope cells by atomic add/min/max of CTA cells.
 //   k_agg_iter_windows, k_agg_iter : per-iteration cells (key = ctx - ctx_lo) of the intervals of a scope.
@@ -19,7 +19,6 @@ namespace {
 
 constexpr int kAggThreads = 256;
 constexpr u32 kCell = 72;  // u64 words per argus_agg_t
-constexpr size_t kAggSmemLimit = 200 * 1024;
 constexpr u32 kAggCompactRegions = 400;  // 112 B each: 44.8 KB of shared memory at most
 constexpr u32 kIterThreads = 512, kIterWarps = kIterThreads / 32;  // k_agg_iter_windows
 constexpr u32 kMaxParts = 16;            // blocks that share a stream in k_agg_streams_compact
@@ -35,7 +34,6 @@ struct AggArgs {
   u64* sm_tab;    // nullable
   u64* kernel_tab;  // nullable
   argus_status_t* status;
-  int use_smem;
   // scope selection
   int scoped;
   u32 ctx_lo, ctx_hi;
@@ -99,14 +97,12 @@ __device__ __forceinline__ void agg_add_interval(u64* tab, u32 region, u64 incl,
 __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
   argus_kernel_begin_long();
   agg_empty_tables(a);
-  extern __shared__ __align__(16) u64 sh_tab[];
   const u32 R = a.num_regions;
   const u32 cells = R * kCell;
   for (u32 s = blockIdx.x; s < a.num_streams; s += gridDim.x) {
     u64* row = a.warp_tab + (size_t)s * cells;
-    u64* tab = a.use_smem ? sh_tab : row;
-    for (u32 i = threadIdx.x; i < cells; i += blockDim.x) tab[i] = (i % kCell == 2) ? ~0ull : 0ull;
-    if (!a.use_smem) __threadfence();
+    for (u32 i = threadIdx.x; i < cells; i += blockDim.x) row[i] = (i % kCell == 2) ? ~0ull : 0ull;
+    __threadfence();
     __syncthreads();
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
     const int sel = stream_in_scope(a, s);
@@ -122,7 +118,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
         const u32 region = q1.z;
         if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
         if (!record_in_scope(a, q1.w, region)) continue;
-        agg_add_interval(tab, region, incl, excl, q2.w >> 16);
+        agg_add_interval(row, region, incl, excl, q2.w >> 16);
       }
     }
     if (a.ambig && a.ambig_offsets && sel == 1) {
@@ -131,13 +127,8 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
         const u32 region = a.ambig[i].tag >> 1;
         if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); continue; }
         if (!record_in_scope(a, a.ambig[i].ctx, region)) continue;
-        atomicAdd(tab + (size_t)region * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
+        atomicAdd(row + (size_t)region * kCell + (a.ambig[i].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
       }
-    }
-    __syncthreads();
-    if (a.use_smem) {
-      for (u32 i = threadIdx.x; i < cells; i += blockDim.x) row[i] = sh_tab[i];
-      __syncthreads();
     }
   }
 }
@@ -250,7 +241,6 @@ __device__ __noinline__ void digest_wide(u64* row, u32 R, uint4 q0, uint4 q1, u3
   atomicAdd(c + 8 + log2_bin(span), 1ull);
 }
 
-//
 // Bound by instruction issue and the atomics' way through the load/store pipe. Bins that need no window, a trash cell instead of
 // selects, a row written once instead of emptied, added to and read back, and a loop of two rounds (the digests asked for
 // ahead change places without moves): decode trace (307 M intervals) 1,215 -> 903 us = 2.7 TB/s of digests, attention 400 -> 323,
@@ -696,11 +686,6 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   if (ov_select) { a.ov = *ov_select; } else { a.ov = ArgusFuseArgs(); }
   a.digest = !scope && !role_tab && !iter_tab && num_regions <= kAggCompactRegions ? (const u64*)digest : nullptr;
   a.parts = digest_parts; a.slices = digest_slices; a.interval_limit = interval_limit;
-  const size_t smem = (size_t)num_regions * sizeof(argus_agg_t);
-  a.use_smem = smem <= kAggSmemLimit;
-  const size_t need = a.use_smem ? smem : 0;
-  if (need > 48 * 1024)
-    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
   const bool windows = iter_tab && num_regions <= kAggCompactRegions;
   a.ranges = windows ? (ulonglong2*)((char*)workspace + L.ranges) : nullptr;
   if (!a.digest) {  // few streams: several blocks share one (how many intervals there are is not known here)
@@ -712,8 +697,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 0);
   if (num_regions <= kAggCompactRegions) {
     const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell);
-    if (compact > 48 * 1024)
-      ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_agg_streams_compact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)compact));
+    static_assert(kAggCompactRegions * sizeof(ArgusAggCell) <= 48 * 1024, "no more shared memory than every kernel gets");
     if (a.digest) {
       const u32 warps = a.slices / a.parts;
       const u32 copies = warps == 16 ? 32 : 8;
@@ -725,7 +709,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
     }
   } else {
-    ARGUS_LAUNCH(k_agg_streams, num_streams, kAggThreads, need, stream, a);
+    ARGUS_LAUNCH(k_agg_streams, num_streams, kAggThreads, 0, stream, a);
   }
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 1);
   if (iter_tab && windows) {

@@ -56,7 +56,7 @@ struct ArgusFuseArgs {    // selection inside the pass over the digests
 };
 
 struct ArgusFuseCtx {     // per CTA, for the stream it is aggregating
-  ArgusAggCell* tab;      // shared memory [R]; null = aggregation off
+  ArgusAggCell* tab;      // shared memory [R]
   u64* row;               // global row of this stream in the warp-scope table
 };
 
@@ -108,7 +108,7 @@ __device__ __forceinline__ void argus_fuse_init(ArgusAggCell* tab, u32 num_regio
   }
 }
 
-// sums of one cell (the part a thread may instead keep in registers for hot regions)
+// sums of one cell
 __device__ __forceinline__ void argus_fuse_agg_sums(ArgusAggCell& c, u64 sum_incl, u64 sum_excl) {
   argus_atomic_add64_split(&c.sum_incl, sum_incl);
   argus_atomic_add64_split(&c.sum_excl, sum_excl);

@@ -616,7 +616,6 @@ extern "C" int argus_pair_intervals_ring(const argus_event_t* ring, uint32_t slo
   if (!status || !stream_offsets || slot_capacity == 0) return ARGUS_ERR_INVALID_ARG;
   if (num_streams && (!ring || !written)) return ARGUS_ERR_INVALID_ARG;
   if (((uintptr_t)written & 7) || ((uintptr_t)dropped & 7)) return ARGUS_ERR_INVALID_ARG;
-  cudaStream_t stream = (cudaStream_t)cuda_stream;
   { const int rc = argus_internal_clear(status, nullptr, 0, cuda_stream); if (rc != ARGUS_OK) return rc; }
   const uint64_t bound = (uint64_t)num_streams * slot_capacity;  // what the slots can hold: sizes the workspace
   int rc = argus_internal_ring_offsets(written, slot_capacity, num_streams, bound, stream_offsets, dropped, status, cuda_stream);

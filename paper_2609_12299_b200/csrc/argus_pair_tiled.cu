@@ -3,11 +3,12 @@
 // One CTA walks one stream tile by tile (T = NT * E events per tile); tiles arrive in shared
 // memory by TMA bulk copies (double buffered, mbarrier completion) and interval records leave with
 // coalesced 16-byte stores, one thread per record. The per-stream region stack is carried from tile
-// to tile in shared memory, so CTAs never wait on one another.
+// to tile in shared memory; a CTA waits for another only when it has nothing to do (see ArgusStreamRecord).
 //
-// Inside a tile the stack height before each event comes from a block-wide prefix sum of +1/-1, so
-// every marker knows its level (stack position) without walking the stack:
-//   - every begin sets its bit in a per-level bitmap over the tile's event positions;
+// Inside a tile the stack height before each event is a count of begins and ends: among 32 in a row by vote, over the
+// warps by one exchange. So every marker knows its level (stack position) without walking the stack:
+//   - the begins of 32 markers in a row that open the same level are one word of that level's bitmap over the tile's
+//     event positions, stored at once (a bit at a time where a window does not cover the tile);
 //   - every end (one thread per end marker) finds its begin as the latest set bit of its own level
 //     before it, and its parent as the latest set bit one level down before that begin; when there
 //     is none in the tile, the frame is in the stack carried from earlier tiles;
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         const int cbase = carlo + cpar * kCar;           // carried level L -> reference cbase + L
         uint4* const car_next = sm.evall + T + (cpar ^ 1) * kCar;
 
-        // ---------------- phase A: heights by prefix sum; begins into per-level bitmaps; ends into `desc` ----------
+        // ---------------- phase A: heights by votes; begins into per-level bitmaps; ends into `desc` ----------
         const bool whole = w0 == 0 && wend == T;  // the usual window: no marker needs a look at the window's bounds
         // a warp looks at 32 E markers in a row, 32 at a time: what lies before a marker is a vote and a count of bits
         const int e0 = w0 + warp * (32 * E) + lane;

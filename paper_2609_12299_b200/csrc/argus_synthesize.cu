@@ -48,7 +48,7 @@ SynLayout syn_layout(uint64_t num_events, uint32_t num_streams, uint32_t num_reg
 }  // namespace
 
 // Where argus_synthesize aggregates and selects overlap spans: -1 automatic, 1 in one pass over the intervals'
-// digests, 2 the plain calls, 3 the same with the aggregation pass over the records (test aid; results are identical).
+// digests, 2 and 3 the plain calls (test aid; results are identical).
 extern "C" void argus_set_synthesize_mode(int mode) { g_synth_mode_knob.store(mode); }
 
 extern "C" size_t argus_synthesize_workspace_bytes(uint64_t num_events, uint32_t num_streams, uint32_t num_regions,

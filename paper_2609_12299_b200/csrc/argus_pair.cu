@@ -1,8 +1,9 @@
 // argus_pair.cu — argus_pair_intervals: marker events -> nested intervals + ambiguity records.
 //
 // Pipeline enqueued on the caller's stream (no host synchronisation):
-//   init, order   : control block and event bitmap cleared; the count of every stream foretold, and from their sum the
-//                   provisional base of its intervals; the order in which streams start
+//   init, order   : control block and event bitmap cleared; the count of every stream foretold, from its ends or, in a malformed
+//                   trace, from all its markers, and from their sum the provisional base of its intervals; the order in which
+//                   streams start
 //   pair pass 1   : intervals written at the provisional bases; per-stream counts; ambiguity notes + bitmap bits
 //   offsets       : scan of counts -> interval_offsets; sets `redo` when a count came out other than foretold;
 //                   popcount prefix over the bitmap if there are notes
@@ -158,12 +159,53 @@ __device__ __forceinline__ bool ends_unclear(const ArgusPairArgs& a, u32 s, u32 
   return !(first & 1u) && (last & 1u) && (first >> 1) != (last >> 1) && !(a.ring_written && a.ring_written[s] > a.ring_capacity);
 }
 
+// A lost or doubled marker inside a stream shows at neither end. Windows of 128 markers all over the trace are looked at: where an
+// end meets, 32 markers at a time, a begin of another region one below it in height, its stream is malformed, and the counts of all
+// streams are then taken from all their markers (recount) instead of from their ends. Seven defects in 10,000 markers show in
+// dozens of the 1,024 windows; a window of a sound trace never tells one. (GEMM trace with that many, 68 M events: 2,263 -> 1,512 us a
+// call, 944 us of a second pass for 208 us of counting; what the look costs a sound one of 2^22 events or more is about 2 us.)
+constexpr u32 kSamples = 1024;  // as many as k_pair_order has threads
+constexpr u32 kSampleRows = 4;
+constexpr u64 kSampledEvents = 1ull << 22;
+// Whether window `w` tells a defect: its stream + 1, or 0. One warp.
+__device__ __forceinline__ u32 sample_window(const ArgusPairArgs& a, u64 off0, u32 w) {
+  const u32 lane = threadIdx.x & 31, lower = (1u << lane) - 1u, s = (u32)(((u64)w * a.num_streams) / kSamples), n = stream_length(a, off0, s);
+  if (n < 32 * kSampleRows) return 0;
+  const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u, at0 = __umulhi(w * 0x9E3779B1u, n - 32 * kSampleRows + 1);
+  const uint4* const src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
+  u32 tags[kSampleRows];
+#pragma unroll
+  for (u32 r = 0; r < kSampleRows; ++r) {
+    u32 at = at0 + 32 * r + lane;
+    if (a.ring_written) { const u32 room = a.ring_capacity - head; at = at >= room ? at - room : head + at; }
+    tags[r] = __ldg(reinterpret_cast<const u32*>(src + at) + 2);
+  }
+  bool bad = false;
+#pragma unroll
+  for (u32 r = 0; r < kSampleRows; ++r) {
+    const bool is_end = tags[r] & 1u;
+    const u32 ends = __ballot_sync(0xffffffffu, is_end);
+    const int level = (int)lane - 2 * __popc(ends & lower) - (int)is_end;  // of the frame it opens or closes
+    const u32 before = __match_any_sync(0xffffffffu, level) & lower;         // (the last of them opened the frame that an end closes)
+    const u32 begin = __shfl_sync(0xffffffffu, tags[r], before ? 31 - __clz((int)before) : 0);
+    bad |= is_end && before && (begin ^ tags[r]) != 1u;
+  }
+  return __any_sync(0xffffffffu, bad) ? s + 1 : 0u;
+}
+
 // A warp takes `per` streams at a time: their first and last markers, a lane each, then a look at those that are not whole.
-__global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uint4* zeroed, u64 zeroed_words, int clear_status, u32 per) {
+// `samples` (nullable): what the windows tell.
+__global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uint4* zeroed, u64 zeroed_words, int clear_status, u32 per, u32* samples) {
   argus_kernel_begin();
   pair_clear(a, zeroed, zeroed_words, clear_status, (u64)blockIdx.x * blockDim.x + threadIdx.x, (u64)gridDim.x * blockDim.x);
   const u32 lane = threadIdx.x & 31;
   const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0, warps = (u64)gridDim.x * (kInitThreads / 32);
+  if (samples && a.num_streams) {
+    for (u32 w = blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5); w < kSamples; w += (u32)warps) {
+      const u32 told = sample_window(a, off0, w);
+      if (lane == 0) samples[w] = told;
+    }
+  }
   int many = -1;  // whether more than a quarter of the streams have unclear ends (a sample of 32 tells, when it is asked for)
   for (u64 s0 = ((u64)blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5)) * per; s0 < a.num_streams; s0 += warps * per) {
     u32 n = 0, f = 0, l = 1;
@@ -222,7 +264,7 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
       c[j] = 0;
       if (s + j < a.num_streams) {
         const u32 n = stream_length(a, off0, (u32)s + j);
-        c[j] = alone ? n >> 1 : a.bases[s + j];
+        c[j] = alone ? n >> 1 : __ldcg(a.bases + s + j);
         cls = n ? 31 - __clz((int)n) : 0;
         *longest = n > *longest ? n : *longest;
         if (RUN == 1) atomicAdd(&cnt[cls], 1u);
@@ -244,13 +286,98 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
   return carry;
 }
 
+// The intervals of stream s as far as its markers' heights tell: ends less those that come below every height before them. Of lost
+// ends and doubled begins this is the exact count. One block.
+__device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, u32 s, int* shi, u32* shu) {
+  const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = stream_length(a, off0, s);
+  const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u, room = a.ring_capacity - head;
+  const uint4* const src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
+  int height = 0, lowest = 0;
+  u32 all_ends = 0;
+  for (u32 i0 = 0; i0 < n; i0 += kScanThreads * 32) {  // 32 markers in a row a thread, read 32 rows of 32 at a time by its warp
+    u32 ends = 0;
+    const u32 w0 = i0 + warp * 1024;
+#pragma unroll 16
+    for (u32 r = 0; r < 32; ++r) {
+      const u32 i = w0 + r * 32 + lane;
+      const u32 at = a.ring_written ? (i >= room ? i - room : head + i) : i;
+      const u32 tag = i < n ? __ldg(reinterpret_cast<const u32*>(src + at) + 2) : 0u;
+      const u32 b = __ballot_sync(0xffffffffu, tag & 1u);
+      if (lane == r) ends = b;
+    }
+    const u32 mine = i0 + tid * 32, have = mine < n ? (n - mine < 32 ? n - mine : 32u) : 0u;
+    const u32 begins = have ? ~ends & (0xffffffffu >> (32 - have)) : 0u;
+    int total;
+    int h = height + argus_block_exclusive_scan<int>(__popc(begins) - __popc(ends), shi, &total);
+#pragma unroll
+    for (u32 r = 0; r < 32; ++r) {
+      h += (int)((begins >> r) & 1u) - (int)((ends >> r) & 1u);
+      lowest = h < lowest ? h : lowest;
+    }
+    all_ends += __popc(ends);
+    height += total;
+  }
+  lowest = __reduce_min_sync(0xffffffffu, lowest);
+  all_ends = __reduce_add_sync(0xffffffffu, all_ends);
+  if (tid == 0) { shi[0] = 0; shu[0] = 0; }
+  __syncthreads();
+  if (lane == 0) { atomicMin(&shi[0], lowest); atomicAdd(&shu[0], all_ends); }
+  __syncthreads();
+  const u32 count = shu[0] - (u32)-shi[0];
+  __syncthreads();
+  return count;
+}
+
+// `samples` (nullable): what the windows that k_pair_init has looked at tell. One block orders; where the trace is malformed, and
+// its first malformed stream lies far enough ahead of the last one that writing the intervals behind it twice would cost more than
+// reading all markers once (a third of a pairing pass), the whole grid counts before the last block orders.
 template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
-                                                            int clear_status, int alone, int ask_split) {
+                                                            int clear_status, int alone, int ask_split, const u32* samples) {
   argus_kernel_begin_long();  // the pairing kernel's blocks spread evenly only over SMs that are free when they come
   __shared__ u32 cnt[64], cur[64];
   __shared__ u64 sh[33];
-  __shared__ u32 one_class, longest_of;
+  __shared__ u32 one_class, longest_of, first_bad;
+  u32 told = 0;
+  if (samples) {
+    static_assert(kSamples == kScanThreads, "a window a thread");
+    told = samples[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x * RUN < a.num_streams) {  // (what comes next, asked for at the same time)
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(a.stream_offsets + threadIdx.x * RUN));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(a.bases + threadIdx.x * RUN));
+    }
+    if (__syncthreads_or(told)) {
+      __shared__ int shi[33];
+      __shared__ u32 next;
+      if (threadIdx.x == 0) first_bad = 0xffffffffu;
+      __syncthreads();
+      if (told) atomicMin(&first_bad, told - 1);
+      __syncthreads();
+      if ((u64)(a.num_streams - first_bad) * 3 > a.num_streams) {
+        const u64 off = a.stream_offsets[0];
+        for (;;) {
+          if (threadIdx.x == 0) next = atomicAdd(&a.ctl->recount_head, 1u);
+          __syncthreads();
+          const u32 s = next;
+          __syncthreads();
+          if (s >= a.num_streams) break;
+          const u32 count = recount_stream(a, off, s, shi, cnt);
+          if (threadIdx.x == 0) a.bases[s] = count;
+        }
+        if (threadIdx.x == 0) {
+          __threadfence();
+          next = atomicAdd(&a.ctl->recount_done, 1u);
+        }
+        __syncthreads();
+        if (next != gridDim.x - 1) return;
+        __threadfence();
+      } else if (blockIdx.x) {
+        return;
+      }
+    } else if (blockIdx.x) {
+      return;
+    }
+  }
   if (threadIdx.x == 0) longest_of = 0;
   if (alone) pair_clear(a, zeroed, zeroed_words, clear_status, threadIdx.x, blockDim.x);
   if (threadIdx.x < 64) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
@@ -263,9 +390,11 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
     if ((threadIdx.x & 31) == 0) atomicMax(&longest_of, longest);
   }
   __syncthreads();
+  // a malformed stream that the split pass would give up together with all others
+  const bool in_vain = ask_split && __syncthreads_or(told && !argus_split_pays(longest_of - stream_length(a, off0, told - 1), a.num_events, a.num_streams));
   if (threadIdx.x == 0) {  // first places, classes in descending order
     a.bases[a.num_streams] = carry;
-    if (ask_split) { a.ctl->split = argus_split_pays(longest_of, a.num_events, a.num_streams); a.ctl->longest = longest_of; }
+    if (ask_split) { a.ctl->split = !in_vain && argus_split_pays(longest_of, a.num_events, a.num_streams); a.ctl->longest = longest_of; }
     u32 base = 0;
     one_class = 0;
     for (int c = 31; c >= 0; --c) {
@@ -547,15 +676,18 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   u32* const order = (u32*)(ws + L.order);
   // Small calls: one block clears and orders. Beyond that a grid clears, and looks at the ends of the streams.
   const bool alone = num_events < (1u << 20) && num_streams <= 8192;
+  // Windows all over the trace are looked at where a second pass would cost much more than the look (50 us against 2).
+  u32* const samples = num_events >= kSampledEvents && num_streams ? (u32*)(ws + L.word_prefix) : nullptr;  // (not used before the offsets kernel)
   if (!alone) {
     // a stream a warp, up to what the chip holds of them
     const u32 per = num_streams <= 148u * 64u ? 1u : num_streams < 32u * 148u * 64u ? (num_streams + 148u * 64u - 1) / (148u * 64u) : 32u;
     const u64 want = ((u64)num_streams / per + kInitThreads / 32 - 1) / (kInitThreads / 32) + zeroed_words / 4096 + 1;
-    ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status, per);
+    ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status, per, samples);
   }
   const bool many = num_streams > kScanThreads;
   const bool split = kernel_choice == 0 && tiled && !ring_written && argus_split_usable(num_events, num_streams);
-  ARGUS_LAUNCH(many ? k_pair_order<kScanRun> : k_pair_order<1>, 1, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone, (int)split);
+  ARGUS_LAUNCH(many ? k_pair_order<kScanRun> : k_pair_order<1>, samples ? 148u : 1u, kScanThreads, 0, stream, a, order, zeroed, zeroed_words, (int)reset_status, (int)alone, (int)split,
+               (const u32*)samples);
   a.order = tiled && num_streams > 1 ? order : nullptr;
   a.segments = nullptr; a.split_failed = nullptr; a.segment_tiles = 0;
 

@@ -37,6 +37,8 @@ struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of
   u32 prefix_done;     // blocks that have counted their share of the ambiguity bitmap
   u32 seg_head;        // segments taken (split pass)
   u32 longest;         // events of the longest stream
+  u32 recount_head;    // streams taken to have their markers counted
+  u32 recount_done;    // blocks that have found no more of them
   alignas(16) u32 num_failed;  // streams that the split pass has to leave to the chained one (read together with the next two)
   u32 num_segments;    // 0 where the segments do not fit their room, too
   u32 split;           // the split pass is worth it (argus_split_pays), and no long stream has been given up

@@ -103,3 +103,74 @@ def test_streams_of_several_outermost_regions(S, length, cut):
     assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)
     assert p.intervals_numpy().tobytes() == iv.tobytes()
     assert p.ambig_numpy().tobytes() == am.tobytes()
+
+
+@pytest.mark.parametrize("defect,where,streams", [("lost ends", 0.0, 900), ("doubled begins", 0.0, 1100), ("lost begins", 0.0, 900), ("lost ends", 0.9, 900),
+                                                  ("cut fronts", 0.0, 900), ("lost ends", 0.0, 300), ("lost ends", 0.98, 300)])
+def test_defects_inside_streams(defect, where, streams):
+    """Defects that show at neither end of a stream, in calls of 2^22 events and more, where windows all over the trace tell them and
+    all markers are counted: in all streams, and in the last ones only; few long streams, too. Stray ends make the count wrong."""
+    rng = np.random.default_rng(streams)
+    spec = tg.config(1).scaled(4, 700)
+    ev, offs = tg.generate_host(spec)
+    source = [ev[offs[s]:offs[s + 1]] for s in range(spec.num_streams)]
+    parts, total = [], 0
+    for s in range(streams):
+        e = source[s % len(source)]
+        if s >= where * streams:
+            is_end = (e["tag"] & 1) == 1
+            hit = rng.random(len(e)) < 0.002
+            hit[0] = hit[-1] = False
+            if defect == "lost ends":
+                e = e[~(hit & is_end)]
+            elif defect == "lost begins":
+                e = e[~(hit & ~is_end)]
+            elif defect == "doubled begins":
+                e = np.repeat(e, 1 + (hit & ~is_end))
+            else:
+                e = e[int(rng.integers(0, 60)):]
+                e = e[~(hit[-len(e):] & ((e["tag"] & 1) == 1))]
+        parts.append(e)
+        total += len(e)
+    while total < 1 << 22:
+        parts += parts[:streams]
+        total *= 2
+    ev = np.concatenate(parts)
+    offs = np.cumsum([0] + [len(e) for e in parts]).astype(np.uint64)
+    _, iv, ioffs, am, aoffs, o_st = oracle.pair(ev, offs, spec.num_regions)
+    assert int(o_st["code"]) == 0 and len(am) > 0
+    p = argus.argus_pair_intervals(torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).to(DEV), torch.from_numpy(offs.view(np.int64).copy()).to(DEV),
+                                   spec.num_regions, ambig_capacity=len(am) + 16)
+    assert int(p.fetch_status()["code"]) == 0
+    assert np.array_equal(p.interval_offsets.cpu().numpy().view(np.uint64), ioffs)
+    assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)
+    assert p.intervals_numpy().tobytes() == iv.tobytes()
+    assert p.ambig_numpy().tobytes() == am.tobytes()
+
+
+def test_wrapped_ring_with_defects():
+    """The same in a ring container: the slots have wrapped, so streams start with ends of lost begins, and ends are missing inside."""
+    rng = np.random.default_rng(3)
+    spec = tg.config(1).scaled(75, 300)
+    ev, offs = tg.generate_host(spec)
+    slot = 4801
+    ring, kept, written = np.zeros((spec.num_streams, slot), argus.EVENT_DTYPE), [], []
+    for s in range(spec.num_streams):
+        e = ev[offs[s]:offs[s + 1]]
+        hit = (rng.random(len(e)) < 0.002) & ((e["tag"] & 1) == 1)
+        e = np.tile(e[~hit], 2)
+        idx = np.arange(max(len(e) - slot, 0), len(e))
+        ring[s, idx % slot] = e[idx]
+        kept.append(e[idx])
+        written.append(len(e))
+    packed = np.concatenate(kept)
+    poffs = np.cumsum([0] + [len(k) for k in kept]).astype(np.uint64)
+    assert len(packed) >= 1 << 22
+    _, iv, ioffs, am, aoffs, o_st = oracle.pair(packed, poffs, spec.num_regions)
+    assert int(o_st["code"]) == 0
+    p, _, _ = argus.argus_pair_intervals_ring(torch.from_numpy(ring.view(np.uint8).reshape(-1).copy()).to(DEV), slot,
+                                              torch.from_numpy(np.array(written, np.int64)).to(DEV), spec.num_regions, ambig_capacity=len(am) + 16)
+    assert int(p.fetch_status()["code"]) == 0
+    assert p.intervals_numpy().tobytes() == iv.tobytes()
+    assert p.ambig_numpy().tobytes() == am.tobytes()
+    assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)

@@ -506,19 +506,65 @@ __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
   }
 }
 
-// iter_tab[ctx - ctx_lo][r] with the compact cells. A block walks a few streams side by side (kIterWarps warps, shared out
+constexpr u32 kIterCopies = 8;  // of the cells of the kDigestHot most frequent regions
+constexpr u32 kItWords = kDgBins + 32;  // a cell: as in the pass over the digests, but with all bins of 32-bit durations (also an odd size)
+static_assert(kItWords % 2 == 1, "an odd cell size keeps the cells of different regions in different banks");
+__host__ __device__ constexpr u32 iter_cells(u32 R) { return R + kDigestHot * kIterCopies; }
+__host__ __device__ constexpr size_t iter_bytes(u32 R) { return 4 * (2 * (size_t)kItWords * iter_cells(R) + R); }
+
+__device__ __forceinline__ void iter_add(u32 cell, u32 incl, u32 excl, u32 flags) {
+  const u32 old_i = dg_add<kDgSumInclLo>(cell, incl), old_e = dg_add<kDgSumExclLo>(cell, excl);
+  dg_max<kDgNotMin>(cell, ~incl);
+  dg_max<kDgMax>(cell, incl);
+  dg_inc<kDgBins>(cell + (31u - (u32)__clz((int)(incl | 1u))) * 4, 1u);
+  if (old_i > ~incl) dg_inc<kDgSumInclHi>(cell, 1u);
+  if (old_e > ~excl) dg_inc<kDgSumExclHi>(cell, 1u);
+  if (flags) dg_inc<kDgFlag>(cell, 1u);
+}
+
+// Adds the cells of an iteration to its row of the table, and empties them. A thread a cell.
+__device__ __forceinline__ void iter_flush(u32* cells, const u32* hot_region, u64* row, u32 R) {
+  for (u32 i = threadIdx.x; i < iter_cells(R); i += kIterThreads) {
+    const u32 r = i < R ? i : hot_region[(i - R) / kIterCopies];
+    if (r >= R) continue;
+    u32* const c = cells + i * kItWords;
+    u64* const g = row + (size_t)r * kCell;
+    u32 cnt = 0;
+#pragma unroll
+    for (u32 j = 0; j < 32; ++j) {
+      const u32 v = c[kDgBins + j];
+      if (v) { atomicAdd(g + 8 + j, (u64)v); c[kDgBins + j] = 0; }
+      cnt += v;
+    }
+    if (!cnt) continue;
+    atomicAdd(g + 0, (u64)cnt);
+    atomicAdd(g + 1, (u64)c[kDgSumInclLo] | ((u64)c[kDgSumInclHi] << 32));
+    atomicMin(g + 2, (u64)~c[kDgNotMin]);
+    atomicMax(g + 3, (u64)c[kDgMax]);
+    atomicAdd(g + 4, (u64)c[kDgSumExclLo] | ((u64)c[kDgSumExclHi] << 32));
+    if (c[kDgFlag]) atomicAdd(g + 7, (u64)c[kDgFlag]);
+#pragma unroll
+    for (u32 f = 0; f < kDgBins; ++f) c[f] = 0;
+  }
+}
+
+// iter_tab[ctx - ctx_lo][r] with cells as in the pass over the digests. A block walks a few streams side by side (kIterWarps warps, shared out
 // among them) and holds the cells of two neighbouring iterations in shared memory; a warp that comes to a later one waits until
 // all have, then the older cells are added to the table. Iterations come in order in a stream, so each is gathered once for
-// all of the block's streams: 550 us for 38 M intervals in 16 iterations of 202 regions, where atomics on the table for every
-// interval took 2.0 ms (adding up the sums of two regions' lanes first: 672 us). An interval of an earlier iteration than the two is added to the table directly. Only the part of a
-// stream that the pass before found to be in the window is read.
+// all of the block's streams; atomics on the table for every interval took 2.0 ms where this took 550 us. An interval of an earlier
+// iteration than the two, or of 2^32 ticks and more, is added to the table directly. Only the part of a stream that the pass before
+// found to be in the window is read, a round ahead. What decides is how many lanes add to one address: with copies of the most
+// frequent regions' cells, and a thread a cell where they are added to the table, the call with all tables goes from 1,616 to 1,508 us
+// for 38 M intervals in 16 iterations of 202 regions, from 2,709 to 2,219 for 115 M in 48, and from 10.1 to 4.4 ms for 34 M in 2,000
+// iterations of five regions. In the same pass as the rows (cells of one stream and iteration) the first took 2,107.
 __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u32 streams_per_block) {
   argus_kernel_begin_long();
   extern __shared__ __align__(16) unsigned char sh_raw[];
   __shared__ u32 need;
   const u32 R = a.num_regions, cells = R * kCell, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  ArgusAggCell* const tab0 = reinterpret_cast<ArgusAggCell*>(sh_raw);
-  ArgusAggCell* const tab1 = tab0 + R;
+  u32 *const tab0 = reinterpret_cast<u32*>(sh_raw), *const tab1 = tab0 + kItWords * iter_cells(R), *const meta = tab1 + kItWords * iter_cells(R);
+  const u32 addr0 = (u32)__cvta_generic_to_shared(tab0), addr1 = (u32)__cvta_generic_to_shared(tab1);
+  __shared__ u32 hot_region[kDigestHot], often[64], num_often;
   constexpr u32 kNone = 0xffffffffu;
   const u32 m = kIterWarps / streams_per_block;  // warps of a stream
   const u32 s = blockIdx.x * streams_per_block + warp / m, mine = warp % m;
@@ -538,40 +584,60 @@ __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u3
       }
     }
   }
-  argus_fuse_init(tab0, 2 * R, threadIdx.x, kIterThreads);
-  if (threadIdx.x == 0) need = kNone;
+  for (u32 i = threadIdx.x; i < 2 * kItWords * iter_cells(R); i += kIterThreads) tab0[i] = 0;
+  for (u32 r = threadIdx.x; r < R; r += kIterThreads) meta[r] = r * (kItWords * 4);
+  if (threadIdx.x < kDigestHot) hot_region[threadIdx.x] = kNone;
+  if (threadIdx.x == 0) { need = kNone; num_often = 0; }
   __syncthreads();
   u64 at = lo < hi ? lo + mine * 32 : ~0ull;
   const u64 end = lo < hi ? hi : 0ull;
   u32 cur = 0;         // the two iterations at hand: cur (in table `odd`) and cur + 1
   u32 odd = 0, want = kNone;
-  bool fresh = true;   // the round at `at` has not been loaded
-  uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
-  u32 flags = 0;
+  bool fresh = true;   // the round at `at` has not been taken up
+  uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0, n0 = q0, n1 = q0;  // the record at hand and the one after it, asked for a round ahead
+  u32 flags = 0, nflags = 0;
+  auto ask = [&](u64 i) {
+    if (i >= end) return;
+    const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
+    n0 = __ldg(p); n1 = __ldg(p + 1);
+    nflags = __ldg(reinterpret_cast<const u32*>(p + 2) + 3) >> 16;
+  };
+  if (at < end) ask(at + lane);
+  // the regions that the first round sees most get copies of their cells, lanes apart: 32 adds to one address take turns
+  if (at < end && at + lane < end && n1.z < R && record_in_scope(a, n1.w, n1.z)) atomicAdd(tab0 + n1.z * kItWords + kDgBins, 1u);
+  __syncthreads();
+  for (u32 r = threadIdx.x; r < R; r += kIterThreads) {
+    const u32 cnt = tab0[r * kItWords + kDgBins];
+    tab0[r * kItWords + kDgBins] = 0;
+    if (cnt >= kIterThreads / 64) often[atomicAdd(&num_often, 1u)] = (cnt << 16) | r;  // at most 64 of them
+  }
+  __syncthreads();
+  if (threadIdx.x < num_often) {
+    const u32 key = often[threadIdx.x], r = key & 0xffffu;
+    u32 rank = 0;
+    for (u32 k = 0; k < num_often; ++k) rank += often[k] > key;
+    if (rank < kDigestHot) { hot_region[rank] = r; meta[r] = ((R + rank * kIterCopies) * (kItWords * 4)) | kDgHot; }
+  }
+  __syncthreads();
+  const u32 own_copy = lane % kIterCopies * (kItWords * 4);
   for (;;) {
     // take what belongs to the two iterations
     while (at < end) {
       if (fresh) {
         const u64 i = at + lane;
-        want = kNone;
-        if (i < end) {
-          const uint4* p = reinterpret_cast<const uint4*>(a.intervals + i);
-          q0 = __ldg(p); q1 = __ldg(p + 1);
-          flags = __ldg(reinterpret_cast<const u32*>(p + 2) + 3) >> 16;
-          if (q1.z < R && record_in_scope(a, q1.w, q1.z)) want = q1.w - a.ctx_lo;
-        }
+        q0 = n0; q1 = n1; flags = nflags;
+        want = i < end && q1.z < R && record_in_scope(a, q1.w, q1.z) ? q1.w - a.ctx_lo : kNone;
+        ask(i + (u64)m * 32);
         fresh = false;
       }
       if (want != kNone && want <= cur + 1) {
         const u64 incl = (u64)q0.z | ((u64)q0.w << 32), excl = (u64)q1.x | ((u64)q1.y << 32);
         u64* const row = a.iter_tab + (u64)want * cells;
-        if (want < cur) {
+        if (want < cur || (q0.w | q1.y)) {
           agg_add_interval(row, q1.z, incl, excl, flags);
         } else {
-          ArgusFuseCtx fx;
-          fx.tab = ((want - cur) ^ odd) ? tab1 : tab0;
-          fx.row = row;
-          argus_fuse_aggregate(fx, q1.z, incl, excl, flags);
+          const u32 mt = meta[q1.z];
+          iter_add((((want - cur) ^ odd) ? addr1 : addr0) + (mt & ~kDgHot) + (mt >> 31) * own_copy, (u32)incl, (u32)excl, flags);
         }
         want = kNone;
       }
@@ -585,13 +651,10 @@ __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u3
     const u32 next = need;
     __syncthreads();
     if (threadIdx.x == 0) need = kNone;
-    ArgusAggCell* const older = odd ? tab1 : tab0;
-    argus_fuse_flush(older, a.iter_tab + (u64)cur * cells, R, threadIdx.x, kIterThreads);
-    if (next != cur + 2 && cur + 1 < a.num_iters) argus_fuse_flush(odd ? tab0 : tab1, a.iter_tab + (u64)(cur + 1) * cells, R, threadIdx.x, kIterThreads);
+    u32* const older = odd ? tab1 : tab0;
+    iter_flush(older, hot_region, a.iter_tab + (u64)cur * cells, R);
+    if (next != cur + 2 && cur + 1 < a.num_iters) iter_flush(odd ? tab0 : tab1, hot_region, a.iter_tab + (u64)(cur + 1) * cells, R);
     if (next == kNone) return;
-    __syncthreads();
-    argus_fuse_init(older, R, threadIdx.x, kIterThreads);
-    if (next != cur + 2) argus_fuse_init(odd ? tab0 : tab1, R, threadIdx.x, kIterThreads);
     if (next == cur + 2) { cur += 1; odd ^= 1; } else { cur = next; }
     __syncthreads();
   }
@@ -715,10 +778,8 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   if (iter_tab && windows) {
     u32 per = kIterWarps;  // streams of a block: at least two blocks for every SM where the streams allow it
     while (per > 1 && num_streams / per < 296) per >>= 1;
-    const size_t two = 2 * (size_t)num_regions * sizeof(ArgusAggCell);
-    if (two > 48 * 1024)
-      ARGUS_CUDA_TRY(argus_allow_smem(k_agg_iter_windows, 2 * (size_t)kAggCompactRegions * sizeof(ArgusAggCell)));
-    ARGUS_LAUNCH(k_agg_iter_windows, (num_streams + per - 1) / per, kIterThreads, two, stream, a, per);
+    if (iter_bytes(num_regions) > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(k_agg_iter_windows, iter_bytes(kAggCompactRegions)));
+    ARGUS_LAUNCH(k_agg_iter_windows, (num_streams + per - 1) / per, kIterThreads, iter_bytes(num_regions), stream, a, per);
   } else if (iter_tab) {
     ARGUS_LAUNCH(k_agg_iter, num_streams < 1184u ? num_streams : 1184u, kAggThreads, 0, stream, a);
   }

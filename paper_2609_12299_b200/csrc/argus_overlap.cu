@@ -146,12 +146,18 @@ __global__ void __launch_bounds__(kSelThreads) k_ov_select(OvSelectArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
-constexpr int kPairThreads = 1024;
-constexpr u32 kPairWarps = kPairThreads / 32;
 constexpr u32 kVT = 9;                                 // spans a thread merges at a time (odd: lanes that far apart hit different banks)
-constexpr u32 kTile = kPairThreads * kVT;              // spans in shared memory at a time (144 KB)
-constexpr u32 kBatch = kPairThreads;                   // slices whose spans are placed at a time
-constexpr size_t kPairSmem = (size_t)kTile * sizeof(ulonglong2);
+__host__ __device__ constexpr u32 bucket_word(u32 b) { return b + (b >> 5); }  // padded: threads sum up runs of counters without bank conflicts
+template <u32 NT>
+struct PairSizes {                                     // of a block of NT threads
+  static constexpr u32 kWarps = NT / 32;
+  static constexpr u32 kTile = NT * kVT;               // spans in shared memory at a time (1,024 threads: 144 KB)
+  static constexpr u32 kBatch = NT;                    // slices whose spans are placed at a time
+  static constexpr u32 kBucketBits = NT == 1024 ? 13 : NT == 512 ? 12 : 11;  // 2^kBucketBits buckets of a role at most
+  static constexpr size_t kSmem = (size_t)kTile * sizeof(ulonglong2);
+  static_assert(kTile <= 1u << 14, "places fit 14 bits");
+  static_assert((2u << kBucketBits) >= kTile && (size_t)kTile * 8 + bucket_word(2u << kBucketBits) * 4 <= kSmem, "a bucket a span, in the tile's room");
+};
 
 struct OvPairArgs {
   const argus_interval_t* intervals;
@@ -212,6 +218,7 @@ __device__ __forceinline__ void merge_serial(const ulonglong2* A, u32 a, u32 na,
 }
 
 // Sorts t[0..cnt) in shared memory by start time: kVT elements a thread in registers, then merges of doubling width.
+template <u32 NT>
 __device__ __noinline__ void sort_tile(ulonglong2* t, u32 cnt) {
   const u32 at = threadIdx.x * kVT;
   ulonglong2 v[kVT];
@@ -246,13 +253,15 @@ __device__ __noinline__ void sort_tile(ulonglong2* t, u32 cnt) {
 }
 
 // Sorts d[0..n) in global memory by start time; `scratch` has as much room. Returns where the sorted spans lie.
+template <u32 NT>
 __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratch, u64 n, ulonglong2* t, u64* sh) {
+  constexpr u32 kTile = PairSizes<NT>::kTile;
   for (u64 t0 = 0; t0 < n; t0 += kTile) {
     const u32 cnt = (u32)(n - t0 < kTile ? n - t0 : kTile);
-    for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) t[i] = d[t0 + i];
+    for (u32 i = threadIdx.x; i < cnt; i += NT) t[i] = d[t0 + i];
     __syncthreads();
-    sort_tile(t, cnt);
-    for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) d[t0 + i] = t[i];
+    sort_tile<NT>(t, cnt);
+    for (u32 i = threadIdx.x; i < cnt; i += NT) d[t0 + i] = t[i];
     __syncthreads();
   }
   const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -267,7 +276,7 @@ __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratc
       __syncthreads();
       const u64 aA = sh[0], aB = sh[1];
       const u32 na = (u32)(aB - aA), cnt = (u32)(d1 - d0), nb = cnt - na;
-      for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) t[i] = i < na ? d[a0 + aA + i] : d[b0 + (d0 - aA) + (i - na)];
+      for (u32 i = threadIdx.x; i < cnt; i += NT) t[i] = i < na ? d[a0 + aA + i] : d[b0 + (d0 - aA) + (i - na)];
       __syncthreads();
       const u32 at = threadIdx.x * kVT;
       ulonglong2 v[kVT];
@@ -279,7 +288,7 @@ __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratc
 #pragma unroll
       for (u32 j = 0; j < kVT; ++j) if (at + j < cnt) t[at + j] = v[j];
       __syncthreads();
-      for (u32 i = threadIdx.x; i < cnt; i += kPairThreads) scratch[t0 + i] = t[i];
+      for (u32 i = threadIdx.x; i < cnt; i += NT) scratch[t0 + i] = t[i];
       __syncthreads();
     }
     ulonglong2* const x = d; d = scratch; scratch = x;
@@ -293,22 +302,21 @@ __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratc
 // bits); the spans follow once (4,096 spans a role: 20 us; merging runs pairwise took 50 us). Returns false, the same for
 // all threads and with nothing written, when a bucket would hold
 // more than kBucketMost (starts that crowd) or a role's starts spread over 2^50 ticks: the caller then merges.
-constexpr u32 kBuckets = 8192, kBucketMost = 32;  // buckets of a role at most
-__host__ __device__ constexpr u32 bucket_word(u32 b) { return b + (b >> 5); }  // padded: threads sum up runs of counters without bank conflicts
-constexpr size_t kBucketSmem = (size_t)kTile * 8 + bucket_word(2 * kBuckets) * 4;
-static_assert(kTile <= 1u << 14 && kBucketSmem <= (size_t)kTile * sizeof(ulonglong2), "places fit 14 bits, buckets the tile's room");
+constexpr u32 kBucketMost = 32;
+template <u32 NT>
 __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong2* in1, u32 n0, u32 n1, ulonglong2* out0, ulonglong2* out1,
-                                          ulonglong2* room, u64 (*red)[kPairWarps + 1], u32* scan) {
+                                          ulonglong2* room, u64 (*red)[NT / 32 + 1], u32* scan) {
+  constexpr u32 kTile = PairSizes<NT>::kTile, kWarps = NT / 32;
   u64* const t = reinterpret_cast<u64*>(room);
   u32* const cnt = reinterpret_cast<u32*>(t + kTile);  // a role's counters after the other's; then where a bucket ends
   const u32 n = n0 + n1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u32 bits = 5;  // 2^bits buckets a role
-  while (bits < 13 && (2u << bits) < n) ++bits;
+  while (bits < PairSizes<NT>::kBucketBits && (2u << bits) < n) ++bits;
   const u32 nb = 2u << bits;
-  for (u32 b = threadIdx.x; b < nb; b += kPairThreads) cnt[bucket_word(b)] = 0;
+  for (u32 b = threadIdx.x; b < nb; b += NT) cnt[bucket_word(b)] = 0;
   u64 low0 = ~0ull, low1 = ~0ull, high0 = 0, high1 = 0;
 #pragma unroll 1
-  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
+  for (u32 i = threadIdx.x; i < n; i += NT) {
     const u64 x = i < n0 ? in0[i].x : in1[i - n0].x;
     if (i < n0) { low0 = x < low0 ? x : low0; high0 = x > high0 ? x : high0; }
     else { low1 = x < low1 ? x : low1; high1 = x > high1 ? x : high1; }
@@ -327,7 +335,7 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
       if (step) break;
       if (lane == 0) { red[0][warp] = mn; red[1][warp] = mx; }
       __syncthreads();
-      mn = red[0][lane]; mx = red[1][lane];
+      mn = lane < kWarps ? red[0][lane] : ~0ull; mx = lane < kWarps ? red[1][lane] : 0ull;
       __syncthreads();
     }
     const u64 range = mx > mn ? mx - mn : 0ull;
@@ -336,13 +344,13 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
     if (role) { low1 = mn; shift1 = sh; } else { low0 = mn; shift0 = sh; }
   }
 #pragma unroll 1
-  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
+  for (u32 i = threadIdx.x; i < n; i += NT) {
     const bool role = i >= n0;
     const u64 x = role ? in1[i - n0].x - low1 : in0[i].x - low0;
     atomicAdd(&cnt[bucket_word((role ? 1u << bits : 0u) + (u32)(x >> (role ? shift1 : shift0)))], 1u);
   }
   __syncthreads();
-  const u32 per = (nb + kPairThreads - 1) / kPairThreads, c0 = threadIdx.x * per;  // counters a thread sums up: consecutive ones
+  const u32 per = (nb + NT - 1) / NT, c0 = threadIdx.x * per;  // counters a thread sums up: consecutive ones
   u32 mine = 0, most = 0;
   for (u32 b = c0; b < c0 + per && b < nb; ++b) { const u32 c = cnt[bucket_word(b)]; mine += c; most = c > most ? c : most; }
   if (__syncthreads_or(most > kBucketMost)) return false;
@@ -351,14 +359,14 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
   for (u32 b = c0; b < c0 + per && b < nb; ++b) { const u32 c = cnt[bucket_word(b)]; cnt[bucket_word(b)] = at; at += c; }
   __syncthreads();
 #pragma unroll 1
-  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {
+  for (u32 i = threadIdx.x; i < n; i += NT) {
     const bool role = i >= n0;
     const u64 x = role ? in1[i - n0].x - low1 : in0[i].x - low0;
     t[atomicAdd(&cnt[bucket_word((role ? 1u << bits : 0u) + (u32)(x >> (role ? shift1 : shift0)))], 1u)] = (x << 14) | i;
   }
   __syncthreads();
 #pragma unroll 1
-  for (u32 i = threadIdx.x; i < n; i += kPairThreads) {  // the counter of a bucket is now where it ends
+  for (u32 i = threadIdx.x; i < n; i += NT) {  // the counter of a bucket is now where it ends
     const bool role = i >= n0;  // (the first n0 elements are role 0's)
     const u64 v = t[i];
     const u32 b = (role ? 1u << bits : 0u) + (u32)((v >> 14) >> (role ? shift1 : shift0)), from = (u32)v & 0x3fffu;
@@ -373,11 +381,12 @@ __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong
 
 // d[0..n) in start order -> the disjoint pieces of their union: piece i = [max(start_i, E), max(end_i, that)) with E the largest
 // end of the spans before i (pieces may be empty). Returns this thread's share of the sum of their lengths.
+template <u32 NT>
 __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
   const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u64 carry = 0, len = 0;
 #pragma unroll 1
-  for (u64 i0 = 0; i0 < n; i0 += kPairThreads) {
+  for (u64 i0 = 0; i0 < n; i0 += NT) {
     const u64 at = i0 + threadIdx.x;
     const ulonglong2 s = at < n ? d[at] : make_ulonglong2(0, 0);
     u64 e = s.y;
@@ -388,7 +397,7 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
     }
     if (lane == 31) red[warp] = e;
     __syncthreads();
-    u64 w = red[lane];
+    u64 w = lane < NT / 32 ? red[lane] : 0ull;
 #pragma unroll
     for (int dd = 1; dd < 32; dd <<= 1) {
       const u64 o = __shfl_up_sync(0xffffffffu, w, dd);
@@ -412,12 +421,15 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
 
 // Latency decides (one block per SM and pair). The entries of up to kBatch slices are taken as one flat sequence, so that
 // every thread has kGather entries and then as many begin times (or pieces of records) in flight, whatever the slices hold.
-// 148 SMs, two roles of 16,000 spans each: 109 us (five kernels before it: 393 us); 2,048 spans a role from 16 interleaved
-// streams: 43 us (178 us); a few hundred spans: 25 us, most of it fixed steps one after the other (45 us): about 12 us go to
-// the gathering, 6 to the sort, 3 to the cutting and 4 to the walk.
+// 148 SMs, two roles of 16,000 spans each: 109 us (five kernels before it: 393 us), about 6.5 a group of 4,096 entries and 10 a tile of
+// the walk; 2,048 spans a role from 16 interleaved streams: 33 us (178 us; 38 with 1,024 threads); a few hundred spans: 25 with 1,024
+// threads, 21 with 512, most of it fixed steps one after the other.
 // DIGEST: entries as the pass over the digests leaves them (argus_fuse.cuh); else {index in the stream, region}.
-template <bool DIGEST, u32 kGather>
-__global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
+template <bool DIGEST, u32 NT>
+__global__ void __launch_bounds__(NT, 1) k_ov_pair(OvPairArgs a) {
+  using Z = PairSizes<NT>;
+  constexpr u32 kGather = 4;  // entries that a thread asks for at a time
+  constexpr u32 kPairThreads = NT, kPairWarps = Z::kWarps, kTile = Z::kTile, kBatch = Z::kBatch;
   argus_kernel_begin_long();
   extern __shared__ __align__(16) unsigned char pair_raw[];
   ulonglong2* const tile = reinterpret_cast<ulonglong2*>(pair_raw);
@@ -510,7 +522,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
               if (e0 + j * kPairThreads >= total) continue;
               const u32 f = e0 + j * kPairThreads + tid, f0 = f - lane;
               // the slice of the warp's first entry: the last one that starts at or before it, 32 probes at a time
-              u32 lo = 32u * ((u32)__popc(__ballot_sync(0xffffffffu, sh_ex[32 * lane] <= f0)) - 1u);
+              u32 lo = 32u * ((u32)__popc(__ballot_sync(0xffffffffu, lane < kBatch / 32 && sh_ex[32 * lane % kBatch] <= f0)) - 1u);
               lo += (u32)__popc(__ballot_sync(0xffffffffu, sh_ex[lo + lane] <= f0)) - 1u;
               if (f < total) while (f >= sh_ex[lo + 1]) ++lo;
               at[j] = lo;
@@ -551,13 +563,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
             if (warp == 0) {
               u32 c[kGather], sum = 0;
 #pragma unroll
-              for (u32 j = 0; j < kGather; ++j) { c[j] = sh_cnt[lane * kGather + j]; sum += c[j]; }
+              for (u32 j = 0; j < kGather; ++j) { c[j] = lane < kPairWarps ? sh_cnt[lane * kGather + j] : 0u; sum += c[j]; }
               u32 incl = sum;
 #pragma unroll
               for (int dd = 1; dd < 32; dd <<= 1) { const u32 o = __shfl_up_sync(0xffffffffu, incl, dd); if (lane >= (u32)dd) incl += o; }
               u32 ex = incl - sum;
 #pragma unroll
-              for (u32 j = 0; j < kGather; ++j) { sh_cnt[lane * kGather + j] = ex; ex += c[j]; }
+              for (u32 j = 0; j < kGather; ++j) { if (lane < kPairWarps) sh_cnt[lane * kGather + j] = ex; ex += c[j]; }
               if (lane == 31) sh_u = incl;
             }
             __syncthreads();
@@ -641,15 +653,15 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_ov_pair(OvPairArgs a) {
     ulonglong2 *const free_a = a.scratch + base + nC, *const free_b = a.spans + base + nP;  // as much room again for either role
     if (cut_a || cut_b) {
       if ((cut_a ? nP : 0ull) + (cut_b ? nC : 0ull) <= kTile &&
-          sort_buckets(A, B, cut_a ? (u32)nP : 0u, cut_b ? (u32)nC : 0u, free_a, free_b, tile, red, sh_scan)) {
+          sort_buckets<NT>(A, B, cut_a ? (u32)nP : 0u, cut_b ? (u32)nC : 0u, free_a, free_b, tile, red, sh_scan)) {
         if (cut_a) A = free_a;
         if (cut_b) B = free_b;
       } else {
-        if (cut_a) A = sort_spans(A, free_a, nP, tile, sh64);
-        if (cut_b) B = sort_spans(B, free_b, nC, tile, sh64);
+        if (cut_a) A = sort_spans<NT>(A, free_a, nP, tile, sh64);
+        if (cut_b) B = sort_spans<NT>(B, free_b, nC, tile, sh64);
       }
-      if (cut_a) len[0] = cut_pieces(A, nP, red[0]);
-      if (cut_b) len[1] = cut_pieces(B, nC, red[1]);
+      if (cut_a) len[0] = cut_pieces<NT>(A, nP, red[0]);
+      if (cut_b) len[1] = cut_pieces<NT>(B, nC, red[1]);
     }
   }
   __syncthreads();
@@ -731,28 +743,32 @@ size_t ov_fixed_bytes(u32 num_streams) {
   return argus_align_up(sizeof(ArgusOvCtl), 256) + argus_align_up((size_t)num_streams * select_slices(num_streams) * sizeof(ArgusOvPiece), 256) + 1024;
 }
 
-template <bool DIGEST, u32 kGather>
-int launch_pair(const OvPairArgs& a, cudaStream_t stream) {
+template <bool DIGEST, u32 NT>
+int launch_pair_as(const OvPairArgs& a, cudaStream_t stream) {
   static std::atomic<bool> opted_in[64];  // the shared-memory opt-in belongs to a device
   int dev = 0;
   ARGUS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return ARGUS_ERR_INVALID_ARG;
   if (!opted_in[dev].load(std::memory_order_acquire)) {
-    ARGUS_CUDA_TRY(cudaFuncSetAttribute(k_ov_pair<DIGEST, kGather>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
+    ARGUS_CUDA_TRY(argus_allow_smem(k_ov_pair<DIGEST, NT>, PairSizes<NT>::kSmem));
     opted_in[dev].store(true, std::memory_order_release);
   }
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);
-  ARGUS_LAUNCH(k_ov_pair<DIGEST, kGather>, a.blocks, kPairThreads, kPairSmem, stream, a);
+  ARGUS_LAUNCH((k_ov_pair<DIGEST, NT>), a.blocks, NT, PairSizes<NT>::kSmem, stream, a);
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 1);
   return ARGUS_OK;
 }
 
-// Entries a thread asks for at a time: four where an SM has many to go through, else two, because a block that runs through its
-// code once waits for that code as well (us for 4 / 2 entries; intervals an SM: 2,500: 27.1 / 25.2, 4,700: 15.9 / 13.9, 90,000 (records): 74.2 /
-// 70.6, 232,000: 108.8 / 113.5, 235,000: 113.0 / 116.9).
+// Threads of a block by how many intervals an SM has on average (how many are spans of a pair is not known here): a block that has
+// little to do waits at its barriers for the warps it has. us with 1,024 / 512 / 256 threads; intervals an SM: 1,200 18.5 / 15.3 /
+// 13.5, 2,500 (all to be sorted) 31.7 / 25.4 / 25.7, 4,700 20.5 / 16.4 / 14.4, 23,000 26.6 / 21.7 / 26.7, 65,000 30.7 / 24.6 / 23.6, 70,000
+// 45.1 / 42.0 / 57.3, 90,000 (records) 77.8 / 72.6 / 93.2, 232,000 112.8 / 127.0 / 195.6, 519,000 (of which 4,000 are spans) 37.7 / 32.5 /
+// 35.9, 4.2 million 82.0 / 115.7 / 177.2. Two entries a thread instead of four: 512 threads 24.7 for the second, 23.5 for the fourth.
 template <bool DIGEST>
 int launch_pair(const OvPairArgs& a, uint64_t num_intervals, cudaStream_t stream) {
-  return num_intervals / a.num_sms < (1u << 17) ? launch_pair<DIGEST, 2>(a, stream) : launch_pair<DIGEST, 4>(a, stream);
+  const u32 ctas = a.num_streams / a.warps_per_cta;  // each is on one SM
+  const u64 sms = ctas < a.num_sms ? (ctas ? ctas : 1u) : a.num_sms, each = num_intervals / sms;
+  return each < 8192 ? launch_pair_as<DIGEST, 256>(a, stream) : each < 1u << 17 ? launch_pair_as<DIGEST, 512>(a, stream) : launch_pair_as<DIGEST, 1024>(a, stream);
 }
 
 }  // namespace

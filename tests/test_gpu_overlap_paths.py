@@ -58,6 +58,24 @@ def test_overlap_sizes_and_orders(order, per_stream):
             assert out.cpu().numpy().view(argus.OVERLAP_DTYPE).reshape(want.shape).tobytes() == want.tobytes()
 
 
+@pytest.mark.parametrize("order", ["disjoint", "overlapping", "shuffled", "crowded"])
+@pytest.mark.parametrize("per_stream,S,W,M", [(1727, 4, 2, 2), (1729, 4, 2, 2), (3455, 4, 2, 2), (3457, 4, 2, 2), (4095, 4, 2, 2), (4096, 4, 2, 2), (100, 16, 16, 1), (700, 32, 16, 1),
+                                              (9, 48, 16, 7)])
+def test_block_sizes(order, per_stream, S, W, M):
+    """Around the spans that blocks of 256 and 512 threads hold, the number of intervals at which a larger one is taken, and with more
+    slices of streams than a block takes at a time."""
+    rng = np.random.default_rng(per_stream)
+    iv = _intervals(rng, per_stream, S, order, 3)
+    offs = (np.arange(S + 1) * per_stream).astype(np.uint64)
+    cta_sm = (np.arange(S // W) % M).astype(np.uint32)
+    pairs_np = np.array([(0, 1), (1, 1), (2, 0)], np.uint32)
+    _, want, _ = oracle.overlap(iv, offs, W, cta_sm, M, pairs_np)
+    out, st = argus.argus_overlap(torch.from_numpy(iv.view(np.uint8).reshape(-1).copy()).to(DEV), len(iv), torch.from_numpy(offs.view(np.int64).copy()).to(DEV),
+                                  W, torch.from_numpy(cta_sm.view(np.int32)).to(DEV), M, torch.from_numpy(pairs_np.view(np.int32)).to(DEV))
+    assert int(argus.argus_status_fetch(st)["code"]) == 0
+    assert out.cpu().numpy().view(argus.OVERLAP_DTYPE).reshape(want.shape).tobytes() == want.tobytes()
+
+
 def test_sm_index_out_of_range_leaves_zeros_and_the_other_tables():
     """A CTA mapped to an SM that does not exist: the call reports it; the overlap is all zeros, and the tables hold every other
     CTA's intervals."""

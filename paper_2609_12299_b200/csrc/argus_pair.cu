@@ -712,7 +712,7 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
       if (pass == 0) argus_prof_mark(ARGUS_PROF_PAIR, stream, 1);
     }
     if (pass == 0)
-      ARGUS_LAUNCH(many ? k_pair_offsets<kScanRun> : k_pair_offsets<1>, (unsigned)(L.num_blocks < 592 ? L.num_blocks : 592) + 1, kScanThreads, 0, stream, g);
+      ARGUS_LAUNCH(many ? k_pair_offsets<kScanRun> : k_pair_offsets<1>, (unsigned)(L.num_blocks < 295 ? L.num_blocks : 295) + 1, kScanThreads, 0, stream, g);
   }
   const u64 want = ((u64)num_streams + 1 + 255) / 256;
   ARGUS_LAUNCH(k_ambig_records, (unsigned)(alone ? (want > 16 ? want : 16) : 296), 256, 0, stream, g);

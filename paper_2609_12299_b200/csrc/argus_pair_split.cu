@@ -14,7 +14,7 @@
 // marker in two of three: 1,922 us when they went on, 1,582 us; 1,385 in the chained passes by themselves).
 //
 // The scan reads the events once more (16 of then 56 bytes an event). 96 streams of 518,656 events: pairing 2,412 -> 660 us
-// (scan 132, chain 36, segments 458, fix 27).
+// (scan 132, chain 29, segments 450, fix 22; 36 and 27 for chain and fix with a warp and a block a stream).
 #include "argus_internal.cuh"
 #include "argus_pair_common.cuh"
 
@@ -120,65 +120,58 @@ __global__ void __launch_bounds__(kScanThreads) k_split_scan(ArgusPairArgs a, u3
   }
 }
 
-// (a segment's summary is asked for four segments ahead: what is left is one round of shared memory per segment)
-__global__ void __launch_bounds__(32) k_split_chain(ArgusPairArgs a, const u32* first_segment) {
+// The summaries of up to kChainBatch segments come into shared memory at once; then one warp goes through them, a round of shared
+// memory per segment (96 streams of 32 segments: 37 us when that warp asked for them itself, four segments ahead, 29 us, of which 20 pass beside the
+// end of the scan).
+constexpr u32 kChainThreads = 256, kChainBatch = 64;
+__global__ void __launch_bounds__(kChainThreads) k_split_chain(ArgusPairArgs a, const u32* first_segment) {
   argus_kernel_begin_long();
   static_assert(ARGUS_MAX_DEPTH == 64, "two levels a lane");
   __shared__ u32 stack[ARGUS_MAX_DEPTH];
-  constexpr u32 kAhead = 4;
+  __shared__ u32 ends[kChainBatch], begins[kChainBatch], open[kChainBatch][ARGUS_MAX_DEPTH];
   const u32 s = blockIdx.x, lane = threadIdx.x;
   if (!__ldcg(&a.ctl->num_segments)) return;  // all streams are left
   const u32 g0 = first_segment[s], g1 = first_segment[s + 1];
   int h = 0;
   bool fail = false;
-  u32 ends[kAhead], begins[kAhead], open0[kAhead], open1[kAhead];
-#pragma unroll
-  for (u32 q = 0; q < kAhead; ++q) {
-    const ArgusSegment* const g = a.segments + (g0 + q < g1 ? g0 + q : g0);
-    ends[q] = __ldcg(&g->unmatched_ends); begins[q] = __ldcg(&g->unmatched_begins);
-    open0[q] = __ldcg(g->open + lane); open1[q] = __ldcg(g->open + lane + 32);
-  }
-  for (u32 k0 = g0; k0 < g1 && !fail; k0 += kAhead) {
-#pragma unroll
-    for (u32 q = 0; q < kAhead; ++q) {
-      const u32 k = k0 + q;
-      if (k >= g1 || fail) break;
-      ArgusSegment* const g = a.segments + k;
-      const int ue = (int)ends[q], ub = (int)begins[q], low = h - ue;
-      const u32 o0 = open0[q], o1 = open1[q];
-      if (k + kAhead < g1) {
-        const ArgusSegment* const n = g + kAhead;
-        ends[q] = __ldcg(&n->unmatched_ends); begins[q] = __ldcg(&n->unmatched_begins);
-        open0[q] = __ldcg(n->open + lane); open1[q] = __ldcg(n->open + lane + 32);
-      }
+  for (u32 k0 = g0; k0 < g1; k0 += kChainBatch) {
+    const u32 have = g1 - k0 < kChainBatch ? g1 - k0 : kChainBatch;
+    const ArgusSegment* const from = a.segments + k0;
+    for (u32 i = threadIdx.x; i < have * ARGUS_MAX_DEPTH; i += kChainThreads) open[i / ARGUS_MAX_DEPTH][i % ARGUS_MAX_DEPTH] = __ldcg(from[i / ARGUS_MAX_DEPTH].open + i % ARGUS_MAX_DEPTH);
+    for (u32 i = threadIdx.x; i < have; i += kChainThreads) { ends[i] = __ldcg(&from[i].unmatched_ends); begins[i] = __ldcg(&from[i].unmatched_begins); }
+    __syncthreads();
+    for (u32 i = 0; lane < 32 && i < have && !fail; ++i) {
+      ArgusSegment* const g = a.segments + k0 + i;
+      const int ue = (int)ends[i], ub = (int)begins[i], low = h - ue;
       if ((int)lane < h) g->idx[lane] = stack[lane];
       if ((int)lane + 32 < h) g->idx[lane + 32] = stack[lane + 32];
       if (lane == 0) g->ch = h;
       if (low < 0 || ub > ARGUS_MAX_DEPTH || low + ub > ARGUS_MAX_DEPTH) { fail = true; break; }
       __syncwarp();
-      if ((int)lane < ub) stack[low + ub - 1 - (int)lane] = o0;
-      if ((int)lane + 32 < ub) stack[low + ub - 1 - (int)lane - 32] = o1;
+      if ((int)lane < ub) stack[low + ub - 1 - (int)lane] = open[i][lane];
+      if ((int)lane + 32 < ub) stack[low + ub - 1 - (int)lane - 32] = open[i][lane + 32];
       h = low + ub;
       __syncwarp();
-      if (k + 1 == g1) {
+      if (k0 + i + 1 == g1) {
         if ((int)lane < h) g->open[lane] = stack[lane];
         if ((int)lane + 32 < h) g->open[lane + 32] = stack[lane + 32];
       }
     }
+    __syncthreads();
   }
   if (fail && lane == 0) argus_split_give_up(a, s, split_length(a, s));
 }
 
-__global__ void __launch_bounds__(kFixThreads) k_split_fix(ArgusPairArgs a, const u32* first_segment) {
+__global__ void __launch_bounds__(kFixThreads) k_split_fix(ArgusPairArgs a, const u32* first_segment, u32 parts) {
   argus_kernel_begin_long();
-  const u32 s = blockIdx.x;
+  const u32 s = blockIdx.x / parts, part = blockIdx.x % parts;  // (blocks that share a stream: a frame a thread)
   bool any_failed;
   if (!argus_split_in_force(a, &any_failed) || (any_failed && __ldcg(a.split_failed + s))) return;
   const u32 g0 = first_segment[s], g1 = first_segment[s + 1], per = a.segment_tiles * kSplitTile;
   const u64 off0 = a.stream_offsets[0];
   u32 ctx = 0, rev = 0, clamp = 0;
   const u64 limit = a.bases[s + 1] < a.interval_capacity ? a.bases[s + 1] : a.interval_capacity;
-  for (u32 i = threadIdx.x; i < (g1 - g0) * ARGUS_MAX_DEPTH; i += blockDim.x) {
+  for (u32 i = part * kFixThreads + threadIdx.x; i < (g1 - g0) * ARGUS_MAX_DEPTH; i += parts * kFixThreads) {
     const u32 k = g0 + i / ARGUS_MAX_DEPTH, l = i % ARGUS_MAX_DEPTH;
     const ArgusSegment* const g = a.segments + k;
     if (l == 0) { ctx += g->flags[0]; rev += g->flags[1]; clamp += g->flags[2]; }
@@ -201,6 +194,7 @@ __global__ void __launch_bounds__(kFixThreads) k_split_fix(ArgusPairArgs a, cons
   if (ctx) atomicAdd((u64*)&a.status->n_ctx_mismatch, (u64)ctx);
   if (rev) atomicAdd((u64*)&a.status->n_time_reversed, (u64)rev);
   if (clamp) atomicAdd((u64*)&a.status->n_child_clamped, (u64)clamp);
+  if (part) return;
   const u32 n = split_length(a, s);
   const ArgusSegment* const last = a.segments + (g1 - 1);
   if (threadIdx.x == 0) a.counts[s] = n ? last->n_int : 0;
@@ -243,9 +237,11 @@ int argus_launch_pair_split(ArgusPairArgs& a, void* room, cudaStream_t stream) {
   a.split_failed = (u32*)w;
   a.segment_tiles = split_tiles(a.num_events);
   ARGUS_LAUNCH(k_split_scan, most, kScanThreads, 0, stream, a, first_segment);
-  ARGUS_LAUNCH(k_split_chain, a.num_streams, 32, 0, stream, a, (const u32*)first_segment);
+  ARGUS_LAUNCH(k_split_chain, a.num_streams, kChainThreads, 0, stream, a, (const u32*)first_segment);
   const int rc = argus_launch_pair_tiled(a, stream, true);
   if (rc != ARGUS_OK) return rc;
-  ARGUS_LAUNCH(k_split_fix, a.num_streams, kFixThreads, 0, stream, a, (const u32*)first_segment);
+  // a level of a segment a thread, on average
+  const u32 each = most / a.num_streams * ARGUS_MAX_DEPTH, parts = (each + kFixThreads - 1) / kFixThreads;
+  ARGUS_LAUNCH(k_split_fix, a.num_streams * parts, kFixThreads, 0, stream, a, (const u32*)first_segment, parts);
   return ARGUS_OK;
 }

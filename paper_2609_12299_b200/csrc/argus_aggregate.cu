@@ -510,7 +510,7 @@ constexpr u32 kIterCopies = 8;  // of the cells of the kDigestHot most frequent 
 constexpr u32 kItWords = kDgBins + 32;  // a cell: as in the pass over the digests, but with all bins of 32-bit durations (also an odd size)
 static_assert(kItWords % 2 == 1, "an odd cell size keeps the cells of different regions in different banks");
 __host__ __device__ constexpr u32 iter_cells(u32 R) { return R + kDigestHot * kIterCopies; }
-__host__ __device__ constexpr size_t iter_bytes(u32 R) { return 4 * (2 * (size_t)kItWords * iter_cells(R) + R); }
+__host__ __device__ constexpr size_t iter_bytes(u32 R) { return 4 * (2 * (size_t)kItWords * iter_cells(R) + R + 4); }
 
 __device__ __forceinline__ void iter_add(u32 cell, u32 incl, u32 excl, u32 flags) {
   const u32 old_i = dg_add<kDgSumInclLo>(cell, incl), old_e = dg_add<kDgSumExclLo>(cell, excl);
@@ -584,7 +584,8 @@ __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u3
       }
     }
   }
-  for (u32 i = threadIdx.x; i < 2 * kItWords * iter_cells(R); i += kIterThreads) tab0[i] = 0;
+  for (u32 i = threadIdx.x; i < (2 * kItWords * iter_cells(R) + 3) / 4; i += kIterThreads) reinterpret_cast<uint4*>(tab0)[i] = make_uint4(0, 0, 0, 0);
+  __syncthreads();  // (the last vector may reach into what follows)
   for (u32 r = threadIdx.x; r < R; r += kIterThreads) meta[r] = r * (kItWords * 4);
   if (threadIdx.x < kDigestHot) hot_region[threadIdx.x] = kNone;
   if (threadIdx.x == 0) { need = kNone; num_often = 0; }

@@ -328,7 +328,9 @@ __device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, 
   return count;
 }
 
-// `samples` (nullable): what the windows that k_pair_init has looked at tell. One block orders; where the trace is malformed, and
+// `samples` (nullable): what the windows that k_pair_init has looked at tell. One block orders; where the trace is malformed (more than
+// one window tells it: a single defect that a window happens to meet is no reason to read everything; 1.2 G markers with one corrupted end
+// at the front 24.5 ms counted, 21.6 not), and
 // its first malformed stream lies far enough ahead of the last one that writing the intervals behind it twice would cost more than
 // reading all markers once (a third of a pairing pass), the whole grid counts before the last block orders.
 template <u32 RUN>
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
       asm volatile("prefetch.global.L1 [%0];" ::"l"(a.stream_offsets + threadIdx.x * RUN));
       asm volatile("prefetch.global.L2 [%0];" ::"l"(a.bases + threadIdx.x * RUN));
     }
-    if (__syncthreads_or(told)) {
+    if (__syncthreads_count(told != 0) > 1) {
       __shared__ int shi[33];
       __shared__ u32 next;
       if (threadIdx.x == 0) first_bad = 0xffffffffu;

@@ -75,10 +75,11 @@ __device__ __forceinline__ void argus_set_error(argus_status_t* st, u32 code, u3
 }
 
 // Exclusive prefix sum over the threads of a block (blockDim.x <= 1024, multiple of 32).
-// `warp_sums` is shared scratch of >= 33 elements. Returns the exclusive prefix of `v`;
-// *total receives the block total. Contains __syncthreads().
-template <typename T>
-__device__ __forceinline__ T argus_block_exclusive_scan(T v, T* warp_sums, T* total) {
+// `warp_sums` is shared scratch of 33 elements whatever the block's size (the first warp writes a full warp of them). Returns the
+// exclusive prefix of `v`; *total receives the block total. Contains __syncthreads().
+template <typename T, int N>
+__device__ __forceinline__ T argus_block_exclusive_scan(T v, T (&warp_sums)[N], T* total) {
+  static_assert(N >= 33, "a full warp's sums and the total");
   const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
   T incl = v;
 #pragma unroll

@@ -305,7 +305,7 @@ __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratc
 constexpr u32 kBucketMost = 32;
 template <u32 NT>
 __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong2* in1, u32 n0, u32 n1, ulonglong2* out0, ulonglong2* out1,
-                                          ulonglong2* room, u64 (*red)[NT / 32 + 1], u32* scan) {
+                                          ulonglong2* room, u64 (*red)[NT / 32 + 1], u32 (&scan)[33]) {
   constexpr u32 kTile = PairSizes<NT>::kTile, kWarps = NT / 32;
   u64* const t = reinterpret_cast<u64*>(room);
   u32* const cnt = reinterpret_cast<u32*>(t + kTile);  // a role's counters after the other's; then where a bucket ends
@@ -437,6 +437,7 @@ __global__ void __launch_bounds__(NT, 1) k_ov_pair(OvPairArgs a) {
   __shared__ u32 sh_ex[kBatch + 1];                // entries of the batch before slice i
   __shared__ u64 sh_pos[kBatch], sh_iv[kBatch];    // where a slice's entries and its stream's intervals start
   __shared__ u32 sh_scan[33];
+  __shared__ u64 sh_scan64[33];
   __shared__ u64 sh64[4];
   __shared__ u64 red[2][kPairWarps + 1];
   __shared__ u32 sh_cnt[kGather * kPairWarps];
@@ -502,7 +503,7 @@ __global__ void __launch_bounds__(NT, 1) k_ov_pair(OvPairArgs a) {
           if (round == 0 && a.num_pairs == 1) { my_all += pc.count; continue; }
           // slices that hold something, one after the other: where each starts in the flat sequence
           u64 all;
-          const u64 ex = argus_block_exclusive_scan<u64>((u64)pc.count | (pc.count ? 1ull << 32 : 0ull), red[0], &all);
+          const u64 ex = argus_block_exclusive_scan<u64>((u64)pc.count | (pc.count ? 1ull << 32 : 0ull), sh_scan64, &all);
           const u32 total = (u32)all, slices = (u32)(all >> 32);
           if (pc.count) {
             const u32 at = (u32)(ex >> 32);

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uin
 // ---------------------------------------------------------------------------------------------
 // Returns the sum of the foretold counts; *longest: events of the longest stream of this thread.
 template <u32 RUN>
-__device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int alone, u32* cnt, u64* sh, u32* longest) {
+__device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int alone, u32* cnt, u64 (&sh)[33], u32* longest) {
   u64 carry = 0;
   for (u64 s0 = 0; s0 < a.num_streams; s0 += kScanThreads * RUN) {
     const u64 s = s0 + threadIdx.x * RUN;
@@ -288,7 +288,7 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
 
 // The intervals of stream s as far as its markers' heights tell: ends less those that come below every height before them. Of lost
 // ends and doubled begins this is the exact count. One block.
-__device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, u32 s, int* shi, u32* shu) {
+__device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, u32 s, int (&shi)[33], u32* shu) {
   const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = stream_length(a, off0, s);
   const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u, room = a.ring_capacity - head;
   const uint4* const src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
@@ -434,7 +434,7 @@ struct AmbigArgs {
 
 // interval_offsets; returns the sum of the counts. *bad: first stream that does not lie right, *used: last one that has any.
 template <u32 RUN>
-__device__ __forceinline__ u64 final_offsets(const ArgusPairArgs& a, u64* sh, u32* bad, u32* used) {
+__device__ __forceinline__ u64 final_offsets(const ArgusPairArgs& a, u64 (&sh)[33], u32* bad, u32* used) {
   u64 carry = 0;
   for (u64 s0 = 0; s0 < a.num_streams; s0 += kScanThreads * RUN) {
     const u64 s = s0 + threadIdx.x * RUN;

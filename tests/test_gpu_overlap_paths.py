@@ -76,6 +76,32 @@ def test_block_sizes(order, per_stream, S, W, M):
     assert out.cpu().numpy().view(argus.OVERLAP_DTYPE).reshape(want.shape).tobytes() == want.tobytes()
 
 
+@pytest.mark.parametrize("order", ["disjoint", "overlapping", "crowded"])
+@pytest.mark.parametrize("S,W,M,per_stream", [(2080, 4, 4, 12), (640, 2, 2, 24), (96, 16, 1, 64)])
+def test_many_ctas_an_sm_and_three_pairs(order, S, W, M, per_stream):
+    """Few intervals an SM (blocks of 256 threads) that lie in more CTAs than a block has threads, and in several batches of
+    slices for each of them: what a block keeps of its CTAs outlives the scans in between. Plain call and one-call pipeline."""
+    rng = np.random.default_rng(S)
+    iv = _intervals(rng, per_stream, S, order, 3)
+    ev = np.zeros((S, per_stream, 2), argus.EVENT_DTYPE)
+    ev["ts"][:, :, 0] = iv["t_begin"].reshape(S, -1)
+    ev["ts"][:, :, 1] = (iv["t_begin"] + iv["inclusive"]).reshape(S, -1)
+    ev["tag"] = np.stack([iv["region"] << 1, (iv["region"] << 1) | 1], axis=-1).reshape(S, per_stream, 2)
+    offs = (np.arange(S + 1) * per_stream).astype(np.uint64)
+    cta_sm = rng.integers(0, M, S // W).astype(np.uint32)
+    pairs_np = np.array([(0, 1), (1, 1), (2, 0)], np.uint32)
+    _, want, _ = oracle.overlap(iv, offs, W, cta_sm, M, pairs_np)
+    d_sm, d_pairs = torch.from_numpy(cta_sm.view(np.int32)).to(DEV), torch.from_numpy(pairs_np.view(np.int32)).to(DEV)
+    out, st = argus.argus_overlap(torch.from_numpy(iv.view(np.uint8).reshape(-1).copy()).to(DEV), len(iv), torch.from_numpy(offs.view(np.int64).copy()).to(DEV),
+                                  W, d_sm, M, d_pairs)
+    assert int(argus.argus_status_fetch(st)["code"]) == 0
+    assert out.cpu().numpy().view(argus.OVERLAP_DTYPE).reshape(want.shape).tobytes() == want.tobytes()
+    r = argus.argus_synthesize(torch.from_numpy(ev.reshape(-1).view(np.uint8).copy()).to(DEV), torch.from_numpy((2 * offs).view(np.int64).copy()).to(DEV), 3, W,
+                               d_sm, M, d_pairs, max_overlap_spans=2 * 3 * len(iv))
+    assert int(r.fetch_status()["code"]) == 0
+    assert r.overlap_numpy(M).tobytes() == want.tobytes()
+
+
 def test_sm_index_out_of_range_leaves_zeros_and_the_other_tables():
     """A CTA mapped to an SM that does not exist: the call reports it; the overlap is all zeros, and the tables hold every other
     CTA's intervals."""

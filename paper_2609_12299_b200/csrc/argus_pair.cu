@@ -289,41 +289,44 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
 // The intervals of stream s as far as its markers' heights tell: ends less those that come below every height before them. Of lost
 // ends and doubled begins this is the exact count. One block.
 __device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, u32 s, int (&shi)[33], u32* shu) {
+  static_assert(kRecountStep == kScanThreads * 32, "32 markers in a row a thread");
   const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = stream_length(a, off0, s);
   const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u, room = a.ring_capacity - head;
   const uint4* const src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
-  int height = 0, lowest = 0;
+  long long height = 0, lowest = 0;
   u32 all_ends = 0;
-  for (u32 i0 = 0; i0 < n; i0 += kScanThreads * 32) {  // 32 markers in a row a thread, read 32 rows of 32 at a time by its warp
+  for (u32 round = 0, rounds = argus_recount_rounds(n); round < rounds; ++round) {  // rows of 32 are read by a warp, 32 at a time
+    const u32 have = argus_recount_markers(n, round), i0 = round * kRecountStep;
     u32 ends = 0;
-    const u32 w0 = i0 + warp * 1024;
 #pragma unroll 16
     for (u32 r = 0; r < 32; ++r) {
-      const u32 i = w0 + r * 32 + lane;
-      const u32 at = a.ring_written ? (i >= room ? i - room : head + i) : i;
-      const u32 tag = i < n ? __ldg(reinterpret_cast<const u32*>(src + at) + 2) : 0u;
+      const u32 j = warp * 1024 + r * 32 + lane;
+      u32 at = i0 + j;
+      if (a.ring_written) at = at >= room ? at - room : head + at;
+      const u32 tag = j < have ? __ldg(reinterpret_cast<const u32*>(src + at) + 2) : 0u;
       const u32 b = __ballot_sync(0xffffffffu, tag & 1u);
       if (lane == r) ends = b;
     }
-    const u32 mine = i0 + tid * 32, have = mine < n ? (n - mine < 32 ? n - mine : 32u) : 0u;
-    const u32 begins = have ? ~ends & (0xffffffffu >> (32 - have)) : 0u;
+    const u32 mine = tid * 32 >= have ? 0u : have - tid * 32 < 32 ? have - tid * 32 : 32u;
+    const u32 begins = mine ? ~ends & (0xffffffffu >> (32 - mine)) : 0u;
     int total;
-    int h = height + argus_block_exclusive_scan<int>(__popc(begins) - __popc(ends), shi, &total);
+    int h = argus_block_exclusive_scan<int>(__popc(begins) - __popc(ends), shi, &total), low = 0;  // (from the round's first marker on)
 #pragma unroll
     for (u32 r = 0; r < 32; ++r) {
       h += (int)((begins >> r) & 1u) - (int)((ends >> r) & 1u);
-      lowest = h < lowest ? h : lowest;
+      low = h < low ? h : low;
     }
+    lowest = height + low < lowest ? height + low : lowest;
     all_ends += __popc(ends);
     height += total;
   }
-  lowest = __reduce_min_sync(0xffffffffu, lowest);
+  const u32 below = __reduce_max_sync(0xffffffffu, (u32)-lowest);
   all_ends = __reduce_add_sync(0xffffffffu, all_ends);
-  if (tid == 0) { shi[0] = 0; shu[0] = 0; }
+  if (tid < 2) shu[tid] = 0;
   __syncthreads();
-  if (lane == 0) { atomicMin(&shi[0], lowest); atomicAdd(&shu[0], all_ends); }
+  if (lane == 0) { atomicMax(&shu[0], below); atomicAdd(&shu[1], all_ends); }
   __syncthreads();
-  const u32 count = shu[0] - (u32)-shi[0];
+  const u32 count = shu[1] - shu[0];
   __syncthreads();
   return count;
 }

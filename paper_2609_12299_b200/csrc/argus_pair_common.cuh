@@ -145,6 +145,14 @@ __device__ __forceinline__ void argus_split_give_up(const ArgusPairArgs& a, u32 
   else atomicExch(&a.ctl->split, 0u);
 }
 
+// The markers of a stream are counted in rounds of kRecountStep. A stream may hold up to 2^32 - 1 markers, so the end of the last
+// round need not fit 32 bits, and no loop may run up to it.
+constexpr u32 kRecountStep = 32768;
+__host__ __device__ constexpr u32 argus_recount_rounds(u32 n) { return n / kRecountStep + (n % kRecountStep != 0); }
+__host__ __device__ constexpr u32 argus_recount_markers(u32 n, u32 round) {  // of that round
+  return n - round * kRecountStep < kRecountStep ? n - round * kRecountStep : kRecountStep;
+}
+
 #define ARGUS_NOTE_POS_BITS 48
 
 // Ring container: slot position of the oldest surviving record of stream s.

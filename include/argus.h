@@ -136,7 +136,8 @@ typedef struct {
 /* Device-resident status block, 64 bytes. */
 typedef struct {
   uint32_t code;       /* ARGUS_OK or the first device error                     */
-  uint32_t bad_stream; /* stream where the first error was seen                  */
+  uint32_t bad_stream; /* stream where the first error was seen; for a CTA whose SM does not
+                          exist, the first stream of the first such CTA            */
   uint64_t bad_event;  /* event index within that stream (or offending count)    */
   uint64_t intervals_required;
   uint64_t ambig_required;

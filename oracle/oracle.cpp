@@ -162,7 +162,7 @@ extern "C" int oracle_aggregate(const OInterval* intervals, const uint64_t* inte
   for (uint32_t s = 0; s < num_streams; ++s) {
     uint32_t keys[4];
     keys_of(s, keys);
-    if (cta_sm && keys[2] >= num_sms && sm_tab) return ERR_INVALID;
+    if (cta_sm && keys[2] >= num_sms && sm_tab) { fail(st, ERR_INVALID, s, keys[2]); return ERR_INVALID; }
     for (uint64_t i = interval_offsets[s]; i < interval_offsets[s + 1]; ++i) {
       const OInterval& v = intervals[i];
       if (v.region >= num_regions) { fail(st, ERR_BAD_REGION, s, i); return OK; }
@@ -228,7 +228,7 @@ extern "C" int oracle_overlap(const OInterval* intervals, const uint64_t* interv
   std::vector<std::vector<uint32_t>> streams_of_sm(num_sms);  // which streams ran on each SM
   for (uint32_t s = 0; s < num_streams; ++s) {
     const uint32_t m = cta_sm[s / warps_per_cta];
-    if (m >= num_sms) return ERR_INVALID;
+    if (m >= num_sms) { fail(st, ERR_INVALID, s, m); return ERR_INVALID; }
     streams_of_sm[m].push_back(s);
   }
   for (uint32_t k = 0; k < num_pairs; ++k) {
@@ -305,7 +305,7 @@ extern "C" int oracle_aggregate_scoped(const OInterval* intervals, const uint64_
     keys[2] = cta_sm ? cta_sm[s / warps_per_cta] : 0;
     keys[3] = 0;
     keys[4] = s % warps_per_cta;
-    if (cta_sm && keys[2] >= num_sms && (sm_tab || (scope && scope->sm_mask))) return ERR_INVALID;
+    if (cta_sm && keys[2] >= num_sms && (sm_tab || (scope && scope->sm_mask))) { fail(st, ERR_INVALID, s, keys[2]); return ERR_INVALID; }
     for (uint64_t i = interval_offsets[s]; i < interval_offsets[s + 1]; ++i) {
       const OInterval& v = intervals[i];
       if (v.region >= num_regions) { fail(st, ERR_BAD_REGION, s, i); return OK; }
@@ -356,7 +356,7 @@ extern "C" int oracle_overlap_scoped(const OInterval* intervals, const uint64_t*
   if (scope && scope->ctx_hi < scope->ctx_lo) return ERR_INVALID;
   std::memset(st, 0, sizeof(*st));
   for (uint32_t s = 0; s < num_streams; ++s)
-    if (cta_sm[s / warps_per_cta] >= num_sms) return ERR_INVALID;
+    if (cta_sm[s / warps_per_cta] >= num_sms) { fail(st, ERR_INVALID, s, cta_sm[s / warps_per_cta]); return ERR_INVALID; }
   for (uint32_t k = 0; k < num_pairs; ++k) {
     const uint32_t P = pairs[2 * k], Cn = pairs[2 * k + 1];
     for (uint32_t sm = 0; sm < num_sms; ++sm) {

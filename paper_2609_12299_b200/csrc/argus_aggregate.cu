@@ -63,6 +63,8 @@ __device__ __forceinline__ void agg_empty_tables(const AggArgs& a) {
 
 __device__ __forceinline__ bool mask_bit(const u32* mask, u32 i) { return !mask || ((mask[i >> 5] >> (i & 31)) & 1u); }
 
+__device__ __forceinline__ void bad_sm(const AggArgs& a, u32 cta) { argus_report_bad_sm(a.status, a.cta_sm, a.num_sms, a.warps_per_cta, cta); }
+
 // Warp-role and SM tests of a scope: one answer per stream. 2 = bad cta_sm entry.
 __device__ __forceinline__ int stream_in_scope(const AggArgs& a, u32 s) {
   if (!a.scoped) return 1;
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
     __syncthreads();
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
     const int sel = stream_in_scope(a, s);
-    if (sel == 2 && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, a.cta_sm[s / a.warps_per_cta]);
+    if (sel == 2 && threadIdx.x == 0) bad_sm(a, s / a.warps_per_cta);
     if (hi < lo || hi > a.interval_limit) {
       if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
     } else if (sel == 1) {
@@ -154,7 +156,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
   fx.tab = ctab; fx.row = row;
   u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
   const int sel = stream_in_scope(a, s);
-  if (sel == 2 && threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, a.cta_sm[s / a.warps_per_cta]);
+  if (sel == 2 && threadIdx.x == 0) bad_sm(a, s / a.warps_per_cta);
   if (hi < lo || hi > a.interval_limit) {
     if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
   } else if (sel == 1) {
@@ -282,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
     meta[r] = (tab_addr + r * (kDgWords * 4)) | (r < R && ((pairbits[r >> 5] >> (r & 31)) & 1u) ? kDgInPair : 0u);
   if (has_ov && tid == 0) {
     const u32 m = a.cta_sm[s / a.warps_per_cta];
-    if (m >= a.num_sms) argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, s, m);
+    if (m >= a.num_sms) bad_sm(a, s / a.warps_per_cta);
   }
   const bool good = hi >= lo && hi <= a.interval_limit && !((hi - lo) >> 32);
   if (!good && tid == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
       if (cta_out) cta_out[(u64)(c0 + q) * per_cta + rem] = v[q];
       if (a.sm_tab && v[q] != none) {
         const u32 m = a.cta_sm[c0 + q];
-        if (m >= a.num_sms) { argus_set_error(a.status, ARGUS_ERR_INVALID_ARG, c0 + q, m); continue; }
+        if (m >= a.num_sms) { bad_sm(a, c0 + q); continue; }
         cell_add(a.sm_tab + (u64)m * per_cta + rem, field, v[q]);
       }
       all = combine(field, all, v[q]);

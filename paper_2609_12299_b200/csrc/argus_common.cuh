@@ -74,6 +74,15 @@ __device__ __forceinline__ void argus_set_error(argus_status_t* st, u32 code, u3
   }
 }
 
+// For whoever meets a CTA that is mapped to an SM that does not exist (CTA `met`): names the first such CTA's first stream, so that
+// the answer is the same whoever comes first.
+static __device__ __noinline__ void argus_report_bad_sm(argus_status_t* st, const u32* cta_sm, u32 num_sms, u32 warps_per_cta, u32 met) {
+  if (*reinterpret_cast<volatile u32*>(&st->code)) return;
+  u32 c = 0;
+  while (c < met && cta_sm[c] < num_sms) ++c;
+  argus_set_error(st, ARGUS_ERR_INVALID_ARG, c * warps_per_cta, cta_sm[c]);
+}
+
 // Exclusive prefix sum over the threads of a block (blockDim.x <= 1024, multiple of 32).
 // `warp_sums` is shared scratch of 33 elements whatever the block's size (the first warp writes a full warp of them). Returns the
 // exclusive prefix of `v`; *total receives the block total. Contains __syncthreads().

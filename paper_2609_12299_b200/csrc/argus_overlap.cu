@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(kSelThreads) k_ov_select(OvSelectArgs a) {
     const u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
     bool take = true;
     if (m >= a.num_sms || hi < lo || hi > a.max_intervals || ((hi - lo) >> 32)) {  // offsets beyond the interval array are reported, not read
-      if (threadIdx.x == 0) argus_set_error(a.status, m >= a.num_sms ? ARGUS_ERR_INVALID_ARG : ARGUS_ERR_BAD_OFFSETS, s, m);
+      if (threadIdx.x == 0 && m >= a.num_sms) argus_report_bad_sm(a.status, a.cta_sm, a.num_sms, a.warps_per_cta, s / a.warps_per_cta);
+      else if (threadIdx.x == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, m);
       take = false;
     } else if (a.scoped) {  // warp-role and SM tests: one answer per stream
       const u32 w = s % a.warps_per_cta;

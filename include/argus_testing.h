@@ -44,10 +44,13 @@ int argus_profile_read(double* ms_total /*host [4]*/, unsigned long long* launch
  * thread, 7 blocks per SM>, 1..3 = <192,5,4>, <64,5,8>, <256,7,2> (tiles end at other places).
  * argus_testing_set_poll_limit: polls after which a block of the tiled pairing kernel that waits for a
  * hand-over gives up with ARGUS_ERR_TIMEOUT (default 2^19, about a second; 0 restores the default). A test
- * sets it to a few polls to see the bounded wait run out and the call return with the status set. */
+ * sets it to a few polls to see the bounded wait run out and the call return with the status set.
+ * argus_testing_pair_passes: after a pairing call (or argus_synthesize) in this workspace is complete, whether the
+ * trace's markers were counted before pairing and whether its second pass rewrote intervals. Waits for the device. */
 void argus_set_synthesize_mode(int mode);
 void argus_set_tile_variant(int variant);
 void argus_testing_set_poll_limit(unsigned int polls);
+int argus_testing_pair_passes(const void* workspace /*device*/, uint32_t* counted /*host*/, uint32_t* second_pass /*host*/);
 
 #ifdef __cplusplus
 }

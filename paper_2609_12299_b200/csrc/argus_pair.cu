@@ -161,16 +161,45 @@ __device__ __forceinline__ bool ends_unclear(const ArgusPairArgs& a, u32 s, u32 
 
 // A lost or doubled marker inside a stream shows at neither end. Windows of 128 markers all over the trace are looked at: where an
 // end meets, 32 markers at a time, a begin of another region one below it in height, its stream is malformed, and the counts of all
-// streams are then taken from all their markers (recount) instead of from their ends. Seven defects in 10,000 markers show in
+// streams may be taken from all their markers (recount) instead of from their ends. Seven defects in 10,000 markers show in
 // dozens of the 1,024 windows; a window of a sound trace never tells one. (GEMM trace with that many, 68 M events: 2,263 -> 1,512 us a
-// call, 944 us of a second pass for 208 us of counting; what the look costs a sound one of 2^22 events or more is about 2 us.)
+// call, 944 us of a second pass for 208 us of counting.) The look costs a sound trace about 2 us. Smaller calls do not look, because
+// sound ones would be longer by more than a thirtieth: pairing of 1.06, 2.1 and 4.1 M sound events takes 33, 43 and 62 us (with seven
+// lost ends in 10,000 markers, and so a second pass, 124, 148 and 246).
+// Counting goes by heights, which lost ends and doubled begins raise for good, and lost begins and doubled ends lower; of either
+// alone it is exact. A marker of which the region has changed leaves the heights as they are but takes its interval away, and of both kinds
+// together one hides the other: counts are then wrong and the second pass comes all the same (68.7 M events, seven in 10,000 ends changed:
+// 2,598 us; counting would add its 205). So a window also tells what kind it has met.
 constexpr u32 kSamples = 1024;  // as many as k_pair_order has threads
 constexpr u32 kSampleRows = 4;
 constexpr u64 kSampledEvents = 1ull << 22;
-// Whether window `w` tells a defect: its stream + 1, or 0. One warp.
+enum : u32 { kNoDefect = 0, kUnclear = 1, kChanged = 2, kLowered = 3, kRaised = 4 };
+__device__ __forceinline__ u32 sample_stream(const ArgusPairArgs& a, u32 w) { return (u32)(((u64)w * a.num_streams) / kSamples); }
+// What kind of defect a row of 32 markers holds, given which of its ends (`bad`) meet the begin of another region. One warp.
+__device__ __noinline__ u32 sample_kind(u32 bad, u32 ends, u32 tag, u32 begin, int level) {
+  u32 kind = kUnclear, passed = 0xffffffffu;  // region of the last begin that was met by another region's end
+  const u32 region = tag >> 1;
+  for (; bad; bad &= bad - 1) {
+    const int i = __ffs((int)bad) - 1;
+    const u32 closing = __shfl_sync(0xffffffffu, region, i), met = __shfl_sync(0xffffffffu, begin >> 1, i);
+    const u32 around = __ballot_sync(0xffffffffu, level == __shfl_sync(0xffffffffu, level, i) - 1);
+    const u32 earlier = around & ((1u << i) - 1u), later = around & ends & ~((2u << i) - 1u);
+    // the begin of the frame around, and the end that closes it
+    const u32 outer = __shfl_sync(0xffffffffu, region, earlier ? 31 - __clz((int)earlier) : 0), next = __shfl_sync(0xffffffffu, region, later ? __ffs((int)later) - 1 : 0);
+    const u32 k = closing == passed ? kLowered                    // the frame that the last such end has passed over
+                  : earlier && closing == outer ? kRaised         // the frame met here is closed along with the one around it
+                  : later && next == met ? kLowered
+                  : earlier && later && next == outer ? kChanged  // as if this end were the right one
+                                                      : kUnclear;
+    kind = k > kind ? k : kind;
+    passed = met;
+  }
+  return kind;
+}
+// What window `w` tells. One warp.
 __device__ __forceinline__ u32 sample_window(const ArgusPairArgs& a, u64 off0, u32 w) {
-  const u32 lane = threadIdx.x & 31, lower = (1u << lane) - 1u, s = (u32)(((u64)w * a.num_streams) / kSamples), n = stream_length(a, off0, s);
-  if (n < 32 * kSampleRows) return 0;
+  const u32 lane = threadIdx.x & 31, lower = (1u << lane) - 1u, s = sample_stream(a, w), n = stream_length(a, off0, s);
+  if (n < 32 * kSampleRows) return kNoDefect;
   const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u, at0 = __umulhi(w * 0x9E3779B1u, n - 32 * kSampleRows + 1);
   const uint4* const src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
   u32 tags[kSampleRows];
@@ -180,7 +209,7 @@ __device__ __forceinline__ u32 sample_window(const ArgusPairArgs& a, u64 off0, u
     if (a.ring_written) { const u32 room = a.ring_capacity - head; at = at >= room ? at - room : head + at; }
     tags[r] = __ldg(reinterpret_cast<const u32*>(src + at) + 2);
   }
-  bool bad = false;
+  u32 kind = kNoDefect;
 #pragma unroll
   for (u32 r = 0; r < kSampleRows; ++r) {
     const bool is_end = tags[r] & 1u;
@@ -188,9 +217,13 @@ __device__ __forceinline__ u32 sample_window(const ArgusPairArgs& a, u64 off0, u
     const int level = (int)lane - 2 * __popc(ends & lower) - (int)is_end;  // of the frame it opens or closes
     const u32 before = __match_any_sync(0xffffffffu, level) & lower;         // (the last of them opened the frame that an end closes)
     const u32 begin = __shfl_sync(0xffffffffu, tags[r], before ? 31 - __clz((int)before) : 0);
-    bad |= is_end && before && (begin ^ tags[r]) != 1u;
+    const u32 bad = __ballot_sync(0xffffffffu, is_end && before && (begin ^ tags[r]) != 1u);
+    if (bad) {
+      const u32 k = sample_kind(bad, ends, tags[r], begin, level);
+      kind = k > kind ? k : kind;
+    }
   }
-  return __any_sync(0xffffffffu, bad) ? s + 1 : 0u;
+  return kind;
 }
 
 // A warp takes `per` streams at a time: their first and last markers, a lane each, then a look at those that are not whole.
@@ -286,8 +319,7 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
   return carry;
 }
 
-// The intervals of stream s as far as its markers' heights tell: ends less those that come below every height before them. Of lost
-// ends and doubled begins this is the exact count. One block.
+// The intervals of stream s as far as its markers' heights tell: ends less those that come below every height before them. One block.
 __device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, u32 s, int (&shi)[33], u32* shu) {
   static_assert(kRecountStep == kScanThreads * 32, "32 markers in a row a thread");
   const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = stream_length(a, off0, s);
@@ -331,11 +363,33 @@ __device__ __forceinline__ u32 recount_stream(const ArgusPairArgs& a, u64 off0, 
   return count;
 }
 
-// `samples` (nullable): what the windows that k_pair_init has looked at tell. One block orders; where the trace is malformed (more than
-// one window tells it: a single defect that a window happens to meet is no reason to read everything; 1.2 G markers with one corrupted end
-// at the front 24.5 ms counted, 21.6 not), and
-// its first malformed stream lies far enough ahead of the last one that writing the intervals behind it twice would cost more than
-// reading all markers once (a third of a pairing pass), the whole grid counts before the last block orders.
+// Whether counting all markers pays: what it costs against a second pass over the streams behind `first_bad`, the first one that
+// is known to be malformed. Both go at the chip's rate (68.6 M events of 1,776 streams: 205 us of counting, 940 of a second pass) or
+// at a block's over the longest stream (96 streams of 405,000: 137 us, 2,150). Lost ends in the last half, fifth and tenth of the
+// streams of the former: 1,428 -> 956 us, 1,343 -> 961 and, not counted, 1,201 -> 1,209; in all of the latter 4,648 -> 2,478. One block.
+__device__ __forceinline__ bool recount_pays(const ArgusPairArgs& a, u32 first_bad, u32* longest /* [2] */) {
+  const u64 off0 = a.stream_offsets[0];
+  u32 all = 0, behind = 0;
+  for (u32 s = threadIdx.x; s < a.num_streams; s += kScanThreads) {
+    const u32 n = stream_length(a, off0, s);
+    all = n > all ? n : all;
+    if (s > first_bad) behind = n > behind ? n : behind;
+  }
+  if (threadIdx.x < 2) longest[threadIdx.x] = 0;
+  __syncthreads();
+  atomicMax(&longest[0], all);
+  atomicMax(&longest[1], behind);
+  __syncthreads();
+  const u64 end = a.stream_offsets[a.num_streams], total = end - off0, left = end - a.stream_offsets[first_bad + 1];
+  const u64 count = total * 3 > longest[0] * 340ull ? total * 3 : longest[0] * 340ull;      // ps, by 3 an event or 340 of the longest
+  const u64 again = left * 14 > longest[1] * 4050ull ? left * 14 : longest[1] * 4050ull;  // by 14, or 4,050
+  return count < again;
+}
+
+// `samples` (nullable): what the windows that k_pair_init has looked at tell. One block orders; where the trace is malformed in a way
+// that counting its markers tells how many intervals it has (windows of one kind, and more than one: a single defect that a window
+// happens to meet is no reason to read everything; 1.2 G markers with one corrupted end at the front 24.5 ms counted, 21.6 not), and
+// counting costs less than the second pass, the whole grid counts before the last block orders.
 template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
                                                             int clear_status, int alone, int ask_split, const u32* samples) {
@@ -343,7 +397,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
   __shared__ u32 cnt[64], cur[64];
   __shared__ u64 sh[33];
   __shared__ u32 one_class, longest_of, first_bad;
-  u32 told = 0;
+  u32 told = kNoDefect;
   if (samples) {
     static_assert(kSamples == kScanThreads, "a window a thread");
     told = samples[threadIdx.x];
@@ -351,34 +405,37 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
       asm volatile("prefetch.global.L1 [%0];" ::"l"(a.stream_offsets + threadIdx.x * RUN));
       asm volatile("prefetch.global.L2 [%0];" ::"l"(a.bases + threadIdx.x * RUN));
     }
-    if (__syncthreads_count(told != 0) > 1) {
+    bool counted = __syncthreads_count(told != kNoDefect) > 1;
+    if (counted) {
+      const int raised = __syncthreads_count(told == kRaised), lowered = __syncthreads_count(told == kLowered);
+      if (threadIdx.x == 0) first_bad = 0xffffffffu;
+      counted = __syncthreads_or(told == kChanged) == 0 && (raised == 0 || lowered == 0) && raised + lowered > 1;
+      if (counted) {
+        if (told) atomicMin(&first_bad, sample_stream(a, threadIdx.x));
+        __syncthreads();
+        counted = recount_pays(a, first_bad, cur);
+      }
+    }
+    if (counted) {
       __shared__ int shi[33];
       __shared__ u32 next;
-      if (threadIdx.x == 0) first_bad = 0xffffffffu;
-      __syncthreads();
-      if (told) atomicMin(&first_bad, told - 1);
-      __syncthreads();
-      if ((u64)(a.num_streams - first_bad) * 3 > a.num_streams) {
-        const u64 off = a.stream_offsets[0];
-        for (;;) {
-          if (threadIdx.x == 0) next = atomicAdd(&a.ctl->recount_head, 1u);
-          __syncthreads();
-          const u32 s = next;
-          __syncthreads();
-          if (s >= a.num_streams) break;
-          const u32 count = recount_stream(a, off, s, shi, cnt);
-          if (threadIdx.x == 0) a.bases[s] = count;
-        }
-        if (threadIdx.x == 0) {
-          __threadfence();
-          next = atomicAdd(&a.ctl->recount_done, 1u);
-        }
+      const u64 off = a.stream_offsets[0];
+      for (;;) {
+        if (threadIdx.x == 0) next = atomicAdd(&a.ctl->recount_head, 1u);
         __syncthreads();
-        if (next != gridDim.x - 1) return;
-        __threadfence();
-      } else if (blockIdx.x) {
-        return;
+        const u32 s = next;
+        __syncthreads();
+        if (s >= a.num_streams) break;
+        const u32 count = recount_stream(a, off, s, shi, cnt);
+        if (threadIdx.x == 0) a.bases[s] = count;
       }
+      if (threadIdx.x == 0) {
+        __threadfence();
+        next = atomicAdd(&a.ctl->recount_done, 1u);
+      }
+      __syncthreads();
+      if (next != gridDim.x - 1) return;
+      __threadfence();
     } else if (blockIdx.x) {
       return;
     }
@@ -396,7 +453,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
   }
   __syncthreads();
   // a malformed stream that the split pass would give up together with all others
-  const bool in_vain = ask_split && __syncthreads_or(told && !argus_split_pays(longest_of - stream_length(a, off0, told - 1), a.num_events, a.num_streams));
+  const bool in_vain = ask_split && __syncthreads_or(told && !argus_split_pays(longest_of - stream_length(a, off0, sample_stream(a, threadIdx.x)), a.num_events, a.num_streams));
   if (threadIdx.x == 0) {  // first places, classes in descending order
     a.bases[a.num_streams] = carry;
     if (ask_split) { a.ctl->split = !in_vain && argus_split_pays(longest_of, a.num_events, a.num_streams); a.ctl->longest = longest_of; }
@@ -629,6 +686,14 @@ bool argus_pair_tiled_usable(const ArgusPairArgs& a);
 
 extern "C" void argus_testing_set_poll_limit(unsigned int polls) { g_poll_limit.store(polls ? polls : 1u << 19); }
 
+extern "C" int argus_testing_pair_passes(const void* workspace, uint32_t* counted, uint32_t* second_pass) {
+  ArgusPairCtl ctl;  // (the first thing in the workspace)
+  ARGUS_CUDA_TRY(cudaMemcpy(&ctl, workspace, sizeof(ctl), cudaMemcpyDeviceToHost));
+  *counted = ctl.recount_done != 0;
+  *second_pass = ctl.redo != 0;
+  return ARGUS_OK;
+}
+
 extern "C" size_t argus_pair_workspace_bytes(uint64_t num_events, uint32_t num_streams, uint64_t ambig_capacity) {
   return make_layout(num_events, num_streams, ambig_capacity).total;
 }
@@ -681,7 +746,7 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   u32* const order = (u32*)(ws + L.order);
   // Small calls: one block clears and orders. Beyond that a grid clears, and looks at the ends of the streams.
   const bool alone = num_events < (1u << 20) && num_streams <= 8192;
-  // Windows all over the trace are looked at where a second pass would cost much more than the look (50 us against 2).
+  // Windows all over the trace are looked at where that is little against the whole call (see kSampledEvents).
   u32* const samples = num_events >= kSampledEvents && num_streams ? (u32*)(ws + L.word_prefix) : nullptr;  // (not used before the offsets kernel)
   if (!alone) {
     // a stream a warp, up to what the chip holds of them

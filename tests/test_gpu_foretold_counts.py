@@ -1,5 +1,7 @@
 """Interval counts foretold from the ends of the streams (calls of 2^20 events and more): streams cut short at the back, at the
 front, at both, and malformed ones for which the foretold count is wrong, against the oracle."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -174,3 +176,59 @@ def test_wrapped_ring_with_defects():
     assert p.intervals_numpy().tobytes() == iv.tobytes()
     assert p.ambig_numpy().tobytes() == am.tobytes()
     assert np.array_equal(p.ambig_offsets.cpu().numpy().view(np.uint64), aoffs)
+
+
+def _passes(p):
+    lib, counted, second = argus.load_library(), ctypes.c_uint32(), ctypes.c_uint32()
+    assert lib.argus_testing_pair_passes(ctypes.c_void_p(p.workspace.data_ptr()), ctypes.byref(counted), ctypes.byref(second)) == 0
+    return bool(counted.value), bool(second.value)
+
+
+def _spoil(e, defect, rng, num_regions):
+    is_end = (e["tag"] & 1) == 1
+    hit = rng.random(len(e)) < 0.002
+    hit[0] = hit[-1] = False
+    if defect == "lost ends":
+        return e[~(hit & is_end)]
+    if defect == "lost begins":
+        return e[~(hit & ~is_end)]
+    if defect == "lost both":
+        return e[~hit]
+    if defect == "doubled begins":
+        return np.repeat(e, 1 + (hit & ~is_end))
+    if defect == "doubled ends":
+        return np.repeat(e, 1 + (hit & is_end))
+    e = e.copy()
+    hit &= is_end == (defect == "changed ends")
+    e["tag"][hit] = (((e["tag"][hit] >> 1) + rng.integers(1, num_regions, hit.sum()).astype(np.uint32)) % num_regions << 1) | (e["tag"][hit] & 1)
+    return e
+
+
+@pytest.mark.parametrize("defect,where,counted,second", [
+    (None, 0.0, False, False), ("lost ends", 0.0, True, False), ("doubled begins", 0.0, True, False), ("lost begins", 0.0, True, False),
+    ("doubled ends", 0.0, True, False), ("changed ends", 0.0, False, True), ("changed begins", 0.0, False, True), ("lost both", 0.0, False, True),
+    ("lost ends", 329.0, False, False), ("one stream", 0.0, False, False)])
+def test_what_is_counted_and_what_is_done_again(defect, where, counted, second):
+    """Markers are counted where that tells the number of intervals, and then nothing is written twice; not where it cannot (markers that
+    have changed, lost begins among lost ends), and not where no stream lies behind the first malformed one. 330 streams."""
+    rng = np.random.default_rng(11)
+    spec = tg.config(1).scaled(4, 700)
+    ev, offs = tg.generate_host(spec)
+    source = [ev[offs[s]:offs[s + 1]] for s in range(spec.num_streams)]
+    parts = [source[s % len(source)] for s in range(330)]
+    if defect == "one stream":
+        parts = [np.concatenate([_spoil(e, "doubled ends", rng, spec.num_regions) for e in parts])]
+    elif defect:
+        parts = [_spoil(e, defect, rng, spec.num_regions) if s >= where else e for s, e in enumerate(parts)]
+    ev = np.concatenate(parts)
+    offs = np.cumsum([0] + [len(e) for e in parts]).astype(np.uint64)
+    assert len(ev) >= 1 << 22
+    _, iv, ioffs, am, aoffs, o_st = oracle.pair(ev, offs, spec.num_regions)
+    assert int(o_st["code"]) == 0
+    p = argus.argus_pair_intervals(torch.from_numpy(ev.view(np.uint8).reshape(-1).copy()).to(DEV), torch.from_numpy(offs.view(np.int64).copy()).to(DEV),
+                                   spec.num_regions, ambig_capacity=len(am) + 16)
+    assert int(p.fetch_status()["code"]) == 0
+    assert _passes(p) == (counted, second)
+    assert np.array_equal(p.interval_offsets.cpu().numpy().view(np.uint64), ioffs)
+    assert p.intervals_numpy().tobytes() == iv.tobytes()
+    assert p.ambig_numpy().tobytes() == am.tobytes()

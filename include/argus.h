@@ -262,7 +262,8 @@ int argus_aggregate(const argus_interval_t* intervals /*device*/,
  * max_intervals is an upper bound of interval_offsets[S] known on the host (for instance
  * the capacity given to argus_pair_intervals); it sizes the workspace, and a stream whose
  * offsets reach beyond it is not read (status->code = ARGUS_ERR_BAD_OFFSETS). If more spans
- * are selected than the workspace holds, status->code = ARGUS_ERR_CAPACITY.
+ * are selected than the workspace holds, status->code = ARGUS_ERR_CAPACITY, and what `out` holds
+ * is unspecified and may differ from call to call.
  * ------------------------------------------------------------------------------------- */
 size_t argus_overlap_workspace_bytes(uint64_t max_intervals, uint32_t num_streams,
                                      uint32_t num_pairs, uint32_t num_sms);

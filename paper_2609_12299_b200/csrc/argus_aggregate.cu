@@ -19,7 +19,7 @@ namespace {
 
 constexpr int kAggThreads = 256;
 constexpr u32 kCell = 72;  // u64 words per argus_agg_t
-constexpr u32 kAggCompactRegions = 400;  // 112 B each: 44.8 KB of shared memory at most
+constexpr u32 kAggCompactRegions = 400;  // 112 B each: 44.8 KB of shared memory at most (k_agg_iter_windows: 136 KB)
 constexpr u32 kIterThreads = 512, kIterWarps = kIterThreads / 32;  // k_agg_iter_windows
 constexpr u32 kMaxParts = 16;            // blocks that share a stream in k_agg_streams_compact
 
@@ -558,7 +558,9 @@ __device__ __forceinline__ void iter_flush(u32* cells, const u32* hot_region, u6
 // found to be in the window is read, a round ahead. What decides is how many lanes add to one address: with copies of the most
 // frequent regions' cells, and a thread a cell where they are added to the table, the call with all tables goes from 1,616 to 1,508 us
 // for 38 M intervals in 16 iterations of 202 regions, from 2,709 to 2,219 for 115 M in 48, and from 10.1 to 4.4 ms for 34 M in 2,000
-// iterations of five regions. In the same pass as the rows (cells of one stream and iteration) the first took 2,107.
+// iterations of five regions. In the same pass as the rows (cells of one stream and iteration) the first took 2,107. More regions leave
+// room for fewer blocks on an SM (136 KB at 400, where two tables of 112-byte cells took 90), which does not turn the gain: 112 M
+// intervals of 292 regions, 16 of 32 iterations, 1,964 -> 1,743 us, 115 M of 400 regions, 16 of 24, 2,487 -> 2,390.
 __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u32 streams_per_block) {
   argus_kernel_begin_long();
   extern __shared__ __align__(16) unsigned char sh_raw[];

@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(NT, 1) k_ov_pair(OvPairArgs a) {
   u64 a0 = 0;  // producer pieces taken so far
   for (u64 t0 = 0; nP && nC && t0 < total; t0 += kTile) {
     const u32 cnt = (u32)(total - t0 < kTile ? total - t0 : kTile), step = (u32)((t0 / kTile) % kPairWarps);
-    if (step == 0) {  // where the next 32 tiles end, one warp each
+    if (step == 0) {  // where the next tiles end, one warp each
       const u64 to = t0 + (u64)(warp + 1) * kTile;
       const u64 s1 = to >= total ? nP : merge_split_warp(A, nP, B, nC, to, lane);
       if (lane == 0) red[0][warp] = s1;

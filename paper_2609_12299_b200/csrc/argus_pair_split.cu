@@ -4,10 +4,11 @@
 // chip has room for blocks (a trace of some of the SMs) the chained pass leaves most of it idle. Here
 //   k_split_scan  : one block per segment reads the markers' kinds only and finds, by heights, how many ends close a frame from
 //                   before the segment and which begins stay open at its end;
-//   k_split_chain : one warp per stream walks its segments and gives every one the stack where it starts;
+//   k_split_chain : one block per stream; its first warp walks the segments, whose summaries the block brings into shared memory,
+//                   and gives every one the stack where it starts;
 //   (the SPLIT instantiation of the tiled kernel walks the segments: argus_pair_tiled.cu)
-//   k_split_fix   : one block per stream completes the child time of the frames that were open across a segment's start, counts
-//                   the stream's intervals and notes the frames open at its end.
+//   k_split_fix   : several blocks per stream complete the child time of the frames that were open across a segment's start; the
+//                   first of them counts the stream's intervals and notes the frames open at its end.
 // Heights know nothing of region ids. A segment that meets a marker which breaks the parallel rules gives its stream up; the
 // chained pass, which follows and does nothing otherwise, walks such streams from their beginning. A stream about as long as the
 // longest takes all others with it, and the blocks stop within eight tiles (384 streams of 129,664 events with a lost or doubled

@@ -43,3 +43,33 @@ def test_iteration_table(order, S, W, R, window):
     assert int(argus.argus_status_fetch(got.status)["code"]) == 0
     for lv in levels:
         assert got.table_numpy(lv).tobytes() == want[lv].tobytes(), lv
+
+
+@pytest.mark.parametrize("shares", ["uniform", "skewed"])
+@pytest.mark.parametrize("S,W,R,window", [(96, 4, 200, 16), (640, 16, 292, 9), (320, 16, 400, 16), (2400, 16, 400, 3)])
+def test_many_regions(shares, S, W, R, window):
+    """Up to the most regions that the tables in shared memory have room for, with regions that have copies of their cells among many
+    that have none: a few hold most intervals, in some streams other ones than in the rest."""
+    rng = np.random.default_rng(S + R)
+    per = 400_000 // S + 65
+    iv = np.zeros(S * per, argus.INTERVAL_DTYPE)
+    iv["ctx"] = np.tile(np.sort(rng.integers(0, window + 6, per)), S)
+    iv["stream"] = np.repeat(np.arange(S), per)
+    iv["region"] = rng.integers(0, R, len(iv))
+    if shares == "skewed":
+        hot = rng.random(len(iv)) < 0.8
+        iv["region"][hot] = (R - 1 - rng.choice(5, hot.sum(), p=[0.5, 0.2, 0.15, 0.1, 0.05]) - iv["stream"][hot] % 2 * 7).astype(np.uint32)
+    iv["t_begin"] = rng.integers(0, 1 << 40, len(iv)).astype(np.uint64)
+    iv["inclusive"] = (2.0 ** rng.uniform(0, 33, len(iv))).astype(np.uint64)  # (some of 2^32 ticks and more)
+    iv["exclusive"] = iv["inclusive"] // np.uint64(2)
+    iv["flags"] = rng.random(len(iv)) < 0.02
+    offs = (np.arange(S + 1) * per).astype(np.uint64)
+    cta_sm = (np.arange(S // W) % 5).astype(np.uint32)
+    levels = ("warp", "kernel", "role", "iter")
+    scope = (4, 4 + window - 1)
+    _, want, _ = oracle.aggregate_scoped(iv, offs, None, None, W, cta_sm, 5, R, scope={"ctx": scope}, levels=levels)
+    got = argus.argus_aggregate_scoped(torch.from_numpy(iv.view(np.uint8).reshape(-1).copy()).to(DEV), torch.from_numpy(offs.view(np.int64).copy()).to(DEV), None,
+                                       None, W, torch.from_numpy(cta_sm.view(np.int32)).to(DEV), 5, R, argus.ArgusScope(*scope), levels=levels)
+    assert int(argus.argus_status_fetch(got.status)["code"]) == 0
+    for lv in levels:
+        assert got.table_numpy(lv).tobytes() == want[lv].tobytes(), lv

@@ -1,6 +1,6 @@
 """argus_overlap's kernel at the sizes where its branches change: spans in order or not, one role or both, around the number of
-spans it holds in shared memory and the number of intervals an SM at which threads ask for more at a time, starts that crowd, and
-a workspace too small for the plain layout of the entries."""
+spans it holds in shared memory and the number of intervals an SM at which blocks have more threads, starts that crowd, many CTAs
+an SM, and a workspace too small for the plain layout of the entries."""
 import numpy as np
 import pytest
 import torch

@@ -149,15 +149,17 @@ __global__ void __launch_bounds__(kSelThreads) k_ov_select(OvSelectArgs a) {
 // ---------------------------------------------------------------------------------------------------------------------
 constexpr u32 kVT = 9;                                 // spans a thread merges at a time (odd: lanes that far apart hit different banks)
 __host__ __device__ constexpr u32 bucket_word(u32 b) { return b + (b >> 5); }  // padded: threads sum up runs of counters without bank conflicts
+constexpr u32 kSorted = 9216;                          // spans of both roles that are sorted at once, whatever the block's size: 144 KB
+constexpr u32 kBucketBits = 13;                        // 2^kBucketBits buckets of a role at most
+constexpr size_t kPairSmem = (size_t)kSorted * sizeof(ulonglong2);
+static_assert(kSorted <= 1u << 14, "places fit 14 bits");
+static_assert((2u << kBucketBits) >= kSorted && (size_t)kSorted * 8 + bucket_word(2u << kBucketBits) * 4 <= kPairSmem, "a bucket a span, in the tile's room");
 template <u32 NT>
 struct PairSizes {                                     // of a block of NT threads
   static constexpr u32 kWarps = NT / 32;
-  static constexpr u32 kTile = NT * kVT;               // spans in shared memory at a time (1,024 threads: 144 KB)
+  static constexpr u32 kTile = NT * kVT;               // spans that are merged at a time
   static constexpr u32 kBatch = NT;                    // slices whose spans are placed at a time
-  static constexpr u32 kBucketBits = NT == 1024 ? 13 : NT == 512 ? 12 : 11;  // 2^kBucketBits buckets of a role at most
-  static constexpr size_t kSmem = (size_t)kTile * sizeof(ulonglong2);
-  static_assert(kTile <= 1u << 14, "places fit 14 bits");
-  static_assert((2u << kBucketBits) >= kTile && (size_t)kTile * 8 + bucket_word(2u << kBucketBits) * 4 <= kSmem, "a bucket a span, in the tile's room");
+  static_assert(kTile <= kSorted, "a tile fits shared memory");
 };
 
 struct OvPairArgs {
@@ -297,7 +299,7 @@ __device__ __noinline__ ulonglong2* sort_spans(ulonglong2* d, ulonglong2* scratc
   return d;
 }
 
-// Sort of both roles together, up to kTile spans (in0[0..n0), in1[0..n1); a role that is in order already comes with n = 0),
+// Sort of both roles together, up to kSorted spans (in0[0..n0), in1[0..n1); a role that is in order already comes with n = 0),
 // into out0 and out1: spans are spread over buckets of equal width in start time, about one for a span, and a span's place is
 // the number of earlier ones in its bucket. Elements are 8 bytes, start time relative to the role's earliest (50 bits) and place (14
 // bits); the spans follow once (4,096 spans a role: 20 us; merging runs pairwise took 50 us). Returns false, the same for
@@ -307,12 +309,12 @@ constexpr u32 kBucketMost = 32;
 template <u32 NT>
 __device__ __noinline__ bool sort_buckets(const ulonglong2* in0, const ulonglong2* in1, u32 n0, u32 n1, ulonglong2* out0, ulonglong2* out1,
                                           ulonglong2* room, u64 (*red)[NT / 32 + 1], u32 (&scan)[33]) {
-  constexpr u32 kTile = PairSizes<NT>::kTile, kWarps = NT / 32;
+  constexpr u32 kWarps = NT / 32;
   u64* const t = reinterpret_cast<u64*>(room);
-  u32* const cnt = reinterpret_cast<u32*>(t + kTile);  // a role's counters after the other's; then where a bucket ends
+  u32* const cnt = reinterpret_cast<u32*>(t + kSorted);  // a role's counters after the other's; then where a bucket ends
   const u32 n = n0 + n1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u32 bits = 5;  // 2^bits buckets a role
-  while (bits < PairSizes<NT>::kBucketBits && (2u << bits) < n) ++bits;
+  while (bits < kBucketBits && (2u << bits) < n) ++bits;
   const u32 nb = 2u << bits;
   for (u32 b = threadIdx.x; b < nb; b += NT) cnt[bucket_word(b)] = 0;
   u64 low0 = ~0ull, low1 = ~0ull, high0 = 0, high1 = 0;
@@ -423,13 +425,11 @@ __device__ __noinline__ u64 cut_pieces(ulonglong2* d, u64 n, u64* red) {
 // Latency decides (one block per SM and pair). The entries of up to kBatch slices are taken as one flat sequence, so that
 // every thread has kGather entries and then as many begin times (or pieces of records) in flight, whatever the slices hold.
 // 148 SMs, two roles of 16,000 spans each: 109 us (five kernels before it: 393 us), about 6.5 a group of 4,096 entries and 10 a tile of
-// the walk; 2,048 spans a role from 16 interleaved streams: 33 us (178 us; 38 with 1,024 threads); a few hundred spans: 25 with 1,024
-// threads, 21 with 512, most of it fixed steps one after the other.
+// the walk; a few hundred spans: 25 with 1,024 threads, 21 with 512, most of it fixed steps one after the other.
 // DIGEST: entries as the pass over the digests leaves them (argus_fuse.cuh); else {index in the stream, region}.
-template <bool DIGEST, u32 NT>
+template <bool DIGEST, u32 NT, u32 kGather>
 __global__ void __launch_bounds__(NT, 1) k_ov_pair(OvPairArgs a) {
   using Z = PairSizes<NT>;
-  constexpr u32 kGather = 4;  // entries that a thread asks for at a time
   constexpr u32 kPairThreads = NT, kPairWarps = Z::kWarps, kTile = Z::kTile, kBatch = Z::kBatch;
   argus_kernel_begin_long();
   extern __shared__ __align__(16) unsigned char pair_raw[];
@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(NT, 1) k_ov_pair(OvPairArgs a) {
     const bool cut_a = __syncthreads_or(suspect[0]), cut_b = __syncthreads_or(suspect[1]);
     ulonglong2 *const free_a = a.scratch + base + nC, *const free_b = a.spans + base + nP;  // as much room again for either role
     if (cut_a || cut_b) {
-      if ((cut_a ? nP : 0ull) + (cut_b ? nC : 0ull) <= kTile &&
+      if ((cut_a ? nP : 0ull) + (cut_b ? nC : 0ull) <= kSorted &&
           sort_buckets<NT>(A, B, cut_a ? (u32)nP : 0u, cut_b ? (u32)nC : 0u, free_a, free_b, tile, red, sh_scan)) {
         if (cut_a) A = free_a;
         if (cut_b) B = free_b;
@@ -745,32 +745,36 @@ size_t ov_fixed_bytes(u32 num_streams) {
   return argus_align_up(sizeof(ArgusOvCtl), 256) + argus_align_up((size_t)num_streams * select_slices(num_streams) * sizeof(ArgusOvPiece), 256) + 1024;
 }
 
-template <bool DIGEST, u32 NT>
+template <bool DIGEST, u32 NT, u32 kGather>
 int launch_pair_as(const OvPairArgs& a, cudaStream_t stream) {
   static std::atomic<bool> opted_in[64];  // the shared-memory opt-in belongs to a device
   int dev = 0;
   ARGUS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return ARGUS_ERR_INVALID_ARG;
   if (!opted_in[dev].load(std::memory_order_acquire)) {
-    ARGUS_CUDA_TRY(argus_allow_smem(k_ov_pair<DIGEST, NT>, PairSizes<NT>::kSmem));
+    ARGUS_CUDA_TRY(argus_allow_smem(k_ov_pair<DIGEST, NT, kGather>, kPairSmem));
     opted_in[dev].store(true, std::memory_order_release);
   }
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);
-  ARGUS_LAUNCH((k_ov_pair<DIGEST, NT>), a.blocks, NT, PairSizes<NT>::kSmem, stream, a);
+  ARGUS_LAUNCH((k_ov_pair<DIGEST, NT, kGather>), a.blocks, NT, kPairSmem, stream, a);
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 1);
   return ARGUS_OK;
 }
 
-// Threads of a block by how many intervals an SM has on average (how many are spans of a pair is not known here): a block that has
-// little to do waits at its barriers for the warps it has. us with 1,024 / 512 / 256 threads; intervals an SM: 1,200 18.5 / 15.3 /
-// 13.5, 2,500 (all to be sorted) 31.7 / 25.4 / 25.7, 4,700 20.5 / 16.4 / 14.4, 23,000 26.6 / 21.7 / 26.7, 65,000 30.7 / 24.6 / 23.6, 70,000
-// 45.1 / 42.0 / 57.3, 90,000 (records) 77.8 / 72.6 / 93.2, 232,000 112.8 / 127.0 / 195.6, 519,000 (of which 4,000 are spans) 37.7 / 32.5 /
-// 35.9, 4.2 million 82.0 / 115.7 / 177.2. Two entries a thread instead of four: 512 threads 24.7 for the second, 23.5 for the fourth.
+// Threads of a block, and entries that a thread asks for at a time, by how many intervals an SM has on average: a block that has little
+// to do waits at its barriers for the warps it has, one that has much to sort and walk needs them. How many intervals are spans
+// of a pair, and whether they come in order, is not known here. us with 1,024 threads and two entries / 512 and four, intervals an SM:
+// spans in order (one pair; 148 SMs): 2,300 18.5 / 16.2, 4,600 18.5 / 16.6, 11,600 21.0 / 18.5, 23,600 22.7 / 20.5, 34,800 35.6 / 35.7, 94,000
+// 43.2 / 43.1; to be sorted (three pairs): 800 27.0 / 22.1, 2,500 30.8 / 24.7, 5,600 36.9 / 33.0, 16,000 57.4 / 57.3; (one pair, 16 CTAs
+// an SM, whole call) 18,600 38.6 / 37.0, 37,000 55.9 / 58.6, 56,000 66.9 / 76.0, 111,000 177 / 195. From 2^17 on four entries with
+// 1,024 threads: 232,000 113.5 / 108.8 (two / four). 256 threads were 1 us less than 512 for spans in order below 6,000 intervals
+// an SM, but 40.3 where 5,600 had to be sorted, and twice the time where a call's CTAs lie on a few of the SMs that it names (37,000 on
+// each of six of 148: 55.9, 58.6 with 512, 114.7 with 256).
 template <bool DIGEST>
 int launch_pair(const OvPairArgs& a, uint64_t num_intervals, cudaStream_t stream) {
   const u32 ctas = a.num_streams / a.warps_per_cta;  // each is on one SM
   const u64 sms = ctas < a.num_sms ? (ctas ? ctas : 1u) : a.num_sms, each = num_intervals / sms;
-  return each < 8192 ? launch_pair_as<DIGEST, 256>(a, stream) : each < 1u << 17 ? launch_pair_as<DIGEST, 512>(a, stream) : launch_pair_as<DIGEST, 1024>(a, stream);
+  return each < 1u << 15 ? launch_pair_as<DIGEST, 512, 4>(a, stream) : each < 1u << 17 ? launch_pair_as<DIGEST, 1024, 2>(a, stream) : launch_pair_as<DIGEST, 1024, 4>(a, stream);
 }
 
 }  // namespace

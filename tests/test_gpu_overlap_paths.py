@@ -60,10 +60,11 @@ def test_overlap_sizes_and_orders(order, per_stream):
 
 @pytest.mark.parametrize("order", ["disjoint", "overlapping", "shuffled", "crowded"])
 @pytest.mark.parametrize("per_stream,S,W,M", [(1727, 4, 2, 2), (1729, 4, 2, 2), (3455, 4, 2, 2), (3457, 4, 2, 2), (4095, 4, 2, 2), (4096, 4, 2, 2), (100, 16, 16, 1), (700, 32, 16, 1),
+                                              (6900, 4, 2, 2), (6912, 4, 2, 2), (6925, 4, 2, 2),
                                               (9, 48, 16, 7)])
 def test_block_sizes(order, per_stream, S, W, M):
-    """Around the spans that blocks of 256 and 512 threads hold, the number of intervals at which a larger one is taken, and with more
-    slices of streams than a block takes at a time."""
+    """Around the spans that a block of 512 threads merges and sorts at a time, and with more slices of streams than a block takes at a
+    time."""
     rng = np.random.default_rng(per_stream)
     iv = _intervals(rng, per_stream, S, order, 3)
     offs = (np.arange(S + 1) * per_stream).astype(np.uint64)
@@ -79,7 +80,7 @@ def test_block_sizes(order, per_stream, S, W, M):
 @pytest.mark.parametrize("order", ["disjoint", "overlapping", "crowded"])
 @pytest.mark.parametrize("S,W,M,per_stream", [(2080, 4, 4, 12), (640, 2, 2, 24), (96, 16, 1, 64)])
 def test_many_ctas_an_sm_and_three_pairs(order, S, W, M, per_stream):
-    """Few intervals an SM (blocks of 256 threads) that lie in more CTAs than a block has threads, and in several batches of
+    """Few intervals an SM that lie in more CTAs than a block looks at at a time, and in several batches of
     slices for each of them: what a block keeps of its CTAs outlives the scans in between. Plain call and one-call pipeline."""
     rng = np.random.default_rng(S)
     iv = _intervals(rng, per_stream, S, order, 3)

@@ -196,19 +196,23 @@ __device__ __noinline__ u32 sample_kind(u32 bad, u32 ends, u32 tag, u32 begin, i
   }
   return kind;
 }
-// What window `w` tells. One warp.
-__device__ __forceinline__ u32 sample_window(const ArgusPairArgs& a, u64 off0, u32 w) {
-  const u32 lane = threadIdx.x & 31, lower = (1u << lane) - 1u, s = sample_stream(a, w), n = stream_length(a, off0, s);
-  if (n < 32 * kSampleRows) return kNoDefect;
+// The tags of window `w`; false where its stream is too short. One warp.
+__device__ __forceinline__ bool sample_load(const ArgusPairArgs& a, u64 off0, u32 w, u32 (&tags)[kSampleRows]) {
+  const u32 lane = threadIdx.x & 31, s = sample_stream(a, w), n = stream_length(a, off0, s);
+  if (n < 32 * kSampleRows) return false;
   const u32 head = a.ring_written ? argus_ring_first(a, s) : 0u, at0 = __umulhi(w * 0x9E3779B1u, n - 32 * kSampleRows + 1);
   const uint4* const src = reinterpret_cast<const uint4*>(a.events) + (a.ring_written ? (u64)s * a.ring_capacity : a.stream_offsets[s]);
-  u32 tags[kSampleRows];
 #pragma unroll
   for (u32 r = 0; r < kSampleRows; ++r) {
     u32 at = at0 + 32 * r + lane;
     if (a.ring_written) { const u32 room = a.ring_capacity - head; at = at >= room ? at - room : head + at; }
     tags[r] = __ldg(reinterpret_cast<const u32*>(src + at) + 2);
   }
+  return true;
+}
+// What they tell. One warp.
+__device__ __forceinline__ u32 sample_tell(const u32 (&tags)[kSampleRows]) {
+  const u32 lane = threadIdx.x & 31, lower = (1u << lane) - 1u;
   u32 kind = kNoDefect;
 #pragma unroll
   for (u32 r = 0; r < kSampleRows; ++r) {
@@ -233,12 +237,9 @@ __global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uin
   pair_clear(a, zeroed, zeroed_words, clear_status, (u64)blockIdx.x * blockDim.x + threadIdx.x, (u64)gridDim.x * blockDim.x);
   const u32 lane = threadIdx.x & 31;
   const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0, warps = (u64)gridDim.x * (kInitThreads / 32);
-  if (samples && a.num_streams) {
-    for (u32 w = blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5); w < kSamples; w += (u32)warps) {
-      const u32 told = sample_window(a, off0, w);
-      if (lane == 0) samples[w] = told;
-    }
-  }
+  // the tags of the warp's first window are on their way while it takes its streams (there are mostly no more windows than warps)
+  u32 window = samples && a.num_streams ? blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5) : kSamples, tags[kSampleRows];
+  bool looked = window < kSamples && sample_load(a, off0, window, tags);
   int many = -1;  // whether more than a quarter of the streams have unclear ends (a sample of 32 tells, when it is asked for)
   for (u64 s0 = ((u64)blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5)) * per; s0 < a.num_streams; s0 += warps * per) {
     u32 n = 0, f = 0, l = 1;
@@ -275,6 +276,12 @@ __global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uin
       }
       if (lane == 0) a.bases[s] = (nk - (unmatched < nk ? unmatched : nk)) >> 1;
     }
+  }
+  while (window < kSamples) {
+    const u32 told = looked ? sample_tell(tags) : kNoDefect;
+    if (lane == 0) samples[window] = told;
+    window += (u32)warps;
+    looked = window < kSamples && sample_load(a, off0, window, tags);
   }
 }
 
@@ -751,7 +758,8 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   if (!alone) {
     // a stream a warp, up to what the chip holds of them
     const u32 per = num_streams <= 148u * 64u ? 1u : num_streams < 32u * 148u * 64u ? (num_streams + 148u * 64u - 1) / (148u * 64u) : 32u;
-    const u64 want = ((u64)num_streams / per + kInitThreads / 32 - 1) / (kInitThreads / 32) + zeroed_words / 4096 + 1;
+    u64 want = ((u64)num_streams / per + kInitThreads / 32 - 1) / (kInitThreads / 32) + zeroed_words / 4096 + 1;
+    if (samples && want < kSamples * 32 / kInitThreads) want = kSamples * 32 / kInitThreads;  // a window a warp
     ARGUS_LAUNCH(k_pair_init, (unsigned)(want < 1184 ? want : 1184), kInitThreads, 0, stream, a, zeroed, zeroed_words, (int)reset_status, per, samples);
   }
   const bool many = num_streams > kScanThreads;

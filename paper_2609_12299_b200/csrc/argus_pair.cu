@@ -287,10 +287,16 @@ __global__ void __launch_bounds__(kInitThreads) k_pair_init(ArgusPairArgs a, uin
 
 // ---------------------------------------------------------------------------------------------
 // order: provisional bases (exclusive sum of the foretold counts), and the streams sorted by length class
-// (floor(log2(events))), longest first. A stream is a chain of chunks that one CTA at a time walks, so when lengths differ
+// (an eighth of an octave), longest first. A stream is a chain of tiles that one CTA at a time walks, so when lengths differ
 // (producer and consumer warps of one kernel) the long chains must start first or they end last, alone. Counting sort in one
 // block; the order inside a class does not matter. Small calls have no init kernel before this one (`alone`).
 // ---------------------------------------------------------------------------------------------
+constexpr u32 kClasses = 256;
+__device__ __forceinline__ u32 length_class(u32 n) {  // 8 floor(log2(n)) and three more bits of n
+  if (!n) return 0;
+  const u32 e = 31 - (u32)__clz((int)n);
+  return e * 8 + (e >= 3 ? (n >> (e - 3)) & 7u : (n << (3 - e)) & 7u);
+}
 // Returns the sum of the foretold counts; *longest: events of the longest stream of this thread.
 template <u32 RUN>
 __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int alone, u32* cnt, u64 (&sh)[33], u32* longest) {
@@ -300,19 +306,19 @@ __device__ __forceinline__ u64 order_bases(const ArgusPairArgs& a, u64 off0, int
     u64 c[RUN], sum = 0, total;
 #pragma unroll
     for (u32 j = 0; j < RUN; ++j) {
-      u32 cls = 64;
+      u32 cls = kClasses;
       c[j] = 0;
       if (s + j < a.num_streams) {
         const u32 n = stream_length(a, off0, (u32)s + j);
         c[j] = alone ? n >> 1 : __ldcg(a.bases + s + j);
-        cls = n ? 31 - __clz((int)n) : 0;
+        cls = length_class(n);
         *longest = n > *longest ? n : *longest;
         if (RUN == 1) atomicAdd(&cnt[cls], 1u);
       }
       sum += c[j];
       if (RUN > 1) {
         const u32 same = __match_any_sync(0xffffffffu, cls);  // a warp's streams are mostly of one class
-        if (cls < 64 && !(same & ((1u << (threadIdx.x & 31)) - 1u))) atomicAdd(&cnt[cls], (u32)__popc(same));
+        if (cls < kClasses && !(same & ((1u << (threadIdx.x & 31)) - 1u))) atomicAdd(&cnt[cls], (u32)__popc(same));
       }
     }
     u64 at = carry + argus_block_exclusive_scan<u64>(sum, sh, &total);
@@ -398,10 +404,10 @@ __device__ __forceinline__ bool recount_pays(const ArgusPairArgs& a, u32 first_b
 // happens to meet is no reason to read everything; 1.2 G markers with one corrupted end at the front 24.5 ms counted, 21.6 not), and
 // counting costs less than the second pass, the whole grid counts before the last block orders.
 template <u32 RUN>
-__global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
+__global__ void __launch_bounds__(kScanThreads, 1) k_pair_order(ArgusPairArgs a, u32* order, uint4* zeroed, u64 zeroed_words,
                                                             int clear_status, int alone, int ask_split, const u32* samples) {
   argus_kernel_begin_long();  // the pairing kernel's blocks spread evenly only over SMs that are free when they come
-  __shared__ u32 cnt[64], cur[64];
+  __shared__ u32 cnt[kClasses], cur[kClasses];
   __shared__ u64 sh[33];
   __shared__ u32 one_class, longest_of, first_bad;
   u32 told = kNoDefect;
@@ -449,7 +455,8 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
   }
   if (threadIdx.x == 0) longest_of = 0;
   if (alone) pair_clear(a, zeroed, zeroed_words, clear_status, threadIdx.x, blockDim.x);
-  if (threadIdx.x < 64) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
+  if (threadIdx.x < kClasses) { cnt[threadIdx.x] = 0; cur[threadIdx.x] = 0; }
+  if (threadIdx.x == 0) one_class = 0;
   __syncthreads();
   const u64 off0 = a.num_streams ? a.stream_offsets[0] : 0;
   u32 longest = 0;
@@ -461,17 +468,24 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
   __syncthreads();
   // a malformed stream that the split pass would give up together with all others
   const bool in_vain = ask_split && __syncthreads_or(told && !argus_split_pays(longest_of - stream_length(a, off0, sample_stream(a, threadIdx.x)), a.num_events, a.num_streams));
-  if (threadIdx.x == 0) {  // first places, classes in descending order
+  if (threadIdx.x == 0) {
     a.bases[a.num_streams] = carry;
     if (ask_split) { a.ctl->split = !in_vain && argus_split_pays(longest_of, a.num_events, a.num_streams); a.ctl->longest = longest_of; }
-    u32 base = 0;
-    one_class = 0;
-    for (int c = 31; c >= 0; --c) {
-      const u32 k = cnt[c];
-      if (k == a.num_streams) one_class = 1;
-      cnt[c] = base;
-      base += k;
+  }
+  if (threadIdx.x < 32) {  // first places, classes in descending order
+    u32 k[kClasses / 32], sum = 0;
+#pragma unroll
+    for (u32 j = 0; j < kClasses / 32; ++j) {
+      k[j] = cnt[kClasses - 1 - (threadIdx.x * (kClasses / 32) + j)];
+      sum += k[j];
+      if (k[j] == a.num_streams) one_class = 1;
     }
+    u32 place = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const u32 o = __shfl_up_sync(0xffffffffu, place, d); if (threadIdx.x >= (u32)d) place += o; }
+    place -= sum;
+#pragma unroll
+    for (u32 j = 0; j < kClasses / 32; ++j) { cnt[kClasses - 1 - (threadIdx.x * (kClasses / 32) + j)] = place; place += k[j]; }
   }
   __syncthreads();
   if (one_class) {  // streams of one length class start in index order, as without this kernel
@@ -479,7 +493,7 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_order(ArgusPairArgs a, u3
     return;
   }
   for (u32 s = threadIdx.x; s < a.num_streams; s += blockDim.x) {
-    const u32 n = stream_length(a, off0, s), c = n ? 31 - __clz((int)n) : 0;
+    const u32 c = length_class(stream_length(a, off0, s));
     order[cnt[c] + atomicAdd(&cur[c], 1u)] = s;
   }
 }
@@ -669,9 +683,11 @@ Layout make_layout(uint64_t num_events, uint32_t num_streams, uint64_t ambig_cap
   size_t o = 0;
   L.ctl = o; o += argus_align_up(sizeof(ArgusPairCtl), 256);
   L.counts = o; o += argus_align_up(((size_t)num_streams + 1) * 8, 256);
-  // every hand-over follows a chunk of at least kChunkEvents events, and only streams longer than that hand over
+  // every hand-over follows a chunk of at least kChunkEvents events, and only streams longer than that hand over (in small calls, for
+  // which the static entry has little scratch, the longest of them)
   L.queue_capacity = num_events / kChunkEvents + 1;
-  L.record_capacity = (u32)(L.queue_capacity < num_streams ? L.queue_capacity : num_streams);
+  const u64 records = num_events > 1u << 20 ? L.queue_capacity : num_events / 32768 + 1;
+  L.record_capacity = (u32)(records < num_streams ? records : num_streams);
   L.queue = o; o += argus_align_up((size_t)L.queue_capacity * 4, 256);
   L.bits = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);
   L.word_prefix = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);

@@ -22,36 +22,51 @@ struct ArgusFrame {  // one open region occurrence, 32 bytes
   u32 pad;
 };
 
-struct ArgusPairCtl {  // control block in the workspace, zeroed at the start of a call
-  u64 n_notes;         // ambiguity notes appended (may exceed the list capacity)
+// Control block in the workspace, zeroed at the start of a call. A word that many blocks change while others look at it is looked at with
+// an atomic, too, and lies on a line with nothing that is read in any other way: loads of a line that changes all the time held
+// up everything else that half of the SMs asked the L2 for (2,368 streams of 16,208 events, blocks that load `level` every 3,840: 69 SMs walked
+// 340 tiles each, the others 485, in 435 us; with atomics 416 each, in 340).
+struct ArgusPairCtl {
+  // written by one kernel, read by the next
   u32 redo;            // 1 = provisional interval bases were wrong; second pass needed
   u32 redo_from;       // first stream whose intervals the second pass writes again
   u64 total_intervals;
   u64 total_ambig;
+  u32 longest;         // events of the longest stream
+  u32 prefix_done;     // blocks that have counted their share of the ambiguity bitmap
+  u32 recount_head;    // streams taken to have their markers counted
+  u32 recount_done;    // blocks that have found no more of them
+  // atomics only
+  alignas(128) u64 n_notes;  // ambiguity notes appended (may exceed the list capacity)
   // work queue of the tiled kernel, one set per pass (0 = first, 1 = redo): positions below num_streams are the
   // streams themselves, later positions are streams handed on after a chunk (see ArgusStreamRecord)
   u64 q_head[2];       // positions taken
   u64 q_tail[2];       // hand-overs published (queue entries written)
-  u32 n_records[2];    // hand-over records allocated
-  u32 n_done[2];       // streams walked to their end (or given up on)
-  u32 prefix_done;     // blocks that have counted their share of the ambiguity bitmap
+  u64 progress[2];     // low half: streams walked to their end (or given up on); high half: moves as long as streams are walked
+  u32 level[2];        // events left of the stream that was taken last, 0 if nothing else waits
   u32 seg_head;        // segments taken (split pass)
-  u32 longest;         // events of the longest stream
-  u32 recount_head;    // streams taken to have their markers counted
-  u32 recount_done;    // blocks that have found no more of them
-  alignas(16) u32 num_failed;  // streams that the split pass has to leave to the chained one (read together with the next two)
+  // read by all blocks, changed when something is given up
+  alignas(128) u32 num_failed;  // streams that the split pass has to leave to the chained one (read together with the next two)
   u32 num_segments;    // 0 where the segments do not fit their room, too
   u32 split;           // the split pass is worth it (argus_split_pays), and no long stream has been given up
   u32 pad;
 };
 
-// A long stream is walked in chunks of about kChunkEvents events. After a chunk the CTA stores the stream's
-// state here and puts the record into the work queue, so that whichever CTA is free next carries on: all
-// streams advance at the same pace and the kernel has no long tail, whatever the number of streams per SM.
+// A stream is a chain of tiles that one CTA at a time walks, and streams rarely share out evenly among the CTAs that the chip holds.
+// So a CTA looks up now and then how much the stream that was taken last had left (ArgusPairCtl::level). If its own has less than half
+// of that left it hands it on: it stores the stream's state here, puts the record into the work queue and takes the next
+// position; whichever CTA is free when the record's turn comes carries on. Streams are taken longest first and what is handed
+// on is about as long as what is taken for it, so what was taken last tells well enough what waits, and the streams that
+// are left get shorter together. A hand-over costs the CTA about 8 us (it waits for its stores, then for a chain of loads), which
+// is why it is not done for a little. Where nothing waits nothing is handed on. Hand-overs every 32,768 events, whatever waited, made
+// long streams wait behind short ones, and left half of the CTAs idle for the last eighth of the time: GEMM trace (68.7 M events in streams
+// of 72,000 and 32,000) 622 -> 571 us, attention (153.5 M in 112,684, 67,628 and 176) 1,412 -> 1,246, 131 x 12 streams (27,972 and
+// 12,432) 244 -> 203, equal streams (2,368 of 129,664) 2,421 -> 2,442; looked up by three quarters instead of a half 576, 1,256 and 2,468.
 // Queue positions are taken with one atomic add each. A CTA whose position has no entry yet is idle anyway
 // (every unfinished stream is in some CTA's hands): it polls until the entry appears or every stream is
-// done, and gives up with ARGUS_ERR_TIMEOUT if no hand-over at all is published for about a second.
-constexpr u32 kChunkEvents = 32768;
+// done, and gives up with ARGUS_ERR_TIMEOUT if nothing moves for about a second.
+constexpr u32 kChunkEvents = 3840;   // walked by a CTA at least before it hands a stream on
+constexpr u32 kLevelMargin = 1280;   // of which the stream has to have less than half as much left
 struct ArgusStreamRecord {
   u32 stream, next_tile;
   int ch;                             // stack height at the hand-over

@@ -81,31 +81,47 @@ constexpr int kBadRef = 0x3fff;   // reference that marks a window as not well n
 constexpr int kSeqChunk = 128;    // markers handed to the sequential machine at once when cuts come densely
 constexpr u32 kNoRec = 0xffffffffu;
 
+__device__ __forceinline__ void tile_progress(const ArgusPairArgs& a, u64 by) {
+  atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->progress[a.redo ? 1 : 0]), by);
+}
+
 // Takes the next piece of work of pass `p`: a stream nobody has started (position below num_streams) or a
-// hand-over from the queue. Returns false when every stream is done (or on a timeout). One thread per CTA.
-__device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64* stream, u32* rec) {
-  const u64 h = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_head[p]), 1ull);
-  if (h < a.num_streams) { *stream = a.order ? a.order[h] : h; *rec = kNoRec; return true; }
+// hand-over from the queue. Returns false when every stream is done (or on a timeout). *rec: the stream's hand-over record (kNoRec: it
+// has none), *resumed: what to start from is in there, *more: others wait. A CTA's first position is its own number, so that every SM
+// gets its share of the long streams, which come first (the CTAs of an SM ask at the same time: with 296 long streams among
+// 1,776, 42 SMs had seven of them each, the others none, and walked 791 tiles instead of 700). One thread per CTA.
+__device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, bool first, u64* stream, u32* rec, bool* resumed, bool* more) {
+  const u64 h = first ? blockIdx.x : gridDim.x + atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_head[p]), 1ull);
+  *resumed = h >= a.num_streams;
+  if (h < a.num_streams) {
+    *stream = a.order ? a.order[h] : h;
+    *rec = h < a.record_capacity ? (u32)h : kNoRec;  // (streams come longest first; those without a record are walked whole)
+    *more = h + 1 < a.num_streams || atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull);
+    return true;
+  }
   const u64 slot = h - a.num_streams;
   if (!a.queue || slot >= a.queue_capacity) return false;  // more positions than hand-overs can ever be published
   volatile u32* q = a.queue + slot;
-  volatile u32* done = &a.ctl->n_done[p];
-  volatile u64* tail = &a.ctl->q_tail[p];
-  u64 seen = *tail;
+  *more = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull) > slot + 1;
+  u64 seen = ~0ull;
   u32 idle = 0, nap = 64;
   for (;;) {
-    const u32 v = *q;
-    if (v) {
-      *q = 0;  // the second pass uses the same entries
-      __threadfence();
-      *rec = v - 1;
-      *stream = *reinterpret_cast<volatile u32*>(&a.records[v - 1].stream);
-      return true;
+    const u64 now = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->progress[p]), 0ull);
+    if (now != seen) {
+      const u32 v = *q;
+      if (v) {
+        *q = 0;  // the second pass uses the same entries
+        __threadfence();
+        *rec = v - 1;
+        *stream = *reinterpret_cast<volatile u32*>(&a.records[v - 1].stream);
+        return true;
+      }
+      if ((u32)now >= a.num_streams) return false;
+      if (seen == ~0ull) atomicExch(&a.ctl->level[p], 0u);
+      seen = now;
+      idle = 0;
     }
-    if (*done >= a.num_streams) return false;
-    const u64 t = *tail;
-    if (t != seen) { seen = t; idle = 0; }
-    if (++idle > a.poll_limit) {  // ~1 s without any hand-over anywhere
+    if (++idle > a.poll_limit) {  // ~1 s without any movement anywhere
       argus_set_error(a.status, ARGUS_ERR_TIMEOUT, 0, slot);
       return false;
     }
@@ -146,6 +162,10 @@ struct TileSmem {
   u64 cur_stream;
   u32 cur_rec;                     // hand-over record of the stream being walked (kNoRec: none)
   int skip;                        // the piece of work taken is not to be walked
+  int resumed;                     // its state is in the record
+  int more, level;                 // others wait; and this CTA says how long they are
+  int started;                     // this CTA has had work
+  u32 ti_end, look;                // where this CTA stops; the tile at which thread 0 looks up what waits
   int stop;                        // split pass: everything is left to the chained pass
   u64 n_int;                       // written by the sequential redo path
   int ch;
@@ -224,7 +244,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);
     fence_mbar_init();
-    sm.dead = 0;
+    sm.dead = sm.started = 0;
     for (int w = NW; w < 32; ++w) sm.warp_tot[w] = 0;
     // the sink of both carried blocks: its tag, shifted arithmetically, reads as ARGUS_NONE
     sm.evall[T + kSink] = sm.evall[T + kCar + kSink] = make_uint4(0, 0, 0xfffffffeu, 0);
@@ -240,16 +260,22 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     if (tid == 0) {
       u64 st = ~0ull;
       u32 rc = kNoRec;
-      bool skip = false;
+      bool skip = false, resumed = false, more = false;
       if (SPLIT) {
         const uint4 w = __ldcg(reinterpret_cast<const uint4*>(&a.ctl->num_failed));  // num_failed, num_segments, split
         rc = atomicAdd(&a.ctl->seg_head, 1u);
         st = w.z && rc < w.y ? a.segments[rc].stream : ~0ull;
         skip = w.x && st < a.num_streams && __ldcg(a.split_failed + st);
-      } else if (!tile_pop_work(a, a.redo ? 1 : 0, &st, &rc)) st = ~0ull;
+      } else if (!tile_pop_work(a, a.redo ? 1 : 0, !sm.started, &st, &rc, &resumed, &more)) st = ~0ull;
       sm.cur_stream = st;
       sm.cur_rec = rc;
-      if (!SPLIT && segments) skip = st < a.num_streams && rc == kNoRec && !__ldcg(a.split_failed + st);
+      if (!SPLIT) {
+        sm.resumed = resumed;
+        sm.level = sm.started || blockIdx.x == gridDim.x - 1;  // (not by all blocks at once when the kernel starts)
+        sm.more = more;
+        sm.started = 1;
+      }
+      if (!SPLIT && segments) skip = st < a.num_streams && !resumed && !__ldcg(a.split_failed + st);
       sm.skip = skip;
       sm.stop = 0;
     }
@@ -257,9 +283,9 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     const u64 s64 = sm.cur_stream;
     if (s64 >= a.num_streams) break;
     const u32 s = (u32)s64;
-    u32 rec = sm.cur_rec;
+    const u32 rec = sm.cur_rec;
     if (sm.skip) {
-      if (!SPLIT && tid == 0) atomicAdd(&a.ctl->n_done[0], 1u);  // walked by the split pass
+      if (!SPLIT && tid == 0) tile_progress(a, 1);  // walked by the split pass
       __syncthreads();
       continue;
     }
@@ -269,7 +295,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       if (tid == 0) {
         argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
         if (!a.redo) a.counts[s] = 0;
-        if (!SPLIT) atomicAdd(&a.ctl->n_done[a.redo ? 1 : 0], 1u);  // (the chained pass counts what the split pass has walked)
+        if (!SPLIT) tile_progress(a, 1);  // (the chained pass counts what the split pass has walked)
       }
       __syncthreads();
       continue;
@@ -279,7 +305,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     const u64 out_base = a.redo ? a.interval_offsets[s] : a.bases[s];
     if (a.redo && s < __ldcg(&a.ctl->redo_from)) {
       // second pass: this stream's intervals (and digests) already lie where they belong
-      if (tid == 0) atomicAdd(&a.ctl->n_done[1], 1u);
+      if (tid == 0) tile_progress(a, 1);
       __syncthreads();
       continue;
     }
@@ -289,11 +315,9 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     int ch = 0;          // carried stack height (uniform)
     u64 n_int = 0;       // intervals of this stream so far (uniform)
     bool stream_failed = false;
-    // Long streams are walked a chunk at a time. A resumed stream takes its state from the record; a new one
-    // reserves a record.
     u32 ti0 = 0;
-    constexpr u32 kChunkTiles = (kChunkEvents + T - 1) / T;
-    bool chunked = !SPLIT && a.queue != nullptr && ntiles > kChunkTiles;
+    constexpr u32 kChunkTiles = (kChunkEvents + T - 1) / T < 2 ? 2 : (kChunkEvents + T - 1) / T;
+    auto look_after = [](u32 left) { return left / 8 > kChunkTiles ? left / 8 : kChunkTiles; };  // tiles; a look costs half a us
     int init_h = 0;      // split: frames of the initial stack that are still open (uniform)
     u64 limit = a.interval_capacity;
     if (SPLIT) {
@@ -308,7 +332,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         sm.cidx[0][tid] = at;
       }
       if (tid == 0) sm.low = 0x7fffffff;
-    } else if (rec != kNoRec) {
+    } else if (sm.resumed) {
       const ArgusStreamRecord* r = a.records + rec;
       ti0 = __ldcg(&r->next_tile);
       ch = __ldcg(&r->ch);
@@ -318,25 +342,26 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         sm.cchild[0][tid] = __ldcg(&r->child[tid]);
         sm.cidx[0][tid] = __ldcg(&r->idx[tid]);
       }
-    } else if (chunked) {
-      __syncthreads();  // everyone has read sm.cur_rec
-      if (tid == 0) {
-        const u32 r = atomicAdd(&a.ctl->n_records[a.redo ? 1 : 0], 1u);
-        sm.cur_rec = r < a.record_capacity ? r : kNoRec;
+    }
+    // thread 0 alone decides where the piece ends
+    if (tid == 0) {
+      const u32 end = SPLIT ? ti0 + seg->num_tiles : ntiles;
+      sm.ti_end = end;
+      if (ti0 < end) {  // first tile of this piece, into the buffer its index selects
+        const u32 start = ti0 * (u32)T;
+        tile_fetch<RING>(a, (ti0 & 1) ? sm.evall + T + 2 * kCar : sm.evall, src, ring_first, start,
+                         (n - start) < (u32)T ? (n - start) : (u32)T, &sm.bar[ti0 & 1]);
       }
-      __syncthreads();
-      rec = sm.cur_rec;
-      if (rec == kNoRec) chunked = false;  // cannot happen (one record per long stream); then the stream is walked whole
+      if (!SPLIT) {
+        sm.look = rec != kNoRec ? ti0 + look_after(ntiles - ti0) - 2 : 0xffffffffu;
+        if (sm.level) atomicExch(&a.ctl->level[a.redo ? 1 : 0], sm.more ? n - ti0 * (u32)T : 0u);
+      }
     }
-    const u32 ti_end = SPLIT ? ti0 + seg->num_tiles : chunked && ti0 + kChunkTiles < ntiles ? ti0 + kChunkTiles : ntiles;
-    if (tid == 0 && ti0 < ti_end) {  // first tile of this chunk, into the buffer its index selects
-      const u32 start = ti0 * (u32)T;
-      tile_fetch<RING>(a, (ti0 & 1) ? sm.evall + T + 2 * kCar : sm.evall, src, ring_first, start,
-                       (n - start) < (u32)T ? (n - start) : (u32)T, &sm.bar[ti0 & 1]);
-    }
+    __syncthreads();
 
     int cpar = 0;        // which carried-frame block holds the current stack
-    for (u32 ti = ti0; ti < ti_end; ++ti) {
+    u32 ti = ti0;
+    for (; ti < sm.ti_end; ++ti) {
       const int b = ti & 1;
       const u32 tile_start = ti * (u32)T;
       const int tn = (int)((n - tile_start) < (u32)T ? (n - tile_start) : (u32)T);
@@ -345,7 +370,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       const uint4* evb = b ? ev1 : ev0;                  // evb[ref] for every reference of this tile
       u32* accb = sm.accall + 2 * kCar;                  // accb[ref], ref in [-2 kCar, T + 2 kCar)
       const int carlo = b ? -2 * kCar : T;               // reference of slot 0 of carried block 0, seen from this buffer
-      if (tid == 0 && ti + 1 < ti_end) {  // prefetch the next tile into the other buffer
+      if (tid == 0 && ti + 1 < sm.ti_end) {  // prefetch the next tile into the other buffer
         const u32 nstart = tile_start + T;
         tile_fetch<RING>(a, b ? ev0 : ev1, src, ring_first, nstart, (n - nstart) < (u32)T ? (n - nstart) : (u32)T, &sm.bar[b ^ 1]);
       }
@@ -355,6 +380,14 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         if (b) ph1 ^= 1; else ph0 ^= 1;
         if (!ok) sm.dead = 1;
         if (SPLIT && !go_on) sm.stop = 1;
+        if (!SPLIT && tid == 0) {
+          if (ti == sm.look && ti + 2 < sm.ti_end) {  // (others read sm.ti_end after the tile's barriers)
+            const u32 half = atomicOr(&a.ctl->level[a.redo ? 1 : 0], 0u) / 2;
+            if (half > kLevelMargin && n - (ti + 2) * (u32)T < half - kLevelMargin) sm.ti_end = ti + 2;
+            sm.look = ti + look_after(ntiles - ti);
+          }
+          if ((ti & 31u) == 31u) tile_progress(a, 1ull << 32);  // whoever waits sees that streams get on
+        }
       }
 
       // The tile is consumed in windows [w0, wend). A well-nested tile is one window. When the parallel
@@ -512,7 +545,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
           if (i == 0 && sm.dead) {  // a bulk copy never arrived: report and leave (uniform decision)
             if (tid == 0) {
               argus_set_error(a.status, ARGUS_ERR_TIMEOUT, s, tile_start);
-              atomicAdd(&a.ctl->n_done[a.redo ? 1 : 0], 1u);  // CTAs that poll for hand-overs must not wait for this stream
+              tile_progress(a, 1);  // CTAs that poll for hand-overs must not wait for this stream
             }
             return;
           }
@@ -638,7 +671,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         }
       }  // windows
       if (stream_failed) {
-        if (ti + 1 < ti_end) {  // drain the prefetched tile before the buffer is reused
+        if (ti + 1 < sm.ti_end) {  // drain the prefetched tile before the buffer is reused
           const bool ok = mbar_wait_bounded(&sm.bar[b ^ 1], (b ^ 1) ? ph1 : ph0);
           if (b ^ 1) ph1 ^= 1; else ph0 ^= 1;
           if (!ok) sm.dead = 1;
@@ -652,7 +685,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
     if (sm.dead) {
       if (tid == 0) {
         argus_set_error(a.status, ARGUS_ERR_TIMEOUT, s, 0);
-        atomicAdd(&a.ctl->n_done[a.redo ? 1 : 0], 1u);
+        tile_progress(a, 1);
       }
       return;
     }
@@ -667,10 +700,11 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         if (tot_clamp) atomicAdd(&seg->flags[2], tot_clamp);
       }
       tot_ctx = tot_rev = tot_clamp = 0;
-    } else if (!stream_failed && ti_end < ntiles) {
+    } else if (!stream_failed && ti < ntiles) {
       // hand the stream on: its state goes into the record, the record into the queue
+      const u32 rec = sm.cur_rec;
       ArgusStreamRecord* r = a.records + rec;
-      if (tid == 0) { r->stream = s; r->next_tile = ti_end; r->ch = ch; r->n_int = n_int; }
+      if (tid == 0) { r->stream = s; r->next_tile = ti; r->ch = ch; r->n_int = n_int; }
       if (tid < ch) {
         r->frames[tid] = sm.evall[T + cpar * kCar + tid];
         r->child[tid] = sm.cchild[cpar][tid];
@@ -681,6 +715,8 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
       if (tid == 0) {
         const u64 slot = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[a.redo ? 1 : 0]), 1ull);
         if (slot < a.queue_capacity) *reinterpret_cast<volatile u32*>(a.queue + slot) = rec + 1;
+        __threadfence();
+        tile_progress(a, 1ull << 32);
       }
     } else {
       if (!a.redo) {
@@ -688,7 +724,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         if (!stream_failed && tid < ch) argus_note_ambiguity(a, gpos0 + sm.cidx[cpar][tid], ARGUS_AMBIG_BEGIN_EOS, (u32)tid);
         if (tid == 0) a.counts[s] = n_int;
       }
-      if (tid == 0) atomicAdd(&a.ctl->n_done[a.redo ? 1 : 0], 1u);
+      if (tid == 0) tile_progress(a, 1);
     }
     __syncthreads();
   }  // streams

@@ -2,7 +2,7 @@
 //
 // One CTA walks one stream tile by tile (T = NT * E events per tile); tiles arrive in shared
 // memory by TMA bulk copies (double buffered, mbarrier completion) and interval records leave with
-// coalesced 16-byte stores, one thread per record. The per-stream region stack is carried from tile
+// 32- and 16-byte stores, one thread per record. The per-stream region stack is carried from tile
 // to tile in shared memory; a CTA waits for another only when it has nothing to do (see ArgusStreamRecord).
 //
 // Inside a tile the stack height before each event is a count of begins and ends: among 32 in a row by vote, over the
@@ -202,6 +202,20 @@ __device__ __forceinline__ int tile_latest_begin(const TileSmem<NT, E>& sm, int 
   return m || earlier ? r : -1;
 }
 
+
+// An interval record, which starts on a 32-byte boundary or 16 bytes behind one, as its aligned 32 bytes and the other 16. Beside a neighbour's
+// 16, stored by the same instruction, every 32-byte sector is written once and whole; three 16-byte stores write each in two
+// halves, and the L2 takes as long for a half as for all of it. (GEMM 573 -> 549 us, attention 1,246 -> 1,191, decode 2,441 -> 2,339;
+// as predicated stores, without selects, 599, 1,283 and 2,531: 16 bytes of registers spilled.)
+__device__ __forceinline__ void tile_store_record(uint4* q, u32 t0, u32 t1, u32 incl, u32 excl, u32 region, u32 ctx, u32 stream, u32 parent,
+                                                  u32 idx, u32 depth_flags) {
+  const bool odd = (reinterpret_cast<uintptr_t>(q) & 16) != 0;
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(q + (odd ? 1 : 0)), "r"(odd ? excl : t0), "r"(odd ? 0u : t1),
+               "r"(odd ? region : incl), "r"(odd ? ctx : 0u), "r"(odd ? stream : excl), "r"(odd ? parent : 0u), "r"(odd ? idx : region),
+               "r"(odd ? depth_flags : ctx)
+               : "memory");
+  q[odd ? 0 : 2] = odd ? make_uint4(t0, t1, incl, 0u) : make_uint4(stream, parent, idx, depth_flags);
+}
 
 // One tile of a stream into shared memory: a bulk copy, or two when the stream lives in a ring slot and the
 // tile straddles the slot's end. `src` is the stream's first record (packed input) or its slot (ring).
@@ -572,10 +586,8 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
             if (over) { flags |= ARGUS_FLAG_CHILD_CLAMPED; excl = 0; }
             if (flags) win_flags += (flags & 1u) | ((flags & 2u) << 9) | ((flags & 4u) << 18);
             if (rk < fit) {
-              uint4* q = rec0 + 3 * rk;
-              q[0] = make_uint4((u32)bts, (u32)(bts >> 32), incl, 0u);
-              q[1] = make_uint4(excl, 0u, btag >> 1, bctx);
-              q[2] = make_uint4(s, preg, bidx, (d >> SM::kDescShift) | (flags << 16));
+              tile_store_record(rec0 + 3 * rk, (u32)bts, (u32)(bts >> 32), incl, excl, btag >> 1, bctx, s, preg, bidx,
+                                (d >> SM::kDescShift) | (flags << 16));
               if (dig0) dig0[rk] = argus_digest_pack32(btag >> 1, incl, excl, flags);
             }
           } else if (incl) {

@@ -3,7 +3,8 @@
 //   k_agg_streams_digest : argus_synthesize's pass: one CTA per stream reads the 8-byte digests the pairing
 //                   kernel wrote beside the interval records (not the records) and gathers the stream's row
 //                   in 124-byte shared-memory cells, with per-lane copies of the most frequent regions' cells;
-//   k_agg_streams_compact : the same over the 48-byte records, with an optional scope: that stream's row in
+//   k_agg_streams_records : the same over the 48-byte records, without the overlap selection;
+//   k_agg_streams_compact : the same over the records that a scope selects: that stream's row in
 //                   a compact shared-memory form (112 B per region: sums, min, max, a 16-bin window, so
 //                   several CTAs fit an SM), for up to kAggCompactRegions regions;
 //   k_agg_streams : the same on the global row itself, for more regions than that. Integer atomics only: the
@@ -13,6 +14,7 @@
 //   k_agg_iter_windows, k_agg_iter : per-iteration cells (key = ctx - ctx_lo) of the intervals of a scope.
 // A scope (iteration window, warp mask, SM mask, region mask) filters what the kernels over intervals
 // take in; without one everything is selected.
+#include "argus_bulk.cuh"
 #include "argus_internal.cuh"
 
 namespace {
@@ -21,7 +23,7 @@ constexpr int kAggThreads = 256;
 constexpr u32 kCell = 72;  // u64 words per argus_agg_t
 constexpr u32 kAggCompactRegions = 400;  // 112 B each: 44.8 KB of shared memory at most (k_agg_iter_windows: 136 KB)
 constexpr u32 kIterThreads = 512, kIterWarps = kIterThreads / 32;  // k_agg_iter_windows
-constexpr u32 kMaxParts = 16;            // blocks that share a stream in k_agg_streams_compact
+constexpr u32 kMaxParts = 16;            // blocks that share a stream in the passes over the records
 
 struct AggArgs {
   const argus_interval_t* intervals;
@@ -46,7 +48,7 @@ struct AggArgs {
   ulonglong2* ranges; // [S][parts] first and last + 1 interval of the part that is in the iteration window (null: not asked for)
   // overlap selection in the pass over the digests (argus_synthesize)
   ArgusFuseArgs ov;
-  u32 parts;          // k_agg_streams_digest, k_agg_streams_compact: blocks that share a stream
+  u32 parts;          // blocks that share a stream
   u32 slices;         // k_agg_streams_digest: slices of a stream, one per warp of its blocks
   const u64* digest;  // digests of the intervals (k_agg_streams_digest; overwritten with entries where overlap is selected), null = read the records
   u64 interval_limit; // records the interval array holds: a stream whose offsets reach beyond it is reported, not read
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams(AggArgs a) {
 __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) {
   argus_kernel_begin_long();
   agg_empty_tables(a);
-  extern __shared__ __align__(16) unsigned char sh_raw[];
+  extern __shared__ __align__(128) unsigned char sh_raw[];
   __shared__ u64 range[2];
   ArgusAggCell* const ctab = reinterpret_cast<ArgusAggCell*>(sh_raw);
   const u32 R = a.num_regions;
@@ -253,7 +255,7 @@ template <u32 kThreads, u32 kCopies, u32 kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArgs a) {
   constexpr u32 kMinProbe = 4 * kThreads;    // shorter streams are gathered without copies
   constexpr u32 kSlices = kThreads / 32;   // slices of a stream, one per warp (also the slices of the overlap entries)
-  extern __shared__ __align__(16) unsigned char sh_raw[];
+  extern __shared__ __align__(128) unsigned char sh_raw[];
   const u32 R = a.num_regions;
   u32* const tab = reinterpret_cast<u32*>(sh_raw);
   u32* const meta = tab + digest_cell_words(R, kCopies);
@@ -550,6 +552,172 @@ __device__ __forceinline__ void iter_flush(u32* cells, const u32* hot_region, u6
   }
 }
 
+// ---- the pass over the records (argus_aggregate) ----
+// One block per stream (or several), as in the pass over the digests: the stream's row in cells of 32-bit words, with copies of the most
+// frequent regions' cells, lanes apart, and the row written once. An interval of 2^32 ticks and more is added to the row
+// afterwards, by the lanes that met one. Bound by HBM where streams are long; the records come by bulk copies, because the cells leave
+// little L1 for what three loads of a lane have in common. k_agg_streams_compact with its 64-bit cells, of which 32 lanes often want the
+// same one, and compare-and-swap loops for minimum and maximum, took (us, then / now): 12.5 M records of 5 regions 162 / 119, 34 M 385 /
+// 293, 42 M of 202 regions 700 / 626, 1.7 M 139 / 72, 207,000 18.5 / 17.3; but of a scope that selects a third of 115 M records 931 /
+// 1,026, because nothing is added for most records and eight blocks of it fit an SM instead of three.
+constexpr u32 kRecCopies = 8;
+constexpr u32 kRecThreads = 256;   // also the records of a tile
+constexpr u32 kRecStages = 2;
+constexpr u32 kRecTileBytes = kRecThreads * (u32)sizeof(argus_interval_t);
+__host__ __device__ constexpr u32 record_cell_words(u32 R) { return (kItWords * (R + kDigestHot * kRecCopies) + 3) & ~3u; }
+__host__ __device__ constexpr size_t record_table_bytes(u32 R) { return kRecStages * kRecTileBytes + 4 * ((size_t)record_cell_words(R) + R); }
+
+__global__ void __launch_bounds__(kRecThreads) k_agg_streams_records(AggArgs a) {
+  extern __shared__ __align__(128) unsigned char sh_raw[];
+  __shared__ u32 hot_region[kDigestHot], often[64], num_often;
+  __shared__ u64 full[kRecStages];
+  constexpr u32 kThreads = kRecThreads;
+  const u32 R = a.num_regions, tid = threadIdx.x, lane = tid & 31;
+  u32 *const tab = reinterpret_cast<u32*>(sh_raw + kRecStages * kRecTileBytes), *const meta = tab + record_cell_words(R);
+  const u32 tab_addr = (u32)__cvta_generic_to_shared(tab);
+  if (tid == 0) {
+#pragma unroll
+    for (u32 k = 0; k < kRecStages; ++k) mbar_init(&full[k], 1);
+    fence_mbar_init();
+    num_often = 0;
+  }
+  argus_kernel_begin_long();
+  const u32 s = blockIdx.x / a.parts, part = blockIdx.x % a.parts;
+  u64* const row = a.warp_tab + (size_t)s * R * kCell;
+  u64 lo = a.interval_offsets[s], hi = a.interval_offsets[s + 1];
+  if (hi < lo || hi > a.interval_limit) {
+    if (tid == 0) argus_set_error(a.status, ARGUS_ERR_BAD_OFFSETS, s, 0);
+    lo = hi = 0;
+  } else if (a.parts > 1) {
+    const u64 per = (hi - lo + a.parts - 1) / a.parts;
+    const u64 from = lo + per * part;
+    lo = from < hi ? from : hi;
+    hi = lo + per < hi ? lo + per : hi;
+  }
+  // a tile of records into its stage (thread 0)
+  auto fetch = [&](u64 first_record, u32 stage) {
+    const u32 bytes = hi - first_record < kThreads ? (u32)(hi - first_record) * (u32)sizeof(argus_interval_t) : kRecTileBytes;
+    mbar_expect_tx(&full[stage], bytes);
+    tma_load_1d(sh_raw + stage * kRecTileBytes, a.intervals + first_record, bytes, &full[stage]);
+  };
+  if (tid == 0) {
+#pragma unroll
+    for (u32 k = 0; k < kRecStages; ++k) if (lo + k * kThreads < hi) fetch(lo + k * kThreads, k);
+  }
+  for (u32 i = tid; i < record_cell_words(R) / 4; i += kThreads) reinterpret_cast<uint4*>(tab)[i] = make_uint4(0, 0, 0, 0);
+  for (u32 r = tid; r < R; r += kThreads) meta[r] = tab_addr + r * (kItWords * 4);
+  if (tid < kDigestHot) hot_region[tid] = 0xffffffffu;
+  agg_empty_tables(a);
+  __syncthreads();
+  const u32 own_copy = lane % kRecCopies * (kItWords * 4);
+  bool wide = false, arrived = true;  // the lane met a wide interval; every copy has arrived
+  u32 stage = 0, parity = 0;
+  for (u64 at = lo; at < hi; at += kThreads) {
+    arrived = mbar_wait_bounded(&full[stage], parity);
+    const u64 i = at + tid;
+    const u32* const p = reinterpret_cast<const u32*>(sh_raw + stage * kRecTileBytes) + tid * (sizeof(argus_interval_t) / 4);
+    bool in = arrived && i < hi;
+    const u32 region = in ? p[6] : 0u;
+    if (region >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, i); in = false; }
+    if (at == lo && hi - lo >= 4 * kThreads) {  // the regions that the first tile has most get copies of their cells, lanes apart: 32 adds to one address take turns
+      if (in) dg_inc<kDgBins>(tab_addr + region * (kItWords * 4), 1u);
+      __syncthreads();
+      for (u32 r = tid; r < R; r += kThreads) {
+        const u32 cnt = tab[r * kItWords + kDgBins];
+        tab[r * kItWords + kDgBins] = 0;
+        if (cnt >= kThreads / 64) often[atomicAdd(&num_often, 1u)] = (cnt << 16) | r;  // at most 64 of them
+      }
+      __syncthreads();
+      if (tid < num_often) {
+        const u32 key = often[tid], r = key & 0xffffu;
+        u32 rank = 0;
+        for (u32 k = 0; k < num_often; ++k) rank += often[k] > key;
+        if (rank < kDigestHot) { hot_region[rank] = r; meta[r] = (tab_addr + (R + rank * kRecCopies) * (kItWords * 4)) | kDgHot; }
+      }
+      __syncthreads();
+    }
+    if (in) {
+      const uint2 incl = *reinterpret_cast<const uint2*>(p + 2), excl = *reinterpret_cast<const uint2*>(p + 4);
+      if (incl.y | excl.y || incl.x == 0xffffffffu) {
+        wide = true;
+      } else {
+        const u32 m = meta[region];
+        iter_add((m & ~kDgHot) + (m >> 31) * own_copy, incl.x, excl.x, p[11] >> 16);
+      }
+    }
+    __syncthreads();  // everybody has read the stage
+    if (tid == 0 && at + kRecStages * kThreads < hi) fetch(at + kRecStages * kThreads, stage);
+    if (++stage == kRecStages) { stage = 0; parity ^= 1; }
+  }
+  if (__syncthreads_or(!arrived) && tid == 0) argus_set_error(a.status, ARGUS_ERR_TIMEOUT, s, 0);
+  // the copies into their region's cell (which nobody added to): a thread per (hot region, field)
+  if (num_often && tid < kDigestHot * kItWords) {
+    const u32 h = tid / kItWords, f = tid % kItWords, r = hot_region[h];
+    if (r != 0xffffffffu && f != kDgSumInclHi && f != kDgSumExclHi) {
+      const u32* src = tab + (R + h * kRecCopies) * kItWords + f;
+      u32* dst = tab + r * kItWords + f;
+      const bool sum = f == kDgSumInclLo || f == kDgSumExclLo, most = f == kDgNotMin || f == kDgMax;
+      u64 acc = 0;
+#pragma unroll
+      for (u32 l = 0; l < kRecCopies; ++l) {
+        const u32 v = src[l * kItWords];
+        if (sum) acc += (u64)v | ((u64)src[l * kItWords + 1] << 32);
+        else acc = most ? (v > acc ? v : acc) : acc + v;
+      }
+      dst[0] = (u32)acc;
+      if (sum) dst[1] = (u32)(acc >> 32);
+    }
+  }
+  __syncthreads();
+  // the regions' cells into the global row; a thread keeps to one field
+  const bool alone = a.parts == 1;  // (else the rows have been initialised: several blocks add to one)
+  auto put = [&](u64* p, u32 field, u64 v) {
+    if (alone) *p = v;
+    else if (field == 2) { if (v != ~0ull) atomicMin(p, v); }
+    else if (field == 3) { if (v) atomicMax(p, v); }
+    else if (v) atomicAdd(p, v);
+  };
+  {
+    const u32 f = tid % 64;
+    for (u32 r = tid / 64; r < R; r += kThreads / 64) put(row + (size_t)r * kCell + 8 + f, 8 + f, f < 32 ? tab[r * kItWords + kDgBins + f] : 0u);
+  }
+  {
+    const u32 f = tid % 8;
+    const u32 w = f == 1 ? kDgSumInclLo : f == 2 ? kDgNotMin : f == 3 ? kDgMax : f == 4 ? kDgSumExclLo : kDgFlag;
+    for (u32 r = tid / 8; r < R; r += kThreads / 8) {
+      const u32* c = tab + r * kItWords;
+      u64 v = c[w];
+      if (f == 0) {
+        u32 cnt = 0;
+#pragma unroll
+        for (u32 j = 0; j < 32; ++j) cnt += c[kDgBins + j];
+        v = cnt;
+      }
+      if (f == 1 || f == 4) v |= (u64)c[w + 1] << 32;
+      if (f == 2) v = v ? (u64)(u32)~(u32)v : ~0ull;
+      if (f == 5 || f == 6) v = 0;  // ambiguity records: below
+      put(row + (size_t)r * kCell + f, f, v);
+    }
+  }
+  u64 alo = 0, ahi = 0;
+  if (a.ambig && a.ambig_offsets && part == 0) { alo = a.ambig_offsets[s]; ahi = a.ambig_offsets[s + 1]; }
+  if (!__syncthreads_or(wide || alo < ahi)) return;
+  __threadfence();
+  __syncthreads();
+  if (wide) {  // (the lane's records are looked at again)
+    for (u64 k = lo + tid; k < hi; k += kThreads) {
+      const uint4* p = reinterpret_cast<const uint4*>(a.intervals + k);
+      const uint4 q0 = __ldg(p), q1 = __ldg(p + 1), q2 = __ldg(p + 2);
+      if (q0.w | q1.y || q0.z == 0xffffffffu) digest_wide(row, R, q0, q1, q2.w >> 16);
+    }
+  }
+  for (u64 k = alo + tid; k < ahi; k += kThreads) {
+    const u32 r = a.ambig[k].tag >> 1;
+    if (r >= R) { argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, k); continue; }
+    atomicAdd(row + (size_t)r * kCell + (a.ambig[k].kind == ARGUS_AMBIG_UNMATCHED_END ? 6 : 5), 1ull);
+  }
+}
+
 // iter_tab[ctx - ctx_lo][r] with cells as in the pass over the digests. A block walks a few streams side by side (kIterWarps warps, shared out
 // among them) and holds the cells of two neighbouring iterations in shared memory; a warp that comes to a later one waits until
 // all have, then the older cells are added to the table. Iterations come in order in a stream, so each is gathered once for
@@ -563,7 +731,7 @@ __device__ __forceinline__ void iter_flush(u32* cells, const u32* hot_region, u6
 // intervals of 292 regions, 16 of 32 iterations, 1,964 -> 1,743 us, 115 M of 400 regions, 16 of 24, 2,487 -> 2,390.
 __global__ void __launch_bounds__(kIterThreads) k_agg_iter_windows(AggArgs a, u32 streams_per_block) {
   argus_kernel_begin_long();
-  extern __shared__ __align__(16) unsigned char sh_raw[];
+  extern __shared__ __align__(128) unsigned char sh_raw[];
   __shared__ u32 need;
   const u32 R = a.num_regions, cells = R * kCell, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u32 *const tab0 = reinterpret_cast<u32*>(sh_raw), *const tab1 = tab0 + kItWords * iter_cells(R), *const meta = tab1 + kItWords * iter_cells(R);
@@ -764,8 +932,6 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
     ARGUS_LAUNCH(k_agg_init, 592, 256, 0, stream, a.warp_tab, (u64)num_streams * num_regions * kCell);
   argus_prof_mark(ARGUS_PROF_AGGREGATE, stream, 0);
   if (num_regions <= kAggCompactRegions) {
-    const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell);
-    static_assert(kAggCompactRegions * sizeof(ArgusAggCell) <= 48 * 1024, "no more shared memory than every kernel gets");
     if (a.digest) {
       const u32 warps = a.slices / a.parts;
       const u32 copies = warps == 16 ? 32 : 8;
@@ -774,7 +940,11 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       if (dg > 48 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, digest_table_bytes(kAggCompactRegions, copies)));
       ARGUS_LAUNCH(kernel, num_streams * a.parts, warps * 32, dg, stream, a);
     } else {
-      ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
+      const size_t bytes = record_table_bytes(num_regions), compact = (size_t)num_regions * sizeof(ArgusAggCell);
+      static_assert(kAggCompactRegions * sizeof(ArgusAggCell) <= 48 * 1024, "no more shared memory than every kernel gets");
+      if (!scope && bytes > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(k_agg_streams_records, record_table_bytes(kAggCompactRegions)));
+      if (scope) ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
+      else ARGUS_LAUNCH(k_agg_streams_records, num_streams * a.parts, kRecThreads, bytes, stream, a);
     }
   } else {
     ARGUS_LAUNCH(k_agg_streams, num_streams, kAggThreads, 0, stream, a);

@@ -22,7 +22,9 @@ constexpr int kScanThreads = 1024;
 // Streams a thread of the one-block scans over all streams takes at a time: four where there are many (10^6 streams: 1,690 -> 1,325 us
 // and 1,640 -> 860), one where a block holds them all (16 streams: a call of 45 us is 1 to 2 us longer with four).
 constexpr u32 kScanRun = 4;
-constexpr u32 kWordsPerBlock = 1024;  // bitmap words per prefix block (32768 events)
+constexpr u32 kGroupWords = 8;                             // bitmap words of a prefix: 256 events, a sector
+constexpr u32 kThreadWords = 4 * kGroupWords;               // a thread's share
+constexpr u32 kWordsPerBlock = kScanThreads * kThreadWords;  // and of a prefix block
 std::atomic<u32> g_poll_limit{1u << 19};  // see argus_testing_set_poll_limit
 
 // ---------------------------------------------------------------------------------------------
@@ -505,7 +507,7 @@ struct AmbigArgs {
   ArgusPairArgs p;
   u64 num_words;     // bitmap words covering [0, span) event positions
   u64 span;          // stream_offsets[S] - stream_offsets[0] is <= num_events; bitmap covers num_events
-  u32* word_prefix;  // per word: set bits before it within its block
+  u32* group_prefix; // per group of words: set bits before it within its block
   u64* block_prefix; // per block: set bits before it (after the scan); [num_blocks + 1]
   u64 num_blocks;
   argus_ambiguity_t* ambig;
@@ -571,8 +573,8 @@ __device__ __forceinline__ void pair_offsets(const ArgusPairArgs& a) {
   }
 }
 
-// The other blocks, when there are notes: set bits before every word within its block of words, and, by the last block to
-// be done, before every block of words.
+// The other blocks, when there are notes: set bits before every group of words within its block of words, and, by the last block to
+// be done, before every block of words. (142 M events with a prefix for every word 46 us, 12 so.)
 template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   // The second pass comes next, and its blocks spread evenly only over SMs that are free when they come (96 streams with a lost end
@@ -588,11 +590,18 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   __shared__ u64 sh64[33];
   __shared__ u32 last;
   for (u64 blk = blockIdx.x - 1; blk < g.num_blocks; blk += gridDim.x - 1) {
-    const u64 w = blk * kWordsPerBlock + threadIdx.x;
-    const u32 c = w < g.num_words ? __popc(g.p.bits[w]) : 0u;
+    const u64 w = blk * kWordsPerBlock + threadIdx.x * kThreadWords;
+    u32 c[4] = {0, 0, 0, 0};
+    if (w < g.num_words) {  // (the last thread's share is filled up with words that are zero)
+#pragma unroll
+      for (u32 j = 0; j < kThreadWords / 4; ++j) {
+        const uint4 b = reinterpret_cast<const uint4*>(g.p.bits + w)[j];
+        c[j / (kGroupWords / 4)] += __popc(b.x) + __popc(b.y) + __popc(b.z) + __popc(b.w);
+      }
+    }
     u32 total;
-    const u32 ex = argus_block_exclusive_scan<u32>(c, sh, &total);
-    if (w < g.num_words) g.word_prefix[w] = ex;
+    const u32 ex = argus_block_exclusive_scan<u32>(c[0] + c[1] + c[2] + c[3], sh, &total);
+    if (w < g.num_words) *reinterpret_cast<uint4*>(g.group_prefix + w / kGroupWords) = make_uint4(ex, ex + c[0], ex + c[0] + c[1], ex + c[0] + c[1] + c[2]);
     if (threadIdx.x == 0) g.block_prefix[blk] = total;
     __syncthreads();
   }
@@ -624,7 +633,13 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
 __device__ __forceinline__ u64 ambig_rank(const AmbigArgs& g, u64 gpos) {
   const u64 w = gpos >> 5;
   if (w >= g.num_words) return g.block_prefix[g.num_blocks];
-  return g.block_prefix[w / kWordsPerBlock] + g.word_prefix[w] + __popc(g.p.bits[w] & ((1u << (gpos & 31)) - 1u));
+  const uint4* const group = reinterpret_cast<const uint4*>(g.p.bits + w / kGroupWords * kGroupWords);
+  const uint4 a = group[0], b = group[1];
+  const u32 v[kGroupWords] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}, k = (u32)w % kGroupWords;
+  u32 c = 0;
+#pragma unroll
+  for (u32 q = 0; q < kGroupWords; ++q) c += q < k ? __popc(v[q]) : q == k ? __popc(v[q] & ((1u << (gpos & 31)) - 1u)) : 0;
+  return g.block_prefix[w / kWordsPerBlock] + g.group_prefix[w / kGroupWords] + c;
 }
 
 __device__ __forceinline__ void ambig_offset(const AmbigArgs& g, u64 s) {
@@ -671,7 +686,7 @@ __global__ void __launch_bounds__(256) k_ambig_records(AmbigArgs g) {
 }
 
 struct Layout {
-  size_t ctl, counts, queue, bits, word_prefix, block_prefix, notes, records, order, bases, split, total;
+  size_t ctl, counts, queue, bits, group_prefix, block_prefix, notes, records, order, bases, split, total;
   u64 num_words, num_blocks, queue_capacity;
   u32 record_capacity;
 };
@@ -689,8 +704,9 @@ Layout make_layout(uint64_t num_events, uint32_t num_streams, uint64_t ambig_cap
   const u64 records = num_events > 1u << 20 ? L.queue_capacity : num_events / 32768 + 1;
   L.record_capacity = (u32)(records < num_streams ? records : num_streams);
   L.queue = o; o += argus_align_up((size_t)L.queue_capacity * 4, 256);
-  L.bits = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);
-  L.word_prefix = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);
+  L.bits = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);  // (whole threads' shares)
+  static_assert(256 % (kThreadWords * 4) == 0, "whole threads' shares");
+  L.group_prefix = o; o += argus_align_up((size_t)(L.num_words + kThreadWords - 1) / kThreadWords * 16 + 4, 256);
   L.block_prefix = o; o += argus_align_up(((size_t)L.num_blocks + 1) * 8, 256);
   L.notes = o; o += argus_align_up((size_t)ambig_capacity * 8 + 8, 256);
   L.records = o; o += argus_align_up((size_t)L.record_capacity * sizeof(ArgusStreamRecord), 256);
@@ -765,12 +781,13 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   const bool tiled = (kernel_choice != 1 && argus_pair_tiled_usable(a)) || ring_written != nullptr;
   // control block, counts, queue and bitmap are contiguous at the start of the workspace and start at zero
   uint4* const zeroed = (uint4*)ws;
-  const u64 zeroed_words = L.word_prefix / 16;
+  const u64 zeroed_words = L.group_prefix / 16;
   u32* const order = (u32*)(ws + L.order);
   // Small calls: one block clears and orders. Beyond that a grid clears, and looks at the ends of the streams.
   const bool alone = num_events < (1u << 20) && num_streams <= 8192;
   // Windows all over the trace are looked at where that is little against the whole call (see kSampledEvents).
-  u32* const samples = num_events >= kSampledEvents && num_streams ? (u32*)(ws + L.word_prefix) : nullptr;  // (not used before the offsets kernel)
+  u32* const samples = num_events >= kSampledEvents && num_streams ? (u32*)(ws + L.group_prefix) : nullptr;  // (not used before the offsets kernel)
+  static_assert(kSampledEvents / 32 / kGroupWords >= kSamples, "room for the samples");
   if (!alone) {
     // a stream a warp, up to what the chip holds of them
     const u32 per = num_streams <= 148u * 64u ? 1u : num_streams < 32u * 148u * 64u ? (num_streams + 148u * 64u - 1) / (148u * 64u) : 32u;
@@ -787,7 +804,7 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
 
   AmbigArgs g;
   g.p = a; g.num_words = L.num_words; g.span = num_events;
-  g.word_prefix = (u32*)(ws + L.word_prefix); g.block_prefix = (u64*)(ws + L.block_prefix);
+  g.group_prefix = (u32*)(ws + L.group_prefix); g.block_prefix = (u64*)(ws + L.block_prefix);
   g.num_blocks = L.num_blocks; g.ambig = ambig; g.ambig_capacity = ambig_capacity; g.ambig_offsets = (u64*)ambig_offsets;
   for (int pass = 0; pass < 2; ++pass) {
     a.redo = pass;

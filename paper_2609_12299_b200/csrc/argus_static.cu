@@ -23,7 +23,7 @@ std::atomic<void*> g_scratch_ptr[kMaxDevices];  // device address of g_pair_scra
 // The documented maxima fit the array together (the run-time check below is then never the one that refuses them).
 static_assert((size_t)ARGUS_STATIC_MAX_EVENTS / 8 * 2 + (size_t)ARGUS_STATIC_MAX_AMBIG * 8 +
                   (size_t)ARGUS_STATIC_MAX_STREAMS * 20 + 64 * 1024 <= kStaticScratchBytes,
-              "bitmap + word prefixes + ambiguity notes + per-stream counters, bases and order + queue, records and control block");
+              "bitmap + prefixes + ambiguity notes + per-stream counters, bases and order + queue, records and control block");
 
 }  // namespace
 

@@ -66,7 +66,8 @@ struct ArgusPairCtl {
 // (every unfinished stream is in some CTA's hands): it polls until the entry appears or every stream is
 // done, and gives up with ARGUS_ERR_TIMEOUT if nothing moves for about a second.
 constexpr u32 kChunkEvents = 3840;   // walked by a CTA at least before it hands a stream on
-constexpr u32 kLevelMargin = 1280;   // of which the stream has to have less than half as much left
+constexpr u32 kLevelMargin = 1280;   // by which the stream has to have less left than half
+constexpr u32 kLeastTiles = 3;       // and what is less than this is walked at once
 struct ArgusStreamRecord {
   u32 stream, next_tile;
   int ch;                             // stack height at the hand-over

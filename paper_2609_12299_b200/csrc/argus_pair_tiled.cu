@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         if (!ok) sm.dead = 1;
         if (SPLIT && !go_on) sm.stop = 1;
         if (!SPLIT && tid == 0) {
-          if (ti == sm.look && ti + 2 < sm.ti_end) {  // (others read sm.ti_end after the tile's barriers)
+          if (ti == sm.look && ti + 2 + kLeastTiles <= ntiles) {  // (others read sm.ti_end after the tile's barriers)
             const u32 half = atomicOr(&a.ctl->level[a.redo ? 1 : 0], 0u) / 2;
             if (half > kLevelMargin && n - (ti + 2) * (u32)T < half - kLevelMargin) sm.ti_end = ti + 2;
             sm.look = ti + look_after(ntiles - ti);

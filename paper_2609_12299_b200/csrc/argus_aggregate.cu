@@ -453,10 +453,6 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
   }
 }
 
-__device__ __forceinline__ u64 combine(u32 field, u64 x, u64 y) {
-  return field == 2 ? (x < y ? x : y) : field == 3 ? (x > y ? x : y) : x + y;
-}
-
 __global__ void __launch_bounds__(256) k_agg_init(u64* tab, u64 n) {
   argus_kernel_begin();
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x)
@@ -464,14 +460,21 @@ __global__ void __launch_bounds__(256) k_agg_init(u64* tab, u64 n) {
 }
 
 // One word of the cells of kGroup CTAs: CTA cells = reduction over the warps of each (written if asked for), warp-role cells over
-// the CTAs; CTA cells go to the SM-scope cells, their reduction over the group to the kernel-scope cells (atomic add / min / max
-// on integers; empty words add nothing). Bound by the one read of the warp-scope table, of which a thread has kGroup words in
-// flight: 64 us for 275 MB; 77 us a CTA a thread, and 288 us more for the roles by themselves.
-__device__ __forceinline__ void cell_add(u64* d, u32 field, u64 v) {
-  if (field == 2 ? v == ~0ull : v == 0ull) return;  // identity element: nothing to add
-  if (field == 2) atomicMin(d, v); else if (field == 3) atomicMax(d, v); else atomicAdd(d, v);
+// the CTAs; CTA cells go to the SM-scope cells, their reduction over the group to the kernel-scope cells (atomic add / max
+// on integers; empty words add nothing). A minimum is taken as the maximum of complements, so that a word is either added or compared.
+// Bound by the one read of the warp-scope table. 275 MB, us without roles / with them, one, two, four and eight CTAs a thread: 60 / 113, 55 /
+// 86, 67 / 61 and 77 / 98; with three ways to combine for every word, and for the roles whether asked for or not (40 M warp
+// instructions, issued on 60 % of the cycles), eight took 69 / 83. Five regions, 1,776 streams: 9.3 -> 7.0.
+__device__ __forceinline__ void cell_add(u64* d, u32 field, u64 v) {  // (v: as roll_in gives it)
+  if (v == 0ull) return;  // nothing to add
+  if (field == 2) atomicMin(d, ~v); else if (field == 3) atomicMax(d, v); else atomicAdd(d, v);
 }
-template <u32 kGroup>
+__device__ __forceinline__ u64 roll_in(bool most, u64 flip, u64 v, u64 x) {
+  x ^= flip;
+  if (most) return x > v ? x : v;
+  return v + x;
+}
+template <u32 kGroup, bool kRoles>
 __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
   argus_kernel_begin_long();
   const u64 per_cta = (u64)a.num_regions * kCell, n = (u64)((a.num_ctas + kGroup - 1) / kGroup) * per_cta;
@@ -479,32 +482,52 @@ __global__ void __launch_bounds__(256) k_agg_rollup(AggArgs a, u64* cta_out) {
     const u32 c0 = (u32)(i / per_cta) * kGroup, have = a.num_ctas - c0 < kGroup ? a.num_ctas - c0 : kGroup;
     const u64 rem = i % per_cta;
     const u32 field = (u32)(rem % kCell);
-    const u64 none = field == 2 ? ~0ull : 0ull;
+    const bool most = field == 2 || field == 3;
+    const u64 flip = field == 2 ? ~0ull : 0ull;
     const u64* src = a.warp_tab + (u64)c0 * a.warps_per_cta * per_cta + rem;
+    const u64 cta = a.warps_per_cta * per_cta;
     u64 v[kGroup];
 #pragma unroll
-    for (u32 q = 0; q < kGroup; ++q) v[q] = none;
-#pragma unroll kGroup == 1 ? 8 : 2
-    for (u32 w = 0; w < a.warps_per_cta; ++w) {
-      u64 x[kGroup];
+    for (u32 q = 0; q < kGroup; ++q) v[q] = 0;
+    if (have == kGroup) {
+#pragma unroll kGroup <= 2 ? 8 : 2
+      for (u32 w = 0; w < a.warps_per_cta; ++w, src += per_cta) {
+        u64 x[kGroup];
 #pragma unroll
-      for (u32 q = 0; q < kGroup; ++q) x[q] = q < have ? src[((u64)q * a.warps_per_cta + w) * per_cta] : none;
-      u64 all = none;
+        for (u32 q = 0; q < kGroup; ++q) x[q] = __ldcg(src + q * cta);
 #pragma unroll
-      for (u32 q = 0; q < kGroup; ++q) { v[q] = combine(field, v[q], x[q]); all = combine(field, all, x[q]); }
-      if (a.role_tab) cell_add(a.role_tab + w * per_cta + rem, field, all);
+        for (u32 q = 0; q < kGroup; ++q) v[q] = roll_in(most, flip, v[q], x[q]);
+        if (kRoles) {
+          u64 all = 0;
+#pragma unroll
+          for (u32 q = 0; q < kGroup; ++q) all = roll_in(most, flip, all, x[q]);
+          cell_add(a.role_tab + w * per_cta + rem, field, all);
+        }
+      }
+    } else {
+      for (u32 w = 0; w < a.warps_per_cta; ++w, src += per_cta) {
+        u64 all = 0;
+#pragma unroll
+        for (u32 q = 0; q < kGroup; ++q) {
+          if (q >= have) break;
+          const u64 x = __ldcg(src + q * cta);
+          v[q] = roll_in(most, flip, v[q], x);
+          all = roll_in(most, flip, all, x);
+        }
+        if (kRoles) cell_add(a.role_tab + w * per_cta + rem, field, all);
+      }
     }
-    u64 all = none;
+    u64 all = 0;
 #pragma unroll
     for (u32 q = 0; q < kGroup; ++q) {
       if (q >= have) break;
-      if (cta_out) cta_out[(u64)(c0 + q) * per_cta + rem] = v[q];
-      if (a.sm_tab && v[q] != none) {
+      if (cta_out) cta_out[(u64)(c0 + q) * per_cta + rem] = v[q] ^ flip;
+      if (a.sm_tab && v[q] != 0ull) {
         const u32 m = a.cta_sm[c0 + q];
         if (m >= a.num_sms) { bad_sm(a, c0 + q); continue; }
         cell_add(a.sm_tab + (u64)m * per_cta + rem, field, v[q]);
       }
-      all = combine(field, all, v[q]);
+      all = roll_in(most, 0ull, all, v[q]);
     }
     if (a.kernel_tab) cell_add(a.kernel_tab + rem, field, all);
   }
@@ -959,12 +982,12 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
     ARGUS_LAUNCH(k_agg_iter, num_streams < 1184u ? num_streams : 1184u, kAggThreads, 0, stream, a);
   }
   if (cta_tab || sm_tab || kernel_tab || role_tab) {
-    // groups of CTAs where that leaves enough threads to fill the chip (148 x 2,048)
-    const u64 words = (u64)num_regions * kCell, groups = ((u64)a.num_ctas + 7) / 8;
-    if (groups * words >= 148 * 1024)
-      ARGUS_LAUNCH(k_agg_rollup<8>, (unsigned)((groups * words + 255) / 256 < 4736 ? (groups * words + 255) / 256 : 4736), 256, 0, stream, a, (u64*)cta_tab);
-    else
-      ARGUS_LAUNCH(k_agg_rollup<1>, (unsigned)((a.num_ctas * words + 255) / 256 < 4736 ? (a.num_ctas * words + 255) / 256 : 4736), 256, 0, stream, a, (u64*)cta_tab);
+    // groups of CTAs where that leaves enough threads to fill the chip (148 x 2,048); larger ones save adds to the tables of roles
+    const u64 words = (u64)num_regions * kCell, of = role_tab ? 4 : 2, groups = ((u64)a.num_ctas + of - 1) / of;
+    const bool grouped = groups * words >= 148 * 1024;
+    const u64 blocks = ((grouped ? groups : a.num_ctas) * words + 255) / 256;
+    const auto kernel = grouped ? (role_tab ? k_agg_rollup<4, true> : k_agg_rollup<2, false>) : role_tab ? k_agg_rollup<1, true> : k_agg_rollup<1, false>;
+    ARGUS_LAUNCH(kernel, (unsigned)(blocks < 4736 ? blocks : 4736), 256, 0, stream, a, (u64*)cta_tab);
   }
   return ARGUS_OK;
 }

@@ -584,17 +584,19 @@ __device__ __forceinline__ void iter_flush(u32* cells, const u32* hot_region, u6
 // 293, 42 M of 202 regions 700 / 626, 1.7 M 139 / 72, 207,000 18.5 / 17.3; but of a scope that selects a third of 115 M records 931 /
 // 1,026, because nothing is added for most records and eight blocks of it fit an SM instead of three.
 constexpr u32 kRecCopies = 8;
-constexpr u32 kRecThreads = 256;   // also the records of a tile
 constexpr u32 kRecStages = 2;
-constexpr u32 kRecTileBytes = kRecThreads * (u32)sizeof(argus_interval_t);
+__host__ __device__ constexpr u32 record_tile_bytes(u32 threads) { return threads * (u32)sizeof(argus_interval_t); }  // a record a thread
 __host__ __device__ constexpr u32 record_cell_words(u32 R) { return (kItWords * (R + kDigestHot * kRecCopies) + 3) & ~3u; }
-__host__ __device__ constexpr size_t record_table_bytes(u32 R) { return kRecStages * kRecTileBytes + 4 * ((size_t)record_cell_words(R) + R); }
+__host__ __device__ constexpr size_t record_table_bytes(u32 R, u32 threads) {
+  return kRecStages * record_tile_bytes(threads) + 4 * ((size_t)record_cell_words(R) + R);
+}
 
-__global__ void __launch_bounds__(kRecThreads) k_agg_streams_records(AggArgs a) {
+template <u32 kThreads>
+__global__ void __launch_bounds__(kThreads) k_agg_streams_records(AggArgs a) {
+  constexpr u32 kRecTileBytes = record_tile_bytes(kThreads);
   extern __shared__ __align__(128) unsigned char sh_raw[];
   __shared__ u32 hot_region[kDigestHot], often[64], num_often;
   __shared__ u64 full[kRecStages];
-  constexpr u32 kThreads = kRecThreads;
   const u32 R = a.num_regions, tid = threadIdx.x, lane = tid & 31;
   u32 *const tab = reinterpret_cast<u32*>(sh_raw + kRecStages * kRecTileBytes), *const meta = tab + record_cell_words(R);
   const u32 tab_addr = (u32)__cvta_generic_to_shared(tab);
@@ -674,8 +676,8 @@ __global__ void __launch_bounds__(kRecThreads) k_agg_streams_records(AggArgs a) 
   }
   if (__syncthreads_or(!arrived) && tid == 0) argus_set_error(a.status, ARGUS_ERR_TIMEOUT, s, 0);
   // the copies into their region's cell (which nobody added to): a thread per (hot region, field)
-  if (num_often && tid < kDigestHot * kItWords) {
-    const u32 h = tid / kItWords, f = tid % kItWords, r = hot_region[h];
+  for (u32 hf = tid; num_often && hf < kDigestHot * kItWords; hf += kThreads) {
+    const u32 h = hf / kItWords, f = hf % kItWords, r = hot_region[h];
     if (r != 0xffffffffu && f != kDgSumInclHi && f != kDgSumExclHi) {
       const u32* src = tab + (R + h * kRecCopies) * kItWords + f;
       u32* dst = tab + r * kItWords + f;
@@ -894,6 +896,20 @@ AggLayout agg_layout(uint32_t num_streams, uint32_t num_regions) {
   return L;
 }
 
+// Threads of a block of the pass over the records. A block takes a stream, and how much of the chip the last round of blocks leaves idle
+// decides: blocks of 192 threads are taken where that makes a tenth of difference. us, 256 / 192 threads, share of the rounds that is
+// filled: 832 streams of 74 regions 454 / 346 (0.56, 0.94), 1,080 of 5 147 / 133 (0.52, 0.81), 960 of 9 117 / 119 (0.93, 0.72), 1,572 of 5 115 / 139
+// (0.76, 0.59), 2,368 of 146 623 / 645 (1, 0.8). 128 threads read the records slower: 34 M 387, 307 and 330 with more.
+u32 record_threads(u32 num_regions, u32 blocks) {
+  auto filled = [&](u32 threads) {
+    const size_t of_sm = 228 * 1024 / (record_table_bytes(num_regions, threads) + 1536);  // (1 KB of the system's and the static part)
+    const u32 most = 65536 / (40 * threads), per_sm = of_sm < most ? (u32)of_sm : most, slots = 148 * (per_sm ? per_sm : 1);
+    const u32 rounds = (blocks + slots - 1) / slots;
+    return (double)blocks / ((double)slots * (rounds ? rounds : 1));
+  };
+  return filled(192) > 1.1 * filled(256) ? 192 : 256;
+}
+
 }  // namespace
 
 extern "C" size_t argus_aggregate_workspace_bytes(uint64_t /*num_intervals*/, uint32_t num_streams, uint32_t num_regions) {
@@ -963,11 +979,17 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       if (dg > 48 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, digest_table_bytes(kAggCompactRegions, copies)));
       ARGUS_LAUNCH(kernel, num_streams * a.parts, warps * 32, dg, stream, a);
     } else {
-      const size_t bytes = record_table_bytes(num_regions), compact = (size_t)num_regions * sizeof(ArgusAggCell);
+      const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell);
       static_assert(kAggCompactRegions * sizeof(ArgusAggCell) <= 48 * 1024, "no more shared memory than every kernel gets");
-      if (!scope && bytes > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(k_agg_streams_records, record_table_bytes(kAggCompactRegions)));
-      if (scope) ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
-      else ARGUS_LAUNCH(k_agg_streams_records, num_streams * a.parts, kRecThreads, bytes, stream, a);
+      if (scope) {
+        ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
+      } else {
+        const u32 threads = record_threads(num_regions, num_streams * a.parts);
+        const size_t bytes = record_table_bytes(num_regions, threads);
+        const auto kernel = threads == 256 ? k_agg_streams_records<256> : k_agg_streams_records<192>;
+        if (bytes > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, record_table_bytes(kAggCompactRegions, threads)));
+        ARGUS_LAUNCH(kernel, num_streams * a.parts, threads, bytes, stream, a);
+      }
     }
   } else {
     ARGUS_LAUNCH(k_agg_streams, num_streams, kAggThreads, 0, stream, a);

@@ -1,4 +1,4 @@
-"""argus_aggregate's pass over the records: streams that end at, before and behind the edges of a tile of 256 records and of the 1,024 from
+"""argus_aggregate's pass over the records: streams that end at, before and behind the edges of a tile of 256 or 192 records and of the four tiles from
 which on frequent regions get copies of their cells, streams that several blocks share, durations around 2^32, one region and 400, and a record
 of a region that does not exist, against the oracle."""
 import numpy as np
@@ -10,7 +10,7 @@ import paper_2609_12299_b200 as argus
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
-EDGES = [0, 1, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 3000]
+EDGES = [0, 1, 191, 192, 193, 255, 256, 257, 385, 511, 512, 513, 767, 768, 769, 1023, 1024, 1025, 3000]
 
 
 def _dev(a):
@@ -18,7 +18,7 @@ def _dev(a):
 
 
 @pytest.mark.parametrize("R", [1, 5, 65, 400])
-@pytest.mark.parametrize("S,W", [(12, 3), (24, 1), (900, 12)])  # blocks share a stream: sixteen, sixteen, none
+@pytest.mark.parametrize("S,W", [(12, 3), (24, 1), (900, 12), (1080, 12)])  # blocks share a stream: sixteen, sixteen, none, none (blocks of 192 threads)
 def test_tables(S, W, R):
     rng = np.random.default_rng(S + R)
     lengths = np.array([EDGES[s % len(EDGES)] for s in range(S)])

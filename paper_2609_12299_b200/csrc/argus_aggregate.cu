@@ -17,6 +17,8 @@
 #include "argus_bulk.cuh"
 #include "argus_internal.cuh"
 
+#include <type_traits>
+
 namespace {
 
 constexpr int kAggThreads = 256;
@@ -201,9 +203,9 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_streams_compact(AggArgs a) 
 // words (an odd size: the cells of 32 different regions start in 32 different banks) that hold all the 23 histogram bins a
 // digest can fall into. All words start at zero: the minimum is kept as the maximum of the complement. A few regions usually
 // own most intervals of a stream, and 32 lanes adding to one address serialise; so after a count of the regions in the first
-// round of every warp the kDigestHot most frequent ones get 32 copies of their cell, one per lane (consecutive cells: never a
+// round of every warp the kDigestHot most frequent ones get copies of their cell, lanes apart (consecutive cells: rarely a
 // bank conflict), which are folded into the region's cell when the stream ends. meta[region] holds the byte address of the
-// cell to add to, whether it is one of 32 copies, and whether the region appears in an overlap pair. What does not count (past
+// cell to add to, whether it is one of the copies, and whether the region appears in an overlap pair. What does not count (past
 // the end, a bad region, a digest marked wide) goes to a cell of its own that nobody reads, so that the common case has no
 // selects. Every warp walks a slice of the stream, so that overlap candidates stay in order; their entries replace digests that
 // the warp has consumed: no list, no atomics. The row is written once, with plain stores; wide intervals (a duration of 2^23
@@ -212,7 +214,7 @@ constexpr u32 kDigestHot = 4;
 constexpr u32 kDgSumInclLo = 0, kDgSumInclHi = 1, kDgSumExclLo = 2, kDgSumExclHi = 3, kDgNotMin = 4, kDgMax = 5, kDgFlag = 6,
               kDgBins = 7, kDgCount = kDgBins + kDigestBits, kDgWords = kDgCount + 1;
 static_assert(kDgWords % 2 == 1, "an odd cell size keeps the cells of different regions in different banks");
-constexpr u32 kDgHot = 1u << 31, kDgInPair = 1u << 30, kDgAddr = (1u << 18) - 1;  // meta
+constexpr u32 kDgHot = 1u << 31, kDgInPair = 1u << 30, kDgNoRegion = 1u << 29, kDgAddr = (1u << 18) - 1;  // meta
 constexpr u64 kDgPad = 0xffffull;              // what a lane past the end looks at: no such region
 
 // cells of the regions, the cell that nobody reads, copies; then meta for each region and for no region
@@ -250,7 +252,9 @@ __device__ __noinline__ void digest_wide(u64* row, u32 R, uint4 q0, uint4 q1, u3
 // ahead change places without moves): decode trace (307 M intervals) 1,215 -> 903 us = 2.7 TB/s of digests, attention 400 -> 323,
 // GEMM 234 -> 188. Unrolled once 1,017, three times 898 (GEMM 191), four times 913. What a stream costs before its first
 // interval and after its last one (85 us of the decode trace's 903) decides for short ones: fewer threads for them and eight
-// copies instead of 32, so that more streams are on the chip (see argus_aggregate_digest_slices).
+// copies instead of 32, so that more streams are on the chip (see argus_aggregate_digest_slices). Whole rounds without a look at the end of the
+// slice, one flag for a region that does not exist, and 16 copies instead of 32 in the large blocks: half of the decode trace 487 -> 465,
+// attention 321 -> 311, GEMM 186 -> 182.
 template <u32 kThreads, u32 kCopies, u32 kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArgs a) {
   constexpr u32 kMinProbe = 4 * kThreads;    // shorter streams are gathered without copies
@@ -283,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
     __syncthreads();
   }
   for (u32 r = tid; r <= R; r += kThreads)
-    meta[r] = (tab_addr + r * (kDgWords * 4)) | (r < R && ((pairbits[r >> 5] >> (r & 31)) & 1u) ? kDgInPair : 0u);
+    meta[r] = (tab_addr + r * (kDgWords * 4)) | (r == R ? kDgNoRegion : (pairbits[r >> 5] >> (r & 31)) & 1u ? kDgInPair : 0u);
   if (has_ov && tid == 0) {
     const u32 m = a.cta_sm[s / a.warps_per_cta];
     if (m >= a.num_sms) bad_sm(a, s / a.warps_per_cta);
@@ -329,14 +333,10 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
   bool late = false;  // the lane's candidate of the round before: its begin time may still be on its way
   u64 late_t0 = 0;
   u64* late_start = nullptr;
-#pragma unroll 2
-  for (u32 b = i0; b < i1; b += 32, i += 32) {
-    const u64 dg = dg_next;
-    dg_next = dg_next2;
-    dg_next2 = i + 64 < i1 ? dgs[i + 64] : kDgPad;
+  auto round = [&](u64 dg, auto FULL) {
     const u32 dlo = (u32)dg, dhi = (u32)(dg >> 32);
     const u32 region = dlo & 0xffffu;
-    const u32 m = meta[region < R ? region : R];
+    const u32 m = meta[min(region, R)];
     const u32 incl = __funnelshift_r(dlo, dhi, 18) & ((1u << kDigestBits) - 1), excl = dhi >> (32 - kDigestBits);
     const u32 normal = (m & kDgAddr) + (m >> 31) * own_copy;
     const u32 cell = dlo & kDigestWide ? tab_addr + R * (kDgWords * 4) : normal;
@@ -347,9 +347,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
     dg_inc<kDgBins>(cell + (31u - (u32)__clz((int)(incl | 1u))) * 4, 1u);
     bool cand = (m & kDgInPair) && incl;
     // whatever is rare (a carry, a flag, a wide digest, no such region) is settled in one place
-    if (old_i > ~incl || old_e > ~excl || (dlo & (kDigestFlag | kDigestWide)) || region >= R) {
-      if (region >= R) {
-        if (i < i1) argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, lo + i);
+    if (old_i > ~incl || old_e > ~excl || ((dlo & (kDigestFlag | kDigestWide)) | (m & kDgNoRegion))) {
+      if (m & kDgNoRegion) {
+        if (decltype(FULL)::value || i < i1) argus_set_error(a.status, ARGUS_ERR_BAD_REGION, s, lo + i);
       } else if (dlo & kDigestWide) {
         wide = true;
         cand = m & kDgInPair;  // (its inclusive duration is not 0: the exclusive one is never longer)
@@ -371,6 +371,21 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
       }
       out_count += __popc(bal);
     }
+  };
+  u32 b = i0;
+#pragma unroll 2
+  for (; b + 96 <= i1; b += 32, i += 32) {  // whole rounds, and those asked for as well
+    const u64 dg = dg_next;
+    dg_next = dg_next2;
+    dg_next2 = dgs[i + 64];
+    round(dg, std::true_type{});
+  }
+#pragma unroll 1
+  for (; b < i1; b += 32, i += 32) {
+    const u64 dg = dg_next;
+    dg_next = dg_next2;
+    dg_next2 = i + 64 < i1 ? dgs[i + 64] : kDgPad;
+    round(dg, std::false_type{});
   }
   if (late) late_start[0] = late_t0;
   if (has_ov && lane == 0) {
@@ -973,9 +988,9 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   if (num_regions <= kAggCompactRegions) {
     if (a.digest) {
       const u32 warps = a.slices / a.parts;
-      const u32 copies = warps == 16 ? 32 : 8;
+      const u32 copies = warps == 16 ? 16 : 8;
       const size_t dg = digest_table_bytes(num_regions, copies);
-      const auto kernel = warps == 16 ? k_agg_streams_digest<512, 32, 3> : warps == 8 ? k_agg_streams_digest<256, 8, 6> : k_agg_streams_digest<128, 8, 12>;
+      const auto kernel = warps == 16 ? k_agg_streams_digest<512, 16, 3> : warps == 8 ? k_agg_streams_digest<256, 8, 6> : k_agg_streams_digest<128, 8, 12>;
       if (dg > 48 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, digest_table_bytes(kAggCompactRegions, copies)));
       ARGUS_LAUNCH(kernel, num_streams * a.parts, warps * 32, dg, stream, a);
     } else {

@@ -22,9 +22,8 @@ constexpr int kScanThreads = 1024;
 // Streams a thread of the one-block scans over all streams takes at a time: four where there are many (10^6 streams: 1,690 -> 1,325 us
 // and 1,640 -> 860), one where a block holds them all (16 streams: a call of 45 us is 1 to 2 us longer with four).
 constexpr u32 kScanRun = 4;
-constexpr u32 kGroupWords = 8;                             // bitmap words of a prefix: 256 events, a sector
-constexpr u32 kThreadWords = 4 * kGroupWords;               // a thread's share
-constexpr u32 kWordsPerBlock = kScanThreads * kThreadWords;  // and of a prefix block
+constexpr u32 kGroupWords = 8;                              // bitmap words of a prefix: 256 events, a sector, a thread's share
+constexpr u32 kWordsPerBlock = kScanThreads * kGroupWords;  // and of a prefix block
 std::atomic<u32> g_poll_limit{1u << 19};  // see argus_testing_set_poll_limit
 
 // ---------------------------------------------------------------------------------------------
@@ -590,18 +589,15 @@ __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   __shared__ u64 sh64[33];
   __shared__ u32 last;
   for (u64 blk = blockIdx.x - 1; blk < g.num_blocks; blk += gridDim.x - 1) {
-    const u64 w = blk * kWordsPerBlock + threadIdx.x * kThreadWords;
-    u32 c[4] = {0, 0, 0, 0};
-    if (w < g.num_words) {  // (the last thread's share is filled up with words that are zero)
-#pragma unroll
-      for (u32 j = 0; j < kThreadWords / 4; ++j) {
-        const uint4 b = reinterpret_cast<const uint4*>(g.p.bits + w)[j];
-        c[j / (kGroupWords / 4)] += __popc(b.x) + __popc(b.y) + __popc(b.z) + __popc(b.w);
-      }
+    const u64 w = blk * kWordsPerBlock + threadIdx.x * kGroupWords;
+    u32 c = 0;
+    if (w < g.num_words) {  // (the last group is filled up with words that are zero)
+      const uint4 x = *reinterpret_cast<const uint4*>(g.p.bits + w), y = *reinterpret_cast<const uint4*>(g.p.bits + w + 4);
+      c = __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w) + __popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w);
     }
     u32 total;
-    const u32 ex = argus_block_exclusive_scan<u32>(c[0] + c[1] + c[2] + c[3], sh, &total);
-    if (w < g.num_words) *reinterpret_cast<uint4*>(g.group_prefix + w / kGroupWords) = make_uint4(ex, ex + c[0], ex + c[0] + c[1], ex + c[0] + c[1] + c[2]);
+    const u32 ex = argus_block_exclusive_scan<u32>(c, sh, &total);
+    if (w < g.num_words) g.group_prefix[w / kGroupWords] = ex;
     if (threadIdx.x == 0) g.block_prefix[blk] = total;
     __syncthreads();
   }
@@ -704,9 +700,9 @@ Layout make_layout(uint64_t num_events, uint32_t num_streams, uint64_t ambig_cap
   const u64 records = num_events > 1u << 20 ? L.queue_capacity : num_events / 32768 + 1;
   L.record_capacity = (u32)(records < num_streams ? records : num_streams);
   L.queue = o; o += argus_align_up((size_t)L.queue_capacity * 4, 256);
-  L.bits = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);  // (whole threads' shares)
-  static_assert(256 % (kThreadWords * 4) == 0, "whole threads' shares");
-  L.group_prefix = o; o += argus_align_up((size_t)(L.num_words + kThreadWords - 1) / kThreadWords * 16 + 4, 256);
+  L.bits = o; o += argus_align_up((size_t)L.num_words * 4 + 4, 256);  // (whole groups)
+  static_assert(256 % (kGroupWords * 4) == 0, "whole groups");
+  L.group_prefix = o; o += argus_align_up((size_t)(L.num_words + kGroupWords - 1) / kGroupWords * 4 + 4, 256);
   L.block_prefix = o; o += argus_align_up(((size_t)L.num_blocks + 1) * 8, 256);
   L.notes = o; o += argus_align_up((size_t)ambig_capacity * 8 + 8, 256);
   L.records = o; o += argus_align_up((size_t)L.record_capacity * sizeof(ArgusStreamRecord), 256);

@@ -14,7 +14,7 @@ extern "C" {
 
 /* argus_pair_intervals (Section 3.2, the nested region context stack per warp) with an explicit
  * kernel choice: 0 = automatic, 1 = one thread per stream (sequential stack, any input),
- * 2 = tiled kernel (CTAs walk streams tile by tile, long streams a chunk at a time, and hand
+ * 2 = tiled kernel (CTAs walk streams tile by tile, may hand a stream on to one another, and hand
  * the markers that break the nesting to the sequential stack). Arguments, ownership and errors
  * as argus_pair_intervals; all choices produce identical output. */
 int argus_pair_intervals_ex(const argus_event_t* events /*device*/, uint64_t num_events,

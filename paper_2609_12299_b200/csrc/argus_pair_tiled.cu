@@ -31,7 +31,8 @@
 // selects (decode trace, 614 M events: 5.42 -> 5.01 ms); then heights by vote over 32 markers in a row instead of a scan over the
 // threads' own five, and a word of a level's bitmap stored at once, by the lowest lane of those that match in level, instead of
 // a bit at a time (4.90 ms = 5.0 TB/s of 16 B read + 24 B written an event, 77 % of the copy rate, 5.5 TB/s with the digests;
-// attention 1.50 -> 1.45 ms; with votes but a bit at a time 5.08 and 1.57). Tiles of 512 events with 8 blocks: GEMM 638 -> 707
+// attention 1.50 -> 1.45 ms; with votes but a bit at a time 5.08 and 1.57); then records in whole sectors (tile_store_record) and streams that
+// change hands where that keeps the SMs busy (ArgusStreamRecord): decode 4.61 ms, attention 1.18, GEMM 0.54. Tiles of 512 events with 8 blocks: GEMM 638 -> 707
 // us, 160 threads with four events each and 6 blocks: 674.
 #include "argus_internal.cuh"
 #include "argus_bulk.cuh"

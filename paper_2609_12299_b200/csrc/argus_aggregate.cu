@@ -247,6 +247,57 @@ __device__ __noinline__ void digest_wide(u64* row, u32 R, uint4 q0, uint4 q1, u3
   atomicAdd(c + 8 + log2_bin(span), 1ull);
 }
 
+// The regions' cells of a stream into its row, 16 bytes at a time where one block has gathered it (`alone`; else the rows have been
+// initialised and several blocks add): a warp takes a region's bins, of which the upper ones are empty, a lane two of them, and then eight
+// regions' other fields. (A word at a time, a field for a thread, took 24 warp instructions for 32 words; 36 lanes' worth of a
+// region in a row, bins and fields in one warp, more: 71 M digests, 2,368 rows of 202 regions 260 us, 281 and 250 so.)
+template <u32 kWords, u32 kBins, u32 kThreads>
+__device__ __forceinline__ void row_out(const u32* tab, u64* row, u32 R, bool alone) {
+  static_assert(kCell == 72 && kBins <= 32, "eight fields, then 32 pairs of bins");
+  const u32 lane = threadIdx.x & 31;
+  const bool vectors = alone && !(reinterpret_cast<uintptr_t>(row) & 15);
+  for (u32 r = threadIdx.x / 32; r < R; r += kThreads / 32) {
+    const u32* const c = tab + r * kWords + kDgBins + 2 * lane;
+    const u64 x = 2 * lane < kBins ? c[0] : 0u, y = 2 * lane + 1 < kBins ? c[1] : 0u;
+    u64* const p = row + (size_t)r * kCell + 8 + 2 * lane;
+    if (vectors) {
+      *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(x, y);
+    } else if (alone) {
+      p[0] = x; p[1] = y;
+    } else {
+      if (x) atomicAdd(p, x);
+      if (y) atomicAdd(p + 1, y);
+    }
+  }
+  for (u32 k = threadIdx.x; k < 4 * R; k += kThreads) {
+    const u32 v = k & 3;
+    const u32* const c = tab + (k >> 2) * kWords;
+    u64 x = 0, y = 0;
+    if (v == 0) {
+#pragma unroll
+      for (u32 j = 0; j < kBins; ++j) x += c[kDgBins + j];
+    }
+    if (v == 1) { const u32 least = c[kDgNotMin]; x = least ? (u64)(u32)~least : ~0ull; y = c[kDgMax]; }
+    if ((v & 1) == 0) {
+      const u32 at = v ? kDgSumExclLo : kDgSumInclLo;
+      (v ? x : y) = (u64)c[at] | ((u64)c[at + 1] << 32);
+    }
+    if (v == 3) y = c[kDgFlag];  // (ambiguity records are added later)
+    u64* const p = row + (size_t)(k >> 2) * kCell + 2 * v;
+    if (vectors) {
+      *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(x, y);
+    } else if (alone) {
+      p[0] = x; p[1] = y;
+    } else if (v == 1) {
+      if (x != ~0ull) atomicMin(p, x);
+      if (y) atomicMax(p + 1, y);
+    } else {
+      if (x) atomicAdd(p, x);
+      if (y) atomicAdd(p + 1, y);
+    }
+  }
+}
+
 // Bound by instruction issue and the atomics' way through the load/store pipe. Bins that need no window, a trash cell instead of
 // selects, a row written once instead of emptied, added to and read back, and a loop of two rounds (the digests asked for
 // ahead change places without moves): decode trace (307 M intervals) 1,215 -> 903 us = 2.7 TB/s of digests, attention 400 -> 323,
@@ -413,38 +464,8 @@ __global__ void __launch_bounds__(kThreads, kBlocks) k_agg_streams_digest(AggArg
     }
   }
   __syncthreads();
-  for (u32 r = tid; r < R; r += kThreads) {
-    u32* c = tab + r * kDgWords;
-    u32 cnt = 0;
-#pragma unroll
-    for (u32 j = 0; j < kDigestBits; ++j) cnt += c[kDgBins + j];
-    c[kDgCount] = cnt;
-  }
-  __syncthreads();
-  // the regions' cells into the global row; a thread keeps to one field
-  const bool alone = a.parts == 1;  // (else the rows have been initialised: several blocks add to one)
-  auto put = [&](u64* p, u32 field, u64 v) {
-    if (alone) *p = v;
-    else if (field == 2) { if (v != ~0ull) atomicMin(p, v); }
-    else if (field == 3) { if (v) atomicMax(p, v); }
-    else if (v) atomicAdd(p, v);
-  };
-  {
-    const u32 f = tid % 64;
-    for (u32 r = tid / 64; r < R; r += kThreads / 64) put(row + (size_t)r * kCell + 8 + f, 8 + f, f < kDigestBits ? tab[r * kDgWords + kDgBins + f] : 0u);
-  }
-  {
-    const u32 f = tid % 8;
-    const u32 w = f == 0 ? kDgCount : f == 1 ? kDgSumInclLo : f == 2 ? kDgNotMin : f == 3 ? kDgMax : f == 4 ? kDgSumExclLo : kDgFlag;
-    for (u32 r = tid / 8; r < R; r += kThreads / 8) {
-      const u32* c = tab + r * kDgWords + w;
-      u64 v = c[0];
-      if (f == 1 || f == 4) v |= (u64)c[1] << 32;
-      if (f == 2) v = v ? (u64)(u32)~(u32)v : ~0ull;
-      if (f == 5 || f == 6) v = 0;  // ambiguity records: below
-      put(row + (size_t)r * kCell + f, f, v);
-    }
-  }
+  // the regions' cells into the global row
+  row_out<kDgWords, kDigestBits, kThreads>(tab, row, R, a.parts == 1);
   u64 alo = 0, ahi = 0;
   if (a.ambig && a.ambig_offsets && part == 0) { alo = a.ambig_offsets[s]; ahi = a.ambig_offsets[s + 1]; }
   wide = __any_sync(0xffffffffu, wide);
@@ -709,36 +730,8 @@ __global__ void __launch_bounds__(kThreads) k_agg_streams_records(AggArgs a) {
     }
   }
   __syncthreads();
-  // the regions' cells into the global row; a thread keeps to one field
-  const bool alone = a.parts == 1;  // (else the rows have been initialised: several blocks add to one)
-  auto put = [&](u64* p, u32 field, u64 v) {
-    if (alone) *p = v;
-    else if (field == 2) { if (v != ~0ull) atomicMin(p, v); }
-    else if (field == 3) { if (v) atomicMax(p, v); }
-    else if (v) atomicAdd(p, v);
-  };
-  {
-    const u32 f = tid % 64;
-    for (u32 r = tid / 64; r < R; r += kThreads / 64) put(row + (size_t)r * kCell + 8 + f, 8 + f, f < 32 ? tab[r * kItWords + kDgBins + f] : 0u);
-  }
-  {
-    const u32 f = tid % 8;
-    const u32 w = f == 1 ? kDgSumInclLo : f == 2 ? kDgNotMin : f == 3 ? kDgMax : f == 4 ? kDgSumExclLo : kDgFlag;
-    for (u32 r = tid / 8; r < R; r += kThreads / 8) {
-      const u32* c = tab + r * kItWords;
-      u64 v = c[w];
-      if (f == 0) {
-        u32 cnt = 0;
-#pragma unroll
-        for (u32 j = 0; j < 32; ++j) cnt += c[kDgBins + j];
-        v = cnt;
-      }
-      if (f == 1 || f == 4) v |= (u64)c[w + 1] << 32;
-      if (f == 2) v = v ? (u64)(u32)~(u32)v : ~0ull;
-      if (f == 5 || f == 6) v = 0;  // ambiguity records: below
-      put(row + (size_t)r * kCell + f, f, v);
-    }
-  }
+  // the regions' cells into the global row
+  row_out<kItWords, 32, kThreads>(tab, row, R, a.parts == 1);
   u64 alo = 0, ahi = 0;
   if (a.ambig && a.ambig_offsets && part == 0) { alo = a.ambig_offsets[s]; ahi = a.ambig_offsets[s + 1]; }
   if (!__syncthreads_or(wide || alo < ahi)) return;

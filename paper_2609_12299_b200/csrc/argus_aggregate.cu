@@ -905,9 +905,10 @@ AggLayout agg_layout(uint32_t num_streams, uint32_t num_regions) {
 }
 
 // Threads of a block of the pass over the records. A block takes a stream, and how much of the chip the last round of blocks leaves idle
-// decides: blocks of 192 threads are taken where that makes a tenth of difference. us, 256 / 192 threads, share of the rounds that is
-// filled: 832 streams of 74 regions 454 / 346 (0.56, 0.94), 1,080 of 5 147 / 133 (0.52, 0.81), 960 of 9 117 / 119 (0.93, 0.72), 1,572 of 5 115 / 139
-// (0.76, 0.59), 2,368 of 146 623 / 645 (1, 0.8). 128 threads read the records slower: 34 M 387, 307 and 330 with more.
+// decides; smaller blocks read the records a little slower (at an equal share 192 threads by a thirteenth, 128 by a fifth). us, 256 / 192
+// threads, share of the rounds that is filled: 832 streams of 74 regions 454 / 346 (0.56, 0.94), 1,080 of 5 147 / 133 (0.52, 0.81), 960 of 9
+// 117 / 119 (0.93, 0.72), 1,572 of 5 115 / 139 (0.76, 0.59), 2,368 of 146 623 / 645 (1, 0.8); 736 of 148 492 with 128 threads
+// (0.99; 0.62 with 256, and 522 for the pass of the scoped calls).
 u32 record_threads(u32 num_regions, u32 blocks) {
   auto filled = [&](u32 threads) {
     const size_t of_sm = 228 * 1024 / (record_table_bytes(num_regions, threads) + 1536);  // (1 KB of the system's and the static part)
@@ -915,7 +916,8 @@ u32 record_threads(u32 num_regions, u32 blocks) {
     const u32 rounds = (blocks + slots - 1) / slots;
     return (double)blocks / ((double)slots * (rounds ? rounds : 1));
   };
-  return filled(192) > 1.1 * filled(256) ? 192 : 256;
+  const double of256 = filled(256), of192 = 0.92 * filled(192), of128 = 0.8 * filled(128);
+  return of256 >= of192 && of256 >= of128 ? 256 : of192 >= of128 ? 192 : 128;
 }
 
 }  // namespace
@@ -994,7 +996,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       } else {
         const u32 threads = record_threads(num_regions, num_streams * a.parts);
         const size_t bytes = record_table_bytes(num_regions, threads);
-        const auto kernel = threads == 256 ? k_agg_streams_records<256> : k_agg_streams_records<192>;
+        const auto kernel = threads == 256 ? k_agg_streams_records<256> : threads == 192 ? k_agg_streams_records<192> : k_agg_streams_records<128>;
         if (bytes > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, record_table_bytes(kAggCompactRegions, threads)));
         ARGUS_LAUNCH(kernel, num_streams * a.parts, threads, bytes, stream, a);
       }

@@ -1,4 +1,4 @@
-"""argus_aggregate's pass over the records: streams that end at, before and behind the edges of a tile of 256 or 192 records and of the four tiles from
+"""argus_aggregate's pass over the records: streams that end at, before and behind the edges of a tile of 256, 192 or 128 records and of the four tiles from
 which on frequent regions get copies of their cells, streams that several blocks share, durations around 2^32, one region and 400, and a record
 of a region that does not exist, against the oracle."""
 import numpy as np
@@ -10,15 +10,15 @@ import paper_2609_12299_b200 as argus
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
-EDGES = [0, 1, 191, 192, 193, 255, 256, 257, 385, 511, 512, 513, 767, 768, 769, 1023, 1024, 1025, 3000]
+EDGES = [0, 1, 127, 128, 129, 191, 192, 193, 255, 256, 257, 385, 511, 512, 513, 767, 768, 769, 1023, 1024, 1025, 3000]
 
 
 def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a).view(np.uint8).reshape(-1).copy()).to(DEV)
 
 
-@pytest.mark.parametrize("R", [1, 5, 65, 400])
-@pytest.mark.parametrize("S,W", [(12, 3), (24, 1), (900, 12), (1080, 12)])  # blocks share a stream: sixteen, sixteen, none, none (blocks of 192 threads)
+@pytest.mark.parametrize("R", [1, 5, 65, 148, 400])
+@pytest.mark.parametrize("S,W", [(12, 3), (24, 1), (900, 12), (1080, 12), (736, 16)])  # sixteen blocks a stream, sixteen, one (of 256, 192 and 128 threads, by R)
 def test_tables(S, W, R):
     rng = np.random.default_rng(S + R)
     lengths = np.array([EDGES[s % len(EDGES)] for s in range(S)])

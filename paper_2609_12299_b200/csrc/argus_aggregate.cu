@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(kThreads) k_agg_streams_records(AggArgs a) {
   agg_empty_tables(a);
   __syncthreads();
   const u32 own_copy = lane % kRecCopies * (kItWords * 4);
-  bool wide = false, arrived = true;  // the lane met a wide interval; every copy has arrived
+  bool wide = false, arrived = true, lost = false;  // the lane met a wide interval; the copy has arrived; one has not
   u32 stage = 0, parity = 0;
   for (u64 at = lo; at < hi; at += kThreads) {
     arrived = mbar_wait_bounded(&full[stage], parity);
@@ -706,11 +706,16 @@ __global__ void __launch_bounds__(kThreads) k_agg_streams_records(AggArgs a) {
         iter_add((m & ~kDgHot) + (m >> 31) * own_copy, incl.x, excl.x, p[11] >> 16);
       }
     }
-    __syncthreads();  // everybody has read the stage
+    lost = __syncthreads_or(!arrived);  // everybody has read the stage
+    if (lost) break;
     if (tid == 0 && at + kRecStages * kThreads < hi) fetch(at + kRecStages * kThreads, stage);
     if (++stage == kRecStages) { stage = 0; parity ^= 1; }
   }
-  if (__syncthreads_or(!arrived) && tid == 0) argus_set_error(a.status, ARGUS_ERR_TIMEOUT, s, 0);
+  if (lost) {  // a copy never arrived: reported, and what else is on its way is waited for (again with a limit)
+    if (tid == 0) argus_set_error(a.status, ARGUS_ERR_TIMEOUT, s, 0);
+    for (u32 k = 0; k < kRecStages; ++k) mbar_wait_bounded(&full[k], k >= stage ? parity : parity ^ 1u);
+    __syncthreads();
+  }
   // the copies into their region's cell (which nobody added to): a thread per (hot region, field)
   for (u32 hf = tid; num_often && hf < kDigestHot * kItWords; hf += kThreads) {
     const u32 h = hf / kItWords, f = hf % kItWords, r = hot_region[h];

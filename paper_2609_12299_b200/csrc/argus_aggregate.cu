@@ -991,7 +991,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       const u32 copies = warps == 16 ? 16 : 8;
       const size_t dg = digest_table_bytes(num_regions, copies);
       const auto kernel = warps == 16 ? k_agg_streams_digest<512, 16, 3> : warps == 8 ? k_agg_streams_digest<256, 8, 6> : k_agg_streams_digest<128, 8, 12>;
-      if (dg > 48 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, digest_table_bytes(kAggCompactRegions, copies)));
+      ARGUS_CUDA_TRY(argus_allow_smem(kernel, dg, digest_table_bytes(kAggCompactRegions, copies)));
       ARGUS_LAUNCH(kernel, num_streams * a.parts, warps * 32, dg, stream, a);
     } else {
       const size_t compact = (size_t)num_regions * sizeof(ArgusAggCell);
@@ -1002,7 +1002,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
         const u32 threads = record_threads(num_regions, num_streams * a.parts);
         const size_t bytes = record_table_bytes(num_regions, threads);
         const auto kernel = threads == 256 ? k_agg_streams_records<256> : threads == 192 ? k_agg_streams_records<192> : k_agg_streams_records<128>;
-        if (bytes > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(kernel, record_table_bytes(kAggCompactRegions, threads)));
+        ARGUS_CUDA_TRY(argus_allow_smem(kernel, bytes, record_table_bytes(kAggCompactRegions, threads)));
         ARGUS_LAUNCH(kernel, num_streams * a.parts, threads, bytes, stream, a);
       }
     }
@@ -1013,7 +1013,7 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
   if (iter_tab && windows) {
     u32 per = kIterWarps;  // streams of a block: at least two blocks for every SM where the streams allow it
     while (per > 1 && num_streams / per < 296) per >>= 1;
-    if (iter_bytes(num_regions) > 47 * 1024) ARGUS_CUDA_TRY(argus_allow_smem(k_agg_iter_windows, iter_bytes(kAggCompactRegions)));
+    ARGUS_CUDA_TRY(argus_allow_smem(k_agg_iter_windows, iter_bytes(num_regions), iter_bytes(kAggCompactRegions)));
     ARGUS_LAUNCH(k_agg_iter_windows, (num_streams + per - 1) / per, kIterThreads, iter_bytes(num_regions), stream, a, per);
   } else if (iter_tab) {
     ARGUS_LAUNCH(k_agg_iter, num_streams < 1184u ? num_streams : 1184u, kAggThreads, 0, stream, a);

@@ -187,8 +187,7 @@ extern "C" int argus_attribute(const uint64_t* counts, uint32_t num_rows, uint32
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   double* partial = (double*)workspace;
   const size_t smem = num_rows <= kAttrRows ? (size_t)num_rows * 32 * 8 : 0;
-  if (smem > 48 * 1024)
-    ARGUS_CUDA_TRY(argus_allow_smem(k_attr_tile, (size_t)kAttrRows * 32 * 8));
+  ARGUS_CUDA_TRY(argus_allow_smem(k_attr_tile, smem, (size_t)kAttrRows * 32 * 8));
   ARGUS_LAUNCH(k_attr_tile, L.blocks, kAttrThreads, smem, stream, (const u64*)counts, num_rows, num_pcs, metric, entropy, alpha, L.blocks,
                partial);
   ARGUS_LAUNCH(k_attr_finish, num_rows, kAttrThreads, 0, stream, (const double*)partial, L.blocks, mhat);

@@ -50,10 +50,13 @@ inline cudaError_t argus_launch(void (*kernel)(P...), dim3 grid, dim3 block, siz
 }
 #define ARGUS_LAUNCH(...) ARGUS_CUDA_TRY(argus_launch(__VA_ARGS__))
 
-// Shared memory of 48 KB and more has to be asked for, and the limit belongs to the kernel and the device, not to a launch: it is
+// A kernel gets 48 KB of shared memory without asking, its static arrays included (4 KB at most where the size of the dynamic part
+// depends on the call). More has to be asked for, and the limit belongs to the kernel and the device, not to a launch: it is
 // always set to the same, the most that any call needs, since another host thread may launch the kernel at the same time.
+constexpr size_t kPlainDynamicSmem = 43 * 1024;
 template <class K>
-inline cudaError_t argus_allow_smem(K* kernel, size_t most) {
+inline cudaError_t argus_allow_smem(K* kernel, size_t dynamic, size_t most) {
+  if (dynamic <= kPlainDynamicSmem) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 

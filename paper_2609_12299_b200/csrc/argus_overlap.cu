@@ -752,7 +752,7 @@ int launch_pair_as(const OvPairArgs& a, cudaStream_t stream) {
   ARGUS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return ARGUS_ERR_INVALID_ARG;
   if (!opted_in[dev].load(std::memory_order_acquire)) {
-    ARGUS_CUDA_TRY(argus_allow_smem(k_ov_pair<DIGEST, NT, kGather>, kPairSmem));
+    ARGUS_CUDA_TRY(argus_allow_smem(k_ov_pair<DIGEST, NT, kGather>, kPairSmem, kPairSmem));
     opted_in[dev].store(true, std::memory_order_release);
   }
   argus_prof_mark(ARGUS_PROF_OVERLAP, stream, 0);

@@ -46,11 +46,15 @@ int argus_profile_read(double* ms_total /*host [4]*/, unsigned long long* launch
  * hand-over gives up with ARGUS_ERR_TIMEOUT (default 2^19, about a second; 0 restores the default). A test
  * sets it to a few polls to see the bounded wait run out and the call return with the status set.
  * argus_testing_pair_passes: after a pairing call (or argus_synthesize) in this workspace is complete, whether the
- * trace's markers were counted before pairing and whether its second pass rewrote intervals. Waits for the device. */
+ * trace's markers were counted before pairing and whether its second pass rewrote intervals. Waits for the device.
+ * argus_testing_hold_sms: a kernel on the stream that holds this many SMs (148 at most; 200 KB of shared memory each, so that no block of the
+ * pairing kernel fits beside it) for this many microseconds (a second at most), and then ends by itself: what another stream's long
+ * kernel does to a call. */
 void argus_set_synthesize_mode(int mode);
 void argus_set_tile_variant(int variant);
 void argus_testing_set_poll_limit(unsigned int polls);
 int argus_testing_pair_passes(const void* workspace /*device*/, uint32_t* counted /*host*/, uint32_t* second_pass /*host*/);
+int argus_testing_hold_sms(unsigned int sms, unsigned int microseconds, void* cuda_stream);
 
 #ifdef __cplusplus
 }

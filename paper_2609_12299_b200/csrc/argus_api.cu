@@ -18,7 +18,27 @@ __global__ void __launch_bounds__(256) k_clear(argus_status_t* status, u64* extr
   if (status && threadIdx.x < sizeof(argus_status_t) / 8) reinterpret_cast<u64*>(status)[threadIdx.x] = 0;
   for (u32 i = threadIdx.x; i < words; i += blockDim.x) extra[i] = 0;
 }
+
+// Holds an SM's shared memory until the time is up (or, whatever the clock does, after as many naps of a us).
+constexpr size_t kHoldSmem = 200 * 1024;
+__global__ void __launch_bounds__(32) k_hold(u32 microseconds) {
+  u64 start, now;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(start));
+  for (u32 i = 0; i < microseconds; ++i) {
+    __nanosleep(1000);
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+    if (now - start >= (u64)microseconds * 1000) return;
+  }
+}
 }  // namespace
+
+extern "C" int argus_testing_hold_sms(unsigned int sms, unsigned int microseconds, void* cuda_stream) {
+  if (sms == 0 || sms > 148 || microseconds > 1000000) return ARGUS_ERR_INVALID_ARG;
+  ARGUS_CUDA_TRY(argus_allow_smem(k_hold, kHoldSmem, kHoldSmem));
+  k_hold<<<sms, 32, kHoldSmem, (cudaStream_t)cuda_stream>>>(microseconds);
+  ARGUS_CUDA_TRY(cudaGetLastError());
+  return ARGUS_OK;
+}
 
 int argus_internal_clear(argus_status_t* status, void* extra, size_t bytes, void* cuda_stream) {
   ARGUS_LAUNCH(k_clear, 1, 256, 0, (cudaStream_t)cuda_stream, status, (u64*)extra, extra ? (u32)(bytes / 8) : 0u);

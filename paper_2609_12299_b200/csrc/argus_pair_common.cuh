@@ -26,6 +26,7 @@ struct ArgusFrame {  // one open region occurrence, 32 bytes
 // an atomic, too, and lies on a line with nothing that is read in any other way: loads of a line that changes all the time held
 // up everything else that half of the SMs asked the L2 for (2,368 streams of 16,208 events, blocks that load `level` every 3,840: 69 SMs walked
 // 340 tiles each, the others 485, in 435 us; with atomics 416 each, in 340).
+constexpr u32 kMostCtas = 2048;  // of the tiled kernel
 struct ArgusPairCtl {
   // written by one kernel, read by the next
   u32 redo;            // 1 = provisional interval bases were wrong; second pass needed
@@ -40,16 +41,19 @@ struct ArgusPairCtl {
   alignas(128) u64 n_notes;  // ambiguity notes appended (may exceed the list capacity)
   // work queue of the tiled kernel, one set per pass (0 = first, 1 = redo): positions below num_streams are the
   // streams themselves, later positions are streams handed on after a chunk (see ArgusStreamRecord)
-  u64 q_head[2];       // positions taken
+  u64 q_head[2];       // positions taken behind those that CTAs start with
   u64 q_tail[2];       // hand-overs published (queue entries written)
   u64 progress[2];     // low half: streams walked to their end (or given up on); high half: moves as long as streams are walked
   u32 level[2];        // events left of the stream that was taken last, 0 if nothing else waits
   u32 seg_head;        // segments taken (split pass)
+  u32 claimed_words[2];  // words of `claimed` of which every position has been claimed
   // read by all blocks, changed when something is given up
   alignas(128) u32 num_failed;  // streams that the split pass has to leave to the chained one (read together with the next two)
   u32 num_segments;    // 0 where the segments do not fit their room, too
   u32 split;           // the split pass is worth it (argus_split_pays), and no long stream has been given up
   u32 pad;
+  // atomics only: positions that CTAs start with, a bit each, a sector for a word (all CTAs claim at once)
+  alignas(128) u32 claimed[2][kMostCtas / 32][8];
 };
 
 // A stream is a chain of tiles that one CTA at a time walks, and streams rarely share out evenly among the CTAs that the chip holds.
@@ -62,9 +66,9 @@ struct ArgusPairCtl {
 // long streams wait behind short ones, and left half of the CTAs idle for the last eighth of the time: GEMM trace (68.7 M events in streams
 // of 72,000 and 32,000) 622 -> 571 us, attention (153.5 M in 112,684, 67,628 and 176) 1,412 -> 1,246, 131 x 12 streams (27,972 and
 // 12,432) 244 -> 203, equal streams (2,368 of 129,664) 2,421 -> 2,442; looked up by three quarters instead of a half 576, 1,256 and 2,468.
-// Queue positions are taken with one atomic add each. A CTA whose position has no entry yet is idle anyway
-// (every unfinished stream is in some CTA's hands): it polls until the entry appears or every stream is
-// done, and gives up with ARGUS_ERR_TIMEOUT if nothing moves for about a second.
+// Positions are only ever taken by CTAs that run (tile_pop_work): other kernels may hold part of the chip, and nothing may wait for a CTA that
+// has not started. So a CTA whose position has no entry yet is idle anyway (every unfinished stream is in a running CTA's hands):
+// it polls until the entry appears or every stream is done, and gives up with ARGUS_ERR_TIMEOUT if nothing moves for about a second.
 constexpr u32 kChunkEvents = 3840;   // walked by a CTA at least before it hands a stream on
 constexpr u32 kLevelMargin = 1280;   // by which the stream has to have less left than half
 constexpr u32 kLeastTiles = 3;       // and what is less than this is walked at once

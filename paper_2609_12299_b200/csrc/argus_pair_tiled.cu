@@ -50,24 +50,63 @@ constexpr int kSink = 64;         // index of the sink slot inside a carried-fra
 constexpr int kBadRef = 0x3fff;   // reference that marks a window as not well nested
 constexpr int kSeqChunk = 128;    // markers handed to the sequential machine at once when cuts come densely
 constexpr u32 kNoRec = 0xffffffffu;
+constexpr u64 kNoWork = ~0ull;
 
 __device__ __forceinline__ void tile_progress(const ArgusPairArgs& a, u64 by) {
   atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->progress[a.redo ? 1 : 0]), by);
+}
+
+// Claims a first position; false if another CTA has. The CTA that claims the last of a word's positions counts the word.
+__device__ __forceinline__ bool tile_claim(ArgusPairCtl* ctl, int p, u32 at) {
+  const u32 bit = 1u << (at & 31), word = at / 32, all = gridDim.x - word * 32 < 32 ? (1u << (gridDim.x & 31)) - 1u : ~0u;
+  const u32 before = atomicOr(ctl->claimed[p][word], bit);
+  if (before & bit) return false;
+  if ((before | bit) == all) atomicAdd(&ctl->claimed_words[p], 1u);
+  return true;
+}
+
+// A first position that no CTA has claimed; kNoRec if there is none.
+__device__ __forceinline__ u32 tile_claim_any(ArgusPairCtl* ctl, int p) {
+#pragma unroll 1
+  for (u32 at = 0; at < gridDim.x; ++at) {
+    const u32 open = ~__ldcg(ctl->claimed[p][at / 32]) >> (at & 31);
+    if (!open) { at |= 31; continue; }
+    at += __ffs((int)open) - 1;
+    if (at < gridDim.x && tile_claim(ctl, p, at)) return at;
+  }
+  return kNoRec;
 }
 
 // Takes the next piece of work of pass `p`: a stream nobody has started (position below num_streams) or a
 // hand-over from the queue. Returns false when every stream is done (or on a timeout). *rec: the stream's hand-over record (kNoRec: it
 // has none), *resumed: what to start from is in there, *more: others wait. A CTA's first position is its own number, so that every SM
 // gets its share of the long streams, which come first (the CTAs of an SM ask at the same time: with 296 long streams among
-// 1,776, 42 SMs had seven of them each, the others none, and walked 791 tiles instead of 700). One thread per CTA.
-__device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, bool first, u64* stream, u32* rec, bool* resumed, bool* more) {
-  const u64 h = first ? blockIdx.x : gridDim.x + atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_head[p]), 1ull);
+// 1,776 taken as they come, 42 SMs had seven of them each, the others none, and walked 791 tiles instead of 700: GEMM trace 545 -> 633 us; the
+// first positions taken seven strata apart, whoever comes: 633, too). But a CTA may start late, when another kernel holds part of the
+// chip, and nothing may wait for one that has not started: so the first position is claimed by a bit, and a CTA that would wait for
+// a hand-over while not all are claimed takes one that is left instead. *drawn: a position that the CTA has, but has not used yet.
+// One thread per CTA.
+__device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64* drawn, u64* stream, u32* rec, bool* resumed, bool* more) {
+  u64 h = *drawn;
+  if (h == kNoWork) h = gridDim.x + atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_head[p]), 1ull);
+  *drawn = kNoWork;
   *resumed = h >= a.num_streams;
   if (h < a.num_streams) {
     *stream = a.order ? a.order[h] : h;
     *rec = h < a.record_capacity ? (u32)h : kNoRec;  // (streams come longest first; those without a record are walked whole)
     *more = h + 1 < a.num_streams || atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull);
     return true;
+  }
+  if (atomicAdd(&a.ctl->claimed_words[p], 0u) < (gridDim.x + 31) / 32) {
+    const u32 left = tile_claim_any(a.ctl, p);
+    if (left != kNoRec) {
+      *drawn = h;
+      *resumed = false;
+      *stream = a.order ? a.order[left] : left;
+      *rec = left < a.record_capacity ? left : kNoRec;
+      *more = true;
+      return true;
+    }
   }
   const u64 slot = h - a.num_streams;
   if (!a.queue || slot >= a.queue_capacity) return false;  // more positions than hand-overs can ever be published
@@ -135,6 +174,7 @@ struct TileSmem {
   int resumed;                     // its state is in the record
   int more, level;                 // others wait; and this CTA says how long they are
   int started;                     // this CTA has had work
+  u64 drawn;                       // a position that it has and has not used yet
   u32 ti_end, look;                // where this CTA stops; the tile at which thread 0 looks up what waits
   int stop;                        // split pass: everything is left to the chained pass
   u64 n_int;                       // written by the sequential redo path
@@ -224,6 +264,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   bool failed = false;
   const bool segments = !SPLIT && !a.redo && a.segments && argus_split_in_force(a, &failed);  // the chained pass after a split one
   if (segments && !failed) return;
+  if (!SPLIT && tid == 32) sm.drawn = tile_claim(a.ctl, a.redo ? 1 : 0, blockIdx.x) ? blockIdx.x : kNoWork;  // (beside what thread 0 does)
   if (tid == 0) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);
@@ -250,7 +291,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         rc = atomicAdd(&a.ctl->seg_head, 1u);
         st = w.z && rc < w.y ? a.segments[rc].stream : ~0ull;
         skip = w.x && st < a.num_streams && __ldcg(a.split_failed + st);
-      } else if (!tile_pop_work(a, a.redo ? 1 : 0, !sm.started, &st, &rc, &resumed, &more)) st = ~0ull;
+      } else if (!tile_pop_work(a, a.redo ? 1 : 0, &sm.drawn, &st, &rc, &resumed, &more)) st = ~0ull;
       sm.cur_stream = st;
       sm.cur_rec = rc;
       if (!SPLIT) {
@@ -747,7 +788,7 @@ int launch_tiled(const ArgusPairArgs& a, cudaStream_t stream) {
       ARGUS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair_tiled<NT, E, MINB, RING, SPLIT>, NT, smem));
       if (per_sm < 1) return ARGUS_ERR_CUDA;
       if (per_sm > MINB) per_sm = MINB;
-      grid_of[dev] = sms * per_sm;
+      grid_of[dev] = sms * per_sm < (int)kMostCtas ? sms * per_sm : (int)kMostCtas;
     }
     grid_cache = grid_of[dev];
   }

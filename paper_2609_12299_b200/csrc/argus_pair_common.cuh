@@ -129,7 +129,7 @@ struct ArgusPairArgs {
   ArgusSegment* segments;  // non-null: split pass; or, in the chained pass after it, what that left: only failed streams are walked
   u32* split_failed;       // [S]
   u32 segment_tiles;       // tiles of a segment
-  u32 poll_limit;          // polls without any hand-over anywhere after which an idle CTA gives up (about a second)
+  u32 poll_limit;          // polls without any movement (ArgusPairCtl::progress) after which an idle CTA gives up (about a second)
 };
 
 // argus_pair_split.cu

@@ -117,6 +117,7 @@ __device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64
   for (;;) {
     const u64 now = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->progress[p]), 0ull);
     if (now != seen) {
+      __threadfence();  // an entry that was stored before the counter moved is seen; it is not looked for again until the counter moves
       const u32 v = *q;
       if (v) {
         *q = 0;  // the second pass uses the same entries

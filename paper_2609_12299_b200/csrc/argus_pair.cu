@@ -578,7 +578,8 @@ template <u32 RUN>
 __global__ void __launch_bounds__(kScanThreads) k_pair_offsets(AmbigArgs g) {
   // The second pass comes next, and its blocks spread evenly only over SMs that are free when they come (96 streams with a lost end
   // each: 5,993 us when they came beside this kernel's blocks, 4,111 us after them). Not so where there are enough of them to fill the
-  // chip or few blocks here; and without notes it has nothing to do (coming early saves 0.5 us of the smallest call, 2 us of others).
+  // chip or few blocks here (up to 9.4 M events: 96 to 960 streams of 1.3, 4 and 8.5 M, whole malformed calls, early / late 450 / 450, 563 / 559
+  // and 531 / 530 us at worst); and without notes it has nothing to do (coming early saves 0.5 us of the smallest call, 2 us of others).
   const bool early = gridDim.x <= 37 || g.p.num_streams >= 1036;
   if (early) argus_launch_next();
   argus_kernel_begin_long();

@@ -17,6 +17,7 @@
 #include "argus_bulk.cuh"
 #include "argus_internal.cuh"
 
+#include <mutex>
 #include <type_traits>
 
 namespace {
@@ -909,23 +910,78 @@ AggLayout agg_layout(uint32_t num_streams, uint32_t num_regions) {
   return L;
 }
 
+auto record_kernel(u32 threads) { return threads == 256 ? k_agg_streams_records<256> : threads == 192 ? k_agg_streams_records<192> : k_agg_streams_records<128>; }
+
+// Blocks of the pass over the records that an SM holds: what registers and threads let fit and the kernel's static shared memory belong to the
+// device and are looked up once, under a lock (two host threads may make their first call at the same time).
+struct RecordFit { int sms, plain[3]; size_t sm_bytes, block_bytes[3]; };
+constexpr u32 kRecThreads[3] = {256, 192, 128};
+int record_fit(RecordFit* fit) {
+  constexpr int kMaxDevices = 64;
+  static RecordFit of[kMaxDevices];
+  static std::mutex mu;
+  int dev = 0;
+  ARGUS_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) return ARGUS_ERR_INVALID_ARG;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!of[dev].sms) {
+    RecordFit f;
+    int sm = 0, reserved = 0;
+    ARGUS_CUDA_TRY(cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    ARGUS_CUDA_TRY(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+    ARGUS_CUDA_TRY(cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev));
+    for (int k = 0; k < 3; ++k) {
+      cudaFuncAttributes attr;
+      ARGUS_CUDA_TRY(cudaFuncGetAttributes(&attr, record_kernel(kRecThreads[k])));
+      ARGUS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.plain[k], record_kernel(kRecThreads[k]), (int)kRecThreads[k], 0));
+      f.block_bytes[k] = attr.sharedSizeBytes + (size_t)reserved;
+    }
+    f.sm_bytes = (size_t)sm;
+    of[dev] = f;
+  }
+  *fit = of[dev];
+  return ARGUS_OK;
+}
+u32 record_blocks(const RecordFit& fit, int k, u32 num_regions) {
+  const size_t held = fit.sm_bytes / argus_align_up(record_table_bytes(num_regions, kRecThreads[k]) + fit.block_bytes[k], 128);
+  return held < (size_t)fit.plain[k] ? (u32)held : (u32)fit.plain[k];
+}
+
 // Threads of a block of the pass over the records. A block takes a stream, and how much of the chip the last round of blocks leaves idle
-// decides; smaller blocks read the records a little slower (at an equal share 192 threads by a thirteenth, 128 by a fifth). us, 256 / 192
-// threads, share of the rounds that is filled: 832 streams of 74 regions 454 / 346 (0.56, 0.94), 1,080 of 5 147 / 133 (0.52, 0.81), 960 of 9
-// 117 / 119 (0.93, 0.72), 1,572 of 5 115 / 139 (0.76, 0.59), 2,368 of 146 623 / 645 (1, 0.8); 736 of 148 492 with 128 threads
-// (0.99; 0.62 with 256, and 522 for the pass of the scoped calls).
-u32 record_threads(u32 num_regions, u32 blocks) {
-  auto filled = [&](u32 threads) {
-    const size_t of_sm = 228 * 1024 / (record_table_bytes(num_regions, threads) + 1536);  // (1 KB of the system's and the static part)
-    const u32 most = 65536 / (40 * threads), per_sm = of_sm < most ? (u32)of_sm : most, slots = 148 * (per_sm ? per_sm : 1);
-    const u32 rounds = (blocks + slots - 1) / slots;
-    return (double)blocks / ((double)slots * (rounds ? rounds : 1));
-  };
-  const double of256 = filled(256), of192 = 0.92 * filled(192), of128 = 0.8 * filled(128);
-  return of256 >= of192 && of256 >= of128 ? 256 : of192 >= of128 ? 192 : 128;
+// decides, weighed against smaller blocks' slower reads (1, 0.96 and 0.8). 20 M records, us with 256 / 192 / 128 threads and the share of
+// the rounds that is filled: 832 streams of 74 regions 194 / 157 / 164 (0.56, 0.94, 0.80), 960 of 5 181 / 146 / 154 (0.54, 0.72, 0.59), 960 of 74 182 / 200
+// / 161 (0.65, 0.54, 0.93), 1,572 of 5 149 / 200 / 159 (0.89, 0.59, 0.97), 2,368 of 146 194 / 202 / 233 (1, 1, 0.8), 736 of 146 199 / 220
+// / 172 (0.62, 0.62, 0.99). 1 and 20 M records in 24 to 4,736 streams of 5 to 400 regions (400 shapes): on average 1.2 % above the best of
+// the three; 256 threads throughout 3.4 %.
+u32 record_threads(const RecordFit& fit, u32 num_regions, u32 blocks) {
+  constexpr double weight[3] = {1.0, 0.96, 0.8};
+  double most = 0;
+  u32 threads = 0;
+  for (int k = 0; k < 3; ++k) {
+    const u32 slots = (u32)fit.sms * (record_blocks(fit, k, num_regions) ? record_blocks(fit, k, num_regions) : 1), rounds = (blocks + slots - 1) / slots;
+    const double share = weight[k] * blocks / ((double)slots * (rounds ? rounds : 1));
+    if (share > most || !threads) { most = share; threads = kRecThreads[k]; }
+  }
+  return threads;
 }
 
 }  // namespace
+
+extern "C" int argus_testing_record_blocks(uint32_t num_regions, uint32_t threads, uint32_t* by_rule, uint32_t* by_device) {
+  if (num_regions == 0 || num_regions > kAggCompactRegions) return ARGUS_ERR_INVALID_ARG;
+  int k = 0;
+  while (k < 3 && kRecThreads[k] != threads) ++k;
+  if (k == 3) return ARGUS_ERR_INVALID_ARG;
+  RecordFit fit;
+  { const int rc = record_fit(&fit); if (rc != ARGUS_OK) return rc; }
+  const size_t bytes = record_table_bytes(num_regions, threads);
+  ARGUS_CUDA_TRY(argus_allow_smem(record_kernel(threads), bytes, record_table_bytes(kAggCompactRegions, threads)));
+  int blocks = 0;
+  ARGUS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, record_kernel(threads), (int)threads, bytes));
+  *by_rule = record_blocks(fit, k, num_regions);
+  *by_device = (uint32_t)blocks;
+  return ARGUS_OK;
+}
 
 extern "C" size_t argus_aggregate_workspace_bytes(uint64_t /*num_intervals*/, uint32_t num_streams, uint32_t num_regions) {
   return agg_layout(num_streams, num_regions).total + 256;
@@ -999,9 +1055,11 @@ int argus_internal_aggregate_scoped(const argus_interval_t* intervals, const uin
       if (scope) {
         ARGUS_LAUNCH(k_agg_streams_compact, num_streams * a.parts, kAggThreads, compact, stream, a);
       } else {
-        const u32 threads = record_threads(num_regions, num_streams * a.parts);
+        RecordFit fit;
+        { const int rc = record_fit(&fit); if (rc != ARGUS_OK) return rc; }
+        const u32 threads = record_threads(fit, num_regions, num_streams * a.parts);
         const size_t bytes = record_table_bytes(num_regions, threads);
-        const auto kernel = threads == 256 ? k_agg_streams_records<256> : threads == 192 ? k_agg_streams_records<192> : k_agg_streams_records<128>;
+        const auto kernel = record_kernel(threads);
         ARGUS_CUDA_TRY(argus_allow_smem(kernel, bytes, record_table_bytes(kAggCompactRegions, threads)));
         ARGUS_LAUNCH(kernel, num_streams * a.parts, threads, bytes, stream, a);
       }

@@ -49,6 +49,10 @@ int argus_profile_read(double* ms_total /*host [4]*/, unsigned long long* launch
  * trace's markers were counted before pairing and whether its second pass rewrote intervals. Waits for the device.
  * argus_testing_record_blocks: blocks of this many threads (256, 192 or 128) of argus_aggregate's pass over the records that an SM holds
  * with this many regions (400 at most): as the library's choice between the three takes it, and as the device says.
+ * argus_testing_set_hand_overs: 1 = a block of the tiled pairing kernel hands its stream on whenever it looks whether to, whatever the others
+ * have left; 0 = the default. Results do not depend on it.
+ * argus_testing_hand_overs: after a pairing call (or argus_synthesize) in this workspace is complete, how many times its two
+ * passes handed a stream on. Waits for the device.
  * argus_testing_hold_sms: a kernel on the stream that holds this many SMs (148 at most; 200 KB of shared memory each, so that no block of the
  * pairing kernel fits beside it) for this many microseconds (a second at most), and then ends by itself: what another stream's long
  * kernel does to a call. */
@@ -57,6 +61,8 @@ void argus_set_tile_variant(int variant);
 void argus_testing_set_poll_limit(unsigned int polls);
 int argus_testing_pair_passes(const void* workspace /*device*/, uint32_t* counted /*host*/, uint32_t* second_pass /*host*/);
 int argus_testing_record_blocks(uint32_t num_regions, uint32_t threads, uint32_t* by_rule /*host*/, uint32_t* by_device /*host*/);
+void argus_testing_set_hand_overs(int always);
+int argus_testing_hand_overs(const void* workspace /*device*/, uint64_t* first_pass /*host*/, uint64_t* second_pass /*host*/);
 int argus_testing_hold_sms(unsigned int sms, unsigned int microseconds, void* cuda_stream);
 
 #ifdef __cplusplus

@@ -25,6 +25,7 @@ constexpr u32 kScanRun = 4;
 constexpr u32 kGroupWords = 8;                              // bitmap words of a prefix: 256 events, a sector, a thread's share
 constexpr u32 kWordsPerBlock = kScanThreads * kGroupWords;  // and of a prefix block
 std::atomic<u32> g_poll_limit{1u << 19};  // see argus_testing_set_poll_limit
+std::atomic<u32> g_hand_on{0};            // see argus_testing_set_hand_overs
 
 // ---------------------------------------------------------------------------------------------
 // Reference-order kernel: one thread walks one stream with its stack in local memory.
@@ -729,6 +730,14 @@ extern "C" int argus_testing_pair_passes(const void* workspace, uint32_t* counte
   *second_pass = ctl.redo != 0;
   return ARGUS_OK;
 }
+extern "C" void argus_testing_set_hand_overs(int always) { g_hand_on.store(always ? 1u : 0u); }
+extern "C" int argus_testing_hand_overs(const void* workspace, uint64_t* first_pass, uint64_t* second_pass) {
+  ArgusPairCtl ctl;
+  ARGUS_CUDA_TRY(cudaMemcpy(&ctl, workspace, sizeof(ctl), cudaMemcpyDeviceToHost));
+  *first_pass = ctl.q_tail[0];
+  *second_pass = ctl.q_tail[1];
+  return ARGUS_OK;
+}
 
 extern "C" size_t argus_pair_workspace_bytes(uint64_t num_events, uint32_t num_streams, uint64_t ambig_capacity) {
   return make_layout(num_events, num_streams, ambig_capacity).total;
@@ -768,6 +777,7 @@ int argus_internal_pair(const argus_event_t* events, uint64_t num_events, const 
   a.queue = (u32*)(ws + L.queue); a.queue_capacity = L.queue_capacity;
   a.records = (ArgusStreamRecord*)(ws + L.records); a.record_capacity = L.record_capacity;
   a.poll_limit = g_poll_limit.load(std::memory_order_relaxed);
+  a.hand_on = g_hand_on.load(std::memory_order_relaxed);
   a.ring_written = (const u64*)ring_written; a.ring_capacity = ring_capacity;
   if (ring_written && (ring_capacity == 0 || kernel_choice == 1)) return ARGUS_ERR_INVALID_ARG;  // only the tiled kernel reads rings
   // Digests lie at their records' positions, so the digest array bounds both. A trace has num_events / 2 intervals at most, which is

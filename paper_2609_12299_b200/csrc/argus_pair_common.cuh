@@ -130,6 +130,7 @@ struct ArgusPairArgs {
   u32* split_failed;       // [S]
   u32 segment_tiles;       // tiles of a segment
   u32 poll_limit;          // polls without any movement (ArgusPairCtl::progress) after which an idle CTA gives up (about a second)
+  u32 hand_on;             // hand on at every look (a test)
 };
 
 // argus_pair_split.cu

@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         if (!SPLIT && tid == 0) {
           if (ti == sm.look && ti + 2 + kLeastTiles <= ntiles) {  // (others read sm.ti_end after the tile's barriers)
             const u32 half = atomicOr(&a.ctl->level[a.redo ? 1 : 0], 0u) / 2;
-            if (half > kLevelMargin && n - (ti + 2) * (u32)T < half - kLevelMargin) sm.ti_end = ti + 2;
+            if (a.hand_on || (half > kLevelMargin && n - (ti + 2) * (u32)T < half - kLevelMargin)) sm.ti_end = ti + 2;
             sm.look = ti + look_after(ntiles - ti);
           }
           if ((ti & 31u) == 31u) tile_progress(a, 1ull << 32);  // whoever waits sees that streams get on

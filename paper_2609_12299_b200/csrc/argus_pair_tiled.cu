@@ -84,20 +84,28 @@ __device__ __forceinline__ u32 tile_claim_any(ArgusPairCtl* ctl, int p) {
 // 1,776 taken as they come, 42 SMs had seven of them each, the others none, and walked 791 tiles instead of 700: GEMM trace 545 -> 633 us; the
 // first positions taken seven strata apart, whoever comes: 633, too). But a CTA may start late, when another kernel holds part of the
 // chip, and nothing may wait for one that has not started: so the first position is claimed by a bit, and a CTA that would wait for
-// a hand-over while not all are claimed takes one that is left instead. *drawn: a position that the CTA has, but has not used yet.
-// One thread per CTA.
-__device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64* drawn, u64* stream, u32* rec, bool* resumed, bool* more) {
+// a hand-over while not all are claimed takes one that is left instead. *drawn: a position that the CTA has, but has not used yet;
+// first_stream: what lies at its own number. Whatever does not depend on one another is asked for together: a round trip is 0.7 us of
+// the smallest call. One thread per CTA.
+__device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64* drawn, u64 first_stream, u64* stream, u32* rec, bool* resumed, bool* more) {
   u64 h = *drawn;
+  const bool first = h < a.num_streams;
+  u32 words = 0;
+  u64 tail = 0;
+  if (!first) {
+    words = atomicAdd(&a.ctl->claimed_words[p], 0u);
+    tail = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull);
+  }
   if (h == kNoWork) h = gridDim.x + atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_head[p]), 1ull);
   *drawn = kNoWork;
   *resumed = h >= a.num_streams;
   if (h < a.num_streams) {
-    *stream = a.order ? a.order[h] : h;
+    *stream = first ? first_stream : a.order ? a.order[h] : h;
     *rec = h < a.record_capacity ? (u32)h : kNoRec;  // (streams come longest first; those without a record are walked whole)
-    *more = h + 1 < a.num_streams || atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull);
+    *more = h + 1 < a.num_streams || (first ? atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull) : tail);
     return true;
   }
-  if (atomicAdd(&a.ctl->claimed_words[p], 0u) < (gridDim.x + 31) / 32) {
+  if (words < (gridDim.x + 31) / 32) {
     const u32 left = tile_claim_any(a.ctl, p);
     if (left != kNoRec) {
       *drawn = h;
@@ -111,13 +119,16 @@ __device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64
   const u64 slot = h - a.num_streams;
   if (!a.queue || slot >= a.queue_capacity) return false;  // more positions than hand-overs can ever be published
   volatile u32* q = a.queue + slot;
-  *more = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->q_tail[p]), 0ull) > slot + 1;
+  *more = tail > slot + 1;
   u64 seen = ~0ull;
   u32 idle = 0, nap = 64;
   for (;;) {
-    const u64 now = atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctl->progress[p]), 0ull);
+    // An entry that was stored before the counter moved has to be seen, since it is not looked for again until the counter moves. (Acquired by the read
+    // itself: a fence in every round, by all who wait, took 10 K markers 41.3 -> 41.0 us, ring of 74 M 1,521 -> 1,512.)
+    u64 now;
+    asm volatile("atom.acquire.gpu.global.add.u64 %0, [%1], 0;" : "=l"(now) : "l"(&a.ctl->progress[p]) : "memory");
     if (now != seen) {
-      __threadfence();  // an entry that was stored before the counter moved is seen; it is not looked for again until the counter moves
+      if ((u32)now >= a.num_streams) return false;
       const u32 v = *q;
       if (v) {
         *q = 0;  // the second pass uses the same entries
@@ -126,7 +137,6 @@ __device__ __forceinline__ bool tile_pop_work(const ArgusPairArgs& a, int p, u64
         *stream = *reinterpret_cast<volatile u32*>(&a.records[v - 1].stream);
         return true;
       }
-      if ((u32)now >= a.num_streams) return false;
       if (seen == ~0ull) atomicExch(&a.ctl->level[p], 0u);
       seen = now;
       idle = 0;
@@ -175,7 +185,7 @@ struct TileSmem {
   int resumed;                     // its state is in the record
   int more, level;                 // others wait; and this CTA says how long they are
   int started;                     // this CTA has had work
-  u64 drawn;                       // a position that it has and has not used yet
+  u64 drawn, first_stream;         // a position that it has and has not used yet; the stream at its own number
   u32 ti_end, look;                // where this CTA stops; the tile at which thread 0 looks up what waits
   int stop;                        // split pass: everything is left to the chained pass
   u64 n_int;                       // written by the sequential redo path
@@ -265,7 +275,10 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
   bool failed = false;
   const bool segments = !SPLIT && !a.redo && a.segments && argus_split_in_force(a, &failed);  // the chained pass after a split one
   if (segments && !failed) return;
-  if (!SPLIT && tid == 32) sm.drawn = tile_claim(a.ctl, a.redo ? 1 : 0, blockIdx.x) ? blockIdx.x : kNoWork;  // (beside what thread 0 does)
+  if (!SPLIT && tid == 32) {  // (beside what thread 0 does)
+    sm.first_stream = a.order ? a.order[blockIdx.x] : blockIdx.x;
+    sm.drawn = tile_claim(a.ctl, a.redo ? 1 : 0, blockIdx.x) ? blockIdx.x : kNoWork;
+  }
   if (tid == 0) {
     mbar_init(&sm.bar[0], 1);
     mbar_init(&sm.bar[1], 1);
@@ -292,7 +305,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pair_tiled(ArgusPairArgs a) {
         rc = atomicAdd(&a.ctl->seg_head, 1u);
         st = w.z && rc < w.y ? a.segments[rc].stream : ~0ull;
         skip = w.x && st < a.num_streams && __ldcg(a.split_failed + st);
-      } else if (!tile_pop_work(a, a.redo ? 1 : 0, &sm.drawn, &st, &rc, &resumed, &more)) st = ~0ull;
+      } else if (!tile_pop_work(a, a.redo ? 1 : 0, &sm.drawn, sm.first_stream, &st, &rc, &resumed, &more)) st = ~0ull;
       sm.cur_stream = st;
       sm.cur_rec = rc;
       if (!SPLIT) {

@@ -53,6 +53,8 @@ int argus_profile_read(double* ms_total /*host [4]*/, unsigned long long* launch
  * have left; 0 = the default. Results do not depend on it.
  * argus_testing_hand_overs: after a pairing call (or argus_synthesize) in this workspace is complete, how many times its two
  * passes handed a stream on. Waits for the device.
+ * argus_testing_limit_requests: how many times since the library was loaded a launch needed more shared memory than a kernel gets without
+ * asking, and asked for it.
  * argus_testing_hold_sms: a kernel on the stream that holds this many SMs (148 at most; 200 KB of shared memory each, so that no block of the
  * pairing kernel fits beside it) for this many microseconds (a second at most), and then ends by itself: what another stream's long
  * kernel does to a call. */
@@ -63,6 +65,7 @@ int argus_testing_pair_passes(const void* workspace /*device*/, uint32_t* counte
 int argus_testing_record_blocks(uint32_t num_regions, uint32_t threads, uint32_t* by_rule /*host*/, uint32_t* by_device /*host*/);
 void argus_testing_set_hand_overs(int always);
 int argus_testing_hand_overs(const void* workspace /*device*/, uint64_t* first_pass /*host*/, uint64_t* second_pass /*host*/);
+unsigned long long argus_testing_limit_requests(void);
 int argus_testing_hold_sms(unsigned int sms, unsigned int microseconds, void* cuda_stream);
 
 #ifdef __cplusplus

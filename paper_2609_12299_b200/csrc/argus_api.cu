@@ -7,6 +7,7 @@
 
 namespace {
 std::atomic<unsigned long long> g_launches{0};
+std::atomic<unsigned long long> g_limit_requests{0};
 std::atomic<int> g_prof_on{0};
 thread_local int g_prof_suppress = 0;  // per host thread: a call that must not create events does not silence others
 std::mutex g_prof_mu;
@@ -66,6 +67,10 @@ void argus_prof_mark(int slot, cudaStream_t stream, int end) {
 void argus_prof_suppress(int delta) { g_prof_suppress += delta; }
 
 extern "C" unsigned long long argus_launch_count(void) { return g_launches.load(); }
+
+void argus_count_limit_request() { g_limit_requests.fetch_add(1, std::memory_order_relaxed); }
+
+extern "C" unsigned long long argus_testing_limit_requests(void) { return g_limit_requests.load(); }
 
 extern "C" void argus_profile_enable(int on) { g_prof_on.store(on ? 1 : 0); }
 

@@ -26,6 +26,7 @@ static_assert(sizeof(argus_status_t) == 64, "status layout");
 
 // host-side bookkeeping implemented in argus_api.cu
 void argus_count_launch();                                      // one more kernel launched by this library
+void argus_count_limit_request();                               // one more call that needed argus_allow_smem
 void argus_prof_mark(int slot, cudaStream_t stream, int end);   // CUDA events around a dominant kernel (if enabled)
 void argus_prof_suppress(int delta);                            // +1 / -1: event recording off while > 0 (it creates events)
 enum { ARGUS_PROF_PAIR = 0, ARGUS_PROF_AGGREGATE = 1, ARGUS_PROF_OVERLAP = 2, ARGUS_PROF_SLOTS = 4 };
@@ -57,6 +58,7 @@ constexpr size_t kPlainDynamicSmem = 43 * 1024;
 template <class K>
 inline cudaError_t argus_allow_smem(K* kernel, size_t dynamic, size_t most) {
   if (dynamic <= kPlainDynamicSmem) return cudaSuccess;
+  argus_count_limit_request();
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 

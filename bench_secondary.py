@@ -76,7 +76,7 @@ def run_scoped(iters: int):
          lambda: argus.argus_aggregate_scoped(*args, argus.ArgusScope(lo, lo + 15, 0b100011, None,
                                                                       argus.ArgusScope.bitmask(range(4), R, dev)),
                                               levels=("kernel", "role", "iter")), 3.0 / 16.0),
-        ("argus_aggregate_scoped, 16 iterations of all regions, + role and iteration tables (iteration table by global atomics)",
+        ("argus_aggregate_scoped, 16 iterations of all regions, + role and iteration tables",
          lambda: argus.argus_aggregate_scoped(*args, argus.ArgusScope(lo, lo + 15),
                                               levels=("warp", "cta", "sm", "kernel", "role", "iter")), 1.0),
         ("argus_overlap_scoped, 16 iterations", lambda: argus.argus_overlap_scoped(p.intervals, n // 2, p.interval_offsets, W,
